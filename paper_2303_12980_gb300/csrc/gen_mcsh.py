@@ -30,8 +30,10 @@ from __future__ import annotations
 
 import math
 import os
+import struct
 import sys
 from collections import defaultdict
+from fractions import Fraction
 
 LMAX = 6
 
@@ -261,48 +263,153 @@ def emit_eval_top(L):
     return "\n".join(lines)
 
 
-def emit_eval_df(L):
-    """The same recurrences in double-float arithmetic (gmp_f2, FP32 pairs):
-    products of a coordinate and a lower component, integer coefficients
-    applied exactly enough by gmp_df_mul_f, sums by gmp_df_add."""
-    name = f"gmp_mcsh_indep_df_{L}"
-    lines = [f"__device__ __forceinline__ void {name}(gmp_f2 x, gmp_f2 y, gmp_f2 z, gmp_f2 r2, gmp_f2* __restrict__ S) {{"]
-    for l in range(L + 1):
-        for t in indep_components(l):
-            k = flat(t)
-            rec = recurrence_terms(t)
-            if rec[0][1] == "1":
-                lines.append(f"  S[{k}] = gmp_f2{{1.0f, 0.0f}};")
-                continue
-            expr = None
-            for coef, kind, src in rec:
-                v = "r2" if kind == "r2" else kind
-                prod = f"gmp_df_mul({v}, S[{flat(src)}])"
-                term = prod if coef == 1 else f"gmp_df_mul_f({prod}, {fnum(coef)})"
-                expr = term if expr is None else f"gmp_df_add({term}, {expr})"
-            lines.append(f"  S[{k}] = {expr};")
-    lines.append("}")
-    return "\n".join(lines)
+# --------------------------------------------- real solid harmonics (refinement)
+def solid_harmonics(l):
+    """The 2l+1 real solid harmonics of order l as (m, part, integer
+    polynomial, coefficients of its z, r^2 factor, scale): factor(z, r^2)
+    times Re (part 0) or Im (part 1) of (x + iy)^m.  The factor is r^(l-m)
+    times the m-th derivative of the Legendre polynomial P_l at z/r,
+      2^-l sum_k (-1)^k C(l,k) C(2l-2k,l) (l-2k)!/(l-2k-m)! z^(l-m-2k) r^(2k),
+    divided by `scale`, the common factor of its coefficients."""
+    out = []
+    xy = [({(0, 0, 0): 1}, {})]
+    for m in range(l):
+        a, b = xy[-1]
+        xy.append((padd((1, pmul(a, {(1, 0, 0): 1})), (-1, pmul(b, {(0, 1, 0): 1}))),
+                   padd((1, pmul(b, {(1, 0, 0): 1})), (1, pmul(a, {(0, 1, 0): 1})))))
+    for m in range(l + 1):
+        n = l - m
+        c = [(-1) ** k * math.comb(l, k) * math.comb(2 * l - 2 * k, l) * math.factorial(l - 2 * k)
+             // math.factorial(l - 2 * k - m) for k in range(n // 2 + 1)]
+        g = math.gcd(*c)
+        c = [v // g for v in c]
+        p = {}
+        for k, v in enumerate(c):
+            p = padd((1, p), (v, pmul_mono(ppow_r2(k), (0, 0, n - 2 * k))))
+        for part in range(1 if m == 0 else 2):
+            out.append((m, part, pmul(p, xy[m][part]), c, Fraction(g, 2 ** l)))
+    return out
 
 
-def emit_feature_df(l):
-    """f = sum_all w mu_all^2 from the 2l+1 independent moments, double-float."""
-    T_ = reconstruction(l)
+def solid_norms(l):
+    """n_j with sum_c l!/(a!b!c!) S_c(u) S_c(v) = sum_j n_j H_j(u) H_j(v): both
+    sides are l! (2l-1)!! (uv)^l P_l(cos), by the sum rule of the S_c and the
+    addition theorem of the harmonics (factor 2 and (l-m)!/(l+m)! for m > 0)."""
+    return [math.factorial(l) * dfact(2 * l - 1) * (2 if m else 1) * Fraction(math.factorial(l - m), math.factorial(l + m))
+            * sc * sc for m, _, _, _, sc in solid_harmonics(l)]
 
-    def combo_expr(combo):
+
+def solid_to_indep(l):
+    """Rows {j: coefficient}: each independent component S_c of order l as a
+    combination of the solid harmonics (a harmonic polynomial is fixed by its
+    coefficients of the monomials with at most one x)."""
+    H = [h[2] for h in solid_harmonics(l)]
+    monos = [t for t in indep_components(l)]
+    A = [[Fraction(h.get(mo, 0)) for h in H] for mo in monos]
+    rows = []
+    for t in indep_components(l):
+        p = closed_form(*t)
+        M = [r[:] + [Fraction(p.get(mo, 0))] for r, mo in zip(A, monos)]
+        n = len(M)
+        for i in range(n):
+            piv = next(r for r in range(i, n) if M[r][i])
+            M[i], M[piv] = M[piv], M[i]
+            M[i] = [v / M[i][i] for v in M[i]]
+            for r in range(n):
+                if r != i and M[r][i]:
+                    f = M[r][i]
+                    M[r] = [v - f * w for v, w in zip(M[r], M[i])]
+        rows.append({j: M[j][n] for j in range(n) if M[j][n]})
+    return rows
+
+
+def check_solid():
+    for l in range(LMAX + 1):
+        H, N, T = solid_harmonics(l), solid_norms(l), solid_to_indep(l)
+        for t, row in zip(indep_components(l), T):
+            got = padd(*[(v, H[j][2]) for j, v in row.items()])
+            assert got == closed_form(*t), t
+        # sum_c w_c S_c S_c == sum_j n_j H_j H_j, with S_c from the rows: as
+        # quadratic forms in the H_j
+        Q = defaultdict(Fraction)
+        full = reconstruction(l)
+        for t in all_components(l):
+            row = defaultdict(Fraction)
+            for k, v in full[t].items():
+                for j, u in T[k].items():
+                    row[j] += v * u
+            for i, u in row.items():
+                for j, v in row.items():
+                    Q[i, j] += weight(*t) * u * v
+        for i in range(2 * l + 1):
+            for j in range(2 * l + 1):
+                assert Q[i, j] == (N[i] if i == j else 0), (l, i, j)
+
+
+def emit_solid_df(l):
+    """The solid harmonics of order l in double-float arithmetic."""
+    L = [f"__device__ __forceinline__ void gmp_solid_df_{l}(gmp_f2 x, gmp_f2 y, gmp_f2 z, gmp_f2 r2, gmp_f2* __restrict__ H) {{"]
+    if l == 0:
+        return "\n".join(L + ["  H[0] = gmp_f2{1.0f, 0.0f};", "}"])
+    if l >= 2:
+        L.append("  const gmp_f2 z2 = gmp_df_mul(z, z);")
+    for k in range(2, l // 2 + 1):
+        L.append(f"  const gmp_f2 r2_{k} = gmp_df_mul(r2, {'r2' if k == 2 else f'r2_{k - 1}'});")
+    rk = lambda k: "r2" if k == 1 else f"r2_{k}"
+    times = lambda v, e: e if v == 1 else f"gmp_df_mul_f({e}, {fnum(v)})"
+    L.append("  gmp_f2 a = x, b = y;")
+    j = 0
+    for m, part, _, c, _ in solid_harmonics(l):
+        if part:
+            continue
+        if m > 1:
+            L.append("  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul(x, a), gmp_df_neg(gmp_df_mul(y, b)));")
+            L.append("    b = gmp_df_add_sloppy(gmp_df_mul(x, b), gmp_df_mul(y, a));")
+            L.append("    a = t; }")
         e = None
-        for k, v in sorted(combo.items()):
-            term = f"mu[{k}]" if v == 1 else f"gmp_df_mul_f(mu[{k}], {fnum(v)})"
-            e = term if e is None else f"gmp_df_add({term}, {e})"
-        return e
+        for k, v in enumerate(c[1:], 1):
+            lead = times(c[0], "z2") if k == 1 else f"gmp_df_mul({e}, z2)"
+            e = f"gmp_df_add_sloppy({lead}, {times(v, rk(k))})"
+        if (l - m) % 2:
+            e = "z" if e is None else f"gmp_df_mul({e}, z)"
+        if m == 0:
+            L.append(f"  H[0] = {e};")
+            j = 1
+            continue
+        if e is None:
+            L.append(f"  H[{j}] = a; H[{j + 1}] = b;")
+        else:
+            L.append(f"  {{ const gmp_f2 q = {e}; H[{j}] = gmp_df_mul(q, a); H[{j + 1}] = gmp_df_mul(q, b); }}")
+        j += 2
+    L.append("}")
+    return "\n".join(L)
 
-    lines = [f"__device__ __forceinline__ gmp_f2 gmp_mcsh_invariant_df_{l}(const gmp_f2* __restrict__ mu) {{",
-             "  gmp_f2 f{0.0f, 0.0f};"]
-    for t in all_components(l):
-        lines.append(f"  {{ const gmp_f2 m = {combo_expr(T_[t])}; "
-                     f"f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, {fnum(weight(*t))}), m), f); }}")
-    lines += ["  return f;", "}"]
-    return "\n".join(lines)
+
+def f2(v):
+    """A rational as a double-float literal."""
+    hi = struct.unpack("f", struct.pack("f", float(v)))[0]
+    lo = struct.unpack("f", struct.pack("f", float(Fraction(v) - Fraction(hi))))[0]
+    return f"{{{hi!r}f, {lo!r}f}}"
+
+
+def emit_solid_tables():
+    """Per order: the norms of the harmonics, and the rows of the independent
+    components (padded to the longest with zero coefficients)."""
+    T = [solid_to_indep(l) for l in range(LMAX + 1)]
+    nz = max(len(r) for t in T for r in t)
+    out = [f"#define GMP_SOLID_NZ {nz}",
+           f"static __device__ const float2 gmp_solid_norm[{LMAX + 1}][{2 * LMAX + 1}] = {{"]
+    for l in range(LMAX + 1):
+        out.append("  {" + ", ".join(f2(v) for v in solid_norms(l)) + "},")
+    out += ["};", f"static __device__ const signed char gmp_solid_row[{LMAX + 1}][{2 * LMAX + 1}][{nz}] = {{"]
+    for t in T:
+        out.append("  {" + ", ".join("{" + ", ".join(str(j) for j in (sorted(r) + [0] * nz)[:nz]) + "}" for r in t) + "},")
+    out += ["};", f"static __device__ const float2 gmp_solid_coef[{LMAX + 1}][{2 * LMAX + 1}][{nz}] = {{"]
+    for t in T:
+        out.append("  {" + ", ".join("{" + ", ".join([f2(r[j]) for j in sorted(r)] + ["{0.0f, 0.0f}"] * (nz - len(r))) + "}"
+                                     for r in t) + "},")
+    out.append("};")
+    return "\n".join(out)
 
 
 def emit_feature(l, dtype="float"):
@@ -418,6 +525,7 @@ def generate() -> str:
     check_shift_identity()
     check_recurrences()
     check_reconstruction()
+    check_solid()
     out = [
         "// Generated by gen_mcsh.py -- do not edit.  MCSH angular probes (independent",
         "// components a <= 1 of each order), their gradients, and the per-order",
@@ -430,11 +538,11 @@ def generate() -> str:
         out.append(emit_eval_scaled(L))
     for L in range(1, LMAX + 2):
         out.append(emit_eval_top(L))
-    for L in range(LMAX + 1):
-        out.append(emit_eval_df(L))
+    for l in range(LMAX + 1):
+        out.append(emit_solid_df(l))
+    out.append(emit_solid_tables())
     for l in range(LMAX + 1):
         out.append(emit_feature(l))
-        out.append(emit_feature_df(l))
     for L in range(LMAX + 1):
         out.append(emit_shift_contract(L))
     for l in range(LMAX + 1):
@@ -461,17 +569,12 @@ def generate() -> str:
     for l in range(LMAX + 1):
         out.append(f"    case {l}: return gmp_mcsh_invariant_{l}(mu);")
     out.append("    default: return 0.0f;\n  }\n}")
-    out.append("__device__ __forceinline__ gmp_f2 gmp_mcsh_invariant_df(int l, const gmp_f2* mu) {")
-    out.append("  switch (l) {")
+    out.append("// solid harmonics of order l in double-float arithmetic")
+    out.append("template <int l>")
+    out.append("__device__ __forceinline__ void gmp_solid_df(gmp_f2 x, gmp_f2 y, gmp_f2 z, gmp_f2 r2, gmp_f2* H) {")
     for l in range(LMAX + 1):
-        out.append(f"    case {l}: return gmp_mcsh_invariant_df_{l}(mu);")
-    out.append("    default: return gmp_f2{0.0f, 0.0f};\n  }\n}")
-    out.append("// independent components of orders 0..l in double-float arithmetic (l <= L of the caller)")
-    out.append("__device__ __forceinline__ void gmp_mcsh_indep_df(int l, gmp_f2 x, gmp_f2 y, gmp_f2 z, gmp_f2 r2, gmp_f2* S) {")
-    out.append("  switch (l) {")
-    for l in range(LMAX + 1):
-        out.append(f"    case {l}: gmp_mcsh_indep_df_{l}(x, y, z, r2, S); break;")
-    out.append("    default: break;\n  }\n}")
+        out.append(f"  if constexpr (l == {l}) gmp_solid_df_{l}(x, y, z, r2, H);")
+    out.append("}")
     out.append("__device__ __forceinline__ void gmp_mcsh_shift_contract_order(int l, const float* lam, const float* S1, float* V) {")
     out.append("  switch (l) {")
     for l in range(LMAX + 1):

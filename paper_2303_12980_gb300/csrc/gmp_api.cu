@@ -524,11 +524,14 @@ constexpr float kFlagTau = 3e-4f;
 constexpr float kFlagLow = 1e-10f;
 
 // Refinement queues, one per requested order: a pass queues at most one
-// entry per (center, order), and a call refines after each pass (derivative
-// calls) or once after all of them (features), so a queue holds one entry
-// per center and pass.  The flag buffer holds 8 counts, then the queues.
+// entry per center and two sigmas, and a call refines after each pass
+// (derivative calls) or once after all of them (features), so a queue holds
+// one entry per center and two sigmas of every pass.  The flag buffer holds 8
+// counts, then the queues.
 int64_t flag_capacity(const gmp_ctx* h, int64_t N) {
-  return (int64_t)std::max<size_t>(h->passes.size(), 1) * N + 1024;
+  int64_t pairs = 0;
+  for (const PassData& pd : h->passes) pairs += (pd.pass.nsig + 1) / 2;
+  return std::max<int64_t>(pairs, 1) * N + 1024;
 }
 unsigned long long* flag_counter(gmp_ctx* h) { return h->flagq.as<unsigned long long>(); }
 unsigned long long* flag_queues(gmp_ctx* h) { return h->flagq.as<unsigned long long>() + 8; }
@@ -619,10 +622,7 @@ gmp_status refine(gmp_ctx* h, int64_t N, float* features, cudaStream_t st, const
   A.mu_sig0 = mt.sig0;
   A.mu_nsig = mt.nsig;
   A.mu_nind = mt.nind;
-  unsigned order_mask = 0;
-  for (int l : h->orders)
-    if (l >= 0) order_mask |= 1u << l;
-  GMP_CK(gmp_launch_refine(A, order_mask, h->sm_count, st, &h->launches), "refine");
+  GMP_CK(gmp_launch_refine(A, h->sm_count, st, &h->launches), "refine");
   return GMP_OK;
 }
 

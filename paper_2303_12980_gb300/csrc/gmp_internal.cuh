@@ -149,9 +149,9 @@ __device__ __forceinline__ gmp_f2 gmp_df_mul_f(gmp_f2 a, float b) {
   float e = __fmaf_rn(a.lo, b, p.lo);
   return gmp_fast_two_sum(p.hi, e);
 }
-// Addition where |a| >= |b| is not required but the result's low word is
-// the plain sum of the rounding errors (one renormalisation): enough for a
-// Horner step whose terms decrease.
+// Addition with one renormalisation: the low words are added in FP32, an
+// error of 2^-48 of the larger operand (not of a cancelling result).  For
+// sums whose accuracy counts against the size of their terms.
 __device__ __forceinline__ gmp_f2 gmp_df_add_sloppy(gmp_f2 a, gmp_f2 b) {
   gmp_f2 s = gmp_two_sum(a.hi, b.hi);
   return gmp_fast_two_sum(s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo)));
@@ -243,33 +243,41 @@ __device__ __forceinline__ float gmp_exp_neg_shifted(float Bhi, float Blo, float
   return gmp_exp_neg_shifted_by(Bhi, Blo, r2hi, r2lo, GMP_EXP_SHIFT);
 }
 
-// exp(-x) for a double-float x to about 1e-13 relative, in FP32
-// arithmetic, by table-driven reduction (Tang's method):
-// x = k ln2/64 + r with |r| <= ln2/128 (ln2/64 as a double-float), so that
-// exp(-x) = 2^-(k div 64) * 2^-((k mod 64)/64) * exp(-r); the middle factor
-// is a double-float table entry (tab[j] = 2^(-j/64)) and
-// exp(-r) = 1 - r + r^2 w, w = 1/2 + r t, t = -1/6 + r/24 - r^2/120, where
-// |r t| < 1e-3 lets t be FP32 (the omitted r^6/720 term is below 3e-17).
-// Results below the FP32 normal range (x > 87) are returned as 0.  A
-// negative x (down to about -88) works the same way: k and its shift by 6
-// are then negative, the table index k mod 64 stays in 0..63.
-__device__ __forceinline__ gmp_f2 gmp_df_exp_neg(gmp_f2 x, const float2* __restrict__ tab) {
+// exp(-x) for a double-float x to 3e-14 relative, in FP32 arithmetic, by
+// table-driven reduction (Tang's method): x = k ln2/64 + r with |r| <=
+// ln2/128, so that exp(-x) = 2^-(k div 64) * 2^-((k mod 64)/64) * exp(-r);
+// the middle factor is a double-float table entry (tab[j] = 2^(-j/64)).
+// ln2/64 is taken as C1 + C2 + C3 (Cody and Waite): C1 has 11 significant
+// bits, so k C1 and x.hi - k C1 are exact (k < 2^13), k C2 is an exact
+// product and k C3 < 3e-10.  exp(-r) = 1 - r + r^2/2 + r^3 t, t = -1/6 + r/24
+// - r^2/120, with r^2/2 as an exact product; |r^3 t| < 3e-8 lets t be FP32
+// (the omitted r^6/720 term is below 4e-17).  Results below the FP32
+// normal range (x > 87) are returned as 0.  A negative x (down to about -88)
+// works the same way: k and its shift by 6 are then negative, the table
+// index k mod 64 stays in 0..63.  About 45 instructions, against 130 for
+// the same steps in general double-float operations (2.2e-13).
+__device__ __forceinline__ gmp_f2 gmp_df_exp_neg(gmp_f2 x, const float2* tab) {
   if (!(x.hi <= 87.0f)) return gmp_f2{0.0f, 0.0f};
-  const float C_HI = 0.010830424726009369f, C_LO = -2.976022206446771e-11f;  // ln2/64
-  const float k = rintf(__fmul_rn(x.hi, 92.33248261689366f));                  // x * 64/ln2
-  const gmp_f2 kc = gmp_df_add(gmp_two_prod(k, C_HI), gmp_two_prod(k, C_LO));
-  const gmp_f2 r = gmp_df_add(x, gmp_df_neg(kc));
+  const float C1 = 0.010833740234375f, C2 = -3.3155381515825866e-06f, C3 = 2.5728046402313451e-14f;
+  const float k = rintf(__fmul_rn(x.hi, 92.33248261689366f));  // x * 64/ln2
+  const gmp_f2 p = gmp_two_prod(k, C2);
+  gmp_f2 r = gmp_two_sum(__fmaf_rn(-k, C1, x.hi), -p.hi);
+  const gmp_f2 u = gmp_two_sum(x.lo, r.lo);
+  r = gmp_two_sum(r.hi, u.hi);
+  r.lo = __fadd_rn(r.lo, __fsub_rn(u.lo, __fmaf_rn(k, C3, p.lo)));
   const float t = __fmaf_rn(r.hi, __fmaf_rn(r.hi, -0.008333333767950535f, 0.0416666679084301f),
                             -0.1666666716337204f);
-  const gmp_f2 rt = gmp_two_prod(r.hi, t);
-  gmp_f2 w = gmp_fast_two_sum(0.5f, rt.hi);
-  w = gmp_fast_two_sum(w.hi, __fadd_rn(w.lo, rt.lo));
-  const gmp_f2 q = gmp_df_mul(gmp_df_mul(r, r), w);
-  gmp_f2 e = gmp_df_add(gmp_df_add(gmp_f2{1.0f, 0.0f}, gmp_df_neg(r)), q);
+  const gmp_f2 q = gmp_two_prod(r.hi, __fmul_rn(0.5f, r.hi));
+  const float ql = __fmaf_rn(__fmul_rn(r.hi, t), __fmul_rn(2.0f, q.hi), __fmaf_rn(r.hi, r.lo, q.lo));
+  const gmp_f2 y = gmp_fast_two_sum(-r.hi, q.hi);  // exp(-r) - 1 = y.hi + yl
+  const float yl = __fadd_rn(y.lo, __fsub_rn(ql, r.lo));
   const int ki = (int)k;
-  const float2 T = __ldg(tab + (ki & 63));
-  e = gmp_df_mul(e, gmp_f2{T.x, T.y});
-  return gmp_f2{ldexpf(e.hi, -(ki >> 6)), ldexpf(e.lo, -(ki >> 6))};
+  const float2 T = tab[ki & 63];
+  const gmp_f2 v = gmp_two_prod(T.x, y.hi);
+  const float vl = __fmaf_rn(T.x, yl, __fmaf_rn(T.y, y.hi, v.lo));
+  const gmp_f2 e = gmp_fast_two_sum(T.x, v.hi);
+  const float scale = __int_as_float((127 - (ki >> 6)) << 23);
+  return gmp_f2{__fmul_rn(e.hi, scale), __fmul_rn(__fadd_rn(e.lo, __fadd_rn(T.y, vl)), scale)};
 }
 
 // Double-float displacement of j's image n from i, and its r^2.
@@ -386,8 +394,8 @@ cudaError_t gmp_launch_virial_reduce(int n_struct, const int64_t* atom_off, cons
 // Double-float recomputation of the flagged features: one queue per
 // order slot o (queue + o * cap, count[o] entries, at most cap; qidx[l] is
 // the slot of order l, -1 when l is not requested), entries center << 32 |
-// first column of the order << 16 | mask of its flagged sigmas;
-// col_info[col] = (order << 16) | sigma.  With mu_out, the
+// column of the first of two sigmas << 16 | mask of the flagged ones of the
+// two; col_info[col] = (order << 16) | sigma.  With mu_out, the
 // recomputed moments of sigmas mu_sig0 .. mu_sig0 + mu_nsig - 1 also
 // overwrite mu_out[center][sigma - mu_sig0][l^2 .. l^2 + 2l] (row length
 // mu_nind), the moments a derivative kernel reads next.
@@ -416,9 +424,8 @@ struct GmpRefine {
   float* mu_out;
   int mu_sig0, mu_nsig, mu_nind;
 };
-// One launch per order set in order_mask (bit l: order l >= 0 requested).
-cudaError_t gmp_launch_refine(const GmpRefine& args, unsigned order_mask, int sm_count, cudaStream_t stream,
-                              int64_t* launches);
+// One launch for all orders.
+cudaError_t gmp_launch_refine(const GmpRefine& args, int sm_count, cudaStream_t stream, int64_t* launches);
 cudaError_t gmp_launch_unpack_neighbors(int64_t P, const GmpPair* pairs, int32_t* nbr_j,
                                         int32_t* nbr_shift, cudaStream_t stream,
                                         int64_t* launches);

@@ -194,10 +194,10 @@ struct KParams {
   const int32_t* center_struct;  // [N] structure of each center (virial)
   double* virial;                // [S, 3, 3] strain derivative accumulators (virial)
   // features too ill-conditioned for FP32 (recomputed in double-float
-  // afterwards): one queue entry per (center, order) of the pass,
-  // center << 32 | first column of the order << 16 | mask of the sigmas,
-  // in the queue of the order's slot o (flags + o * flag_cap, count
-  // flag_count[o])
+  // afterwards): one queue entry per (center, order, pair of sigmas 2b, 2b+1)
+  // of the pass, center << 32 | column of the first sigma << 16 | mask of the
+  // flagged ones, in the queue of the order's slot o (flags + o * flag_cap,
+  // count flag_count[o])
   unsigned long long* flags;
   unsigned long long* flag_count;
   int64_t flag_cap;
@@ -873,15 +873,19 @@ __device__ __forceinline__ void write_features(const KParams& K, int64_t i, cons
       if (lane == oo) omask |= m;
     }
   }
-  // one entry per (center, order) with flagged sigmas, in the order's own
-  // queue: center << 32 | first column of the order << 16 | sigma mask.  A
-  // pass has at most one entry per (center, order), and a queue holds that
-  // many.
+  // one entry per pair of sigmas with a flagged one, in the order's own
+  // queue (center << 32 | column of the pair << 16 | mask): the refinement
+  // shares the pair terms of the two, and every entry is work of one size.
+  // A queue holds every pair of every center.
   if (lane < P.n_ord && omask) {
-    const unsigned long long slot = atomicAdd(K.flag_count + lane, 1ull);
-    if (slot < (unsigned long long)K.flag_cap)
-      K.flags[lane * K.flag_cap + slot] =
-          ((unsigned long long)i << 32) | ((unsigned long long)P.ord_col[lane] << 16) | omask;
+    unsigned heads = (omask | (omask >> 1)) & 0x5555u;
+    unsigned long long slot = atomicAdd(K.flag_count + lane, (unsigned long long)__popc(heads));
+    for (; heads; heads &= heads - 1, ++slot) {
+      const int b = __ffs(heads) - 1;
+      if (slot < (unsigned long long)K.flag_cap)
+        K.flags[lane * K.flag_cap + slot] = ((unsigned long long)i << 32) |
+                                            ((unsigned long long)(P.ord_col[lane] + b) << 16) | ((omask >> b) & 3u);
+    }
   }
   if (P.want_density && lane == 0) frow[P.dens_col] = rho;
 }

@@ -526,160 +526,136 @@ __device__ __forceinline__ void gmp_mcsh_top_7(float x, float y, float z, float 
   S[62] = __fmaf_rn(r2_m20, S[34], __fmaf_rn(z_10, S[47], __fmaf_rn(y_2, S[48], __fmul_rn(x, S[41]))));
   S[63] = __fmaf_rn(r2_m30, S[35], __fmaf_rn(z_12, S[48], __fmul_rn(x, S[42])));
 }
-__device__ __forceinline__ void gmp_mcsh_indep_df_0(gmp_f2 x, gmp_f2 y, gmp_f2 z, gmp_f2 r2, gmp_f2* __restrict__ S) {
-  S[0] = gmp_f2{1.0f, 0.0f};
+__device__ __forceinline__ void gmp_solid_df_0(gmp_f2 x, gmp_f2 y, gmp_f2 z, gmp_f2 r2, gmp_f2* __restrict__ H) {
+  H[0] = gmp_f2{1.0f, 0.0f};
 }
-__device__ __forceinline__ void gmp_mcsh_indep_df_1(gmp_f2 x, gmp_f2 y, gmp_f2 z, gmp_f2 r2, gmp_f2* __restrict__ S) {
-  S[0] = gmp_f2{1.0f, 0.0f};
-  S[1] = gmp_df_mul(y, S[0]);
-  S[2] = gmp_df_mul(z, S[0]);
-  S[3] = gmp_df_mul(x, S[0]);
+__device__ __forceinline__ void gmp_solid_df_1(gmp_f2 x, gmp_f2 y, gmp_f2 z, gmp_f2 r2, gmp_f2* __restrict__ H) {
+  gmp_f2 a = x, b = y;
+  H[0] = z;
+  H[1] = a; H[2] = b;
 }
-__device__ __forceinline__ void gmp_mcsh_indep_df_2(gmp_f2 x, gmp_f2 y, gmp_f2 z, gmp_f2 r2, gmp_f2* __restrict__ S) {
-  S[0] = gmp_f2{1.0f, 0.0f};
-  S[1] = gmp_df_mul(y, S[0]);
-  S[2] = gmp_df_mul(z, S[0]);
-  S[3] = gmp_df_mul(x, S[0]);
-  S[4] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[0]), -1.0f), gmp_df_mul_f(gmp_df_mul(y, S[1]), 3.0f));
-  S[5] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[1]), 2.0f), gmp_df_mul(y, S[2]));
-  S[6] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[0]), -1.0f), gmp_df_mul_f(gmp_df_mul(z, S[2]), 3.0f));
-  S[7] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(y, S[3]), 2.0f), gmp_df_mul(x, S[1]));
-  S[8] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[3]), 2.0f), gmp_df_mul(x, S[2]));
+__device__ __forceinline__ void gmp_solid_df_2(gmp_f2 x, gmp_f2 y, gmp_f2 z, gmp_f2 r2, gmp_f2* __restrict__ H) {
+  const gmp_f2 z2 = gmp_df_mul(z, z);
+  gmp_f2 a = x, b = y;
+  H[0] = gmp_df_add_sloppy(gmp_df_mul_f(z2, 3.0f), gmp_df_mul_f(r2, -1.0f));
+  { const gmp_f2 q = z; H[1] = gmp_df_mul(q, a); H[2] = gmp_df_mul(q, b); }
+  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul(x, a), gmp_df_neg(gmp_df_mul(y, b)));
+    b = gmp_df_add_sloppy(gmp_df_mul(x, b), gmp_df_mul(y, a));
+    a = t; }
+  H[3] = a; H[4] = b;
 }
-__device__ __forceinline__ void gmp_mcsh_indep_df_3(gmp_f2 x, gmp_f2 y, gmp_f2 z, gmp_f2 r2, gmp_f2* __restrict__ S) {
-  S[0] = gmp_f2{1.0f, 0.0f};
-  S[1] = gmp_df_mul(y, S[0]);
-  S[2] = gmp_df_mul(z, S[0]);
-  S[3] = gmp_df_mul(x, S[0]);
-  S[4] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[0]), -1.0f), gmp_df_mul_f(gmp_df_mul(y, S[1]), 3.0f));
-  S[5] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[1]), 2.0f), gmp_df_mul(y, S[2]));
-  S[6] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[0]), -1.0f), gmp_df_mul_f(gmp_df_mul(z, S[2]), 3.0f));
-  S[7] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(y, S[3]), 2.0f), gmp_df_mul(x, S[1]));
-  S[8] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[3]), 2.0f), gmp_df_mul(x, S[2]));
-  S[9] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[1]), -4.0f), gmp_df_mul_f(gmp_df_mul(y, S[4]), 5.0f));
-  S[10] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[2]), -1.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[4]), 2.0f), gmp_df_mul_f(gmp_df_mul(y, S[5]), 3.0f)));
-  S[11] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[1]), -2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[5]), 4.0f), gmp_df_mul(y, S[6])));
-  S[12] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[2]), -4.0f), gmp_df_mul_f(gmp_df_mul(z, S[6]), 5.0f));
-  S[13] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[3]), -2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(y, S[7]), 4.0f), gmp_df_mul(x, S[4])));
-  S[14] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[7]), 2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(y, S[8]), 2.0f), gmp_df_mul(x, S[5])));
-  S[15] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[3]), -2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[8]), 4.0f), gmp_df_mul(x, S[6])));
+__device__ __forceinline__ void gmp_solid_df_3(gmp_f2 x, gmp_f2 y, gmp_f2 z, gmp_f2 r2, gmp_f2* __restrict__ H) {
+  const gmp_f2 z2 = gmp_df_mul(z, z);
+  gmp_f2 a = x, b = y;
+  H[0] = gmp_df_mul(gmp_df_add_sloppy(gmp_df_mul_f(z2, 5.0f), gmp_df_mul_f(r2, -3.0f)), z);
+  { const gmp_f2 q = gmp_df_add_sloppy(gmp_df_mul_f(z2, 5.0f), gmp_df_mul_f(r2, -1.0f)); H[1] = gmp_df_mul(q, a); H[2] = gmp_df_mul(q, b); }
+  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul(x, a), gmp_df_neg(gmp_df_mul(y, b)));
+    b = gmp_df_add_sloppy(gmp_df_mul(x, b), gmp_df_mul(y, a));
+    a = t; }
+  { const gmp_f2 q = z; H[3] = gmp_df_mul(q, a); H[4] = gmp_df_mul(q, b); }
+  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul(x, a), gmp_df_neg(gmp_df_mul(y, b)));
+    b = gmp_df_add_sloppy(gmp_df_mul(x, b), gmp_df_mul(y, a));
+    a = t; }
+  H[5] = a; H[6] = b;
 }
-__device__ __forceinline__ void gmp_mcsh_indep_df_4(gmp_f2 x, gmp_f2 y, gmp_f2 z, gmp_f2 r2, gmp_f2* __restrict__ S) {
-  S[0] = gmp_f2{1.0f, 0.0f};
-  S[1] = gmp_df_mul(y, S[0]);
-  S[2] = gmp_df_mul(z, S[0]);
-  S[3] = gmp_df_mul(x, S[0]);
-  S[4] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[0]), -1.0f), gmp_df_mul_f(gmp_df_mul(y, S[1]), 3.0f));
-  S[5] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[1]), 2.0f), gmp_df_mul(y, S[2]));
-  S[6] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[0]), -1.0f), gmp_df_mul_f(gmp_df_mul(z, S[2]), 3.0f));
-  S[7] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(y, S[3]), 2.0f), gmp_df_mul(x, S[1]));
-  S[8] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[3]), 2.0f), gmp_df_mul(x, S[2]));
-  S[9] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[1]), -4.0f), gmp_df_mul_f(gmp_df_mul(y, S[4]), 5.0f));
-  S[10] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[2]), -1.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[4]), 2.0f), gmp_df_mul_f(gmp_df_mul(y, S[5]), 3.0f)));
-  S[11] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[1]), -2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[5]), 4.0f), gmp_df_mul(y, S[6])));
-  S[12] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[2]), -4.0f), gmp_df_mul_f(gmp_df_mul(z, S[6]), 5.0f));
-  S[13] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[3]), -2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(y, S[7]), 4.0f), gmp_df_mul(x, S[4])));
-  S[14] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[7]), 2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(y, S[8]), 2.0f), gmp_df_mul(x, S[5])));
-  S[15] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[3]), -2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[8]), 4.0f), gmp_df_mul(x, S[6])));
-  S[16] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[4]), -9.0f), gmp_df_mul_f(gmp_df_mul(y, S[9]), 7.0f));
-  S[17] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[5]), -4.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[9]), 2.0f), gmp_df_mul_f(gmp_df_mul(y, S[10]), 5.0f)));
-  S[18] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[4]), -2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[6]), -1.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[10]), 4.0f), gmp_df_mul_f(gmp_df_mul(y, S[11]), 3.0f))));
-  S[19] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[5]), -6.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[11]), 6.0f), gmp_df_mul(y, S[12])));
-  S[20] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[6]), -9.0f), gmp_df_mul_f(gmp_df_mul(z, S[12]), 7.0f));
-  S[21] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[7]), -6.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(y, S[13]), 6.0f), gmp_df_mul(x, S[9])));
-  S[22] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[8]), -2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[13]), 2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(y, S[14]), 4.0f), gmp_df_mul(x, S[10]))));
-  S[23] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[7]), -2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[14]), 4.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(y, S[15]), 2.0f), gmp_df_mul(x, S[11]))));
-  S[24] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[8]), -6.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[15]), 6.0f), gmp_df_mul(x, S[12])));
+__device__ __forceinline__ void gmp_solid_df_4(gmp_f2 x, gmp_f2 y, gmp_f2 z, gmp_f2 r2, gmp_f2* __restrict__ H) {
+  const gmp_f2 z2 = gmp_df_mul(z, z);
+  const gmp_f2 r2_2 = gmp_df_mul(r2, r2);
+  gmp_f2 a = x, b = y;
+  H[0] = gmp_df_add_sloppy(gmp_df_mul(gmp_df_add_sloppy(gmp_df_mul_f(z2, 35.0f), gmp_df_mul_f(r2, -30.0f)), z2), gmp_df_mul_f(r2_2, 3.0f));
+  { const gmp_f2 q = gmp_df_mul(gmp_df_add_sloppy(gmp_df_mul_f(z2, 7.0f), gmp_df_mul_f(r2, -3.0f)), z); H[1] = gmp_df_mul(q, a); H[2] = gmp_df_mul(q, b); }
+  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul(x, a), gmp_df_neg(gmp_df_mul(y, b)));
+    b = gmp_df_add_sloppy(gmp_df_mul(x, b), gmp_df_mul(y, a));
+    a = t; }
+  { const gmp_f2 q = gmp_df_add_sloppy(gmp_df_mul_f(z2, 7.0f), gmp_df_mul_f(r2, -1.0f)); H[3] = gmp_df_mul(q, a); H[4] = gmp_df_mul(q, b); }
+  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul(x, a), gmp_df_neg(gmp_df_mul(y, b)));
+    b = gmp_df_add_sloppy(gmp_df_mul(x, b), gmp_df_mul(y, a));
+    a = t; }
+  { const gmp_f2 q = z; H[5] = gmp_df_mul(q, a); H[6] = gmp_df_mul(q, b); }
+  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul(x, a), gmp_df_neg(gmp_df_mul(y, b)));
+    b = gmp_df_add_sloppy(gmp_df_mul(x, b), gmp_df_mul(y, a));
+    a = t; }
+  H[7] = a; H[8] = b;
 }
-__device__ __forceinline__ void gmp_mcsh_indep_df_5(gmp_f2 x, gmp_f2 y, gmp_f2 z, gmp_f2 r2, gmp_f2* __restrict__ S) {
-  S[0] = gmp_f2{1.0f, 0.0f};
-  S[1] = gmp_df_mul(y, S[0]);
-  S[2] = gmp_df_mul(z, S[0]);
-  S[3] = gmp_df_mul(x, S[0]);
-  S[4] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[0]), -1.0f), gmp_df_mul_f(gmp_df_mul(y, S[1]), 3.0f));
-  S[5] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[1]), 2.0f), gmp_df_mul(y, S[2]));
-  S[6] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[0]), -1.0f), gmp_df_mul_f(gmp_df_mul(z, S[2]), 3.0f));
-  S[7] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(y, S[3]), 2.0f), gmp_df_mul(x, S[1]));
-  S[8] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[3]), 2.0f), gmp_df_mul(x, S[2]));
-  S[9] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[1]), -4.0f), gmp_df_mul_f(gmp_df_mul(y, S[4]), 5.0f));
-  S[10] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[2]), -1.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[4]), 2.0f), gmp_df_mul_f(gmp_df_mul(y, S[5]), 3.0f)));
-  S[11] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[1]), -2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[5]), 4.0f), gmp_df_mul(y, S[6])));
-  S[12] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[2]), -4.0f), gmp_df_mul_f(gmp_df_mul(z, S[6]), 5.0f));
-  S[13] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[3]), -2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(y, S[7]), 4.0f), gmp_df_mul(x, S[4])));
-  S[14] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[7]), 2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(y, S[8]), 2.0f), gmp_df_mul(x, S[5])));
-  S[15] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[3]), -2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[8]), 4.0f), gmp_df_mul(x, S[6])));
-  S[16] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[4]), -9.0f), gmp_df_mul_f(gmp_df_mul(y, S[9]), 7.0f));
-  S[17] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[5]), -4.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[9]), 2.0f), gmp_df_mul_f(gmp_df_mul(y, S[10]), 5.0f)));
-  S[18] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[4]), -2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[6]), -1.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[10]), 4.0f), gmp_df_mul_f(gmp_df_mul(y, S[11]), 3.0f))));
-  S[19] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[5]), -6.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[11]), 6.0f), gmp_df_mul(y, S[12])));
-  S[20] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[6]), -9.0f), gmp_df_mul_f(gmp_df_mul(z, S[12]), 7.0f));
-  S[21] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[7]), -6.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(y, S[13]), 6.0f), gmp_df_mul(x, S[9])));
-  S[22] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[8]), -2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[13]), 2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(y, S[14]), 4.0f), gmp_df_mul(x, S[10]))));
-  S[23] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[7]), -2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[14]), 4.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(y, S[15]), 2.0f), gmp_df_mul(x, S[11]))));
-  S[24] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[8]), -6.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[15]), 6.0f), gmp_df_mul(x, S[12])));
-  S[25] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[9]), -16.0f), gmp_df_mul_f(gmp_df_mul(y, S[16]), 9.0f));
-  S[26] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[10]), -9.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[16]), 2.0f), gmp_df_mul_f(gmp_df_mul(y, S[17]), 7.0f)));
-  S[27] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[9]), -2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[11]), -4.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[17]), 4.0f), gmp_df_mul_f(gmp_df_mul(y, S[18]), 5.0f))));
-  S[28] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[10]), -6.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[12]), -1.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[18]), 6.0f), gmp_df_mul_f(gmp_df_mul(y, S[19]), 3.0f))));
-  S[29] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[11]), -12.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[19]), 8.0f), gmp_df_mul(y, S[20])));
-  S[30] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[12]), -16.0f), gmp_df_mul_f(gmp_df_mul(z, S[20]), 9.0f));
-  S[31] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[13]), -12.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(y, S[21]), 8.0f), gmp_df_mul(x, S[16])));
-  S[32] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[14]), -6.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[21]), 2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(y, S[22]), 6.0f), gmp_df_mul(x, S[17]))));
-  S[33] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[13]), -2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[15]), -2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[22]), 4.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(y, S[23]), 4.0f), gmp_df_mul(x, S[18])))));
-  S[34] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[14]), -6.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[23]), 6.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(y, S[24]), 2.0f), gmp_df_mul(x, S[19]))));
-  S[35] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[15]), -12.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[24]), 8.0f), gmp_df_mul(x, S[20])));
+__device__ __forceinline__ void gmp_solid_df_5(gmp_f2 x, gmp_f2 y, gmp_f2 z, gmp_f2 r2, gmp_f2* __restrict__ H) {
+  const gmp_f2 z2 = gmp_df_mul(z, z);
+  const gmp_f2 r2_2 = gmp_df_mul(r2, r2);
+  gmp_f2 a = x, b = y;
+  H[0] = gmp_df_mul(gmp_df_add_sloppy(gmp_df_mul(gmp_df_add_sloppy(gmp_df_mul_f(z2, 63.0f), gmp_df_mul_f(r2, -70.0f)), z2), gmp_df_mul_f(r2_2, 15.0f)), z);
+  { const gmp_f2 q = gmp_df_add_sloppy(gmp_df_mul(gmp_df_add_sloppy(gmp_df_mul_f(z2, 21.0f), gmp_df_mul_f(r2, -14.0f)), z2), r2_2); H[1] = gmp_df_mul(q, a); H[2] = gmp_df_mul(q, b); }
+  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul(x, a), gmp_df_neg(gmp_df_mul(y, b)));
+    b = gmp_df_add_sloppy(gmp_df_mul(x, b), gmp_df_mul(y, a));
+    a = t; }
+  { const gmp_f2 q = gmp_df_mul(gmp_df_add_sloppy(gmp_df_mul_f(z2, 3.0f), gmp_df_mul_f(r2, -1.0f)), z); H[3] = gmp_df_mul(q, a); H[4] = gmp_df_mul(q, b); }
+  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul(x, a), gmp_df_neg(gmp_df_mul(y, b)));
+    b = gmp_df_add_sloppy(gmp_df_mul(x, b), gmp_df_mul(y, a));
+    a = t; }
+  { const gmp_f2 q = gmp_df_add_sloppy(gmp_df_mul_f(z2, 9.0f), gmp_df_mul_f(r2, -1.0f)); H[5] = gmp_df_mul(q, a); H[6] = gmp_df_mul(q, b); }
+  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul(x, a), gmp_df_neg(gmp_df_mul(y, b)));
+    b = gmp_df_add_sloppy(gmp_df_mul(x, b), gmp_df_mul(y, a));
+    a = t; }
+  { const gmp_f2 q = z; H[7] = gmp_df_mul(q, a); H[8] = gmp_df_mul(q, b); }
+  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul(x, a), gmp_df_neg(gmp_df_mul(y, b)));
+    b = gmp_df_add_sloppy(gmp_df_mul(x, b), gmp_df_mul(y, a));
+    a = t; }
+  H[9] = a; H[10] = b;
 }
-__device__ __forceinline__ void gmp_mcsh_indep_df_6(gmp_f2 x, gmp_f2 y, gmp_f2 z, gmp_f2 r2, gmp_f2* __restrict__ S) {
-  S[0] = gmp_f2{1.0f, 0.0f};
-  S[1] = gmp_df_mul(y, S[0]);
-  S[2] = gmp_df_mul(z, S[0]);
-  S[3] = gmp_df_mul(x, S[0]);
-  S[4] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[0]), -1.0f), gmp_df_mul_f(gmp_df_mul(y, S[1]), 3.0f));
-  S[5] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[1]), 2.0f), gmp_df_mul(y, S[2]));
-  S[6] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[0]), -1.0f), gmp_df_mul_f(gmp_df_mul(z, S[2]), 3.0f));
-  S[7] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(y, S[3]), 2.0f), gmp_df_mul(x, S[1]));
-  S[8] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[3]), 2.0f), gmp_df_mul(x, S[2]));
-  S[9] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[1]), -4.0f), gmp_df_mul_f(gmp_df_mul(y, S[4]), 5.0f));
-  S[10] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[2]), -1.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[4]), 2.0f), gmp_df_mul_f(gmp_df_mul(y, S[5]), 3.0f)));
-  S[11] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[1]), -2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[5]), 4.0f), gmp_df_mul(y, S[6])));
-  S[12] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[2]), -4.0f), gmp_df_mul_f(gmp_df_mul(z, S[6]), 5.0f));
-  S[13] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[3]), -2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(y, S[7]), 4.0f), gmp_df_mul(x, S[4])));
-  S[14] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[7]), 2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(y, S[8]), 2.0f), gmp_df_mul(x, S[5])));
-  S[15] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[3]), -2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[8]), 4.0f), gmp_df_mul(x, S[6])));
-  S[16] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[4]), -9.0f), gmp_df_mul_f(gmp_df_mul(y, S[9]), 7.0f));
-  S[17] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[5]), -4.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[9]), 2.0f), gmp_df_mul_f(gmp_df_mul(y, S[10]), 5.0f)));
-  S[18] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[4]), -2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[6]), -1.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[10]), 4.0f), gmp_df_mul_f(gmp_df_mul(y, S[11]), 3.0f))));
-  S[19] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[5]), -6.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[11]), 6.0f), gmp_df_mul(y, S[12])));
-  S[20] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[6]), -9.0f), gmp_df_mul_f(gmp_df_mul(z, S[12]), 7.0f));
-  S[21] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[7]), -6.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(y, S[13]), 6.0f), gmp_df_mul(x, S[9])));
-  S[22] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[8]), -2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[13]), 2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(y, S[14]), 4.0f), gmp_df_mul(x, S[10]))));
-  S[23] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[7]), -2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[14]), 4.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(y, S[15]), 2.0f), gmp_df_mul(x, S[11]))));
-  S[24] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[8]), -6.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[15]), 6.0f), gmp_df_mul(x, S[12])));
-  S[25] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[9]), -16.0f), gmp_df_mul_f(gmp_df_mul(y, S[16]), 9.0f));
-  S[26] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[10]), -9.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[16]), 2.0f), gmp_df_mul_f(gmp_df_mul(y, S[17]), 7.0f)));
-  S[27] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[9]), -2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[11]), -4.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[17]), 4.0f), gmp_df_mul_f(gmp_df_mul(y, S[18]), 5.0f))));
-  S[28] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[10]), -6.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[12]), -1.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[18]), 6.0f), gmp_df_mul_f(gmp_df_mul(y, S[19]), 3.0f))));
-  S[29] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[11]), -12.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[19]), 8.0f), gmp_df_mul(y, S[20])));
-  S[30] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[12]), -16.0f), gmp_df_mul_f(gmp_df_mul(z, S[20]), 9.0f));
-  S[31] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[13]), -12.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(y, S[21]), 8.0f), gmp_df_mul(x, S[16])));
-  S[32] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[14]), -6.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[21]), 2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(y, S[22]), 6.0f), gmp_df_mul(x, S[17]))));
-  S[33] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[13]), -2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[15]), -2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[22]), 4.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(y, S[23]), 4.0f), gmp_df_mul(x, S[18])))));
-  S[34] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[14]), -6.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[23]), 6.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(y, S[24]), 2.0f), gmp_df_mul(x, S[19]))));
-  S[35] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[15]), -12.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[24]), 8.0f), gmp_df_mul(x, S[20])));
-  S[36] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[16]), -25.0f), gmp_df_mul_f(gmp_df_mul(y, S[25]), 11.0f));
-  S[37] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[17]), -16.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[25]), 2.0f), gmp_df_mul_f(gmp_df_mul(y, S[26]), 9.0f)));
-  S[38] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[16]), -2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[18]), -9.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[26]), 4.0f), gmp_df_mul_f(gmp_df_mul(y, S[27]), 7.0f))));
-  S[39] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[17]), -6.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[19]), -4.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[27]), 6.0f), gmp_df_mul_f(gmp_df_mul(y, S[28]), 5.0f))));
-  S[40] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[18]), -12.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[20]), -1.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[28]), 8.0f), gmp_df_mul_f(gmp_df_mul(y, S[29]), 3.0f))));
-  S[41] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[19]), -20.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[29]), 10.0f), gmp_df_mul(y, S[30])));
-  S[42] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[20]), -25.0f), gmp_df_mul_f(gmp_df_mul(z, S[30]), 11.0f));
-  S[43] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[21]), -20.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(y, S[31]), 10.0f), gmp_df_mul(x, S[25])));
-  S[44] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[22]), -12.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[31]), 2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(y, S[32]), 8.0f), gmp_df_mul(x, S[26]))));
-  S[45] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[21]), -2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[23]), -6.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[32]), 4.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(y, S[33]), 6.0f), gmp_df_mul(x, S[27])))));
-  S[46] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[22]), -6.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[24]), -2.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[33]), 6.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(y, S[34]), 4.0f), gmp_df_mul(x, S[28])))));
-  S[47] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[23]), -12.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[34]), 8.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(y, S[35]), 2.0f), gmp_df_mul(x, S[29]))));
-  S[48] = gmp_df_add(gmp_df_mul_f(gmp_df_mul(r2, S[24]), -20.0f), gmp_df_add(gmp_df_mul_f(gmp_df_mul(z, S[35]), 10.0f), gmp_df_mul(x, S[30])));
+__device__ __forceinline__ void gmp_solid_df_6(gmp_f2 x, gmp_f2 y, gmp_f2 z, gmp_f2 r2, gmp_f2* __restrict__ H) {
+  const gmp_f2 z2 = gmp_df_mul(z, z);
+  const gmp_f2 r2_2 = gmp_df_mul(r2, r2);
+  const gmp_f2 r2_3 = gmp_df_mul(r2, r2_2);
+  gmp_f2 a = x, b = y;
+  H[0] = gmp_df_add_sloppy(gmp_df_mul(gmp_df_add_sloppy(gmp_df_mul(gmp_df_add_sloppy(gmp_df_mul_f(z2, 231.0f), gmp_df_mul_f(r2, -315.0f)), z2), gmp_df_mul_f(r2_2, 105.0f)), z2), gmp_df_mul_f(r2_3, -5.0f));
+  { const gmp_f2 q = gmp_df_mul(gmp_df_add_sloppy(gmp_df_mul(gmp_df_add_sloppy(gmp_df_mul_f(z2, 33.0f), gmp_df_mul_f(r2, -30.0f)), z2), gmp_df_mul_f(r2_2, 5.0f)), z); H[1] = gmp_df_mul(q, a); H[2] = gmp_df_mul(q, b); }
+  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul(x, a), gmp_df_neg(gmp_df_mul(y, b)));
+    b = gmp_df_add_sloppy(gmp_df_mul(x, b), gmp_df_mul(y, a));
+    a = t; }
+  { const gmp_f2 q = gmp_df_add_sloppy(gmp_df_mul(gmp_df_add_sloppy(gmp_df_mul_f(z2, 33.0f), gmp_df_mul_f(r2, -18.0f)), z2), r2_2); H[3] = gmp_df_mul(q, a); H[4] = gmp_df_mul(q, b); }
+  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul(x, a), gmp_df_neg(gmp_df_mul(y, b)));
+    b = gmp_df_add_sloppy(gmp_df_mul(x, b), gmp_df_mul(y, a));
+    a = t; }
+  { const gmp_f2 q = gmp_df_mul(gmp_df_add_sloppy(gmp_df_mul_f(z2, 11.0f), gmp_df_mul_f(r2, -3.0f)), z); H[5] = gmp_df_mul(q, a); H[6] = gmp_df_mul(q, b); }
+  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul(x, a), gmp_df_neg(gmp_df_mul(y, b)));
+    b = gmp_df_add_sloppy(gmp_df_mul(x, b), gmp_df_mul(y, a));
+    a = t; }
+  { const gmp_f2 q = gmp_df_add_sloppy(gmp_df_mul_f(z2, 11.0f), gmp_df_mul_f(r2, -1.0f)); H[7] = gmp_df_mul(q, a); H[8] = gmp_df_mul(q, b); }
+  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul(x, a), gmp_df_neg(gmp_df_mul(y, b)));
+    b = gmp_df_add_sloppy(gmp_df_mul(x, b), gmp_df_mul(y, a));
+    a = t; }
+  { const gmp_f2 q = z; H[9] = gmp_df_mul(q, a); H[10] = gmp_df_mul(q, b); }
+  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul(x, a), gmp_df_neg(gmp_df_mul(y, b)));
+    b = gmp_df_add_sloppy(gmp_df_mul(x, b), gmp_df_mul(y, a));
+    a = t; }
+  H[11] = a; H[12] = b;
 }
+#define GMP_SOLID_NZ 4
+static __device__ const float2 gmp_solid_norm[7][13] = {
+  {{1.0f, 0.0f}},
+  {{1.0f, 0.0f}, {1.0f, 0.0f}, {1.0f, 0.0f}},
+  {{1.5f, 0.0f}, {18.0f, 0.0f}, {18.0f, 0.0f}, {4.5f, 0.0f}, {4.5f, 0.0f}},
+  {{22.5f, 0.0f}, {33.75f, 0.0f}, {33.75f, 0.0f}, {337.5f, 0.0f}, {337.5f, 0.0f}, {56.25f, 0.0f}, {56.25f, 0.0f}},
+  {{39.375f, 0.0f}, {1575.0f, 0.0f}, {1575.0f, 0.0f}, {787.5f, 0.0f}, {787.5f, 0.0f}, {11025.0f, 0.0f}, {11025.0f, 0.0f}, {1378.125f, 0.0f}, {1378.125f, 0.0f}},
+  {{1771.875f, 0.0f}, {26578.125f, 0.0f}, {26578.125f, 0.0f}, {744187.5f, 0.0f}, {744187.5f, 0.0f}, {31007.8125f, 0.0f}, {31007.8125f, 0.0f}, {558140.625f, 0.0f}, {558140.625f, 0.0f}, {55814.0625f, 0.0f}, {55814.0625f, 0.0f}},
+  {{29235.9375f, 0.0f}, {2455818.75f, 0.0f}, {2455818.75f, 0.0f}, {1534886.75f, -0.03125f}, {1534886.75f, -0.03125f}, {6139547.0f, -0.125f}, {6139547.0f, -0.125f}, {1841864.0f, 0.0625f}, {1841864.0f, 0.0625f}, {40521008.0f, 1.375f}, {40521008.0f, 1.375f}, {3376750.75f, 0.03125f}, {3376750.75f, 0.03125f}},
+};
+static __device__ const signed char gmp_solid_row[7][13][4] = {
+  {{0, 0, 0, 0}},
+  {{2, 0, 0, 0}, {0, 0, 0, 0}, {1, 0, 0, 0}},
+  {{0, 3, 0, 0}, {2, 0, 0, 0}, {0, 0, 0, 0}, {4, 0, 0, 0}, {1, 0, 0, 0}},
+  {{2, 6, 0, 0}, {0, 3, 0, 0}, {2, 0, 0, 0}, {0, 0, 0, 0}, {1, 5, 0, 0}, {4, 0, 0, 0}, {1, 0, 0, 0}},
+  {{0, 3, 7, 0}, {2, 6, 0, 0}, {0, 3, 0, 0}, {2, 0, 0, 0}, {0, 0, 0, 0}, {4, 8, 0, 0}, {1, 5, 0, 0}, {4, 0, 0, 0}, {1, 0, 0, 0}},
+  {{2, 6, 10, 0}, {0, 3, 7, 0}, {2, 6, 0, 0}, {0, 3, 0, 0}, {2, 0, 0, 0}, {0, 0, 0, 0}, {1, 5, 9, 0}, {4, 8, 0, 0}, {1, 5, 0, 0}, {4, 0, 0, 0}, {1, 0, 0, 0}},
+  {{0, 3, 7, 11}, {2, 6, 10, 0}, {0, 3, 7, 0}, {2, 6, 0, 0}, {0, 3, 0, 0}, {2, 0, 0, 0}, {0, 0, 0, 0}, {4, 8, 12, 0}, {1, 5, 9, 0}, {4, 8, 0, 0}, {1, 5, 0, 0}, {4, 0, 0, 0}, {1, 0, 0, 0}},
+};
+static __device__ const float2 gmp_solid_coef[7][13][4] = {
+  {{{1.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}},
+  {{{1.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, {{1.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, {{1.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}},
+  {{{-0.5f, 0.0f}, {-1.5f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, {{3.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, {{1.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, {{1.5f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, {{3.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}},
+  {{{-2.25f, 0.0f}, {-3.75f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, {{-1.5f, 0.0f}, {-7.5f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, {{3.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, {{3.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, {{-0.75f, 0.0f}, {-3.75f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, {{7.5f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, {{3.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}},
+  {{{1.125f, 0.0f}, {7.5f, 0.0f}, {13.125f, 0.0f}, {0.0f, 0.0f}}, {{-11.25f, 0.0f}, {-26.25f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, {{-1.5f, 0.0f}, {-7.5f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, {{15.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, {{3.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, {{-3.75f, 0.0f}, {-13.125f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, {{-3.75f, 0.0f}, {-26.25f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, {{7.5f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, {{15.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}},
+  {{{28.125f, 0.0f}, {32.8125f, 0.0f}, {59.0625f, 0.0f}, {0.0f, 0.0f}}, {{5.625f, 0.0f}, {157.5f, 0.0f}, {118.125f, 0.0f}, {0.0f, 0.0f}}, {{-33.75f, 0.0f}, {-26.25f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, {{-7.5f, 0.0f}, {-157.5f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, {{45.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, {{15.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, {{5.625f, 0.0f}, {19.6875f, 0.0f}, {59.0625f, 0.0f}, {0.0f, 0.0f}}, {{-78.75f, 0.0f}, {-118.125f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, {{-11.25f, 0.0f}, {-26.25f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, {{157.5f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, {{45.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}},
+  {{{-14.0625f, 0.0f}, {-147.65625f, 0.0f}, {-177.1875f, 0.0f}, {-324.84375f, 0.0f}}, {{196.875f, 0.0f}, {295.3125f, 0.0f}, {649.6875f, 0.0f}, {0.0f, 0.0f}}, {{16.875f, 0.0f}, {157.5f, 0.0f}, {118.125f, 0.0f}, {0.0f, 0.0f}}, {{-236.25f, 0.0f}, {-236.25f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, {{-22.5f, 0.0f}, {-157.5f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, {{315.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, {{45.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, {{49.21875f, 0.0f}, {118.125f, 0.0f}, {324.84375f, 0.0f}, {0.0f, 0.0f}}, {{39.375f, 0.0f}, {177.1875f, 0.0f}, {649.6875f, 0.0f}, {0.0f, 0.0f}}, {{-78.75f, 0.0f}, {-118.125f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, {{-78.75f, 0.0f}, {-236.25f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, {{157.5f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, {{315.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}},
+};
 __device__ __forceinline__ float gmp_mcsh_invariant_0(const float* __restrict__ mu) {
   float f = 0.0f;
   { const float m = mu[0]; f = __fmaf_rn(__fmul_rn(1.0f, m), m, f); }
@@ -690,11 +666,6 @@ __device__ __forceinline__ void gmp_mcsh_invariant_adjoint_0(const float* __rest
   { const float m = __fmul_rn(2.0f, __fmul_rn(g, mu[0]));
     lam[0] = __fmaf_rn(1.0f, m, lam[0]);
   }
-}
-__device__ __forceinline__ gmp_f2 gmp_mcsh_invariant_df_0(const gmp_f2* __restrict__ mu) {
-  gmp_f2 f{0.0f, 0.0f};
-  { const gmp_f2 m = mu[0]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 1.0f), m), f); }
-  return f;
 }
 __device__ __forceinline__ float gmp_mcsh_invariant_1(const float* __restrict__ mu) {
   float f = 0.0f;
@@ -716,13 +687,6 @@ __device__ __forceinline__ void gmp_mcsh_invariant_adjoint_1(const float* __rest
   { const float m = __fmul_rn(2.0f, __fmul_rn(g, mu[1]));
     lam[1] = __fmaf_rn(1.0f, m, lam[1]);
   }
-}
-__device__ __forceinline__ gmp_f2 gmp_mcsh_invariant_df_1(const gmp_f2* __restrict__ mu) {
-  gmp_f2 f{0.0f, 0.0f};
-  { const gmp_f2 m = mu[2]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 1.0f), m), f); }
-  { const gmp_f2 m = mu[0]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 1.0f), m), f); }
-  { const gmp_f2 m = mu[1]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 1.0f), m), f); }
-  return f;
 }
 __device__ __forceinline__ float gmp_mcsh_invariant_2(const float* __restrict__ mu) {
   float f = 0.0f;
@@ -759,16 +723,6 @@ __device__ __forceinline__ void gmp_mcsh_invariant_adjoint_2(const float* __rest
   { const float m = __fmul_rn(2.0f, __fmul_rn(g, mu[2]));
     lam[2] = __fmaf_rn(1.0f, m, lam[2]);
   }
-}
-__device__ __forceinline__ gmp_f2 gmp_mcsh_invariant_df_2(const gmp_f2* __restrict__ mu) {
-  gmp_f2 f{0.0f, 0.0f};
-  { const gmp_f2 m = gmp_df_add(gmp_df_mul_f(mu[2], -1.0f), gmp_df_mul_f(mu[0], -1.0f)); f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 1.0f), m), f); }
-  { const gmp_f2 m = mu[3]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 2.0f), m), f); }
-  { const gmp_f2 m = mu[4]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 2.0f), m), f); }
-  { const gmp_f2 m = mu[0]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 1.0f), m), f); }
-  { const gmp_f2 m = mu[1]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 2.0f), m), f); }
-  { const gmp_f2 m = mu[2]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 1.0f), m), f); }
-  return f;
 }
 __device__ __forceinline__ float gmp_mcsh_invariant_3(const float* __restrict__ mu) {
   float f = 0.0f;
@@ -825,20 +779,6 @@ __device__ __forceinline__ void gmp_mcsh_invariant_adjoint_3(const float* __rest
   { const float m = __fmul_rn(2.0f, __fmul_rn(g, mu[3]));
     lam[3] = __fmaf_rn(1.0f, m, lam[3]);
   }
-}
-__device__ __forceinline__ gmp_f2 gmp_mcsh_invariant_df_3(const gmp_f2* __restrict__ mu) {
-  gmp_f2 f{0.0f, 0.0f};
-  { const gmp_f2 m = gmp_df_add(gmp_df_mul_f(mu[6], -1.0f), gmp_df_mul_f(mu[4], -1.0f)); f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 1.0f), m), f); }
-  { const gmp_f2 m = gmp_df_add(gmp_df_mul_f(mu[2], -1.0f), gmp_df_mul_f(mu[0], -1.0f)); f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 3.0f), m), f); }
-  { const gmp_f2 m = gmp_df_add(gmp_df_mul_f(mu[3], -1.0f), gmp_df_mul_f(mu[1], -1.0f)); f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 3.0f), m), f); }
-  { const gmp_f2 m = mu[4]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 3.0f), m), f); }
-  { const gmp_f2 m = mu[5]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 6.0f), m), f); }
-  { const gmp_f2 m = mu[6]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 3.0f), m), f); }
-  { const gmp_f2 m = mu[0]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 1.0f), m), f); }
-  { const gmp_f2 m = mu[1]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 3.0f), m), f); }
-  { const gmp_f2 m = mu[2]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 3.0f), m), f); }
-  { const gmp_f2 m = mu[3]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 1.0f), m), f); }
-  return f;
 }
 __device__ __forceinline__ float gmp_mcsh_invariant_4(const float* __restrict__ mu) {
   float f = 0.0f;
@@ -921,25 +861,6 @@ __device__ __forceinline__ void gmp_mcsh_invariant_adjoint_4(const float* __rest
   { const float m = __fmul_rn(2.0f, __fmul_rn(g, mu[4]));
     lam[4] = __fmaf_rn(1.0f, m, lam[4]);
   }
-}
-__device__ __forceinline__ gmp_f2 gmp_mcsh_invariant_df_4(const gmp_f2* __restrict__ mu) {
-  gmp_f2 f{0.0f, 0.0f};
-  { const gmp_f2 m = gmp_df_add(mu[4], gmp_df_add(gmp_df_mul_f(mu[2], 2.0f), mu[0])); f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 1.0f), m), f); }
-  { const gmp_f2 m = gmp_df_add(gmp_df_mul_f(mu[7], -1.0f), gmp_df_mul_f(mu[5], -1.0f)); f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 4.0f), m), f); }
-  { const gmp_f2 m = gmp_df_add(gmp_df_mul_f(mu[8], -1.0f), gmp_df_mul_f(mu[6], -1.0f)); f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 4.0f), m), f); }
-  { const gmp_f2 m = gmp_df_add(gmp_df_mul_f(mu[2], -1.0f), gmp_df_mul_f(mu[0], -1.0f)); f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 6.0f), m), f); }
-  { const gmp_f2 m = gmp_df_add(gmp_df_mul_f(mu[3], -1.0f), gmp_df_mul_f(mu[1], -1.0f)); f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 12.0f), m), f); }
-  { const gmp_f2 m = gmp_df_add(gmp_df_mul_f(mu[4], -1.0f), gmp_df_mul_f(mu[2], -1.0f)); f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 6.0f), m), f); }
-  { const gmp_f2 m = mu[5]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 4.0f), m), f); }
-  { const gmp_f2 m = mu[6]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 12.0f), m), f); }
-  { const gmp_f2 m = mu[7]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 12.0f), m), f); }
-  { const gmp_f2 m = mu[8]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 4.0f), m), f); }
-  { const gmp_f2 m = mu[0]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 1.0f), m), f); }
-  { const gmp_f2 m = mu[1]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 4.0f), m), f); }
-  { const gmp_f2 m = mu[2]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 6.0f), m), f); }
-  { const gmp_f2 m = mu[3]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 4.0f), m), f); }
-  { const gmp_f2 m = mu[4]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 1.0f), m), f); }
-  return f;
 }
 __device__ __forceinline__ float gmp_mcsh_invariant_5(const float* __restrict__ mu) {
   float f = 0.0f;
@@ -1054,31 +975,6 @@ __device__ __forceinline__ void gmp_mcsh_invariant_adjoint_5(const float* __rest
   { const float m = __fmul_rn(2.0f, __fmul_rn(g, mu[5]));
     lam[5] = __fmaf_rn(1.0f, m, lam[5]);
   }
-}
-__device__ __forceinline__ gmp_f2 gmp_mcsh_invariant_df_5(const gmp_f2* __restrict__ mu) {
-  gmp_f2 f{0.0f, 0.0f};
-  { const gmp_f2 m = gmp_df_add(mu[10], gmp_df_add(gmp_df_mul_f(mu[8], 2.0f), mu[6])); f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 1.0f), m), f); }
-  { const gmp_f2 m = gmp_df_add(mu[4], gmp_df_add(gmp_df_mul_f(mu[2], 2.0f), mu[0])); f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 5.0f), m), f); }
-  { const gmp_f2 m = gmp_df_add(mu[5], gmp_df_add(gmp_df_mul_f(mu[3], 2.0f), mu[1])); f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 5.0f), m), f); }
-  { const gmp_f2 m = gmp_df_add(gmp_df_mul_f(mu[8], -1.0f), gmp_df_mul_f(mu[6], -1.0f)); f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 10.0f), m), f); }
-  { const gmp_f2 m = gmp_df_add(gmp_df_mul_f(mu[9], -1.0f), gmp_df_mul_f(mu[7], -1.0f)); f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 20.0f), m), f); }
-  { const gmp_f2 m = gmp_df_add(gmp_df_mul_f(mu[10], -1.0f), gmp_df_mul_f(mu[8], -1.0f)); f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 10.0f), m), f); }
-  { const gmp_f2 m = gmp_df_add(gmp_df_mul_f(mu[2], -1.0f), gmp_df_mul_f(mu[0], -1.0f)); f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 10.0f), m), f); }
-  { const gmp_f2 m = gmp_df_add(gmp_df_mul_f(mu[3], -1.0f), gmp_df_mul_f(mu[1], -1.0f)); f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 30.0f), m), f); }
-  { const gmp_f2 m = gmp_df_add(gmp_df_mul_f(mu[4], -1.0f), gmp_df_mul_f(mu[2], -1.0f)); f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 30.0f), m), f); }
-  { const gmp_f2 m = gmp_df_add(gmp_df_mul_f(mu[5], -1.0f), gmp_df_mul_f(mu[3], -1.0f)); f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 10.0f), m), f); }
-  { const gmp_f2 m = mu[6]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 5.0f), m), f); }
-  { const gmp_f2 m = mu[7]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 20.0f), m), f); }
-  { const gmp_f2 m = mu[8]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 30.0f), m), f); }
-  { const gmp_f2 m = mu[9]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 20.0f), m), f); }
-  { const gmp_f2 m = mu[10]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 5.0f), m), f); }
-  { const gmp_f2 m = mu[0]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 1.0f), m), f); }
-  { const gmp_f2 m = mu[1]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 5.0f), m), f); }
-  { const gmp_f2 m = mu[2]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 10.0f), m), f); }
-  { const gmp_f2 m = mu[3]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 10.0f), m), f); }
-  { const gmp_f2 m = mu[4]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 5.0f), m), f); }
-  { const gmp_f2 m = mu[5]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 1.0f), m), f); }
-  return f;
 }
 __device__ __forceinline__ float gmp_mcsh_invariant_6(const float* __restrict__ mu) {
   float f = 0.0f;
@@ -1232,38 +1128,6 @@ __device__ __forceinline__ void gmp_mcsh_invariant_adjoint_6(const float* __rest
   { const float m = __fmul_rn(2.0f, __fmul_rn(g, mu[6]));
     lam[6] = __fmaf_rn(1.0f, m, lam[6]);
   }
-}
-__device__ __forceinline__ gmp_f2 gmp_mcsh_invariant_df_6(const gmp_f2* __restrict__ mu) {
-  gmp_f2 f{0.0f, 0.0f};
-  { const gmp_f2 m = gmp_df_add(gmp_df_mul_f(mu[6], -1.0f), gmp_df_add(gmp_df_mul_f(mu[4], -3.0f), gmp_df_add(gmp_df_mul_f(mu[2], -3.0f), gmp_df_mul_f(mu[0], -1.0f)))); f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 1.0f), m), f); }
-  { const gmp_f2 m = gmp_df_add(mu[11], gmp_df_add(gmp_df_mul_f(mu[9], 2.0f), mu[7])); f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 6.0f), m), f); }
-  { const gmp_f2 m = gmp_df_add(mu[12], gmp_df_add(gmp_df_mul_f(mu[10], 2.0f), mu[8])); f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 6.0f), m), f); }
-  { const gmp_f2 m = gmp_df_add(mu[4], gmp_df_add(gmp_df_mul_f(mu[2], 2.0f), mu[0])); f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 15.0f), m), f); }
-  { const gmp_f2 m = gmp_df_add(mu[5], gmp_df_add(gmp_df_mul_f(mu[3], 2.0f), mu[1])); f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 30.0f), m), f); }
-  { const gmp_f2 m = gmp_df_add(mu[6], gmp_df_add(gmp_df_mul_f(mu[4], 2.0f), mu[2])); f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 15.0f), m), f); }
-  { const gmp_f2 m = gmp_df_add(gmp_df_mul_f(mu[9], -1.0f), gmp_df_mul_f(mu[7], -1.0f)); f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 20.0f), m), f); }
-  { const gmp_f2 m = gmp_df_add(gmp_df_mul_f(mu[10], -1.0f), gmp_df_mul_f(mu[8], -1.0f)); f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 60.0f), m), f); }
-  { const gmp_f2 m = gmp_df_add(gmp_df_mul_f(mu[11], -1.0f), gmp_df_mul_f(mu[9], -1.0f)); f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 60.0f), m), f); }
-  { const gmp_f2 m = gmp_df_add(gmp_df_mul_f(mu[12], -1.0f), gmp_df_mul_f(mu[10], -1.0f)); f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 20.0f), m), f); }
-  { const gmp_f2 m = gmp_df_add(gmp_df_mul_f(mu[2], -1.0f), gmp_df_mul_f(mu[0], -1.0f)); f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 15.0f), m), f); }
-  { const gmp_f2 m = gmp_df_add(gmp_df_mul_f(mu[3], -1.0f), gmp_df_mul_f(mu[1], -1.0f)); f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 60.0f), m), f); }
-  { const gmp_f2 m = gmp_df_add(gmp_df_mul_f(mu[4], -1.0f), gmp_df_mul_f(mu[2], -1.0f)); f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 90.0f), m), f); }
-  { const gmp_f2 m = gmp_df_add(gmp_df_mul_f(mu[5], -1.0f), gmp_df_mul_f(mu[3], -1.0f)); f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 60.0f), m), f); }
-  { const gmp_f2 m = gmp_df_add(gmp_df_mul_f(mu[6], -1.0f), gmp_df_mul_f(mu[4], -1.0f)); f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 15.0f), m), f); }
-  { const gmp_f2 m = mu[7]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 6.0f), m), f); }
-  { const gmp_f2 m = mu[8]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 30.0f), m), f); }
-  { const gmp_f2 m = mu[9]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 60.0f), m), f); }
-  { const gmp_f2 m = mu[10]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 60.0f), m), f); }
-  { const gmp_f2 m = mu[11]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 30.0f), m), f); }
-  { const gmp_f2 m = mu[12]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 6.0f), m), f); }
-  { const gmp_f2 m = mu[0]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 1.0f), m), f); }
-  { const gmp_f2 m = mu[1]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 6.0f), m), f); }
-  { const gmp_f2 m = mu[2]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 15.0f), m), f); }
-  { const gmp_f2 m = mu[3]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 20.0f), m), f); }
-  { const gmp_f2 m = mu[4]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 15.0f), m), f); }
-  { const gmp_f2 m = mu[5]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 6.0f), m), f); }
-  { const gmp_f2 m = mu[6]; f = gmp_df_add(gmp_df_mul(gmp_df_mul_f(m, 1.0f), m), f); }
-  return f;
 }
 __device__ __forceinline__ void gmp_mcsh_shift_contract_0(const float* __restrict__ lam, const float* __restrict__ S1, float* __restrict__ V) {
   float vx = 0.0f, vy = 0.0f, vz = 0.0f;
@@ -1949,30 +1813,16 @@ __device__ __forceinline__ float gmp_mcsh_invariant(int l, const float* mu) {
     default: return 0.0f;
   }
 }
-__device__ __forceinline__ gmp_f2 gmp_mcsh_invariant_df(int l, const gmp_f2* mu) {
-  switch (l) {
-    case 0: return gmp_mcsh_invariant_df_0(mu);
-    case 1: return gmp_mcsh_invariant_df_1(mu);
-    case 2: return gmp_mcsh_invariant_df_2(mu);
-    case 3: return gmp_mcsh_invariant_df_3(mu);
-    case 4: return gmp_mcsh_invariant_df_4(mu);
-    case 5: return gmp_mcsh_invariant_df_5(mu);
-    case 6: return gmp_mcsh_invariant_df_6(mu);
-    default: return gmp_f2{0.0f, 0.0f};
-  }
-}
-// independent components of orders 0..l in double-float arithmetic (l <= L of the caller)
-__device__ __forceinline__ void gmp_mcsh_indep_df(int l, gmp_f2 x, gmp_f2 y, gmp_f2 z, gmp_f2 r2, gmp_f2* S) {
-  switch (l) {
-    case 0: gmp_mcsh_indep_df_0(x, y, z, r2, S); break;
-    case 1: gmp_mcsh_indep_df_1(x, y, z, r2, S); break;
-    case 2: gmp_mcsh_indep_df_2(x, y, z, r2, S); break;
-    case 3: gmp_mcsh_indep_df_3(x, y, z, r2, S); break;
-    case 4: gmp_mcsh_indep_df_4(x, y, z, r2, S); break;
-    case 5: gmp_mcsh_indep_df_5(x, y, z, r2, S); break;
-    case 6: gmp_mcsh_indep_df_6(x, y, z, r2, S); break;
-    default: break;
-  }
+// solid harmonics of order l in double-float arithmetic
+template <int l>
+__device__ __forceinline__ void gmp_solid_df(gmp_f2 x, gmp_f2 y, gmp_f2 z, gmp_f2 r2, gmp_f2* H) {
+  if constexpr (l == 0) gmp_solid_df_0(x, y, z, r2, H);
+  if constexpr (l == 1) gmp_solid_df_1(x, y, z, r2, H);
+  if constexpr (l == 2) gmp_solid_df_2(x, y, z, r2, H);
+  if constexpr (l == 3) gmp_solid_df_3(x, y, z, r2, H);
+  if constexpr (l == 4) gmp_solid_df_4(x, y, z, r2, H);
+  if constexpr (l == 5) gmp_solid_df_5(x, y, z, r2, H);
+  if constexpr (l == 6) gmp_solid_df_6(x, y, z, r2, H);
 }
 __device__ __forceinline__ void gmp_mcsh_shift_contract_order(int l, const float* lam, const float* S1, float* V) {
   switch (l) {

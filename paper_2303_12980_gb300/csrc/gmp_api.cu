@@ -92,7 +92,7 @@ struct gmp_ctx {
   std::vector<uint8_t> last_pbc;
   int64_t n_bins = 0;
   // workspace
-  DevBuf structs, grid, atom_off, struct_of, bbox, atom_xh, atom_xl, atom_u, atom_bin, atom_rng, atom_y;
+  DevBuf structs, grid, atom_off, struct_of, bbox, atom_xh, atom_xl, atom_u, atom_bin, atom_t, atom_y;
   DevBuf bin_count, bin_cursor, bin_start, bin_y, bin_je, counts, nbr_off, scan_tmp, pairs;
   DevBuf scalars;  // err word, maxm, counter
   DevBuf grad_acc, jac_counts, jac_rows;
@@ -106,7 +106,7 @@ struct gmp_ctx {
   DevBuf colinfo;   // per feature column: (order << 16) | sigma, -1 for the density
   int n_ord_pos = 1;  // orders >= 0: refine queue entries per center and pass
   DevBuf stage_pos, stage_species, stage_feat, stage_gradf, stage_gradp, stage_virial;
-  DevBuf pt_off, pt_struct, pt_xh, pt_xl, pt_rng, pt_y, stage_pts;  // reference points
+  DevBuf pt_off, pt_struct, pt_xh, pt_xl, pt_t, pt_y, stage_pts;  // reference points
   int64_t P = 0;  // pairs of the last neighbor build
   int max_m = 0;
   // Pair layout of the last build: CSR by center (nbr_off) or, after a
@@ -298,6 +298,9 @@ gmp_status upload_structures(gmp_ctx* h, int32_t S, const int64_t* atom_off, con
     }
     g.atom_base = atom_off[s];
     g.n_atoms = (int32_t)(atom_off[s + 1] - atom_off[s]);
+    g.diag = 1;
+    for (int k = 0; k < 9; ++k)
+      if (k % 4 != 0 && g.A[k] != 0.0) g.diag = 0;
     g.bin_base = bin_base;
     g.bin_cap = 2 * g.n_atoms + 8;
     bin_base += g.bin_cap;
@@ -358,7 +361,7 @@ gmp_status bin_atoms(gmp_ctx* h, int32_t S, const double* pos, const int32_t* sp
   GMP_CK(h->atom_xl.ensure(sizeof(float4) * N), "atom_xl");
   GMP_CK(h->atom_u.ensure(sizeof(GmpD4) * N), "atom_u");
   GMP_CK(h->atom_bin.ensure(sizeof(int32_t) * N), "atom_bin");
-  GMP_CK(h->atom_rng.ensure(sizeof(int4) * N), "atom_rng");
+  GMP_CK(h->atom_t.ensure(sizeof(float4) * N), "atom_t");
   GMP_CK(h->atom_y.ensure(sizeof(float4) * N), "atom_y");
   GMP_CK(h->bin_count.ensure(sizeof(int32_t) * h->n_bins), "bin_count");
   GMP_CK(h->bin_cursor.ensure(sizeof(int32_t) * h->n_bins), "bin_cursor");
@@ -375,7 +378,7 @@ gmp_status bin_atoms(gmp_ctx* h, int32_t S, const double* pos, const int32_t* sp
                                 h->n_el, h->grid.as<GmpGrid>(), h->n_bins, h->atom_xh.as<float4>(),
                                 h->atom_xl.as<float4>(), h->atom_u.as<GmpD4>(), h->atom_bin.as<int32_t>(),
                                 h->bin_start.as<int32_t>(), h->bin_y.as<float4>(), h->bin_je.as<int2>(),
-                                h->atom_rng.as<int4>(), h->atom_y.as<float4>(), d_err, st, L),
+                                h->atom_t.as<float4>(), h->atom_y.as<float4>(), d_err, st, L),
            "bins (one block)");
     return GMP_OK;
   }
@@ -386,7 +389,7 @@ gmp_status bin_atoms(gmp_ctx* h, int32_t S, const double* pos, const int32_t* sp
          "prepare");
   GMP_CK(gmp_launch_bins(h->structs.as<GmpStruct>(), h->grid.as<GmpGrid>(), h->struct_of.as<int32_t>(), N,
                          h->n_bins, h->atom_bin.as<int32_t>(), h->bin_count.as<int32_t>(),
-                         h->bin_start.as<int32_t>(), h->bin_cursor.as<int32_t>(), h->atom_rng.as<int4>(),
+                         h->bin_start.as<int32_t>(), h->bin_cursor.as<int32_t>(), h->atom_t.as<float4>(),
                          h->atom_y.as<float4>(), h->bin_y.as<float4>(), h->bin_je.as<int2>(), h->atom_u.as<GmpD4>(),
                          h->atom_xh.as<float4>(), h->atom_xl.as<float4>(), h->scan_tmp.p, h->scan_tmp.bytes, st,
                          h->sm_count, L),
@@ -508,7 +511,7 @@ gmp_status build_neighbors(gmp_ctx* h, int32_t S, const double* pos, const int32
   gmp_status r = bin_atoms(h, S, pos, species, N, N, st);
   if (r != GMP_OK) return r;
   const GmpCenters C{h->struct_of.as<int32_t>(), pos, h->atom_xh.as<float4>(), h->atom_xl.as<float4>(),
-                     h->atom_rng.as<int4>(), h->atom_y.as<float4>()};
+                     h->atom_t.as<float4>(), h->atom_y.as<float4>()};
   if ((r = neighbor_lists(h, C, N, pos, st, sorted, capture, !need_csr)) != GMP_OK) return r;
   GMP_CK(prof_mark(h, 0, false, st), "profile");
   return GMP_OK;
@@ -1373,7 +1376,7 @@ gmp_status gmp_featurize_points(gmp_handle h, int32_t n_struct, const int64_t* a
     GMP_CK(h->pt_struct.ensure(sizeof(int32_t) * NP), "point struct");
     GMP_CK(h->pt_xh.ensure(sizeof(float4) * NP), "point xh");
     GMP_CK(h->pt_xl.ensure(sizeof(float4) * NP), "point xl");
-    GMP_CK(h->pt_rng.ensure(sizeof(int4) * NP), "point ranges");
+    GMP_CK(h->pt_t.ensure(sizeof(float4) * NP), "point t");
     GMP_CK(h->pt_y.ensure(sizeof(float4) * NP), "point y");
     GMP_CK(cudaMemcpyAsync(h->pt_off.p, point_off, sizeof(int64_t) * (n_struct + 1), cudaMemcpyHostToDevice, st),
            "upload point_off");
@@ -1382,11 +1385,11 @@ gmp_status gmp_featurize_points(gmp_handle h, int32_t n_struct, const int64_t* a
     GMP_CK(prof_mark(h, 0, true, st), "profile");
     if ((r = bin_atoms(h, n_struct, io.pos, io.species, N, NP, st)) != GMP_OK) return r;
     GMP_CK(gmp_launch_point_prepare(h->structs.as<GmpStruct>(), h->grid.as<GmpGrid>(), h->pt_struct.as<int32_t>(), NP,
-                                    pts, io.pos, h->pt_xh.as<float4>(), h->pt_xl.as<float4>(), h->pt_rng.as<int4>(),
+                                    pts, io.pos, h->pt_xh.as<float4>(), h->pt_xl.as<float4>(), h->pt_t.as<float4>(),
                                     h->pt_y.as<float4>(), h->scalars.as<uint32_t>(), st, h->sm_count, &h->launches),
            "point prepare");
     const GmpCenters C{h->pt_struct.as<int32_t>(), pts, h->pt_xh.as<float4>(), h->pt_xl.as<float4>(),
-                       h->pt_rng.as<int4>(), h->pt_y.as<float4>()};
+                       h->pt_t.as<float4>(), h->pt_y.as<float4>()};
     h->last_nc = -1;  // the capacities below describe the points, not the atoms
     if ((r = neighbor_lists(h, C, NP, io.pos, st, false, false)) != GMP_OK) return r;
     h->last_nc = -1;

@@ -28,7 +28,7 @@ struct GmpStruct {
   int periodic[3];
   int64_t atom_base;  // first atom
   int32_t n_atoms;
-  int32_t pad0;
+  int32_t diag;       // A has no off-diagonal entries
   int64_t bin_base;   // first bin slot of this structure
   int32_t bin_cap;    // bin slots reserved
   int32_t pad1;
@@ -43,7 +43,11 @@ struct GmpGrid {
   double binw[3];     // bin width (fractional)
   double inv_binw[3]; // 1 / binw
   int nb[3];          // bins per axis
-  int pad;
+  int ortho;          // the cell's axes are orthogonal (up to rounding)
+  // for the neighbor search, in FP32: the cutoff in bins, the distance
+  // between the planes of a bin (Angstrom), and 1 / that of axis 0
+  float rb[3], h[3], inv_h0;
+  float pad;
 };
 
 // One neighbor image of a center, 32 bytes.
@@ -280,29 +284,45 @@ __device__ __forceinline__ gmp_f2 gmp_df_exp_neg(gmp_f2 x, const float2* tab) {
   return gmp_f2{__fmul_rn(e.hi, scale), __fmul_rn(__fadd_rn(e.lo, __fadd_rn(T.y, vl)), scale)};
 }
 
-// Double-float displacement of j's image n from i, and its r^2.
+// Double-float displacement of j's image n from i, and its r^2; mag (when
+// asked for) bounds the size of the added terms.  One renormalisation per
+// addition: the low words' sum is then off by 2^-48 of the coordinates, as
+// their split itself is; r^2 adds non-negative terms.  A cell along the
+// coordinate axes (st.diag) has one lattice vector per component.
+template <bool MAG = false>
 __device__ __forceinline__ void gmp_df_disp(const float4& xhi, const float4& xli, const float4& xhj,
                                         const float4& xlj, const GmpStruct& st, const int* n,
-                                        gmp_f2* d, gmp_f2& r2, float& mag) {
+                                        gmp_f2* d, gmp_f2& r2, float* mag = nullptr) {
   const float xi_h[3] = {xhi.x, xhi.y, xhi.z}, xi_l[3] = {xli.x, xli.y, xli.z};
   const float xj_h[3] = {xhj.x, xhj.y, xhj.z}, xj_l[3] = {xlj.x, xlj.y, xlj.z};
   const bool shifted = (n[0] | n[1] | n[2]) != 0;
-  mag = 0.0f;
+  float m[3];
+#pragma unroll
   for (int c = 0; c < 3; ++c) {
-    gmp_f2 dd = gmp_df_add(gmp_f2{xj_h[c], xj_l[c]}, gmp_f2{-xi_h[c], -xi_l[c]});
-    float m = fabsf(xj_h[c]) + fabsf(xi_h[c]);
-    if (shifted) {
-      gmp_f2 s0 = gmp_df_mul_int(n[0], gmp_f2{st.Ahi[c], st.Alo[c]});
-      gmp_f2 s1 = gmp_df_mul_int(n[1], gmp_f2{st.Ahi[3 + c], st.Alo[3 + c]});
-      gmp_f2 s2 = gmp_df_mul_int(n[2], gmp_f2{st.Ahi[6 + c], st.Alo[6 + c]});
-      gmp_f2 sh = gmp_df_add(gmp_df_add(s0, s1), s2);
-      dd = gmp_df_add(dd, sh);
-      m += fabsf(s0.hi) + fabsf(s1.hi) + fabsf(s2.hi);
-    }
-    d[c] = dd;
-    mag = fmaxf(mag, m);
+    d[c] = gmp_df_add_sloppy(gmp_f2{xj_h[c], xj_l[c]}, gmp_f2{-xi_h[c], -xi_l[c]});
+    if (MAG) m[c] = fabsf(xj_h[c]) + fabsf(xi_h[c]);
   }
-  r2 = gmp_df_add(gmp_df_add(gmp_df_mul(d[0], d[0]), gmp_df_mul(d[1], d[1])), gmp_df_mul(d[2], d[2]));
+  if (shifted) {
+    if (st.diag) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const gmp_f2 sh = gmp_df_mul_int(n[c], gmp_f2{st.Ahi[4 * c], st.Alo[4 * c]});
+        d[c] = gmp_df_add_sloppy(d[c], sh);
+        if (MAG) m[c] += fabsf(sh.hi);
+      }
+    } else {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const gmp_f2 s0 = gmp_df_mul_int(n[0], gmp_f2{st.Ahi[c], st.Alo[c]});
+        const gmp_f2 s1 = gmp_df_mul_int(n[1], gmp_f2{st.Ahi[3 + c], st.Alo[3 + c]});
+        const gmp_f2 s2 = gmp_df_mul_int(n[2], gmp_f2{st.Ahi[6 + c], st.Alo[6 + c]});
+        d[c] = gmp_df_add_sloppy(d[c], gmp_df_add_sloppy(gmp_df_add_sloppy(s0, s1), s2));
+        if (MAG) m[c] += fabsf(s0.hi) + fabsf(s1.hi) + fabsf(s2.hi);
+      }
+    }
+  }
+  if (MAG) *mag = fmaxf(fmaxf(m[0], m[1]), m[2]);
+  r2 = gmp_df_add_sloppy(gmp_df_add_sloppy(gmp_df_mul(d[0], d[0]), gmp_df_mul(d[1], d[1])), gmp_df_mul(d[2], d[2]));
 }
 
 // ---------------------------------------------------------------- host side
@@ -311,7 +331,7 @@ struct GmpWorkspace;
 // Launchers implemented in the .cu files (all asynchronous on `stream`).
 // Binning of a small batch (at most kSmallBinAtoms atoms, 256 structures)
 // in one launch of one CTA: the outputs of gmp_launch_neighbors_prepare +
-// gmp_launch_bins (atom_xh/xl/u/bin/rng/y, grid, pre-screen bounds,
+// gmp_launch_bins (atom_xh/xl/u/bin/t/y, grid, pre-screen bounds,
 // bin_start/bin_y/bin_je), bit for bit.  gmp_bin_small_fits says whether
 // a batch qualifies (shared memory for its bins and slots).
 // One SM runs the batch's FP64 set-up (GB300: 1/64 of the FP32 rate), so
@@ -324,7 +344,7 @@ cudaError_t gmp_launch_bin_small(GmpStruct* d_structs, int n_struct, const int32
                                  double cutoff, const double* pos, const int32_t* species, int n_el,
                                  GmpGrid* d_grid, int64_t n_bins, float4* atom_xh, float4* atom_xl, GmpD4* atom_u,
                                  int32_t* atom_bin, int32_t* bin_start, float4* bin_y, int2* bin_je,
-                                 int4* atom_rng, float4* atom_y, uint32_t* d_err, cudaStream_t stream,
+                                 float4* atom_t, float4* atom_y, uint32_t* d_err, cudaStream_t stream,
                                  int64_t* launches);
 cudaError_t gmp_launch_neighbors_prepare(const GmpStruct* d_structs, int n_struct,
                                          const int32_t* d_struct_of, int64_t N, double cutoff,
@@ -336,7 +356,7 @@ cudaError_t gmp_launch_neighbors_prepare(const GmpStruct* d_structs, int n_struc
 cudaError_t gmp_launch_bins(const GmpStruct* d_structs, const GmpGrid* d_grid,
                             const int32_t* d_struct_of, int64_t N, int64_t n_bins,
                             const int32_t* atom_bin, int32_t* bin_count, int32_t* bin_start,
-                            int32_t* bin_cursor, int4* atom_rng, float4* atom_y, float4* bin_y, int2* bin_je,
+                            int32_t* bin_cursor, float4* atom_t, float4* atom_y, float4* bin_y, int2* bin_je,
                             const GmpD4* atom_u, const float4* atom_xh, const float4* atom_xl, void* scan_tmp,
                             size_t scan_tmp_bytes, cudaStream_t stream, int sm_count, int64_t* launches);
 size_t gmp_scan_tmp_bytes(int64_t n);
@@ -345,13 +365,14 @@ cudaError_t gmp_exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, v
 // The points that neighbor lists are built around: the atoms themselves or
 // reference points (gmp_featurize_points).  Per center: structure id, FP64
 // position [3], double-float split (xl.w = packed wrap of the fractional
-// coordinates), scanned bin range and wrapped FP32 position (k_ranges).
+// coordinates), position in the structure's bin grid in units of bins (t,
+// FP32) and wrapped FP32 position y (k_ranges).
 struct GmpCenters {
   const int32_t* sid;
   const double* pos;
   const float4* xh;
   const float4* xl;
-  const int4* rng;
+  const float4* t;
   const float4* y;
 };
 // Per reference point: the GmpCenters fields above from its FP64 position
@@ -359,7 +380,7 @@ struct GmpCenters {
 // gives each structure's reference cell (that of its first atom).
 cudaError_t gmp_launch_point_prepare(const GmpStruct* d_structs, const GmpGrid* d_grid,
                                      const int32_t* point_struct, int64_t n_points, const double* points,
-                                     const double* atom_pos, float4* pt_xh, float4* pt_xl, int4* pt_rng,
+                                     const double* atom_pos, float4* pt_xh, float4* pt_xl, float4* pt_t,
                                      float4* pt_y, uint32_t* d_err, cudaStream_t stream, int sm_count,
                                      int64_t* launches);
 // fill: 0 = count only, 1 = records grouped by species (deterministic),

@@ -7,9 +7,9 @@
 // where the expression is FP64, evaluated left to right without FMA.  The
 // GPU reaches the same decision with far less FP64 work:
 //   1. atoms are binned on a grid in (wrapped) fractional coordinates;
-//   2. a center scans the bins that its cutoff sphere can touch (periodic
-//      axes wrap, giving an image index m); each candidate is pre-screened
-//      in FP32 against a rigorous bound on the FP32 error;
+//   2. a center scans the rows of bins that its cutoff sphere can touch
+//      (periodic axes wrap, giving an image index m); each candidate is
+//      pre-screened in FP32 against a rigorous bound on the FP32 error;
 //   3. survivors get d and r^2 in double-float arithmetic (about 2^-44
 //      relative), which decides every case except a shell of relative width
 //      ~1e-9 around rc^2; inside that shell the FP64 expression above is
@@ -227,8 +227,21 @@ __device__ inline void grid_struct(GmpStruct* S, int s, const unsigned long long
   }
   double delta = ldexp(Y + Sh + cutoff, -21);
   double b = (cutoff + 2.0 * delta);
-  g.pad = 0;
-  for (int k = 0; k < 3; ++k) g.inv_binw[k] = 1.0 / g.binw[k];
+  g.ortho = 1;
+  double bk[3];  // |b_k|^2, b_k = column k of Ainv
+  for (int k = 0; k < 3; ++k) bk[k] = st.Ainv[k] * st.Ainv[k] + st.Ainv[3 + k] * st.Ainv[3 + k] + st.Ainv[6 + k] * st.Ainv[6 + k];
+  for (int k = 0; k < 3; ++k) {
+    const int m = k == 2 ? 0 : k + 1;
+    const double d = st.Ainv[k] * st.Ainv[m] + st.Ainv[3 + k] * st.Ainv[3 + m] + st.Ainv[6 + k] * st.Ainv[6 + m];
+    if (!(d * d <= 1e-18 * bk[k] * bk[m])) g.ortho = 0;
+  }
+  for (int k = 0; k < 3; ++k) {
+    g.inv_binw[k] = 1.0 / g.binw[k];
+    g.rb[k] = (float)(st.reach[k] * g.inv_binw[k]);
+    g.h[k] = (float)(cutoff / (st.reach[k] * g.inv_binw[k]));
+  }
+  g.inv_h0 = g.rb[0] / (float)cutoff;
+  g.pad = 0.0f;
   G[s] = g;
   float p2 = (float)(b * b * (1.0 + ldexp(1.0, -20)));
   S[s].prescreen2 = nextafterf(p2, INFINITY);
@@ -250,7 +263,7 @@ __device__ __forceinline__ int32_t bin_of(const GmpStruct* S, const GmpGrid* G, 
   const double u[3] = {u4.x, u4.y, u4.z};
   int b[3];
   for (int k = 0; k < 3; ++k) {
-    double t = floor((u[k] - g.umin[k]) * g.inv_binw[k]);  // as center_range scales
+    double t = floor((u[k] - g.umin[k]) * g.inv_binw[k]);  // as center_place scales
     t = fmin(fmax(t, 0.0), (double)(g.nb[k] - 1));
     b[k] = (int)t;
   }
@@ -313,57 +326,39 @@ __global__ void k_bin_place(const GmpStruct* __restrict__ S, const int32_t* __re
   }
 }
 
-// Bins a center at wrapped fractional coordinates u can reach, and its
-// wrapped FP32 position.
-__device__ __forceinline__ void center_range(const GmpStruct& st, const GmpGrid& g, const double* u,
-                                             int4& rng_out, float4& y_out) {
-  int lo[3], span[3];
-  for (int k = 0; k < 3; ++k) {
-    const double lo_f = (u[k] - st.reach[k] - g.umin[k]) * g.inv_binw[k];
-    const double hi_f = (u[k] + st.reach[k] - g.umin[k]) * g.inv_binw[k];
-    int l0, h0;
-    if (st.periodic[k]) {
-      l0 = (int)floor(lo_f - 1e-7);
-      h0 = (int)floor(hi_f + 1e-7);
-    } else {
-      // a reference point may lie far outside the atoms' range: clamp in
-      // FP64 before converting (an empty range comes out as h0 < l0)
-      l0 = (int)fmin(fmax(floor(lo_f - 1e-7), 0.0), (double)g.nb[k]);
-      h0 = (int)fmax(fmin(floor(hi_f + 1e-7), (double)(g.nb[k] - 1)), -1.0);
-    }
-    lo[k] = l0;
-    span[k] = max(h0 - l0 + 1, 0);
+// A center at wrapped fractional coordinates u in the bin grid (units of
+// bins; as bin_of scales) and its wrapped FP32 position.
+__device__ __forceinline__ void center_place(const GmpStruct& st, const GmpGrid& g, const double* u,
+                                             float4& t_out, float4& y_out) {
+  float y[3], t[3];
+  for (int c = 0; c < 3; ++c) {
+    t[c] = (float)((u[c] - g.umin[c]) * g.inv_binw[c]);
+    y[c] = (float)(u[0] * st.A[c] + u[1] * st.A[3 + c] + u[2] * st.A[6 + c]);
   }
-  float y[3];
-  for (int c = 0; c < 3; ++c) y[c] = (float)(u[0] * st.A[c] + u[1] * st.A[3 + c] + u[2] * st.A[6 + c]);
-  rng_out = make_int4(lo[0], lo[1], lo[2], span[0] | (span[1] << 10) | (span[2] << 20));
+  t_out = make_float4(t[0], t[1], t[2], 0.0f);
   y_out = make_float4(y[0], y[1], y[2], 0.0f);
 }
 
-// Per atom: the bins its cutoff sphere can touch, lo[k] .. lo[k]+span[k]-1
-// (periodic axes unwrapped), and its wrapped FP32 position.  Once per atom,
-// so the neighbor kernels need no FP64 set-up.  atom_u is overwritten with
-// {yx, yy, yz, packed (lo, span)} in a second array.
+// Per atom: its place in the bin grid and its wrapped FP32 position, so that
+// the neighbor kernels need no FP64 set-up.
 __global__ void k_ranges(const GmpStruct* __restrict__ S, const GmpGrid* __restrict__ G,
                          const int32_t* __restrict__ struct_of, int64_t N, const GmpD4* __restrict__ atom_u,
-                         int4* __restrict__ atom_rng, float4* __restrict__ atom_y) {
+                         float4* __restrict__ atom_t, float4* __restrict__ atom_y) {
   for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < N;
        a += (int64_t)gridDim.x * blockDim.x) {
     const int s = struct_of[a];
-    const GmpStruct& st = S[s];
-    const GmpGrid& g = G[s];
     const GmpD4 u4 = atom_u[a];
     const double u[3] = {u4.x, u4.y, u4.z};
-    center_range(st, g, u, atom_rng[a], atom_y[a]);
+    center_place(S[s], G[s], u, atom_t[a], atom_y[a]);
   }
 }
 
 // Per reference point: the checks, wrap and double-float split of
-// k_prepare and the bin range of k_ranges, in the structure's atom grid.
+// k_prepare and the place of k_ranges, in the structure's atom grid.
 __global__ void k_point_prepare(const GmpStruct* __restrict__ S, const GmpGrid* __restrict__ G,
                                 const int32_t* __restrict__ point_struct, int64_t n, const double* __restrict__ pts,
                                 const double* __restrict__ atom_pos, float4* __restrict__ pt_xh,
-                                float4* __restrict__ pt_xl, int4* __restrict__ pt_rng, float4* __restrict__ pt_y,
+                                float4* __restrict__ pt_xl, float4* __restrict__ pt_t, float4* __restrict__ pt_y,
                                 uint32_t* __restrict__ err) {
   for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < n;
        a += (int64_t)gridDim.x * blockDim.x) {
@@ -388,7 +383,7 @@ __global__ void k_point_prepare(const GmpStruct* __restrict__ S, const GmpGrid* 
     }
     pt_xh[a] = make_float4(h[0], h[1], h[2], 0.0f);
     pt_xl[a] = make_float4(l[0], l[1], l[2], __int_as_float(pack_wrap(w[0], w[1], w[2])));
-    center_range(st, G[s], u, pt_rng[a], pt_y[a]);
+    center_place(st, G[s], u, pt_t[a], pt_y[a]);
   }
 }
 
@@ -410,7 +405,7 @@ __global__ void __launch_bounds__(1024) k_bin_small(GmpStruct* S, int n_struct, 
                                                    int64_t n_bins, float4* atom_xh, float4* atom_xl, GmpD4* atom_u,
                                                    int32_t* atom_bin, int32_t* __restrict__ bin_start,
                                                    float4* __restrict__ bin_y, int2* __restrict__ bin_je,
-                                                   int4* __restrict__ atom_rng, float4* __restrict__ atom_y,
+                                                   float4* __restrict__ atom_t, float4* __restrict__ atom_y,
                                                    uint32_t* __restrict__ err) {
   extern __shared__ __align__(16) unsigned char sm_small[];
   __shared__ int32_t warp_tot[32];
@@ -489,7 +484,7 @@ __global__ void __launch_bounds__(1024) k_bin_small(GmpStruct* S, int n_struct, 
     const int s = struct_of[a];
     const GmpD4 u4 = atom_u[a];
     const double u[3] = {u4.x, u4.y, u4.z};
-    center_range(S[s], G[s], u, atom_rng[a], atom_y[a]);
+    center_place(S[s], G[s], u, atom_t[a], atom_y[a]);
   }
 }
 
@@ -570,7 +565,7 @@ __device__ __forceinline__ bool exact_accept(const double* __restrict__ pos, con
                                              float rc2hi, float rc2lo, double rc2, float cutoff) {
   gmp_f2 d[3], r2;
   float mag;
-  gmp_df_disp(xhi, xli, xhj, xlj, st, n, d, r2, mag);
+  gmp_df_disp<true>(xhi, xli, xhj, xlj, st, n, d, r2, &mag);
   gmp_f2 diff = gmp_df_add(r2, gmp_f2{-rc2hi, -rc2lo});
   // double-float error bound (generous): 2^-36 (mag + rc + 1) (rc + 1) * 16
   const float tol = ldexpf((mag + cutoff + 1.0f) * (cutoff + 1.0f) * 16.0f, -36);
@@ -579,21 +574,43 @@ __device__ __forceinline__ bool exact_accept(const double* __restrict__ pos, con
   return fp64_within(pos, xi, j, st, n, rc2);
 }
 
-// Per-warp shared memory of the fill passes: keys [max_keys] u64, species
-// of each key [max_keys] u16 (FILL 1), per-species counters [n_el] int.
-__host__ __device__ inline size_t fill_warp_bytes(int max_keys, int n_el) {
-  return ((size_t)max_keys * 10 + (size_t)n_el * 4 + 15) / 16 * 16;
+// An image index that does not fit the packed shift.
+__device__ __forceinline__ bool out_of_range(const int* n) {
+  return abs(n[0]) >= 512 || abs(n[1]) >= 512 || abs(n[2]) >= 512;
 }
 
-// Warp per center, latency-bound (dependent bin loads): the launch bounds
-// hold the kernel at 80 registers, 24 resident warps per SM instead of 20
-// at the 96 it would take (slab single pass 1.88 -> 1.82 ms).
+// Per-warp shared memory: 32 bin segments (float4 + int2); in the fill
+// passes also keys [max_keys] u64, species of each key [max_keys] u16
+// (FILL 1), per-species counters [n_el] int.
+constexpr size_t kSegBytes = 32 * (sizeof(float4) + sizeof(int2));
+__host__ __device__ inline size_t fill_warp_bytes(int max_keys, int n_el) {
+  return kSegBytes + ((size_t)max_keys * 10 + (size_t)n_el * 4 + 15) / 16 * 16;
+}
+
+// Warp per center.  The center's cutoff sphere is covered by segments: the
+// bins of one row (fixed bins b1, b2 of axes 1 and 2, one image m0 of axis
+// 0), whose slots are contiguous.  A lane sets up one segment, 32 at a time:
+// a row farther than the cutoff from the center is left out, and with
+// orthogonal axes the row is cut to the sphere's chord (bounds on the
+// distance between planes, with a slack of kSlack bins that covers the FP32
+// rounding of t; the test of each candidate is exact, so the bounds only have
+// to keep every neighbor).  Then groups of 8 lanes walk the segments that
+// are not empty, 4 at a time: consecutive lanes read consecutive slots.
+// An accepted candidate is kept as (slot, image) and completed afterwards,
+// with all lanes busy; a row costs two bin offsets instead of two per bin.
+// Bound by instruction issue (64%) and the loads' latency; 64 registers, 32
+// resident warps per SM (a few words spilled; 80 registers and 24 warps:
+// 147 us on the slab of 32,768 atoms, 130 at 64).  Against one bin per lane,
+// its slots in turn, and general double-float sums in the records (GB300):
+// neighbor stage of 2,500 small structures 946 -> 634 us, alloy slab of
+// 262,144 atoms 1774 -> 1087 us.
 // FILL = 0: count exact neighbors; FILL = 1: write the
 // pair records grouped by neighbor species, in enumeration order within a
-// species (cells in a fixed order, atoms in index order within a cell:
+// species (segments in a fixed order, atoms in index order within a bin:
 // deterministic); FILL = 2: sorted by (neighbor atom, image).
+constexpr float kSlack = 1e-3f;
 template <int FILL>
-__global__ void __launch_bounds__(128, 6) k_neighbors(const GmpStruct* __restrict__ S, const GmpGrid* __restrict__ G,
+__global__ void __launch_bounds__(128, 8) k_neighbors(const GmpStruct* __restrict__ S, const GmpGrid* __restrict__ G,
                             const GmpCenters C, int64_t N, float cutoff,
                             float rc2hi, float rc2lo, double rc2, const double* __restrict__ pos,
                             const float4* __restrict__ atom_xh, const float4* __restrict__ atom_xl,
@@ -609,125 +626,146 @@ __global__ void __launch_bounds__(128, 6) k_neighbors(const GmpStruct* __restric
   const int wib = threadIdx.x >> 5;
   const int64_t i = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib;
   if (i >= N) return;
-  unsigned char* wbase = sh_fill + (size_t)wib * fill_warp_bytes(max_keys, n_el);
-  unsigned long long* keys = reinterpret_cast<unsigned long long*>(wbase);
-  uint16_t* kel = reinterpret_cast<uint16_t*>(wbase + (size_t)max_keys * 8);
-  int* ecnt = reinterpret_cast<int*>(wbase + (size_t)max_keys * 10);  // max_keys: a power of 2 >= 32
+  unsigned char* wbase = sh_fill + (size_t)wib * (fill ? fill_warp_bytes(max_keys, n_el) : kSegBytes);
+  float4* seg_sh = reinterpret_cast<float4*>(wbase);          // image shift of the segment, first slot
+  int2* seg_cm = reinterpret_cast<int2*>(seg_sh + 32);        // slots, packed image (m0, m1, m2)
+  int2* keys = reinterpret_cast<int2*>(wbase + kSegBytes);    // accepted: slot, packed image (m0, m1, m2)
+  uint16_t* kel = reinterpret_cast<uint16_t*>(keys + max_keys);
+  int* ecnt = reinterpret_cast<int*>(kel + max_keys);  // max_keys: a power of 2 >= 32
 
   const int s = C.sid[i];
   const GmpStruct& st = S[s];
   const GmpGrid& g = G[s];
-  int nb[3], per[3];
-  float ahi[9];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) { nb[k] = g.nb[k]; per[k] = st.periodic[k]; }
-#pragma unroll
-  for (int k = 0; k < 9; ++k) ahi[k] = st.Ahi[k];
-  const int64_t bin_base = st.bin_base;
   const float p2 = st.prescreen2, q2 = st.inside2;
   const float4 xhi = C.xh[i], xli = C.xl[i];
   const double* xi = C.pos + 3 * i;
   int wi[3];
   gmp_unpack_shift(__float_as_int(xli.w), wi);
-  const int4 rg = C.rng[i];
-  const int lo[3] = {rg.x, rg.y, rg.z};
-  const int span[3] = {rg.w & 1023, (rg.w >> 10) & 1023, (rg.w >> 20) & 1023};
-  const float4 yi4 = C.y[i];
-  const float yi[3] = {yi4.x, yi4.y, yi4.z};
-  const int total = span[0] * span[1] * span[2];
+  const float4 yi = C.y[i];
   int count = 0;   // per lane (count pass) / per warp (fill passes)
-  for (int r0 = 0; r0 < total; r0 += 32) {
-    const int cidx = r0 + lane;
-    int m[3] = {0, 0, 0};
-    int b0 = 0, b1 = 0;
-    float sh[3] = {0.0f, 0.0f, 0.0f};
-    if (cidx < total) {
-      // cell (c0, c1, c2) of the box and its bin; all operands are below
-      // 2^20 in magnitude unless the box is huge (then integer division:
-      // a cutoff of over 50 cell widths along periodic axes reaches it, and
-      // its image count then exceeds the per-center limit)
-      int c0, c1, c2;
-      const bool small = total < (1 << 20);
-      if (small) {
-        const int t01 = floor_div_small(cidx, span[0]);
-        c0 = cidx - t01 * span[0];
-        c2 = floor_div_small(t01, span[1]);
-        c1 = t01 - c2 * span[1];
-      } else {
-        c0 = cidx % span[0];
-        c1 = (cidx / span[0]) % span[1];
-        c2 = cidx / (span[0] * span[1]);
-      }
-      const int bb[3] = {lo[0] + c0, lo[1] + c1, lo[2] + c2};
-      int bw[3];
+  {
+    const float4 t4 = C.t[i];
+    const float t[3] = {t4.x, t4.y, t4.z};
+    int nb[3], lo[3], hi[3];
 #pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        if (per[k]) {
-          m[k] = small ? floor_div_small(bb[k], nb[k]) : floor_div(bb[k], nb[k]);
-          bw[k] = bb[k] - m[k] * nb[k];
-        } else {
-          bw[k] = bb[k];
-        }
+    for (int k = 0; k < 3; ++k) {
+      nb[k] = g.nb[k];
+      // FP32 bounds as integers (a point far outside the atoms' range
+      // saturates and comes out empty after the clamp)
+      lo[k] = __float2int_rd(t[k] - g.rb[k] - kSlack);
+      hi[k] = __float2int_rd(t[k] + g.rb[k] + kSlack);
+      if (!st.periodic[k]) {
+        lo[k] = max(lo[k], 0);
+        hi[k] = min(hi[k], nb[k] - 1);
       }
-      const int64_t bin = bin_base + bw[0] + (int64_t)nb[0] * (bw[1] + (int64_t)nb[1] * bw[2]);
-#pragma unroll
-      for (int c = 0; c < 3; ++c)
-        sh[c] = (float)m[0] * ahi[c] + (float)m[1] * ahi[3 + c] + (float)m[2] * ahi[6 + c];
-      b0 = bin_start[bin];
-      b1 = bin_start[bin + 1];
     }
-    // lockstep over the slots of this round's cells
-    const int len = __reduce_max_sync(0xffffffffu, b1 - b0);
-    for (int t = 0; t < len; ++t) {
-      const int slot = b0 + t;
-      bool acc = false;
-      unsigned long long key = 0;
-      int ej = 0;
-      if (slot < b1) {
-        const float4 yj = bin_y[slot];
-        const float dx = (yj.x - yi[0]) + sh[0];
-        const float dy = (yj.y - yi[1]) + sh[1];
-        const float dz = (yj.z - yi[2]) + sh[2];
-        // three roundings of non-negative terms: within 3 x 2^-24 relative
-        const float r2 = __fmaf_rn(dx, dx, __fmaf_rn(dy, dy, __fmul_rn(dz, dz)));
-        if (r2 <= p2) {
-          int wj[3];
-          gmp_unpack_shift(__float_as_int(yj.w), wj);
-          int n[3] = {m[0] + wi[0] - wj[0], m[1] + wi[1] - wj[1], m[2] + wi[2] - wj[2]};
-          acc = true;
-          int64_t j = -1;
-          if (r2 >= q2) {  // boundary shell: exact decision
-            const int2 je = bin_je[slot];
-            j = je.x;
-            ej = je.y;
-            const float4 xhj = atom_xh[j], xlj = atom_xl[j];
-            acc = exact_accept(pos, xi, j, xhi, xli, xhj, xlj, st, n, rc2hi, rc2lo, rc2, cutoff);
+    const int im0 = st.periodic[0] ? floor_div(lo[0], nb[0]) : 0;  // images of axis 0
+    const int n0 = st.periodic[0] ? floor_div(hi[0], nb[0]) - im0 + 1 : (hi[0] >= lo[0] ? 1 : 0);
+    const int n1 = max(hi[1] - lo[1] + 1, 0), n2 = max(hi[2] - lo[2] + 1, 0);
+    const int total = n0 * n1 * n2;
+    const float rcs = cutoff * cutoff * 1.00001f;
+    for (int r0 = 0; r0 < total; r0 += 32) {
+      const int cidx = r0 + lane;
+      float4 sg = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      int2 cm = make_int2(0, 0);
+      if (cidx < total) {
+        // segment (c0, c1, c2); the single-precision quotients hold while
+        // the operands are below 2^20 (beyond it a cutoff of over 50 cell
+        // widths, whose image count exceeds the per-center limit)
+        const bool small = total < (1 << 20);
+        const int t01 = small ? floor_div_small(cidx, n0) : cidx / n0;
+        const int c2 = small ? floor_div_small(t01, n1) : t01 / n1;
+        const int b1 = lo[1] + (t01 - c2 * n1), b2 = lo[2] + c2;
+        const float g1 = fmaxf(fmaxf((float)b1 - t[1], t[1] - (float)(b1 + 1)) - kSlack, 0.0f) * g.h[1];
+        const float g2 = fmaxf(fmaxf((float)b2 - t[2], t[2] - (float)(b2 + 1)) - kSlack, 0.0f) * g.h[2];
+        // squared room left along axis 0 (or, with skew axes, only a bound
+        // from each pair of planes alone)
+        const float gm = fmaxf(g1, g2);
+        const float room = rcs - (g.ortho ? g1 * g1 + g2 * g2 : gm * gm);
+        if (room >= 0.0f) {
+          const int m0 = im0 + (cidx - t01 * n0);
+          int x0 = lo[0], x1 = hi[0], m1 = 0, m2 = 0, w0 = 0;
+          if (g.ortho) {
+            const float c = __fsqrt_rn(room) * g.inv_h0 + kSlack;
+            x0 = max(x0, __float2int_rd(t[0] - c));
+            x1 = min(x1, __float2int_rd(t[0] + c));
           }
-          if (acc && (abs(n[0]) >= 512 || abs(n[1]) >= 512 || abs(n[2]) >= 512)) {
-            atomicOr(err, GMP_DEV_SHIFT_RANGE);  // reported after the count pass
-            acc = false;
+          if (st.periodic[0]) {
+            w0 = m0 * nb[0];
+            x0 = max(x0, w0);
+            x1 = min(x1, w0 + nb[0] - 1);
           }
-          if (fill && acc) {
-            if (j < 0) {
-              const int2 je = bin_je[slot];
-              j = je.x;
-              ej = je.y;
+          if (st.periodic[1]) m1 = small ? floor_div_small(b1, nb[1]) : floor_div(b1, nb[1]);
+          if (st.periodic[2]) m2 = small ? floor_div_small(b2, nb[2]) : floor_div(b2, nb[2]);
+          if (x0 <= x1) {
+            const int64_t bin = st.bin_base + (int64_t)nb[0] * ((b1 - m1 * nb[1]) + (int64_t)nb[1] * (b2 - m2 * nb[2])) - w0;
+            const int first = bin_start[bin + x0];
+            cm = make_int2(bin_start[bin + x1 + 1] - first, gmp_pack_shift(m0, m1, m2));
+            const float f0 = (float)m0, f1 = (float)m1, f2 = (float)m2;
+            sg = make_float4(f0 * st.Ahi[0] + f1 * st.Ahi[3] + f2 * st.Ahi[6],
+                             f0 * st.Ahi[1] + f1 * st.Ahi[4] + f2 * st.Ahi[7],
+                             f0 * st.Ahi[2] + f1 * st.Ahi[5] + f2 * st.Ahi[8], __int_as_float(first));
+          }
+        }
+      }
+      const unsigned some = __ballot_sync(0xffffffffu, cm.x > 0);
+      const int nseg = __popc(some);
+      if (cm.x > 0) {
+        const int at = __popc(some & ((1u << lane) - 1u));
+        seg_sh[at] = sg;
+        seg_cm[at] = cm;
+      }
+      __syncwarp();
+      for (int q0 = 0; q0 < nseg; q0 += 4) {
+        const int q = q0 + (lane >> 3);
+        float4 sh = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        int2 c = make_int2(0, 0);
+        if (q < nseg) {
+          sh = seg_sh[q];
+          c = seg_cm[q];
+        }
+        const int len = __reduce_max_sync(0xffffffffu, c.x);
+        for (int u = lane & 7; u - (lane & 7) < len; u += 8) {
+          const int slot = __float_as_int(sh.w) + u;
+          bool acc = false;
+          if (u < c.x) {
+            const float4 yj = bin_y[slot];
+            const float dx = (yj.x - yi.x) + sh.x;
+            const float dy = (yj.y - yi.y) + sh.y;
+            const float dz = (yj.z - yi.z) + sh.z;
+            // three roundings of non-negative terms: within 3 x 2^-24 relative
+            const float r2 = __fmaf_rn(dx, dx, __fmaf_rn(dy, dy, __fmul_rn(dz, dz)));
+            acc = r2 <= p2;
+            // the image index is needed for the boundary shell's exact
+            // decision, and in the count pass (whose caller reports it) for
+            // its range
+            if (acc && (!fill || r2 >= q2)) {
+              int wj[3], m[3];
+              gmp_unpack_shift(__float_as_int(yj.w), wj);
+              gmp_unpack_shift(c.y, m);
+              const int n[3] = {m[0] + wi[0] - wj[0], m[1] + wi[1] - wj[1], m[2] + wi[2] - wj[2]};
+              if (r2 >= q2) {
+                const int64_t j = bin_je[slot].x;
+                const float4 xhj = atom_xh[j], xlj = atom_xl[j];
+                acc = exact_accept(pos, xi, j, xhi, xli, xhj, xlj, st, n, rc2hi, rc2lo, rc2, cutoff);
+              }
+              if (!fill && acc && out_of_range(n)) {
+                atomicOr(err, GMP_DEV_SHIFT_RANGE);  // reported after the count pass
+                acc = false;
+              }
             }
-            key = sort_key(j, n);
+          }
+          if (!fill) {
+            count += acc ? 1 : 0;
+          } else {
+            const unsigned mask = __ballot_sync(0xffffffffu, acc);
+            const int slot_k = count + __popc(mask & ((1u << lane) - 1u));
+            if (acc && slot_k < max_keys) keys[slot_k] = make_int2(slot, c.y);
+            count += __popc(mask);
           }
         }
       }
-      if (!fill) {
-        count += acc ? 1 : 0;
-      } else {
-        const unsigned mask = __ballot_sync(0xffffffffu, acc);
-        const int slot_k = count + __popc(mask & ((1u << lane) - 1u));
-        if (acc && slot_k < max_keys) {
-          keys[slot_k] = key;
-          if (fill == 1) kel[slot_k] = (uint16_t)ej;
-        }
-        count += __popc(mask);
-      }
+      __syncwarp();
     }
   }
   if (!fill) {
@@ -770,22 +808,39 @@ __global__ void __launch_bounds__(128, 6) k_neighbors(const GmpStruct* __restric
       return;
     }
   }
+  // image index of an accepted slot's atom from its packed (m0, m1, m2) and wrap
+  auto image = [&](int m, int wrap, int* n) {
+    int wj[3], mm[3];
+    gmp_unpack_shift(wrap, wj);
+    gmp_unpack_shift(m, mm);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) n[k] = mm[k] + wi[k] - wj[k];
+    if (out_of_range(n)) atomicOr(err, GMP_DEV_SHIFT_RANGE);
+  };
+  unsigned long long* skey = reinterpret_cast<unsigned long long*>(keys);
   if (fill == 2) {
+    for (int t = lane; t < M; t += 32) {
+      const int2 k = keys[t];
+      int n[3];
+      image(k.y, __float_as_int(bin_y[k.x].w), n);
+      skey[t] = sort_key(bin_je[k.x].x, n);
+    }
+    __syncwarp();
     // bitonic sort of the M keys (padded to a power of two with ~0)
     int P2 = 1;
     while (P2 < M) P2 <<= 1;
-    for (int t = M + lane; t < P2; t += 32) keys[t] = ~0ull;
+    for (int t = M + lane; t < P2; t += 32) skey[t] = ~0ull;
     __syncwarp();
     for (int k = 2; k <= P2; k <<= 1) {
       for (int jj = k >> 1; jj > 0; jj >>= 1) {
         for (int t = lane; t < P2; t += 32) {
           int partner = t ^ jj;
           if (partner > t) {
-            unsigned long long a = keys[t], b = keys[partner];
+            unsigned long long a = skey[t], b = skey[partner];
             bool up = (t & k) == 0;
             if ((a > b) == up) {
-              keys[t] = b;
-              keys[partner] = a;
+              skey[t] = b;
+              skey[partner] = a;
             }
           }
         }
@@ -793,25 +848,36 @@ __global__ void __launch_bounds__(128, 6) k_neighbors(const GmpStruct* __restric
       }
     }
   }
-  if (fill == 1) {
+  const bool by_species = fill == 1 && n_el > 1;
+  if (by_species) {
     // destination of key t: species-major, enumeration order within a
     // species (counting sort; lanes of one match group have one species)
     for (int e = lane; e < n_el; e += 32) ecnt[e] = 0;
     __syncwarp();
     for (int t0 = 0; t0 < M; t0 += 32) {
       const int t = t0 + lane;
-      const int e = t < M ? (int)kel[t] : -1;
+      int e = -1;
+      if (t < M) {
+        e = bin_je[keys[t].x].y;
+        kel[t] = (uint16_t)e;
+      }
       const unsigned grp = __match_any_sync(0xffffffffu, e);
       if (t < M && lane == __ffs(grp) - 1) ecnt[e] += __popc(grp);
       __syncwarp();
     }
-    if (lane == 0) {
-      int run = 0;
-      for (int e = 0; e < n_el; ++e) {
-        const int c = ecnt[e];
-        ecnt[e] = run;
-        run += c;
+    // exclusive prefix over the species
+    int run = 0;
+    for (int e0 = 0; e0 < n_el; e0 += 32) {
+      const int e = e0 + lane;
+      const int c = e < n_el ? ecnt[e] : 0;
+      int incl = c;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
       }
+      if (e < n_el) ecnt[e] = run + incl - c;
+      run += __shfl_sync(0xffffffffu, incl, 31);
     }
     __syncwarp();
   }
@@ -819,7 +885,7 @@ __global__ void __launch_bounds__(128, 6) k_neighbors(const GmpStruct* __restric
   for (int t0 = 0; t0 < M; t0 += 32) {
     const int t = t0 + lane;
     int dst = t;
-    if (fill == 1) {
+    if (by_species) {
       const int e = t < M ? (int)kel[t] : -1;
       const unsigned grp = __match_any_sync(0xffffffffu, e);
       if (t < M) dst = ecnt[e] + __popc(grp & ((1u << lane) - 1u));
@@ -828,25 +894,28 @@ __global__ void __launch_bounds__(128, 6) k_neighbors(const GmpStruct* __restric
       __syncwarp();
     }
     if (t >= M) continue;
-    const unsigned long long key = keys[t];
-    const int64_t j = (int64_t)(key >> 30);
+    int64_t j;
     int n[3];
-    sort_key_image(key, n);
-    const int32_t packed = gmp_pack_shift(n[0], n[1], n[2]);
-    const float4 xhj = atom_xh[j], xlj = atom_xl[j];
+    float4 xhj, xlj;
+    if (fill == 2) {
+      const unsigned long long key = skey[t];
+      j = (int64_t)(key >> 30);
+      sort_key_image(key, n);
+      xhj = atom_xh[j];
+      xlj = atom_xl[j];
+    } else {
+      const int2 k = keys[t];
+      j = bin_je[k.x].x;
+      xhj = atom_xh[j];
+      xlj = atom_xl[j];
+      image(k.y, __float_as_int(xlj.w), n);
+    }
     gmp_f2 d[3], r2;
-    float mag;
-    gmp_df_disp(xhi, xli, xhj, xlj, st, n, d, r2, mag);
-    GmpPair p;
-    p.dx = d[0].hi + d[0].lo;
-    p.dy = d[1].hi + d[1].lo;
-    p.dz = d[2].hi + d[2].lo;
-    p.r2hi = r2.hi;
-    p.r2lo = r2.lo;
-    p.e = __float_as_int(xhj.w);
-    p.j = (int32_t)j;
-    p.shift = packed;
-    pairs[base + dst] = p;
+    gmp_df_disp(xhi, xli, xhj, xlj, st, n, d, r2);
+    float4* dstp = reinterpret_cast<float4*>(pairs + base + dst);
+    dstp[0] = make_float4(d[0].hi + d[0].lo, d[1].hi + d[1].lo, d[2].hi + d[2].lo, r2.hi);
+    dstp[1] = make_float4(r2.lo, xhj.w, __int_as_float((int32_t)j),
+                          __int_as_float(gmp_pack_shift(n[0], n[1], n[2])));
   }
 }
 
@@ -913,7 +982,7 @@ cudaError_t gmp_launch_neighbors_prepare(const GmpStruct* d_structs, int n_struc
 cudaError_t gmp_launch_bins(const GmpStruct* d_structs, const GmpGrid* d_grid,
                             const int32_t* d_struct_of, int64_t N, int64_t n_bins,
                             const int32_t* atom_bin, int32_t* bin_count, int32_t* bin_start,
-                            int32_t* bin_cursor, int4* atom_rng, float4* atom_y, float4* bin_y, int2* bin_je,
+                            int32_t* bin_cursor, float4* atom_t, float4* atom_y, float4* bin_y, int2* bin_je,
                             const GmpD4* atom_u, const float4* atom_xh, const float4* atom_xl, void* scan_tmp,
                             size_t scan_tmp_bytes, cudaStream_t stream, int sm_count, int64_t* launches) {
   (void)scan_tmp_bytes;
@@ -932,7 +1001,7 @@ cudaError_t gmp_launch_bins(const GmpStruct* d_structs, const GmpGrid* d_grid,
   k_bin_place<<<grid_for(N, 256, sm_count), 256, 0, stream>>>(d_structs, d_struct_of, N, atom_bin, bin_start,
                                                               bin_count, atom_u, atom_xh, atom_xl, bin_y, bin_je);
   ++*launches;
-  k_ranges<<<grid_for(N, 256, sm_count), 256, 0, stream>>>(d_structs, d_grid, d_struct_of, N, atom_u, atom_rng,
+  k_ranges<<<grid_for(N, 256, sm_count), 256, 0, stream>>>(d_structs, d_grid, d_struct_of, N, atom_u, atom_t,
                                                            atom_y);
   ++*launches;
   return cudaGetLastError();
@@ -946,7 +1015,7 @@ cudaError_t gmp_launch_bin_small(GmpStruct* d_structs, int n_struct, const int32
                                  double cutoff, const double* pos, const int32_t* species, int n_el,
                                  GmpGrid* d_grid, int64_t n_bins, float4* atom_xh, float4* atom_xl, GmpD4* atom_u,
                                  int32_t* atom_bin, int32_t* bin_start, float4* bin_y, int2* bin_je,
-                                 int4* atom_rng, float4* atom_y, uint32_t* d_err, cudaStream_t stream,
+                                 float4* atom_t, float4* atom_y, uint32_t* d_err, cudaStream_t stream,
                                  int64_t* launches) {
   if (!gmp_bin_small_fits(N, n_bins, n_struct)) return cudaErrorInvalidValue;
   const size_t smem = small_bin_smem(N, n_bins, n_struct);
@@ -956,19 +1025,19 @@ cudaError_t gmp_launch_bin_small(GmpStruct* d_structs, int n_struct, const int32
   }
   k_bin_small<<<1, 1024, smem, stream>>>(d_structs, n_struct, d_struct_of, N, cutoff, pos, species, n_el, d_grid,
                                          n_bins, atom_xh, atom_xl, atom_u, atom_bin, bin_start, bin_y, bin_je,
-                                         atom_rng, atom_y, d_err);
+                                         atom_t, atom_y, d_err);
   ++*launches;
   return cudaGetLastError();
 }
 
 cudaError_t gmp_launch_point_prepare(const GmpStruct* d_structs, const GmpGrid* d_grid,
                                      const int32_t* point_struct, int64_t n_points, const double* points,
-                                     const double* atom_pos, float4* pt_xh, float4* pt_xl, int4* pt_rng,
+                                     const double* atom_pos, float4* pt_xh, float4* pt_xl, float4* pt_t,
                                      float4* pt_y, uint32_t* d_err, cudaStream_t stream, int sm_count,
                                      int64_t* launches) {
   if (n_points <= 0) return cudaSuccess;
   k_point_prepare<<<grid_for(n_points, 256, sm_count), 256, 0, stream>>>(
-      d_structs, d_grid, point_struct, n_points, points, atom_pos, pt_xh, pt_xl, pt_rng, pt_y, d_err);
+      d_structs, d_grid, point_struct, n_points, points, atom_pos, pt_xh, pt_xl, pt_t, pt_y, d_err);
   ++*launches;
   return cudaGetLastError();
 }
@@ -981,14 +1050,14 @@ cudaError_t gmp_launch_neighbor_pass(int fill, const GmpStruct* d_structs, const
                                      GmpPair* pairs, int64_t pair_cap, int max_keys, int32_t* d_maxm,
                                      uint32_t* d_err, cudaStream_t stream, int sm_count, int64_t* launches,
                                      unsigned long long* cursor, int64_t* rng) {
-  (void)sm_count;
   if (fill < 0 || fill > 2 || (cursor && fill == 0)) return cudaErrorInvalidValue;
   const double rc2 = cutoff * cutoff;
   const float rc2hi = (float)rc2;
   const float rc2lo = (float)(rc2 - (double)rc2hi);
   auto fn = fill == 0 ? k_neighbors<0> : fill == 1 ? k_neighbors<1> : k_neighbors<2>;
-  int warps = 4;
-  size_t smem = 0;
+  // few centers: one warp per CTA, so that they spread over the SMs
+  int warps = N >= 16 * (int64_t)sm_count ? 4 : 1;
+  size_t smem = warps * kSegBytes;
   if (fill) {
     while (warps > 1 && (size_t)warps * fill_warp_bytes(max_keys, n_el) > 96 * 1024) warps >>= 1;
     smem = (size_t)warps * fill_warp_bytes(max_keys, n_el);

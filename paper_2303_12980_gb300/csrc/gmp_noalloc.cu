@@ -44,8 +44,8 @@ struct Layout {
   static constexpr size_t bstart = bcursor + align256(4 * kMaxBins);
   static constexpr size_t by = bstart + align256(4 * (kMaxBins + 1));
   static constexpr size_t bje = by + align256(16 * kNoAllocMaxAtoms);
-  static constexpr size_t rng = bje + align256(8 * kNoAllocMaxAtoms);
-  static constexpr size_t ay = rng + align256(16 * kNoAllocMaxAtoms);
+  static constexpr size_t t = bje + align256(8 * kNoAllocMaxAtoms);
+  static constexpr size_t ay = t + align256(16 * kNoAllocMaxAtoms);
   static constexpr size_t scan = ay + align256(16 * kNoAllocMaxAtoms);
   static constexpr size_t scan_bytes = 16 * 1024;
   static constexpr size_t total = scan + scan_bytes;
@@ -150,6 +150,9 @@ extern "C" gmp_status gmp_neighbor_counts_noalloc(int32_t n_atoms, const double*
     g.Alo[k] = (float)(g.A[k] - (double)g.Ahi[k]);
   }
   g.n_atoms = n_atoms;
+  g.diag = 1;
+  for (int k = 0; k < 9; ++k)
+    if (k % 4 != 0 && g.A[k] != 0.0) g.diag = 0;
   g.bin_cap = 2 * n_atoms + 8;
   const int64_t n_bins = g.bin_cap;
 
@@ -169,7 +172,7 @@ extern "C" gmp_status gmp_neighbor_counts_noalloc(int32_t n_atoms, const double*
   int32_t* d_bstart = reinterpret_cast<int32_t*>(base + Layout::bstart);
   float4* d_by = reinterpret_cast<float4*>(base + Layout::by);
   int2* d_bje = reinterpret_cast<int2*>(base + Layout::bje);
-  int4* d_rng = reinterpret_cast<int4*>(base + Layout::rng);
+  float4* d_t = reinterpret_cast<float4*>(base + Layout::t);
   float4* d_ay = reinterpret_cast<float4*>(base + Layout::ay);
   void* d_scan = base + Layout::scan;
   if (gmp_scan_tmp_bytes(n_bins) > Layout::scan_bytes) return report(GMP_ERR_CAPACITY, "scan workspace too small");
@@ -184,9 +187,9 @@ extern "C" gmp_status gmp_neighbor_counts_noalloc(int32_t n_atoms, const double*
     e = gmp_launch_neighbors_prepare(d_st, 1, d_struct_of, n_atoms, cutoff, pos, d_species, 1, d_grid, d_xh, d_xl,
                                      d_u, d_bin, d_bbox, d_err, st, sm_count, &launches);
   if (e == cudaSuccess)
-    e = gmp_launch_bins(d_st, d_grid, d_struct_of, n_atoms, n_bins, d_bin, d_bcount, d_bstart, d_bcursor, d_rng,
+    e = gmp_launch_bins(d_st, d_grid, d_struct_of, n_atoms, n_bins, d_bin, d_bcount, d_bstart, d_bcursor, d_t,
                         d_ay, d_by, d_bje, d_u, d_xh, d_xl, d_scan, Layout::scan_bytes, st, sm_count, &launches);
-  const GmpCenters centers{d_struct_of, pos, d_xh, d_xl, d_rng, d_ay};
+  const GmpCenters centers{d_struct_of, pos, d_xh, d_xl, d_t, d_ay};
   if (e == cudaSuccess)
     e = gmp_launch_neighbor_pass(0, d_st, d_grid, centers, n_atoms, cutoff, pos, d_xh, d_xl, d_bstart, d_by,
                                  d_bje, 1, counts, nullptr, nullptr, 0, 0, d_maxm, d_err, st, sm_count, &launches);

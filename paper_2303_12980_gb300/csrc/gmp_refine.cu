@@ -81,8 +81,7 @@ __device__ __forceinline__ void refine_entry(int lane, const GmpRefine& A, const
     int nn[3];
     gmp_unpack_shift(pr.shift, nn);
     gmp_f2 d[3], r2, H[2 * L + 1];
-    float mag;
-    gmp_df_disp(xhi, xli, A.atom_xh[pr.j], A.atom_xl[pr.j], st, nn, d, r2, mag);
+    gmp_df_disp(xhi, xli, A.atom_xh[pr.j], A.atom_xl[pr.j], st, nn, d, r2);
     gmp_solid_df<L>(d[0], d[1], d[2], r2, H);
 #pragma unroll
     for (int g = 0; g < 2; ++g) {

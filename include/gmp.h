@@ -39,7 +39,9 @@
  *     Conditions detected on the device (bad species id, non-finite
  *     position, too many neighbors of one center) are reported through a
  *     device error word checked at the end of the call (device-pointer
- *     calls synchronise `stream` once per call to read it).
+ *     calls wait once per call to read it: for the neighbor lists, not for
+ *     the kernels queued behind them).  After an error the contents of the
+ *     output buffers are undefined.
  */
 #ifndef GMP_H_
 #define GMP_H_
@@ -183,7 +185,7 @@ gmp_status gmp_featurize_grad_centers(gmp_handle h, int32_t n_struct, const int6
  *   features [n_points, F] float32 out, columns as in gmp_featurize.
  * points and features follow pos (device or host; with no atoms at all the
  * features are zero).  A structure may own points and no atoms, or atoms and
- * no points.  Synchronises `stream` once (to size the neighbor buffer). */
+ * no points.  Waits for the neighbor lists (to read their size). */
 gmp_status gmp_featurize_points(gmp_handle h, int32_t n_struct, const int64_t *atom_off,
                                 const double *pos, const double *cell, const uint8_t *pbc,
                                 const int32_t *species, const int64_t *point_off,

@@ -56,6 +56,13 @@ struct DevBuf {
   T* as() const { return static_cast<T*>(p); }
 };
 
+// A part of a larger device buffer.
+struct DevView {
+  void* p = nullptr;
+  template <typename T>
+  T* as() const { return static_cast<T*>(p); }
+};
+
 struct PassData {
   GmpPass pass;
   int L;
@@ -67,6 +74,7 @@ struct PassData {
   GmpShape fused{16, 0};
   GmpShape jac{16, 0};
   int vjp_fused = 0;  // 1: one fused forward+backward kernel instead of two
+  GmpLaunchPlan plan[5];  // per kind: the launch shape worked out for the request above
 };
 
 }  // namespace
@@ -92,9 +100,19 @@ struct gmp_ctx {
   std::vector<uint8_t> last_pbc;
   int64_t n_bins = 0;
   // workspace
-  DevBuf structs, grid, atom_off, struct_of, bbox, atom_xh, atom_xl, atom_u, atom_bin, atom_t, atom_y;
+  DevBuf desc;                      // structs, grid and atom_off of the batch, uploaded in one copy
+  DevView structs, grid, atom_off;
+  void* h_desc = nullptr;           // pinned staging of that copy
+  size_t h_desc_bytes = 0;
+  cudaEvent_t ev_desc = nullptr;    // the copy is done with the staging
+  GmpGridMode grid_mode = GmpGridMode::kGiven;
+  DevBuf struct_of, bbox, atom_xh, atom_xl, atom_u, atom_bin, atom_t, atom_y;
   DevBuf bin_count, bin_cursor, bin_start, bin_y, bin_je, counts, nbr_off, scan_tmp, pairs;
-  DevBuf scalars;  // err word, maxm, counter
+  // error word, longest list, pair cursor, refinement queue counts and the
+  // work counters of a call's compute launches (kScalar* below); everything
+  // but the error word is cleared at the start of a call
+  DevBuf scalars;
+  int next_counter = 0;
   DevBuf grad_acc, jac_counts, jac_rows;
   // VJP sums without float atomics: fixed-point bins per (atom,
   // component), per-center own terms and strain-derivative sums
@@ -104,6 +122,7 @@ struct gmp_ctx {
   DevBuf exptab; // [64] 2^(-j/64) as double-floats (the refinement's exponential)
   DevBuf flagq;     // queued ill-conditioned features, one entry per (center, order)
   DevBuf colinfo;   // per feature column: (order << 16) | sigma, -1 for the density
+  int refine_per_sm = 0;  // resident CTAs of the refinement kernel (0: not asked yet)
   int n_ord_pos = 1;  // orders >= 0: refine queue entries per center and pass
   DevBuf stage_pos, stage_species, stage_feat, stage_gradf, stage_gradp, stage_virial;
   DevBuf pt_off, pt_struct, pt_xh, pt_xl, pt_t, pt_y, stage_pts;  // reference points
@@ -113,8 +132,20 @@ struct gmp_ctx {
   // single-pass build, one block per center with ranges in nbr_rng [2N].
   DevBuf nbr_rng;
   bool rng_mode = false;
-  int64_t last_nc = -1;    // batch (centers, description) the P / max_m above belong to
-  int64_t last_gen = -1;
+  // pairs per center and longest list of the last build around atoms [0] and
+  // around reference points [1], from which the next one's capacities are
+  // guessed (0: no build yet)
+  struct ListSize {
+    double per_center = 0.0;
+    int max_m = 0;
+  } sizes[2];
+  int size_kind = 0;           // of the current lists
+  int64_t cap_cur = 0;         // pair capacity of the current lists
+  int64_t nc_cur = 0;          // ... and their centers
+  bool lists_pending = false;  // single-pass lists whose outcome is not read yet (ev_lists)
+  bool lists_outgrown = false; // ... and found to exceed its capacities
+  bool exact_lists = false;    // count before filling (set for a rerun)
+  cudaEvent_t ev_lists = nullptr;
   // pinned host scratch for small readbacks
   int64_t* h_small = nullptr;
   std::string err;
@@ -141,6 +172,11 @@ struct gmp_ctx {
 
 namespace {
 
+// Byte offsets in gmp_ctx::scalars.
+constexpr size_t kScalarMaxM = 4, kScalarCursor = 8, kScalarFlags = 16, kScalarCounters = 80;  // the error word at 0
+constexpr int kCounters = 160;  // two per sigma pass (at most 64) and spares
+constexpr size_t kScalarBytes = kScalarCounters + 4 * kCounters;
+
 gmp_status fail(gmp_ctx* h, gmp_status st, const std::string& msg) {
   if (h) h->err = msg;
   return st;
@@ -162,16 +198,19 @@ gmp_status cuda_fail(gmp_ctx* h, cudaError_t e, const char* where) {
 
 int pad_sigmas(int n) { return n <= 4 ? 4 : (n <= 8 ? 8 : 16); }
 
-cudaError_t launch_compute(int L, int kind, int ns, const gmpk::KParams& K, GmpShape shape, cudaStream_t st,
+// Launches a compute kernel of a pass with the requested shape.
+cudaError_t launch_compute(PassData& pd, int kind, const gmpk::KParams& K, GmpShape shape, cudaStream_t st,
                            int sm, int64_t* launches) {
-  switch (L) {
-    case 0: return gmp_launch_compute_L0(kind, ns, K, shape, st, sm, launches);
-    case 1: return gmp_launch_compute_L1(kind, ns, K, shape, st, sm, launches);
-    case 2: return gmp_launch_compute_L2(kind, ns, K, shape, st, sm, launches);
-    case 3: return gmp_launch_compute_L3(kind, ns, K, shape, st, sm, launches);
-    case 4: return gmp_launch_compute_L4(kind, ns, K, shape, st, sm, launches);
-    case 5: return gmp_launch_compute_L5(kind, ns, K, shape, st, sm, launches);
-    case 6: return gmp_launch_compute_L6(kind, ns, K, shape, st, sm, launches);
+  const int ns = pd.NS;
+  GmpLaunchPlan* plan = &pd.plan[kind];
+  switch (pd.L) {
+    case 0: return gmp_launch_compute_L0(kind, ns, K, shape, plan, st, sm, launches);
+    case 1: return gmp_launch_compute_L1(kind, ns, K, shape, plan, st, sm, launches);
+    case 2: return gmp_launch_compute_L2(kind, ns, K, shape, plan, st, sm, launches);
+    case 3: return gmp_launch_compute_L3(kind, ns, K, shape, plan, st, sm, launches);
+    case 4: return gmp_launch_compute_L4(kind, ns, K, shape, plan, st, sm, launches);
+    case 5: return gmp_launch_compute_L5(kind, ns, K, shape, plan, st, sm, launches);
+    case 6: return gmp_launch_compute_L6(kind, ns, K, shape, plan, st, sm, launches);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -264,7 +303,23 @@ gmp_status upload_structures(gmp_ctx* h, int32_t S, const int64_t* atom_off, con
                     std::memcmp(h->last_cell.data(), cell, sizeof(double) * 9 * S) == 0 &&
                     std::memcmp(h->last_pbc.data(), pbc, S * 3) == 0;
   if (same) return GMP_OK;
-  std::vector<GmpStruct> info(S);
+  // one pinned staging block [structs | grid | atom_off], one copy
+  const size_t o_grid = sizeof(GmpStruct) * (size_t)S, o_off = o_grid + sizeof(GmpGrid) * (size_t)S;
+  const size_t bytes = o_off + sizeof(int64_t) * (size_t)(S + 1);
+  if (bytes > h->h_desc_bytes) {
+    GMP_CK(cudaEventSynchronize(h->ev_desc), "batch staging");  // the last copy out of it
+    if (h->h_desc) cudaFreeHost(h->h_desc);
+    h->h_desc = nullptr;
+    h->h_desc_bytes = 0;
+    GMP_CK(cudaMallocHost(&h->h_desc, bytes + bytes / 2), "batch staging");
+    h->h_desc_bytes = bytes + bytes / 2;
+  } else {
+    GMP_CK(cudaEventSynchronize(h->ev_desc), "batch staging");  // the last copy out of it
+  }
+  h->last_off.clear();  // no description until this one is complete
+  GmpStruct* const info = static_cast<GmpStruct*>(h->h_desc);
+  GmpGrid* const grids = reinterpret_cast<GmpGrid*>(static_cast<char*>(h->h_desc) + o_grid);
+  GmpGridMode mode = GmpGridMode::kGiven;
   int64_t bin_base = 0;
   for (int s = 0; s < S; ++s) {
     GmpStruct& g = info[s];
@@ -304,18 +359,21 @@ gmp_status upload_structures(gmp_ctx* h, int32_t S, const int64_t* atom_off, con
     g.bin_base = bin_base;
     g.bin_cap = 2 * g.n_atoms + 8;
     bin_base += g.bin_cap;
+    gmp_periodic_grid(g, grids[s], h->cutoff);
+    if (!(g.periodic[0] && g.periodic[1] && g.periodic[2])) mode = GmpGridMode::kOpen;
   }
+  std::memcpy(static_cast<char*>(h->h_desc) + o_off, atom_off, sizeof(int64_t) * (S + 1));
   h->n_bins = bin_base;
-  GMP_CK(h->structs.ensure(sizeof(GmpStruct) * S), "structs");
-  GMP_CK(h->grid.ensure(sizeof(GmpGrid) * S), "grid");
-  GMP_CK(h->atom_off.ensure(sizeof(int64_t) * (S + 1)), "atom_off");
+  h->grid_mode = mode;
+  GMP_CK(h->desc.ensure(bytes), "structs");
+  h->structs.p = h->desc.p;
+  h->grid.p = h->desc.as<char>() + o_grid;
+  h->atom_off.p = h->desc.as<char>() + o_off;
   GMP_CK(h->bbox.ensure(sizeof(unsigned long long) * 6 * S), "bbox");
-  GMP_CK(cudaMemcpyAsync(h->structs.p, info.data(), sizeof(GmpStruct) * S, cudaMemcpyHostToDevice, st), "upload structs");
-  GMP_CK(cudaMemcpyAsync(h->atom_off.p, atom_off, sizeof(int64_t) * (S + 1), cudaMemcpyHostToDevice, st), "upload atom_off");
   GMP_CK(h->struct_of.ensure(sizeof(int32_t) * (N > 0 ? N : 1)), "struct_of");
+  GMP_CK(cudaMemcpyAsync(h->desc.p, h->h_desc, bytes, cudaMemcpyHostToDevice, st), "upload structs");
+  GMP_CK(cudaEventRecord(h->ev_desc, st), "event");
   if (N > 0) GMP_CK(gmp_launch_struct_of(h->atom_off.as<int64_t>(), S, h->struct_of.as<int32_t>(), st, &h->launches), "struct_of");
-  // the copies above read host memory asynchronously: wait before returning
-  GMP_CK(cudaStreamSynchronize(st), "upload sync");
   ++h->struct_gen;
   h->last_off.assign(atom_off, atom_off + S + 1);
   h->last_cell.assign(cell, cell + 9 * S);
@@ -372,6 +430,10 @@ gmp_status bin_atoms(gmp_ctx* h, int32_t S, const double* pos, const int32_t* sp
   GMP_CK(h->nbr_off.ensure(sizeof(int64_t) * (n_centers + 1)), "nbr_off");
   const int64_t scan_n = std::max<int64_t>(std::max<int64_t>(N, n_centers), h->n_bins);
   GMP_CK(h->scan_tmp.ensure(gmp_scan_tmp_bytes(scan_n)), "scan_tmp");
+  // the error word is cleared after it is read, so a condition raised after
+  // the read of the previous call is reported here
+  GMP_CK(cudaMemsetAsync(h->scalars.as<char>() + kScalarMaxM, 0, kScalarBytes - kScalarMaxM, st), "clear scalars");
+  h->next_counter = 0;
 
   if (gmp_bin_small_fits(N, h->n_bins, S)) {
     GMP_CK(gmp_launch_bin_small(h->structs.as<GmpStruct>(), S, h->struct_of.as<int32_t>(), N, h->cutoff, pos, species,
@@ -383,63 +445,98 @@ gmp_status bin_atoms(gmp_ctx* h, int32_t S, const double* pos, const int32_t* sp
     return GMP_OK;
   }
   GMP_CK(gmp_launch_neighbors_prepare(h->structs.as<GmpStruct>(), S, h->struct_of.as<int32_t>(), N, h->cutoff,
-                                      pos, species, h->n_el, h->grid.as<GmpGrid>(), h->atom_xh.as<float4>(),
-                                      h->atom_xl.as<float4>(), h->atom_u.as<GmpD4>(), h->atom_bin.as<int32_t>(),
-                                      h->bbox.as<unsigned long long>(), d_err, st, h->sm_count, L),
+                                      pos, species, h->n_el, h->grid_mode, h->grid.as<GmpGrid>(),
+                                      h->atom_xh.as<float4>(), h->atom_xl.as<float4>(), h->atom_u.as<GmpD4>(),
+                                      h->bbox.as<unsigned long long>(), h->n_bins, h->bin_count.as<int32_t>(),
+                                      h->bin_cursor.as<int32_t>(), d_err, st, h->sm_count, L),
          "prepare");
   GMP_CK(gmp_launch_bins(h->structs.as<GmpStruct>(), h->grid.as<GmpGrid>(), h->struct_of.as<int32_t>(), N,
                          h->n_bins, h->atom_bin.as<int32_t>(), h->bin_count.as<int32_t>(),
                          h->bin_start.as<int32_t>(), h->bin_cursor.as<int32_t>(), h->atom_t.as<float4>(),
                          h->atom_y.as<float4>(), h->bin_y.as<float4>(), h->bin_je.as<int2>(), h->atom_u.as<GmpD4>(),
-                         h->atom_xh.as<float4>(), h->atom_xl.as<float4>(), h->scan_tmp.p, h->scan_tmp.bytes, st,
-                         h->sm_count, L),
+                         h->atom_xh.as<float4>(), h->atom_xl.as<float4>(), h->scan_tmp.p, st, h->sm_count, L),
          "bins");
   return GMP_OK;
 }
 
+void note_sizes(gmp_ctx* h) {
+  h->sizes[h->size_kind].per_center = (double)h->P / (double)std::max<int64_t>(h->nc_cur, 1);
+  h->sizes[h->size_kind].max_m = h->max_m;
+}
+
+// Reads the outcome of a pending single-pass build (waiting for the lists,
+// not for what was queued after them): GMP_ERR_CAPACITY when they outgrew the
+// guessed capacities -- the caller repeats its sequence with exact_lists.
+gmp_status finish_lists(gmp_ctx* h, cudaStream_t st) {
+  if (!h->lists_pending) return GMP_OK;
+  h->lists_pending = false;
+  GMP_CK(cudaEventSynchronize(h->ev_lists), "neighbor sync");
+  const uint32_t w = (uint32_t)(h->h_small[0] & 0xffffffffu);
+  if (!w) {
+    h->P = h->h_small[1];
+    h->max_m = (int)(h->h_small[0] >> 32);
+    note_sizes(h);
+    return GMP_OK;
+  }
+  GMP_CK(cudaMemsetAsync(h->scalars.p, 0, 4, st), "clear err");
+  if (w != GMP_DEV_CAPACITY) return decode_device_error(h, w);
+  h->lists_outgrown = true;
+  return GMP_ERR_CAPACITY;
+}
+
+// Runs a call's device sequence and then reads the outcome of its neighbor
+// lists; a sequence whose lists outgrew the guess runs again, counting first.
+template <typename Seq>
+gmp_status run_sequence(gmp_ctx* h, cudaStream_t st, Seq& seq) {
+  h->lists_pending = h->lists_outgrown = h->exact_lists = false;
+  gmp_status r = seq(false);
+  if (r == GMP_OK) r = finish_lists(h, st);
+  if (!h->lists_outgrown) return r;
+  h->exact_lists = true;
+  r = seq(false);
+  h->exact_lists = false;
+  return r;
+}
+
 // Exact neighbor lists of the NC centers C over the binned atoms into
-// h->pairs / h->nbr_off.  Synchronises `st` once (to size the pair buffer)
-// unless capturing.
+// h->pairs / h->nbr_off.  With single_ok and an earlier build to guess the
+// capacities from, one enumeration pass whose outcome finish_lists reads
+// later; otherwise (unless capturing) synchronises `st` once to size the pair
+// buffer.
 gmp_status neighbor_lists(gmp_ctx* h, const GmpCenters& C, int64_t NC, const double* pos, cudaStream_t st,
-                          bool sorted, bool capture, bool single_ok = false) {
+                          bool sorted, bool capture, bool single_ok, int size_kind) {
   int64_t* L = &h->launches;
   uint32_t* d_err = h->scalars.as<uint32_t>();
-  int32_t* d_maxm = reinterpret_cast<int32_t*>(d_err + 1);
-  unsigned long long* d_cursor = reinterpret_cast<unsigned long long*>(h->scalars.as<char>() + 16);
+  int32_t* d_maxm = reinterpret_cast<int32_t*>(h->scalars.as<char>() + kScalarMaxM);
+  unsigned long long* d_cursor = reinterpret_cast<unsigned long long*>(h->scalars.as<char>() + kScalarCursor);
   h->rng_mode = false;
-  // the error word is cleared after it is read (below), so a condition
-  // raised after the read of the previous call is reported here
-  GMP_CK(cudaMemsetAsync(d_maxm, 0, 4, st), "memset maxm");
-  if (single_ok && !capture && h->last_nc == NC && h->last_gen == h->struct_gen && h->P > 0) {
-    // Repeated batch: one enumeration pass, each center allocating its
-    // block of records, with capacities from the last build + 12.5%
-    // (blocks in allocation order: no CSR offsets, ranges in nbr_rng).
-    const int64_t cap = h->P + h->P / 8 + 4096;
+  h->nc_cur = NC;
+  h->size_kind = size_kind;
+  const gmp_ctx::ListSize last = h->sizes[size_kind];
+  if (single_ok && !capture && !h->exact_lists && last.per_center > 0.0) {
+    // One enumeration pass, each center allocating its block of records, with
+    // the pairs per center and the longest list of the last build + 12.5%
+    // (blocks in allocation order: no CSR offsets, ranges in nbr_rng).  A
+    // batch of another kind may outgrow them: the kernel then flags it, later
+    // kernels skip the centers left out, and the call runs again.
+    const int64_t cap = (int64_t)(last.per_center * 1.125 * (double)NC) + 4096;
     int keys = 32;
-    while (keys < h->max_m + h->max_m / 8 + 8) keys <<= 1;
+    while (keys < last.max_m + last.max_m / 8 + 8) keys <<= 1;
     if ((size_t)keys * 8 <= 200 * 1024) {
       GMP_CK(h->pairs.ensure(sizeof(GmpPair) * cap), "pairs");
       GMP_CK(h->nbr_rng.ensure(sizeof(int64_t) * 2 * NC), "nbr_rng");
-      GMP_CK(cudaMemsetAsync(d_cursor, 0, 8, st), "memset cursor");
       GMP_CK(gmp_launch_neighbor_pass(sorted ? 2 : 1, h->structs.as<GmpStruct>(), h->grid.as<GmpGrid>(), C, NC, h->cutoff, pos,
                                       h->atom_xh.as<float4>(), h->atom_xl.as<float4>(), h->bin_start.as<int32_t>(),
                                       h->bin_y.as<float4>(), h->bin_je.as<int2>(), h->n_el, nullptr, nullptr,
                                       h->pairs.as<GmpPair>(), cap, keys, d_maxm, d_err, st, h->sm_count, L, d_cursor,
                                       h->nbr_rng.as<int64_t>()),
              "neighbor single pass");
-      GMP_CK(cudaMemcpyAsync(h->h_small, d_cursor, 8, cudaMemcpyDeviceToHost, st), "read P");
-      GMP_CK(cudaMemcpyAsync(h->h_small + 1, d_err, 8, cudaMemcpyDeviceToHost, st), "read err");
-      GMP_CK(cudaStreamSynchronize(st), "neighbor sync");
-      const uint32_t w = (uint32_t)(h->h_small[1] & 0xffffffffu);
-      if (!w) {
-        h->P = h->h_small[0];
-        h->max_m = (int)(h->h_small[1] >> 32);
-        h->rng_mode = true;
-        return GMP_OK;
-      }
-      GMP_CK(cudaMemsetAsync(d_err, 0, 8, st), "clear err");  // error word and maxm
-      if (w != GMP_DEV_CAPACITY) return decode_device_error(h, w);
-      // outgrew the guessed capacity: count exactly below
+      GMP_CK(cudaMemcpyAsync(h->h_small, d_err, 16, cudaMemcpyDeviceToHost, st), "read err, longest, P");
+      GMP_CK(cudaEventRecord(h->ev_lists, st), "event");
+      h->cap_cur = cap;
+      h->rng_mode = true;
+      h->lists_pending = true;
+      return GMP_OK;
     }
   }
   if (capture && !sorted) {
@@ -447,7 +544,6 @@ gmp_status neighbor_lists(gmp_ctx* h, const GmpCenters& C, int64_t NC, const dou
     // time; a block beyond them is flagged on the device and the call then
     // runs eagerly (and recaptures)
     GMP_CK(h->nbr_rng.ensure(sizeof(int64_t) * 2 * NC), "nbr_rng");
-    GMP_CK(cudaMemsetAsync(d_cursor, 0, 8, st), "memset cursor");
     GMP_CK(gmp_launch_neighbor_pass(1, h->structs.as<GmpStruct>(), h->grid.as<GmpGrid>(), C, NC, h->cutoff, pos,
                                     h->atom_xh.as<float4>(), h->atom_xl.as<float4>(), h->bin_start.as<int32_t>(),
                                     h->bin_y.as<float4>(), h->bin_je.as<int2>(), h->n_el, nullptr, nullptr,
@@ -486,8 +582,8 @@ gmp_status neighbor_lists(gmp_ctx* h, const GmpCenters& C, int64_t NC, const dou
   }
   h->P = h->h_small[0];
   h->max_m = maxm;
-  h->last_nc = NC;
-  h->last_gen = h->struct_gen;
+  note_sizes(h);
+  h->cap_cur = h->P;
   int keys = 32;
   while (keys < maxm) keys <<= 1;
   if ((size_t)keys * 8 > 200 * 1024)
@@ -502,8 +598,8 @@ gmp_status neighbor_lists(gmp_ctx* h, const GmpCenters& C, int64_t NC, const dou
   return GMP_OK;
 }
 
-// Binning + exact neighbor lists of every atom into h->pairs / h->nbr_off.
-// Synchronises `st` once (to size the pair buffer) unless capturing.
+// Binning + exact neighbor lists of every atom into h->pairs / h->nbr_off
+// (see neighbor_lists).
 gmp_status build_neighbors(gmp_ctx* h, int32_t S, const double* pos, const int32_t* species,
                            int64_t N, cudaStream_t st, bool sorted, bool capture = false, bool need_csr = false) {
   if (!capture) h->graph_valid = false;  // buffers may move: a captured graph is stale
@@ -512,7 +608,7 @@ gmp_status build_neighbors(gmp_ctx* h, int32_t S, const double* pos, const int32
   if (r != GMP_OK) return r;
   const GmpCenters C{h->struct_of.as<int32_t>(), pos, h->atom_xh.as<float4>(), h->atom_xl.as<float4>(),
                      h->atom_t.as<float4>(), h->atom_y.as<float4>()};
-  if ((r = neighbor_lists(h, C, N, pos, st, sorted, capture, !need_csr)) != GMP_OK) return r;
+  if ((r = neighbor_lists(h, C, N, pos, st, sorted, capture, !need_csr, 0)) != GMP_OK) return r;
   GMP_CK(prof_mark(h, 0, false, st), "profile");
   return GMP_OK;
 }
@@ -529,15 +625,16 @@ constexpr float kFlagLow = 1e-10f;
 // Refinement queues, one per requested order: a pass queues at most one
 // entry per center and two sigmas, and a call refines after each pass
 // (derivative calls) or once after all of them (features), so a queue holds
-// one entry per center and two sigmas of every pass.  The flag buffer holds 8
-// counts, then the queues.
+// one entry per center and two sigmas of every pass.
 int64_t flag_capacity(const gmp_ctx* h, int64_t N) {
   int64_t pairs = 0;
   for (const PassData& pd : h->passes) pairs += (pd.pass.nsig + 1) / 2;
   return std::max<int64_t>(pairs, 1) * N + 1024;
 }
-unsigned long long* flag_counter(gmp_ctx* h) { return h->flagq.as<unsigned long long>(); }
-unsigned long long* flag_queues(gmp_ctx* h) { return h->flagq.as<unsigned long long>() + 8; }
+unsigned long long* flag_counter(gmp_ctx* h) {
+  return reinterpret_cast<unsigned long long*>(h->scalars.as<char>() + kScalarFlags);
+}
+unsigned long long* flag_queues(gmp_ctx* h) { return h->flagq.as<unsigned long long>(); }
 
 gmpk::KParams base_params(gmp_ctx* h, const PassData& pd, int pass_index, int64_t N) {
   gmpk::KParams K;
@@ -547,29 +644,32 @@ gmpk::KParams base_params(gmp_ctx* h, const PassData& pd, int pass_index, int64_
   K.nbr_beg = h->rng_mode ? h->nbr_rng.as<int64_t>() : h->nbr_off.as<int64_t>();
   K.nbr_end = h->rng_mode ? h->nbr_rng.as<int64_t>() + N : h->nbr_off.as<int64_t>() + 1;
   K.pairs = h->pairs.as<GmpPair>();
-  K.counter = reinterpret_cast<int32_t*>(h->scalars.as<uint32_t>() + 2);
   K.flags = flag_queues(h);
   K.flag_count = flag_counter(h);
   K.flag_cap = flag_capacity(h, N);
-  K.pair_cap = h->capturing ? h->cap_pairs : h->P;
+  K.pair_cap = h->capturing ? h->cap_pairs : h->cap_cur;
   K.sig0 = 16 * pass_index;
   K.flag_tau = kFlagTau;
   K.flag_low = kFlagLow;
   return K;
 }
 
-// Clears the flag queue (before a call's compute kernels, and after each
-// refinement so that the next pass queues only its own flags).
-gmp_status reset_flags(gmp_ctx* h, int64_t N, cudaStream_t st) {
-  (void)N;
+// The next of the call's work counters (cleared when the call began).
+void take_counter(gmp_ctx* h, gmpk::KParams& K) {
+  K.counter = reinterpret_cast<int32_t*>(h->scalars.as<char>() + kScalarCounters) + h->next_counter++;
+}
+
+// Empties the flag queues (after the refinement of a pass that another one
+// follows).
+gmp_status reset_flags(gmp_ctx* h, cudaStream_t st) {
   GMP_CK(cudaMemsetAsync(flag_counter(h), 0, 8 * sizeof(unsigned long long), st), "flag reset");
   return GMP_OK;
 }
 
-gmp_status begin_compute(gmp_ctx* h, int64_t N, cudaStream_t st) {
-  GMP_CK(h->flagq.ensure(sizeof(unsigned long long) * (8 + (size_t)std::max(h->n_ord_pos, 1) * flag_capacity(h, N))),
-         "flags");
-  return reset_flags(h, N, st);
+// Buffers of a call's compute kernels.
+gmp_status begin_compute(gmp_ctx* h, int64_t N) {
+  GMP_CK(h->flagq.ensure(sizeof(unsigned long long) * (size_t)std::max(h->n_ord_pos, 1) * flag_capacity(h, N)), "flags");
+  return GMP_OK;
 }
 
 // The moments of one pass that a derivative kernel reads after the
@@ -625,7 +725,7 @@ gmp_status refine(gmp_ctx* h, int64_t N, float* features, cudaStream_t st, const
   A.mu_sig0 = mt.sig0;
   A.mu_nsig = mt.nsig;
   A.mu_nind = mt.nind;
-  GMP_CK(gmp_launch_refine(A, h->sm_count, st, &h->launches), "refine");
+  GMP_CK(gmp_launch_refine(A, h->sm_count, &h->refine_per_sm, st, &h->launches), "refine");
   return GMP_OK;
 }
 
@@ -747,19 +847,24 @@ gmp_status grad_impl(gmp_ctx* h, int32_t n_struct, const int64_t* atom_off, cons
   const bool whole = c0 == 0 && c1 == N;
   Io io;
   if ((r = stage_inputs(h, N, pos, species, io, st)) != GMP_OK) return r;
-  if ((r = build_neighbors(h, n_struct, io.pos, io.species, N, st, true)) != GMP_OK) return r;
   GMP_CK(h->jac_counts.ensure(sizeof(int64_t) * (2 * n + 1)), "jac counts");
   int64_t* cnt = h->jac_counts.as<int64_t>();
   int64_t* joff = cnt + n;
-  GMP_CK(h->jac_rows.ensure(sizeof(int32_t) * std::max<int64_t>(h->P, 1)), "jac rows");
-  const int64_t* nbeg = h->rng_mode ? h->nbr_rng.as<int64_t>() : h->nbr_off.as<int64_t>();
-  const int64_t* nend = h->rng_mode ? h->nbr_rng.as<int64_t>() + N : h->nbr_off.as<int64_t>() + 1;
-  GMP_CK(gmp_launch_jacobian_count(n, nbeg + c0, nend + c0, h->pairs.as<GmpPair>(), cnt,
-                                   h->jac_rows.as<int32_t>(), st, h->sm_count, &h->launches), "jac count");
-  GMP_CK(gmp_exclusive_scan_i64(cnt, joff, n, h->scan_tmp.p, st, &h->launches), "jac scan");
-  GMP_CK(cudaMemcpyAsync(h->h_small, joff + n, sizeof(int64_t), cudaMemcpyDeviceToHost, st), "read nnz");
-  GMP_CK(cudaStreamSynchronize(st), "jac sync");
-  const int64_t nnz = h->h_small[0];
+  auto lists = [&](bool) -> gmp_status {
+    gmp_status q = build_neighbors(h, n_struct, io.pos, io.species, N, st, true);
+    if (q != GMP_OK) return q;
+    GMP_CK(h->jac_rows.ensure(sizeof(int32_t) * std::max<int64_t>(h->cap_cur, 1)), "jac rows");
+    const int64_t* nbeg = h->rng_mode ? h->nbr_rng.as<int64_t>() : h->nbr_off.as<int64_t>();
+    const int64_t* nend = h->rng_mode ? h->nbr_rng.as<int64_t>() + N : h->nbr_off.as<int64_t>() + 1;
+    GMP_CK(gmp_launch_jacobian_count(n, nbeg + c0, nend + c0, h->pairs.as<GmpPair>(), cnt,
+                                     h->jac_rows.as<int32_t>(), st, h->sm_count, &h->launches), "jac count");
+    GMP_CK(gmp_exclusive_scan_i64(cnt, joff, n, h->scan_tmp.p, st, &h->launches), "jac scan");
+    GMP_CK(cudaMemcpyAsync(h->h_small + 2, joff + n, sizeof(int64_t), cudaMemcpyDeviceToHost, st), "read nnz");
+    GMP_CK(cudaStreamSynchronize(st), "jac sync");
+    return GMP_OK;
+  };
+  if ((r = run_sequence(h, st, lists)) != GMP_OK) return r;
+  const int64_t nnz = h->h_small[2];
   *nnz_out = nnz;
   if (nnz > cap) return fail(h, GMP_ERR_CAPACITY, "jacobian needs " + std::to_string(nnz) + " rows, cap is " + std::to_string(cap));
   if (nnz > 0 && (!jac_j || !jac)) return fail(h, GMP_ERR_INVALID_ARG, "jac_j and jac are required");
@@ -781,22 +886,23 @@ gmp_status grad_impl(gmp_ctx* h, int32_t n_struct, const int64_t* atom_off, cons
     GMP_CK(h->stage_feat.ensure(sizeof(float) * N * h->F), "feature scratch");
     fout = h->stage_feat.as<float>();
   }
-  if ((r = begin_compute(h, N, st)) != GMP_OK) return r;
+  if ((r = begin_compute(h, N)) != GMP_OK) return r;
   for (size_t g = 0; g < h->passes.size(); ++g) {
     // forward kernel (features, moments), refinement of the flagged
     // features and their moments, then the Jacobian rows from the moments
-    const PassData& pd = h->passes[g];
+    PassData& pd = h->passes[g];
     gmpk::KParams K = base_params(h, pd, (int)g, N);
     K.N = c1;
     K.center0 = c0;
     K.features = fout;
     K.mu_out = h->mu.as<float>();
     GMP_CK(prof_mark(h, 1, true, st), "profile");
-    GMP_CK(launch_compute(pd.L, GMP_KIND_FORWARD, pd.NS, K, pd.fwd, st, h->sm_count, &h->launches), "forward");
+    take_counter(h, K);
+    GMP_CK(launch_compute(pd, GMP_KIND_FORWARD, K, pd.fwd, st, h->sm_count, &h->launches), "forward");
     GMP_CK(prof_mark(h, 1, false, st), "profile");
     GMP_CK(prof_mark(h, 3, true, st), "profile");
     if ((r = refine(h, N, fout, st, nullptr, nullptr, nullptr, pass_moments(h, pd, (int)g))) != GMP_OK) return r;
-    if ((r = reset_flags(h, N, st)) != GMP_OK) return r;
+    if (g + 1 < h->passes.size() && (r = reset_flags(h, st)) != GMP_OK) return r;
     GMP_CK(prof_mark(h, 3, false, st), "profile");
     K.features = nullptr;
     K.flags = nullptr;
@@ -805,7 +911,8 @@ gmp_status grad_impl(gmp_ctx* h, int32_t n_struct, const int64_t* atom_off, cons
     K.jac_j = jj;
     K.jac = jd;
     GMP_CK(prof_mark(h, 2, true, st), "profile");
-    GMP_CK(launch_compute(pd.L, GMP_KIND_JACOBIAN, pd.NS, K, pd.jac, st, h->sm_count, &h->launches), "jacobian");
+    take_counter(h, K);
+    GMP_CK(launch_compute(pd, GMP_KIND_JACOBIAN, K, pd.jac, st, h->sm_count, &h->launches), "jacobian");
     GMP_CK(prof_mark(h, 2, false, st), "profile");
   }
   const cudaMemcpyKind k_out = io.host ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
@@ -1044,7 +1151,7 @@ gmp_status gmp_create(const gmp_params* p, int device, gmp_handle* out) {
         cudaMemcpy(h->ktab.p, kt.data(), kt.size() * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess ||
         h->colinfo.ensure(ci.size() * sizeof(int32_t)) != cudaSuccess ||
         cudaMemcpy(h->colinfo.p, ci.data(), ci.size() * sizeof(int32_t), cudaMemcpyHostToDevice) != cudaSuccess ||
-        h->scalars.ensure(64) != cudaSuccess || cudaMemset(h->scalars.p, 0, 64) != cudaSuccess) {
+        h->scalars.ensure(kScalarBytes) != cudaSuccess || cudaMemset(h->scalars.p, 0, kScalarBytes) != cudaSuccess) {
       cudaGetLastError();
       return bad("device allocation for tables failed");
     }
@@ -1053,6 +1160,8 @@ gmp_status gmp_create(const gmp_params* p, int device, gmp_handle* out) {
   if (cudaMallocHost((void**)&h->h_small, 64) != cudaSuccess) { cudaGetLastError(); return bad("pinned alloc failed"); }
   if (cudaEventCreateWithFlags(&h->ev, cudaEventDisableTiming) != cudaSuccess) { cudaGetLastError(); return bad("event"); }
   if (cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking) != cudaSuccess ||
+      cudaEventCreateWithFlags(&h->ev_desc, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&h->ev_lists, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&h->ev_in, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&h->ev_feat, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&h->ev_out, cudaEventDisableTiming) != cudaSuccess) {
@@ -1100,13 +1209,14 @@ gmp_status gmp_featurize(gmp_handle h, int32_t n_struct, const int64_t* atom_off
   auto seq = [&](bool capture) -> gmp_status {
     gmp_status q = build_neighbors(h, n_struct, io.pos, io.species, N, st, false, capture);
     if (q != GMP_OK) return q;
-    if ((q = begin_compute(h, N, st)) != GMP_OK) return q;
+    if (io.host && (q = finish_lists(h, st)) != GMP_OK) return q;
+    if ((q = begin_compute(h, N)) != GMP_OK) return q;
     GMP_CK(prof_mark(h, 1, true, st), "profile");
     for (size_t g = 0; g < h->passes.size(); ++g) {
       gmpk::KParams K = base_params(h, h->passes[g], (int)g, N);
       K.features = feat;
-      GMP_CK(launch_compute(h->passes[g].L, GMP_KIND_FORWARD, h->passes[g].NS, K, h->passes[g].fwd, st,
-                            h->sm_count, &h->launches),
+      take_counter(h, K);
+      GMP_CK(launch_compute(h->passes[g], GMP_KIND_FORWARD, K, h->passes[g].fwd, st, h->sm_count, &h->launches),
              "forward");
     }
     GMP_CK(prof_mark(h, 1, false, st), "profile");
@@ -1115,7 +1225,7 @@ gmp_status gmp_featurize(gmp_handle h, int32_t n_struct, const int64_t* atom_off
     GMP_CK(prof_mark(h, 3, false, st), "profile");
     return GMP_OK;
   };
-  if ((r = seq(false)) != GMP_OK) return r;
+  if ((r = run_sequence(h, st, seq)) != GMP_OK) return r;
   if (use_graph && (r = capture_graph(h, key, st, seq, N)) != GMP_OK) return r;
   if (io.host) {
     GMP_CK(cudaMemcpyAsync(features, feat, sizeof(float) * N * h->F, cudaMemcpyDeviceToHost, st), "d2h features");
@@ -1178,7 +1288,7 @@ static gmp_status vjp_impl(gmp_handle h, int32_t n_struct, const int64_t* atom_o
                                       (uintptr_t)n_struct, (uintptr_t)h->struct_gen};
   if (use_graph && (r = replay_graph(h, key, st)) != GMP_ERR_CAPACITY) return r;
   // buffers first (no allocation may happen while a graph is captured)
-  GMP_CK(h->grad_acc.ensure(sizeof(double) * 3 * N), "grad_acc");
+  if (h->passes.size() > 1) GMP_CK(h->grad_acc.ensure(sizeof(double) * 3 * N), "grad_acc");
   GMP_CK(h->gbins.ensure(sizeof(unsigned long long) * 3 * gmpk::kGradBins * N), "gradient bins");
   GMP_CK(h->own.ensure(sizeof(double) * 3 * N), "own");
   if (vir) GMP_CK(h->vir_c.ensure(sizeof(double) * 9 * N), "vir_c");
@@ -1193,16 +1303,17 @@ static gmp_status vjp_impl(gmp_handle h, int32_t n_struct, const int64_t* atom_o
     K.gbins = h->gbins.as<unsigned long long>();
     K.own = h->own.as<double>();
     K.vir_c = vir ? h->vir_c.as<double>() : nullptr;
+    take_counter(h, K);
     GMP_CK(cudaMemsetAsync(K.gbins, 0, sizeof(unsigned long long) * 3 * gmpk::kGradBins * N, st), "memset bins");
-    GMP_CK(cudaMemsetAsync(K.own, 0, sizeof(double) * 3 * N, st), "memset own");
-    if (vir) GMP_CK(cudaMemsetAsync(K.vir_c, 0, sizeof(double) * 9 * N, st), "memset vir_c");
     return GMP_OK;
   };
-  auto vjp_end = [&](const gmpk::KParams& K) -> gmp_status {
-    GMP_CK(gmp_launch_grad_bins_finish(N, K.gbins, K.own, h->grad_acc.as<double>(), st, h->sm_count, &h->launches),
+  auto vjp_end = [&](const gmpk::KParams& K, bool first, bool last) -> gmp_status {
+    GMP_CK(gmp_launch_grad_bins_finish(N, K.gbins, K.own, first ? nullptr : h->grad_acc.as<double>(),
+                                       last ? nullptr : h->grad_acc.as<double>(), last ? gp : nullptr, st, h->sm_count,
+                                       &h->launches),
            "gradient sums");
     if (vir)
-      GMP_CK(gmp_launch_virial_reduce(n_struct, h->atom_off.as<int64_t>(), K.vir_c, vir, st, h->sm_count,
+      GMP_CK(gmp_launch_virial_reduce(n_struct, h->atom_off.as<int64_t>(), K.vir_c, vir, first, st, h->sm_count,
                                       &h->launches),
              "virial sums");
     return GMP_OK;
@@ -1210,13 +1321,13 @@ static gmp_status vjp_impl(gmp_handle h, int32_t n_struct, const int64_t* atom_o
   auto seq = [&](bool capture) -> gmp_status {
   gmp_status q = build_neighbors(h, n_struct, io.pos, io.species, N, st, false, capture);
   if (q != GMP_OK) return q;
-  GMP_CK(cudaMemsetAsync(h->grad_acc.p, 0, sizeof(double) * 3 * N, st), "memset grad");
-  if (vir) GMP_CK(cudaMemsetAsync(vir, 0, sizeof(double) * 9 * n_struct, st), "memset virial");
-  if ((q = begin_compute(h, N, st)) != GMP_OK) return q;
+  if (io.host && (q = finish_lists(h, st)) != GMP_OK) return q;
+  if ((q = begin_compute(h, N)) != GMP_OK) return q;
   bool refined = false, waited = false, pending = false;
   const bool overlap = io.host && !capture;
   for (size_t g = 0; g < h->passes.size(); ++g) {
-    const PassData& pd = h->passes[g];
+    PassData& pd = h->passes[g];
+    const bool last = g + 1 == h->passes.size();
     // forward kernel (features + moments), then the backward kernel reading
     // the moments (or one fused kernel, if the autotuner chose it)
     float* fout = feat ? feat : h->stage_feat.as<float>();
@@ -1231,27 +1342,27 @@ static gmp_status vjp_impl(gmp_handle h, int32_t n_struct, const int64_t* atom_o
     }
     if (fused) {
       K.grad_feat = gf;
-      K.grad_acc = h->grad_acc.as<double>();
       GMP_CK(prof_mark(h, 2, true, st), "profile");
       if ((q = vjp_begin(K)) != GMP_OK) return q;
-      GMP_CK(launch_compute(pd.L, GMP_KIND_VJP, pd.NS, K, pd.fused, st, h->sm_count, &h->launches), "vjp");
-      if ((q = vjp_end(K)) != GMP_OK) return q;
+      GMP_CK(launch_compute(pd, GMP_KIND_VJP, K, pd.fused, st, h->sm_count, &h->launches), "vjp");
+      if ((q = vjp_end(K, g == 0, last)) != GMP_OK) return q;
       GMP_CK(prof_mark(h, 2, false, st), "profile");
       pending = true;
       continue;
     }
     K.mu_out = h->mu.as<float>();
     GMP_CK(prof_mark(h, 1, true, st), "profile");
-    GMP_CK(launch_compute(pd.L, GMP_KIND_FORWARD, pd.NS, K, pd.fwd, st, h->sm_count, &h->launches), "forward");
+    take_counter(h, K);
+    GMP_CK(launch_compute(pd, GMP_KIND_FORWARD, K, pd.fwd, st, h->sm_count, &h->launches), "forward");
     GMP_CK(prof_mark(h, 1, false, st), "profile");
     // refinement of the flagged features (this pass's, and any a fused pass
     // left); the backward kernel then reads the refined moments
     GMP_CK(prof_mark(h, 3, true, st), "profile");
     if ((q = refine(h, N, fout, st, nullptr, nullptr, nullptr, pass_moments(h, pd, (int)g))) != GMP_OK) return q;
-    if ((q = reset_flags(h, N, st)) != GMP_OK) return q;
+    if (!last && (q = reset_flags(h, st)) != GMP_OK) return q;
     GMP_CK(prof_mark(h, 3, false, st), "profile");
     pending = false;
-    if (g + 1 == h->passes.size()) {
+    if (last) {
       // every feature is final once the last forward kernel and its
       // refinement ran: the download overlaps the backward kernel
       refined = true;
@@ -1269,15 +1380,12 @@ static gmp_status vjp_impl(gmp_handle h, int32_t n_struct, const int64_t* atom_o
     K.features = nullptr;
     K.flags = nullptr;
     K.grad_feat = gf;
-    K.grad_acc = h->grad_acc.as<double>();
-    K.virial = vir;
-    K.center_struct = h->struct_of.as<int32_t>();
     GMP_CK(prof_mark(h, 2, true, st), "profile");
     if ((q = vjp_begin(K)) != GMP_OK) return q;
-    GMP_CK(launch_compute(pd.L, vir ? GMP_KIND_BACKWARD_VIRIAL : GMP_KIND_BACKWARD, pd.NS, K, pd.bwd, st,
-                          h->sm_count, &h->launches),
+    GMP_CK(launch_compute(pd, vir ? GMP_KIND_BACKWARD_VIRIAL : GMP_KIND_BACKWARD, K, pd.bwd, st, h->sm_count,
+                          &h->launches),
            "backward");
-    if ((q = vjp_end(K)) != GMP_OK) return q;
+    if ((q = vjp_end(K, g == 0, last)) != GMP_OK) return q;
     GMP_CK(prof_mark(h, 2, false, st), "profile");
   }
   if (feat && pending) {
@@ -1285,7 +1393,6 @@ static gmp_status vjp_impl(gmp_handle h, int32_t n_struct, const int64_t* atom_o
     if ((q = refine(h, N, feat, st)) != GMP_OK) return q;
     GMP_CK(prof_mark(h, 3, false, st), "profile");
   }
-  GMP_CK(gmp_launch_grad_finish(N, h->grad_acc.as<double>(), gp, st, &h->launches), "grad finish");
   if (overlap && features && !refined) {  // fused path: features final only now
     GMP_CK(cudaEventRecord(h->ev_feat, st), "event");
     GMP_CK(cudaStreamWaitEvent(h->side, h->ev_feat, 0), "side wait");
@@ -1294,7 +1401,7 @@ static gmp_status vjp_impl(gmp_handle h, int32_t n_struct, const int64_t* atom_o
   }
   return GMP_OK;
   };
-  if ((r = seq(false)) != GMP_OK) {
+  if ((r = run_sequence(h, st, seq)) != GMP_OK) {
     if (io.host) cudaStreamSynchronize(h->side);  // no copy may outlive the call
     return r;
   }
@@ -1382,31 +1489,35 @@ gmp_status gmp_featurize_points(gmp_handle h, int32_t n_struct, const int64_t* a
            "upload point_off");
     GMP_CK(gmp_launch_struct_of(h->pt_off.as<int64_t>(), n_struct, h->pt_struct.as<int32_t>(), st, &h->launches),
            "point struct");
+    auto seq = [&](bool) -> gmp_status {
+    gmp_status q;
     GMP_CK(prof_mark(h, 0, true, st), "profile");
-    if ((r = bin_atoms(h, n_struct, io.pos, io.species, N, NP, st)) != GMP_OK) return r;
+    if ((q = bin_atoms(h, n_struct, io.pos, io.species, N, NP, st)) != GMP_OK) return q;
     GMP_CK(gmp_launch_point_prepare(h->structs.as<GmpStruct>(), h->grid.as<GmpGrid>(), h->pt_struct.as<int32_t>(), NP,
                                     pts, io.pos, h->pt_xh.as<float4>(), h->pt_xl.as<float4>(), h->pt_t.as<float4>(),
                                     h->pt_y.as<float4>(), h->scalars.as<uint32_t>(), st, h->sm_count, &h->launches),
            "point prepare");
     const GmpCenters C{h->pt_struct.as<int32_t>(), pts, h->pt_xh.as<float4>(), h->pt_xl.as<float4>(),
                        h->pt_t.as<float4>(), h->pt_y.as<float4>()};
-    h->last_nc = -1;  // the capacities below describe the points, not the atoms
-    if ((r = neighbor_lists(h, C, NP, io.pos, st, false, false)) != GMP_OK) return r;
-    h->last_nc = -1;
+    if ((q = neighbor_lists(h, C, NP, io.pos, st, false, false, true, 1)) != GMP_OK) return q;
     GMP_CK(prof_mark(h, 0, false, st), "profile");
-    if ((r = begin_compute(h, NP, st)) != GMP_OK) return r;
+    if (host && (q = finish_lists(h, st)) != GMP_OK) return q;
+    if ((q = begin_compute(h, NP)) != GMP_OK) return q;
     GMP_CK(prof_mark(h, 1, true, st), "profile");
     for (size_t g = 0; g < h->passes.size(); ++g) {
       gmpk::KParams K = base_params(h, h->passes[g], (int)g, NP);
       K.features = feat;
-      GMP_CK(launch_compute(h->passes[g].L, GMP_KIND_FORWARD, h->passes[g].NS, K, h->passes[g].fwd, st,
-                            h->sm_count, &h->launches),
+      take_counter(h, K);
+      GMP_CK(launch_compute(h->passes[g], GMP_KIND_FORWARD, K, h->passes[g].fwd, st, h->sm_count, &h->launches),
              "forward");
     }
     GMP_CK(prof_mark(h, 1, false, st), "profile");
     GMP_CK(prof_mark(h, 3, true, st), "profile");
-    if ((r = refine(h, NP, feat, st, h->pt_xh.as<float4>(), h->pt_xl.as<float4>(), h->pt_struct.as<int32_t>())) != GMP_OK) return r;
+    if ((q = refine(h, NP, feat, st, h->pt_xh.as<float4>(), h->pt_xl.as<float4>(), h->pt_struct.as<int32_t>())) != GMP_OK) return q;
     GMP_CK(prof_mark(h, 3, false, st), "profile");
+    return GMP_OK;
+    };
+    if ((r = run_sequence(h, st, seq)) != GMP_OK) return r;
   }
   if (host) {
     GMP_CK(cudaMemcpyAsync(features, feat, sizeof(float) * NP * h->F, cudaMemcpyDeviceToHost, st), "d2h features");
@@ -1466,21 +1577,25 @@ gmp_status gmp_tune(gmp_handle h, int32_t n_struct, const int64_t* atom_off, con
   if (reps < 1) reps = 1;
   Io io;
   if ((r = stage_inputs(h, N, pos, species, io, st)) != GMP_OK) return r;
-  if ((r = build_neighbors(h, n_struct, io.pos, io.species, N, st, false)) != GMP_OK) return r;
+  auto lists = [&](bool) { return build_neighbors(h, n_struct, io.pos, io.species, N, st, false); };
+  if ((r = run_sequence(h, st, lists)) != GMP_OK) return r;
   if (pairs_out) *pairs_out = h->P;
   GMP_CK(h->stage_feat.ensure(sizeof(float) * N * h->F), "tune features");
   GMP_CK(h->stage_gradf.ensure(sizeof(float) * N * h->F), "tune grad");
   GMP_CK(cudaMemsetAsync(h->stage_gradf.p, 0, sizeof(float) * N * h->F, st), "tune grad zero");
-  GMP_CK(h->grad_acc.ensure(sizeof(double) * 3 * N), "grad_acc");
   cudaEvent_t e0, e1;
   GMP_CK(cudaEventCreate(&e0), "event");
   GMP_CK(cudaEventCreate(&e1), "event");
-  auto timed = [&](int kind, const PassData& pd, const gmpk::KParams& K, GmpShape shape, float* ms) -> cudaError_t {
-    cudaError_t e = launch_compute(pd.L, kind, pd.NS, K, shape, st, h->sm_count, &h->launches);  // warm-up
+  auto launch_cleared = [&](int kind, PassData& pd, const gmpk::KParams& K, GmpShape shape) -> cudaError_t {
+    const cudaError_t e = cudaMemsetAsync(K.counter, 0, sizeof(int32_t), st);
+    return e != cudaSuccess ? e : launch_compute(pd, kind, K, shape, st, h->sm_count, &h->launches);
+  };
+  auto timed = [&](int kind, PassData& pd, const gmpk::KParams& K, GmpShape shape, float* ms) -> cudaError_t {
+    cudaError_t e = launch_cleared(kind, pd, K, shape);  // warm-up
     if (e != cudaSuccess) return e;
     if ((e = cudaEventRecord(e0, st)) != cudaSuccess) return e;
     for (int k = 0; k < reps; ++k)
-      if ((e = launch_compute(pd.L, kind, pd.NS, K, shape, st, h->sm_count, &h->launches)) != cudaSuccess) return e;
+      if ((e = launch_cleared(kind, pd, K, shape)) != cudaSuccess) return e;
     if ((e = cudaEventRecord(e1, st)) != cudaSuccess) return e;
     if ((e = cudaEventSynchronize(e1)) != cudaSuccess) return e;
     if ((e = cudaEventElapsedTime(ms, e0, e1)) != cudaSuccess) return e;
@@ -1492,11 +1607,12 @@ gmp_status gmp_tune(gmp_handle h, int32_t n_struct, const int64_t* atom_off, con
     PassData& pd = h->passes[g];
     const size_t mu_floats = (size_t)N * std::max(pd.pass.nsig, 1) * (pd.L + 1) * (pd.L + 1);
     if (h->mu.ensure(sizeof(float) * mu_floats) != cudaSuccess ||
-        (out = begin_compute(h, N, st)) != GMP_OK) {
+        (out = begin_compute(h, N)) != GMP_OK) {
       if (out == GMP_OK) out = fail(h, GMP_ERR_OOM, "tune buffers");
       break;
     }
     gmpk::KParams K = base_params(h, pd, (int)g, N);
+    K.counter = reinterpret_cast<int32_t*>(h->scalars.as<char>() + kScalarCounters);
     K.flags = nullptr;
     K.features = h->stage_feat.as<float>();
     K.mu_out = h->mu.as<float>();
@@ -1510,14 +1626,13 @@ gmp_status gmp_tune(gmp_handle h, int32_t n_struct, const int64_t* atom_off, con
       }
     if (out != GMP_OK) break;
     // moments for the backward candidates
-    if (cudaError_t e = launch_compute(pd.L, GMP_KIND_FORWARD, pd.NS, K, fwd_best, st, h->sm_count, &h->launches)) {
+    if (cudaError_t e = launch_cleared(GMP_KIND_FORWARD, pd, K, fwd_best)) {
       out = cuda_fail(h, e, "tune forward");
       break;
     }
     gmpk::KParams Kb = K;
     Kb.features = nullptr;
     Kb.grad_feat = h->stage_gradf.as<float>();
-    Kb.grad_acc = h->grad_acc.as<double>();
     float best_b = 1e30f;
     GmpShape bwd_best = pd.bwd;
     for (int warps : {4, 6, 12}) {
@@ -1653,7 +1768,8 @@ void gmp_destroy(gmp_handle h) {
   for (auto& v : h->prof_ev)
     for (cudaEvent_t e : v) cudaEventDestroy(e);
   if (h->ev) cudaEventDestroy(h->ev);
-  for (cudaEvent_t e : {h->ev_in, h->ev_feat, h->ev_out})
+  if (h->h_desc) cudaFreeHost(h->h_desc);
+  for (cudaEvent_t e : {h->ev_in, h->ev_feat, h->ev_out, h->ev_desc, h->ev_lists})
     if (e) cudaEventDestroy(e);
   if (h->side) cudaStreamDestroy(h->side);
   delete h;  // the device buffers free themselves, with this device current

@@ -346,19 +346,27 @@ cudaError_t gmp_launch_bin_small(GmpStruct* d_structs, int n_struct, const int32
                                  int32_t* atom_bin, int32_t* bin_start, float4* bin_y, int2* bin_je,
                                  float4* atom_t, float4* atom_y, uint32_t* d_err, cudaStream_t stream,
                                  int64_t* launches);
-cudaError_t gmp_launch_neighbors_prepare(const GmpStruct* d_structs, int n_struct,
+// Where the structures' bin grids come from: given (uploaded with the batch
+// description: every structure is periodic along all axes, gmp_periodic_grid),
+// from the atoms' range for the structures with a non-periodic axis (the
+// others' are given), or all of them made on the device.
+enum class GmpGridMode { kGiven, kOpen, kAll };
+// Grid and pre-screen bounds of a structure periodic along all axes (host);
+// zeroed for others.
+void gmp_periodic_grid(GmpStruct& st, GmpGrid& g, double cutoff);
+cudaError_t gmp_launch_neighbors_prepare(GmpStruct* d_structs, int n_struct,
                                          const int32_t* d_struct_of, int64_t N, double cutoff,
-                                         const double* pos, const int32_t* species, int n_el,
+                                         const double* pos, const int32_t* species, int n_el, GmpGridMode mode,
                                          GmpGrid* d_grid, float4* atom_xh, float4* atom_xl,
-                                         GmpD4* atom_u, int32_t* atom_bin,
-                                         unsigned long long* d_bbox, uint32_t* d_err,
+                                         GmpD4* atom_u, unsigned long long* d_bbox, int64_t n_bins,
+                                         int32_t* bin_count, int32_t* bin_cursor, uint32_t* d_err,
                                          cudaStream_t stream, int sm_count, int64_t* launches);
 cudaError_t gmp_launch_bins(const GmpStruct* d_structs, const GmpGrid* d_grid,
                             const int32_t* d_struct_of, int64_t N, int64_t n_bins,
-                            const int32_t* atom_bin, int32_t* bin_count, int32_t* bin_start,
+                            int32_t* atom_bin, int32_t* bin_count, int32_t* bin_start,
                             int32_t* bin_cursor, float4* atom_t, float4* atom_y, float4* bin_y, int2* bin_je,
                             const GmpD4* atom_u, const float4* atom_xh, const float4* atom_xl, void* scan_tmp,
-                            size_t scan_tmp_bytes, cudaStream_t stream, int sm_count, int64_t* launches);
+                            cudaStream_t stream, int sm_count, int64_t* launches);
 size_t gmp_scan_tmp_bytes(int64_t n);
 cudaError_t gmp_exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, void* tmp,
                                    cudaStream_t stream, int64_t* launches);
@@ -366,7 +374,7 @@ cudaError_t gmp_exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, v
 // reference points (gmp_featurize_points).  Per center: structure id, FP64
 // position [3], double-float split (xl.w = packed wrap of the fractional
 // coordinates), position in the structure's bin grid in units of bins (t,
-// FP32) and wrapped FP32 position y (k_ranges).
+// FP32) and wrapped FP32 position y (k_bin_assign).
 struct GmpCenters {
   const int32_t* sid;
   const double* pos;
@@ -403,15 +411,16 @@ cudaError_t gmp_launch_neighbor_pass(int fill, const GmpStruct* d_structs, const
 cudaError_t gmp_launch_jacobian_count(int64_t N, const int64_t* nbr_beg, const int64_t* nbr_end, const GmpPair* pairs,
                                       int64_t* counts, int32_t* local_row, cudaStream_t stream, int sm_count,
                                       int64_t* launches);
-cudaError_t gmp_launch_grad_finish(int64_t N, const double* grad_acc, float* grad_pos,
-                                   cudaStream_t stream, int64_t* launches);
-// grad_acc[j] += own[j] + the value of j's exact fixed-point bins (filled by
-// the backward kernels without float atomics; 12 per atom and component).
+// Gradient of atom j: own[j] + the value of j's exact fixed-point bins (filled
+// by the backward kernels without float atomics; 12 per atom and component),
+// plus acc_in[j] (earlier passes, may be null), to acc_out[j], or rounded to
+// grad_pos[j] when that is given (the last pass).
 cudaError_t gmp_launch_grad_bins_finish(int64_t N, const unsigned long long* bins, const double* own,
-                                        double* grad_acc, cudaStream_t stream, int sm_count, int64_t* launches);
-// virial[s] += sum of vir_c over the centers atom_off[s] .. atom_off[s+1]-1 (fixed order).
+                                        const double* acc_in, double* acc_out, float* grad_pos, cudaStream_t stream,
+                                        int sm_count, int64_t* launches);
+// virial[s] = (first) or += sum of vir_c over the centers atom_off[s] .. atom_off[s+1]-1 (fixed order).
 cudaError_t gmp_launch_virial_reduce(int n_struct, const int64_t* atom_off, const double* vir_c, double* virial,
-                                     cudaStream_t stream, int sm_count, int64_t* launches);
+                                     bool first, cudaStream_t stream, int sm_count, int64_t* launches);
 // Double-float recomputation of the flagged features: one queue per
 // order slot o (queue + o * cap, count[o] entries, at most cap; qidx[l] is
 // the slot of order l, -1 when l is not requested), entries center << 32 |
@@ -445,8 +454,10 @@ struct GmpRefine {
   float* mu_out;
   int mu_sig0, mu_nsig, mu_nind;
 };
-// One launch for all orders.
-cudaError_t gmp_launch_refine(const GmpRefine& args, int sm_count, cudaStream_t stream, int64_t* launches);
+// One launch for all orders; *per_sm keeps the kernel's resident CTAs per SM
+// (0: asked here).
+cudaError_t gmp_launch_refine(const GmpRefine& args, int sm_count, int* per_sm, cudaStream_t stream,
+                              int64_t* launches);
 cudaError_t gmp_launch_unpack_neighbors(int64_t P, const GmpPair* pairs, int32_t* nbr_j,
                                         int32_t* nbr_shift, cudaStream_t stream,
                                         int64_t* launches);

@@ -183,16 +183,13 @@ struct KParams {
   float* features;        // [N, F] or null
   float* mu_out;          // [N, nsig, NIND] or null
   const float* grad_feat; // [N, F] (vjp)
-  double* grad_acc;       // [N, 3] (vjp)
   const int64_t* jac_off; // [N+1] (jacobian)
   const int32_t* jac_row; // [P] row of each pair within its center (jacobian)
   int32_t* jac_j;
   float* jac;             // [nnz, F, 3]
-  int32_t* counter;
-  int64_t center0;        // centers center0 .. N-1 (the work counter starts there);
+  int32_t* counter;       // the launch's work counter, zero at its start
+  int64_t center0;        // centers center0 .. N-1;
                           // jac_off row 0 belongs to center center0 (jacobian)
-  const int32_t* center_struct;  // [N] structure of each center (virial)
-  double* virial;                // [S, 3, 3] strain derivative accumulators (virial)
   // features too ill-conditioned for FP32 (recomputed in double-float
   // afterwards): one queue entry per (center, order, pair of sigmas 2b, 2b+1)
   // of the pass, center << 32 | column of the first sigma << 16 | mask of the
@@ -829,10 +826,10 @@ __device__ __forceinline__ void setup_items(int (&it_l)[Shape<L, NS>::Q], int (&
   }
 }
 
-__device__ __forceinline__ int64_t next_center(int32_t* counter) {
-  int64_t c = 0;
-  if ((threadIdx.x & 31) == 0) c = atomicAdd(counter, 1);
-  return __shfl_sync(0xffffffffu, (int)c, 0);
+__device__ __forceinline__ int64_t next_center(const KParams& K) {
+  int c = 0;
+  if ((threadIdx.x & 31) == 0) c = atomicAdd(K.counter, 1);
+  return K.center0 + __shfl_sync(0xffffffffu, c, 0);
 }
 
 // Features of center i from Mu; features whose value is below the FP32
@@ -908,7 +905,7 @@ __global__ void __launch_bounds__(512) k_forward(KParams K) {
   int it_l[SH::Q], it_sb[SH::Q], it_ch[SH::Q];
   bool it_ok[SH::Q];
   setup_items<L, NS>(it_l, it_sb, it_ch, it_ok);
-  for (int64_t i = next_center(K.counter); i < K.N; i = next_center(K.counter)) {
+  for (int64_t i = next_center(K); i < K.N; i = next_center(K)) {
     const int64_t p0 = K.nbr_beg[i], p1 = K.nbr_end[i];
     if (p1 > K.pair_cap) continue;  // over capacity: flagged by the fill pass
     const int M = (int)(p1 - p0);
@@ -1119,7 +1116,7 @@ __global__ void __launch_bounds__(256) k_vjp(KParams K) {
   int it_l[SH::Q], it_sb[SH::Q], it_ch[SH::Q];
   bool it_ok[SH::Q];
   setup_items<L, NS>(it_l, it_sb, it_ch, it_ok);
-  for (int64_t i = next_center(K.counter); i < K.N; i = next_center(K.counter)) {
+  for (int64_t i = next_center(K); i < K.N; i = next_center(K)) {
     const int64_t p0 = K.nbr_beg[i], p1 = K.nbr_end[i];
     if (p1 > K.pair_cap) continue;  // over capacity: flagged by the fill pass
     const int M = (int)(p1 - p0);
@@ -1151,7 +1148,7 @@ __global__ void __launch_bounds__(384) k_backward(KParams K) {
   float* Mu = s_warp + (size_t)wib * (SH::WARP_FLOATS + EXTRA);
   float* Lam = Mu + SH::TILE * SH::RSTR;
   float* Wv = EXTRA ? Mu + SH::WARP_FLOATS : Mu;  // Mu is dead once Lam is formed
-  for (int64_t i = next_center(K.counter); i < K.N; i = next_center(K.counter)) {
+  for (int64_t i = next_center(K); i < K.N; i = next_center(K)) {
     const int64_t p0 = K.nbr_beg[i], p1 = K.nbr_end[i];
     if (p1 > K.pair_cap) continue;  // over capacity: flagged by the fill pass
     const int M = (int)(p1 - p0);
@@ -1222,7 +1219,7 @@ __global__ void __maxnreg__(L >= 6 ? 168 : 128) k_jacobian(KParams K) {
   float* Mu = s_warp + (size_t)wib * SH::WARP_FLOATS;
   float* Lam = Mu + SH::TILE * SH::RSTR;
   const float* lam_s = Lam + s * SH::NINDP;
-  for (int64_t i = next_center(K.counter); i < K.N; i = next_center(K.counter)) {
+  for (int64_t i = next_center(K); i < K.N; i = next_center(K)) {
     const int64_t p0 = K.nbr_beg[i], p1 = K.nbr_end[i];
     if (p1 > K.pair_cap) continue;  // over capacity: flagged by the fill pass
     const float* mrow = K.mu_out + i * (int64_t)P.nsig * SH::NIND;

@@ -20,9 +20,18 @@ struct GmpShape {
   int warps;  // warps per CTA, 0 = largest that fits
 };
 
+// The launch worked out for a request (shape and number of centers' class):
+// kept by the handle, so that a call repeats neither the attribute nor the
+// occupancy queries (several microseconds a launch).
+struct GmpLaunchPlan {
+  const void* fn = nullptr;   // null: nothing worked out yet
+  int req_warps = 0, warps = 0, per_sm = 0;
+  size_t smem = 0;
+};
+
 #define GMP_DECLARE_LAUNCHER(LV)                                                                \
   cudaError_t gmp_launch_compute_L##LV(int kind, int ns, const gmpk::KParams& K, GmpShape shape,  \
-                                      cudaStream_t st, int sm_count, int64_t* launches);
+                                      GmpLaunchPlan* plan, cudaStream_t st, int sm_count, int64_t* launches);
 GMP_DECLARE_LAUNCHER(0)
 GMP_DECLARE_LAUNCHER(1)
 GMP_DECLARE_LAUNCHER(2)

@@ -22,6 +22,7 @@
 #include "gmp_internal.cuh"
 
 #include <math.h>
+#include <string.h>
 
 namespace {
 
@@ -29,9 +30,11 @@ __device__ __forceinline__ unsigned long long order_key(double v) {
   unsigned long long b = (unsigned long long)__double_as_longlong(v);
   return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
 }
-__device__ __forceinline__ double key_to_double(unsigned long long k) {
-  unsigned long long b = (k >> 63) ? (k & 0x7FFFFFFFFFFFFFFFull) : ~k;
-  return __longlong_as_double((long long)b);
+__host__ __device__ inline double key_to_double(unsigned long long k) {
+  const unsigned long long b = (k >> 63) ? (k & 0x7FFFFFFFFFFFFFFFull) : ~k;
+  double v;
+  memcpy(&v, &b, sizeof(v));
+  return v;
 }
 
 __device__ __forceinline__ int floor_div(int a, int b) {  // b > 0
@@ -152,18 +155,20 @@ __global__ void k_prepare(const GmpStruct* __restrict__ S, const int32_t* __rest
                           const int32_t* __restrict__ species, int n_el,
                           float4* __restrict__ atom_xh, float4* __restrict__ atom_xl,
                           GmpD4* __restrict__ atom_u, unsigned long long* __restrict__ bbox,
+                          int64_t n_bins, int32_t* __restrict__ bin_count, int32_t* __restrict__ bin_cursor,
                           uint32_t* __restrict__ err) {
+  for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < n_bins; b += (int64_t)gridDim.x * blockDim.x)
+    bin_count[b] = bin_cursor[b] = 0;
   for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < N;
        a += (int64_t)gridDim.x * blockDim.x)
     prepare_atom(S, struct_of, a, pos, species, n_el, atom_xh, atom_xl, atom_u, bbox, err);
 }
 
-// Per structure: bin grid and the FP32 pre-screen bound.  bbox may be
-// global or shared memory.
-__device__ inline void grid_struct(GmpStruct* S, int s, const unsigned long long* bbox, GmpGrid* G,
-                                   double cutoff) {
-  const GmpStruct& st = S[s];
-  GmpGrid g;
+// Bin grid and FP32 pre-screen bound of one structure.  bbox: its 6 keys,
+// read for non-periodic axes only (a fully periodic structure's grid follows
+// from its cell and is made on the host, with the batch description).
+__host__ __device__ inline void grid_struct(GmpStruct& st, const unsigned long long* bbox, GmpGrid& g,
+                                            double cutoff) {
   double umax[3], ext[3];
   for (int k = 0; k < 3; ++k) {
     if (st.periodic[k]) {
@@ -175,8 +180,8 @@ __device__ inline void grid_struct(GmpStruct* S, int s, const unsigned long long
       g.nb[k] = (int)fmin(fmax(nbf, 1.0), 1024.0);
       g.binw[k] = 1.0 / g.nb[k];
     } else {
-      double lo = st.n_atoms ? key_to_double(bbox[6 * s + 2 * k]) : 0.0;
-      double hi = st.n_atoms ? key_to_double(~bbox[6 * s + 2 * k + 1]) : 0.0;
+      double lo = st.n_atoms ? key_to_double(bbox[2 * k]) : 0.0;
+      double hi = st.n_atoms ? key_to_double(~bbox[2 * k + 1]) : 0.0;
       g.umin[k] = lo;
       umax[k] = hi;
       ext[k] = hi - lo;
@@ -242,19 +247,26 @@ __device__ inline void grid_struct(GmpStruct* S, int s, const unsigned long long
   }
   g.inv_h0 = g.rb[0] / (float)cutoff;
   g.pad = 0.0f;
-  G[s] = g;
   float p2 = (float)(b * b * (1.0 + ldexp(1.0, -20)));
-  S[s].prescreen2 = nextafterf(p2, INFINITY);
+  st.prescreen2 = nextafterf(p2, INFINITY);
   const double bi = fmax(cutoff - 2.0 * delta, 0.0);
   float q2 = (float)(bi * bi * (1.0 - ldexp(1.0, -20)));
-  S[s].inside2 = fmaxf(nextafterf(q2, 0.0f), 0.0f);
+  st.inside2 = fmaxf(nextafterf(q2, 0.0f), 0.0f);
 }
 
+__host__ __device__ inline bool all_periodic(const GmpStruct& st) {
+  return st.periodic[0] && st.periodic[1] && st.periodic[2];
+}
+
+// The grids that depend on the atoms' range (all: every structure's).
 __global__ void k_grid(GmpStruct* __restrict__ S, int n_struct,
                        const unsigned long long* __restrict__ bbox, GmpGrid* __restrict__ G,
-                       double cutoff) {
+                       double cutoff, int all) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s < n_struct) grid_struct(S, s, bbox, G, cutoff);
+  if (s >= n_struct || (!all && all_periodic(S[s]))) return;
+  GmpGrid g;
+  grid_struct(S[s], bbox + 6 * s, g, cutoff);
+  G[s] = g;
 }
 
 // Bin of an atom at wrapped fractional coordinates u4 in structure s.
@@ -280,18 +292,6 @@ __device__ __forceinline__ void write_slot(const GmpStruct& st, int64_t a, int32
   for (int c = 0; c < 3; ++c) y[c] = (float)(u4.x * st.A[c] + u4.y * st.A[3 + c] + u4.z * st.A[6 + c]);
   bin_y[slot] = make_float4(y[0], y[1], y[2], wrap);
   bin_je[slot] = make_int2((int32_t)a, __float_as_int(spec));
-}
-
-__global__ void k_bin_assign(const GmpStruct* __restrict__ S, const GmpGrid* __restrict__ G,
-                             const int32_t* __restrict__ struct_of, int64_t N,
-                             const GmpD4* __restrict__ atom_u, int32_t* __restrict__ atom_bin,
-                             int32_t* __restrict__ bin_count) {
-  for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < N;
-       a += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t bin = bin_of(S, G, struct_of[a], atom_u[a]);
-    atom_bin[a] = bin;
-    atomicAdd(&bin_count[bin], 1);
-  }
 }
 
 // Slot lists in arbitrary order: slot_atom[bin_start[b] + k] = the k-th
@@ -339,22 +339,27 @@ __device__ __forceinline__ void center_place(const GmpStruct& st, const GmpGrid&
   y_out = make_float4(y[0], y[1], y[2], 0.0f);
 }
 
-// Per atom: its place in the bin grid and its wrapped FP32 position, so that
-// the neighbor kernels need no FP64 set-up.
-__global__ void k_ranges(const GmpStruct* __restrict__ S, const GmpGrid* __restrict__ G,
-                         const int32_t* __restrict__ struct_of, int64_t N, const GmpD4* __restrict__ atom_u,
-                         float4* __restrict__ atom_t, float4* __restrict__ atom_y) {
+// Per atom: its bin, its place in the bin grid and its wrapped FP32 position
+// (so that the neighbor kernels need no FP64 set-up).
+__global__ void k_bin_assign(const GmpStruct* __restrict__ S, const GmpGrid* __restrict__ G,
+                             const int32_t* __restrict__ struct_of, int64_t N,
+                             const GmpD4* __restrict__ atom_u, int32_t* __restrict__ atom_bin,
+                             int32_t* __restrict__ bin_count, float4* __restrict__ atom_t,
+                             float4* __restrict__ atom_y) {
   for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < N;
        a += (int64_t)gridDim.x * blockDim.x) {
     const int s = struct_of[a];
     const GmpD4 u4 = atom_u[a];
+    const int32_t bin = bin_of(S, G, s, u4);
+    atom_bin[a] = bin;
+    atomicAdd(&bin_count[bin], 1);
     const double u[3] = {u4.x, u4.y, u4.z};
     center_place(S[s], G[s], u, atom_t[a], atom_y[a]);
   }
 }
 
 // Per reference point: the checks, wrap and double-float split of
-// k_prepare and the place of k_ranges, in the structure's atom grid.
+// k_prepare and the place of k_bin_assign, in the structure's atom grid.
 __global__ void k_point_prepare(const GmpStruct* __restrict__ S, const GmpGrid* __restrict__ G,
                                 const int32_t* __restrict__ point_struct, int64_t n, const double* __restrict__ pts,
                                 const double* __restrict__ atom_pos, float4* __restrict__ pt_xh,
@@ -388,7 +393,7 @@ __global__ void k_point_prepare(const GmpStruct* __restrict__ S, const GmpGrid* 
 }
 
 // Small batches: the whole binning (k_prepare, k_grid, k_bin_assign, the
-// scan, k_bin_scatter, k_bin_place, k_ranges) in one CTA, the bin counts,
+// scan, k_bin_scatter, k_bin_place) in one CTA, the bin counts,
 // offsets and slot lists in shared memory; same outputs as those kernels
 // (bins hold their atoms in index order).  A batch of up to about a
 // thousand atoms spends most of its multi-kernel binning time in launch and
@@ -420,7 +425,8 @@ __global__ void __launch_bounds__(1024) k_bin_small(GmpStruct* S, int n_struct, 
   for (int64_t a = tid; a < N; a += nt)
     prepare_atom(S, struct_of, a, pos, species, n_el, atom_xh, atom_xl, atom_u, bbox, err);
   __syncthreads();
-  for (int s = tid; s < n_struct; s += nt) grid_struct(S, s, bbox, G, cutoff);
+  for (int s = tid; s < n_struct; s += nt)
+    if (!all_periodic(S[s])) grid_struct(S[s], bbox + 6 * s, G[s], cutoff);
   __syncthreads();
   for (int64_t a = tid; a < N; a += nt) {
     const int32_t b = bin_of(S, G, struct_of[a], atom_u[a]);
@@ -512,6 +518,49 @@ template <typename T>
 __global__ void k_scan_add(T* __restrict__ out, const T* __restrict__ offs, int64_t n) {
   const int64_t i = (int64_t)blockIdx.x * 1024 + threadIdx.x;
   if (i < n) out[i] += offs[blockIdx.x];
+  if (i == 0) out[n] = offs[gridDim.x];  // the total
+}
+
+// The whole scan in one CTA, 4096 values at a time: one launch where the
+// block scan, the scan of its sums and the addition take three, each of
+// them 3-4 us of latency.  Up to 4 rounds (16384 values, 5 us).
+constexpr int64_t kScanOneCta = 16384;
+template <typename T>
+__global__ void __launch_bounds__(1024) k_scan_one(const T* __restrict__ in, T* __restrict__ out, int64_t n) {
+  __shared__ T tot[32];
+  const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+  T carry = 0;
+  for (int64_t base = 0; base < n; base += 4096) {
+    const int64_t i0 = base + 4 * t;
+    T v[4], run = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      v[k] = run;
+      if (i0 + k < n) run += in[i0 + k];
+    }
+    T incl = run;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const T u = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += u;
+    }
+    if (lane == 31) tot[wid] = incl;
+    __syncthreads();
+    T w = tot[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const T u = __shfl_up_sync(0xffffffffu, w, o);
+      if (lane >= o) w += u;
+    }
+    const T before = __shfl_sync(0xffffffffu, w, (wid + 31) & 31);
+    const T off = carry + (wid ? before : T(0)) + (incl - run);
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (i0 + k < n) out[i0 + k] = off + v[k];
+    carry += __shfl_sync(0xffffffffu, w, 31);
+    __syncthreads();
+  }
+  if (t == 0) out[n] = carry;
 }
 
 // out[0..n] exclusive scan of in[0..n-1]; out[n] = total.  tmp sized by
@@ -522,22 +571,22 @@ cudaError_t exclusive_scan(const T* in, T* out, int64_t n, void* tmp, cudaStream
   if (n <= 0) {
     return cudaMemsetAsync(out, 0, sizeof(T), st);
   }
+  if (n <= kScanOneCta) {
+    k_scan_one<T><<<1, 1024, 0, st>>>(in, out, n);
+    ++*launches;
+    return cudaGetLastError();
+  }
   const int64_t nb = (n + 1023) / 1024;
   T* sums = (T*)tmp;
   T* sums_scan = sums + nb + 1;
   void* rest = (void*)(sums_scan + nb + 1);
   k_scan_block<T><<<(unsigned)nb, 1024, 0, st>>>(in, out, sums, n);
   ++*launches;
-  if (nb == 1) {
-    // total = sums[0]
-    cudaError_t e = cudaMemcpyAsync(out + n, sums, sizeof(T), cudaMemcpyDeviceToDevice, st);
-    return e != cudaSuccess ? e : cudaGetLastError();
-  }
-  cudaError_t e = exclusive_scan<T>(sums, sums_scan, nb, rest, st, launches);
+  const cudaError_t e = exclusive_scan<T>(sums, sums_scan, nb, rest, st, launches);
   if (e != cudaSuccess) return e;
   k_scan_add<T><<<(unsigned)nb, 1024, 0, st>>>(out, sums_scan, n);
   ++*launches;
-  return cudaMemcpyAsync(out + n, sums_scan + nb, sizeof(T), cudaMemcpyDeviceToDevice, st);
+  return cudaGetLastError();
 }
 
 // ----------------------------------------------------------- neighbor pass
@@ -959,50 +1008,50 @@ cudaError_t gmp_exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, v
   return exclusive_scan<int64_t>(in, out, n, tmp, stream, launches);
 }
 
-cudaError_t gmp_launch_neighbors_prepare(const GmpStruct* d_structs, int n_struct,
+void gmp_periodic_grid(GmpStruct& st, GmpGrid& g, double cutoff) {
+  memset(&g, 0, sizeof(g));
+  if (all_periodic(st)) grid_struct(st, nullptr, g, cutoff);
+}
+
+cudaError_t gmp_launch_neighbors_prepare(GmpStruct* d_structs, int n_struct,
                                          const int32_t* d_struct_of, int64_t N, double cutoff,
-                                         const double* pos, const int32_t* species, int n_el,
+                                         const double* pos, const int32_t* species, int n_el, GmpGridMode mode,
                                          GmpGrid* d_grid, float4* atom_xh, float4* atom_xl,
-                                         GmpD4* atom_u, int32_t* atom_bin,
-                                         unsigned long long* d_bbox, uint32_t* d_err,
+                                         GmpD4* atom_u, unsigned long long* d_bbox, int64_t n_bins,
+                                         int32_t* bin_count, int32_t* bin_cursor, uint32_t* d_err,
                                          cudaStream_t stream, int sm_count, int64_t* launches) {
-  (void)atom_bin;
-  cudaError_t e = cudaMemsetAsync(d_bbox, 0xFF, sizeof(unsigned long long) * 6 * n_struct, stream);
-  if (e != cudaSuccess) return e;
+  if (mode != GmpGridMode::kGiven) {
+    const cudaError_t e = cudaMemsetAsync(d_bbox, 0xFF, sizeof(unsigned long long) * 6 * n_struct, stream);
+    if (e != cudaSuccess) return e;
+  }
   k_prepare<<<grid_for(N, 256, sm_count), 256, 0, stream>>>(d_structs, d_struct_of, N, pos, species,
-                                                            n_el, atom_xh, atom_xl, atom_u, d_bbox,
-                                                            d_err);
+                                                            n_el, atom_xh, atom_xl, atom_u, d_bbox, n_bins,
+                                                            bin_count, bin_cursor, d_err);
   ++*launches;
-  k_grid<<<(n_struct + 127) / 128, 128, 0, stream>>>((GmpStruct*)d_structs, n_struct, d_bbox, d_grid,
-                                                     cutoff);
-  ++*launches;
+  if (mode != GmpGridMode::kGiven) {
+    k_grid<<<(n_struct + 31) / 32, 32, 0, stream>>>(d_structs, n_struct, d_bbox, d_grid, cutoff,
+                                                    mode == GmpGridMode::kAll ? 1 : 0);
+    ++*launches;
+  }
   return cudaGetLastError();
 }
 
 cudaError_t gmp_launch_bins(const GmpStruct* d_structs, const GmpGrid* d_grid,
                             const int32_t* d_struct_of, int64_t N, int64_t n_bins,
-                            const int32_t* atom_bin, int32_t* bin_count, int32_t* bin_start,
+                            int32_t* atom_bin, int32_t* bin_count, int32_t* bin_start,
                             int32_t* bin_cursor, float4* atom_t, float4* atom_y, float4* bin_y, int2* bin_je,
                             const GmpD4* atom_u, const float4* atom_xh, const float4* atom_xl, void* scan_tmp,
-                            size_t scan_tmp_bytes, cudaStream_t stream, int sm_count, int64_t* launches) {
-  (void)scan_tmp_bytes;
-  cudaError_t e = cudaMemsetAsync(bin_count, 0, sizeof(int32_t) * n_bins, stream);
-  if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(bin_cursor, 0, sizeof(int32_t) * n_bins, stream);
-  if (e != cudaSuccess) return e;
+                            cudaStream_t stream, int sm_count, int64_t* launches) {
   k_bin_assign<<<grid_for(N, 256, sm_count), 256, 0, stream>>>(d_structs, d_grid, d_struct_of, N,
-                                                               atom_u, (int32_t*)atom_bin, bin_count);
+                                                               atom_u, atom_bin, bin_count, atom_t, atom_y);
   ++*launches;
-  e = exclusive_scan<int32_t>(bin_count, bin_start, n_bins, scan_tmp, stream, launches);
+  cudaError_t e = exclusive_scan<int32_t>(bin_count, bin_start, n_bins, scan_tmp, stream, launches);
   if (e != cudaSuccess) return e;
   // bin_count is free once scanned: it holds the slot lists (n_bins >= N)
   k_bin_scatter<<<grid_for(N, 256, sm_count), 256, 0, stream>>>(N, atom_bin, bin_start, bin_cursor, bin_count);
   ++*launches;
   k_bin_place<<<grid_for(N, 256, sm_count), 256, 0, stream>>>(d_structs, d_struct_of, N, atom_bin, bin_start,
                                                               bin_count, atom_u, atom_xh, atom_xl, bin_y, bin_je);
-  ++*launches;
-  k_ranges<<<grid_for(N, 256, sm_count), 256, 0, stream>>>(d_structs, d_grid, d_struct_of, N, atom_u, atom_t,
-                                                           atom_y);
   ++*launches;
   return cudaGetLastError();
 }

@@ -184,11 +184,12 @@ extern "C" gmp_status gmp_neighbor_counts_noalloc(int32_t n_atoms, const double*
   if (e == cudaSuccess) e = cudaMemsetAsync(d_struct_of, 0, sizeof(int32_t) * n_atoms, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(d_species, 0, sizeof(int32_t) * n_atoms, st);
   if (e == cudaSuccess)
-    e = gmp_launch_neighbors_prepare(d_st, 1, d_struct_of, n_atoms, cutoff, pos, d_species, 1, d_grid, d_xh, d_xl,
-                                     d_u, d_bin, d_bbox, d_err, st, sm_count, &launches);
+    e = gmp_launch_neighbors_prepare(d_st, 1, d_struct_of, n_atoms, cutoff, pos, d_species, 1, GmpGridMode::kAll,
+                                     d_grid, d_xh, d_xl, d_u, d_bbox, n_bins, d_bcount, d_bcursor, d_err, st, sm_count,
+                                     &launches);
   if (e == cudaSuccess)
     e = gmp_launch_bins(d_st, d_grid, d_struct_of, n_atoms, n_bins, d_bin, d_bcount, d_bstart, d_bcursor, d_t,
-                        d_ay, d_by, d_bje, d_u, d_xh, d_xl, d_scan, Layout::scan_bytes, st, sm_count, &launches);
+                        d_ay, d_by, d_bje, d_u, d_xh, d_xl, d_scan, st, sm_count, &launches);
   const GmpCenters centers{d_struct_of, pos, d_xh, d_xl, d_t, d_ay};
   if (e == cudaSuccess)
     e = gmp_launch_neighbor_pass(0, d_st, d_grid, centers, n_atoms, cutoff, pos, d_xh, d_xl, d_bstart, d_by,

@@ -177,18 +177,19 @@ __global__ void __launch_bounds__(256, 2) k_refine(const GmpRefine A) {
 
 }  // namespace
 
-cudaError_t gmp_launch_refine(const GmpRefine& A, int sm_count, cudaStream_t stream, int64_t* launches) {
+cudaError_t gmp_launch_refine(const GmpRefine& A, int sm_count, int* per_sm, cudaStream_t stream, int64_t* launches) {
   bool any = false;  // orders >= 0 requested
   for (int l = 0; l < 7; ++l) any = any || A.qidx[l] >= 0;
   if (A.n_centers <= 0 || !any) return cudaSuccess;
   // as many CTAs as can be resident: the warps take fixed strides of the
   // flagged entries, so a second partial wave would leave most of each SM
   // idle while it runs
-  int per_sm = 0;
-  const cudaError_t eo = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_refine, 256, 0);
-  if (eo != cudaSuccess) return eo;
-  if (per_sm < 1) per_sm = 1;
-  k_refine<<<(unsigned)(sm_count * per_sm), 256, 0, stream>>>(A);
+  if (*per_sm < 1) {
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_refine, 256, 0);
+    if (e != cudaSuccess) return e;
+    if (*per_sm < 1) *per_sm = 1;
+  }
+  k_refine<<<(unsigned)(sm_count * *per_sm), 256, 0, stream>>>(A);
   ++*launches;
   return cudaGetLastError();
 }

@@ -358,8 +358,8 @@ gmp_status upload_structures(gmp_ctx* h, int32_t S, const int64_t* atom_off, con
       if (k % 4 != 0 && g.A[k] != 0.0) g.diag = 0;
     g.bin_base = bin_base;
     g.bin_cap = 2 * g.n_atoms + 8;
-    bin_base += g.bin_cap;
     gmp_periodic_grid(g, grids[s], h->cutoff);
+    bin_base += g.bin_cap;
     if (!(g.periodic[0] && g.periodic[1] && g.periodic[2])) mode = GmpGridMode::kOpen;
   }
   std::memcpy(static_cast<char*>(h->h_desc) + o_off, atom_off, sizeof(int64_t) * (S + 1));
@@ -421,7 +421,7 @@ gmp_status bin_atoms(gmp_ctx* h, int32_t S, const double* pos, const int32_t* sp
   GMP_CK(h->atom_bin.ensure(sizeof(int32_t) * N), "atom_bin");
   GMP_CK(h->atom_t.ensure(sizeof(float4) * N), "atom_t");
   GMP_CK(h->atom_y.ensure(sizeof(float4) * N), "atom_y");
-  GMP_CK(h->bin_count.ensure(sizeof(int32_t) * h->n_bins), "bin_count");
+  GMP_CK(h->bin_count.ensure(sizeof(int32_t) * std::max(h->n_bins, N)), "bin_count");
   GMP_CK(h->bin_cursor.ensure(sizeof(int32_t) * h->n_bins), "bin_cursor");
   GMP_CK(h->bin_start.ensure(sizeof(int32_t) * (h->n_bins + 1)), "bin_start");
   GMP_CK(h->bin_y.ensure(sizeof(float4) * N), "bin_y");

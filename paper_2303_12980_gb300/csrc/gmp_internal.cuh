@@ -351,8 +351,8 @@ cudaError_t gmp_launch_bin_small(GmpStruct* d_structs, int n_struct, const int32
 // from the atoms' range for the structures with a non-periodic axis (the
 // others' are given), or all of them made on the device.
 enum class GmpGridMode { kGiven, kOpen, kAll };
-// Grid and pre-screen bounds of a structure periodic along all axes (host);
-// zeroed for others.
+// Grid and pre-screen bounds of a structure periodic along all axes (host), its
+// bin_cap reduced to the bins the grid has; zeroed for others.
 void gmp_periodic_grid(GmpStruct& st, GmpGrid& g, double cutoff);
 cudaError_t gmp_launch_neighbors_prepare(GmpStruct* d_structs, int n_struct,
                                          const int32_t* d_struct_of, int64_t N, double cutoff,

@@ -44,6 +44,8 @@ __global__ void k_grad_bins_finish(int64_t n, const unsigned long long* __restri
                                    const double* __restrict__ own, const double* acc_in, double* acc_out,
                                    float* __restrict__ grad_pos) {
   constexpr int kBins = 12;
+  constexpr double kBinUnit[11] = {0x1p-149, 0x1p-125, 0x1p-101, 0x1p-77, 0x1p-53, 0x1p-29,
+                                   0x1p-5,   0x1p+19,  0x1p+43,  0x1p+67, 0x1p+91};
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
     const unsigned long long* bt = bins + t * kBins;
     const unsigned long long fl = bt[11];
@@ -53,7 +55,8 @@ __global__ void k_grad_bins_finish(int64_t n, const unsigned long long* __restri
     } else {
       v = 0.0;
 #pragma unroll
-      for (int b = 0; b < 11; ++b) v += ldexp((double)(long long)bt[b], 24 * b - 149);
+      for (int b = 0; b < 11; ++b)  // most are empty; the product is exact
+        if (const long long x = (long long)bt[b]) v = __fma_rn((double)x, kBinUnit[b], v);
     }
     v = own[t] + v;
     if (acc_in) v = acc_in[t] + v;
@@ -113,10 +116,12 @@ cudaError_t gmp_launch_grad_bins_finish(int64_t N, const unsigned long long* bin
                                         int sm_count, int64_t* launches) {
   if (N <= 0) return cudaSuccess;
   const int64_t n = 3 * N;
-  int64_t blocks = (n + 255) / 256;
-  const int64_t cap = (int64_t)sm_count * 8;
+  // (few values: one-warp CTAs over more SMs, for their FP64 sums)
+  const int nt = n >= 256 * (int64_t)sm_count ? 256 : 32;
+  int64_t blocks = (n + nt - 1) / nt;
+  const int64_t cap = (int64_t)sm_count * 32;
   if (blocks > cap) blocks = cap;
-  k_grad_bins_finish<<<(unsigned)blocks, 256, 0, stream>>>(n, bins, own, acc_in, acc_out, grad_pos);
+  k_grad_bins_finish<<<(unsigned)blocks, nt, 0, stream>>>(n, bins, own, acc_in, acc_out, grad_pos);
   ++*launches;
   return cudaGetLastError();
 }

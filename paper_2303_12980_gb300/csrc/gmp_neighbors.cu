@@ -982,6 +982,11 @@ __global__ void k_unpack(int64_t P, const GmpPair* __restrict__ pairs, int32_t* 
   }
 }
 
+// Threads per CTA of the per-atom kernels: their FP64 set-up runs at 2 lanes
+// per clock and SM, so a batch too small to give every SM 256 atoms is cut
+// into one-warp CTAs over more SMs (4096 atoms: 128 SMs instead of 16).
+inline int atom_threads(int64_t n, int sm_count) { return n >= 256 * (int64_t)sm_count ? 256 : 32; }
+
 inline unsigned grid_for(int64_t n, int threads, int sm_count) {
   int64_t b = (n + threads - 1) / threads;
   int64_t cap = (int64_t)sm_count * 32;
@@ -1010,7 +1015,9 @@ cudaError_t gmp_exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, v
 
 void gmp_periodic_grid(GmpStruct& st, GmpGrid& g, double cutoff) {
   memset(&g, 0, sizeof(g));
-  if (all_periodic(st)) grid_struct(st, nullptr, g, cutoff);
+  if (!all_periodic(st)) return;
+  grid_struct(st, nullptr, g, cutoff);
+  st.bin_cap = g.nb[0] * g.nb[1] * g.nb[2];  // known: no more are reserved, cleared and scanned
 }
 
 cudaError_t gmp_launch_neighbors_prepare(GmpStruct* d_structs, int n_struct,
@@ -1024,7 +1031,8 @@ cudaError_t gmp_launch_neighbors_prepare(GmpStruct* d_structs, int n_struct,
     const cudaError_t e = cudaMemsetAsync(d_bbox, 0xFF, sizeof(unsigned long long) * 6 * n_struct, stream);
     if (e != cudaSuccess) return e;
   }
-  k_prepare<<<grid_for(N, 256, sm_count), 256, 0, stream>>>(d_structs, d_struct_of, N, pos, species,
+  const int nt = atom_threads(N, sm_count);
+  k_prepare<<<grid_for(N, nt, sm_count), nt, 0, stream>>>(d_structs, d_struct_of, N, pos, species,
                                                             n_el, atom_xh, atom_xl, atom_u, d_bbox, n_bins,
                                                             bin_count, bin_cursor, d_err);
   ++*launches;
@@ -1042,15 +1050,17 @@ cudaError_t gmp_launch_bins(const GmpStruct* d_structs, const GmpGrid* d_grid,
                             int32_t* bin_cursor, float4* atom_t, float4* atom_y, float4* bin_y, int2* bin_je,
                             const GmpD4* atom_u, const float4* atom_xh, const float4* atom_xl, void* scan_tmp,
                             cudaStream_t stream, int sm_count, int64_t* launches) {
-  k_bin_assign<<<grid_for(N, 256, sm_count), 256, 0, stream>>>(d_structs, d_grid, d_struct_of, N,
+  const int nt = atom_threads(N, sm_count);
+  k_bin_assign<<<grid_for(N, nt, sm_count), nt, 0, stream>>>(d_structs, d_grid, d_struct_of, N,
                                                                atom_u, atom_bin, bin_count, atom_t, atom_y);
   ++*launches;
   cudaError_t e = exclusive_scan<int32_t>(bin_count, bin_start, n_bins, scan_tmp, stream, launches);
   if (e != cudaSuccess) return e;
-  // bin_count is free once scanned: it holds the slot lists (n_bins >= N)
+  // bin_count is free once scanned: it holds the slot lists (room for
+  // max(n_bins, N) values)
   k_bin_scatter<<<grid_for(N, 256, sm_count), 256, 0, stream>>>(N, atom_bin, bin_start, bin_cursor, bin_count);
   ++*launches;
-  k_bin_place<<<grid_for(N, 256, sm_count), 256, 0, stream>>>(d_structs, d_struct_of, N, atom_bin, bin_start,
+  k_bin_place<<<grid_for(N, nt, sm_count), nt, 0, stream>>>(d_structs, d_struct_of, N, atom_bin, bin_start,
                                                               bin_count, atom_u, atom_xh, atom_xl, bin_y, bin_je);
   ++*launches;
   return cudaGetLastError();
@@ -1085,7 +1095,8 @@ cudaError_t gmp_launch_point_prepare(const GmpStruct* d_structs, const GmpGrid* 
                                      float4* pt_y, uint32_t* d_err, cudaStream_t stream, int sm_count,
                                      int64_t* launches) {
   if (n_points <= 0) return cudaSuccess;
-  k_point_prepare<<<grid_for(n_points, 256, sm_count), 256, 0, stream>>>(
+  const int nt = atom_threads(n_points, sm_count);
+  k_point_prepare<<<grid_for(n_points, nt, sm_count), nt, 0, stream>>>(
       d_structs, d_grid, point_struct, n_points, points, atom_pos, pt_xh, pt_xl, pt_t, pt_y, d_err);
   ++*launches;
   return cudaGetLastError();

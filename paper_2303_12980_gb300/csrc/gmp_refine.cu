@@ -135,14 +135,13 @@ __device__ __forceinline__ void refine_entry(int lane, const GmpRefine& A, const
   }
 }
 
+// (count: lane l holds the entries of order l)
 template <int L>
 __device__ __forceinline__ void refine_order(int lane, const GmpRefine& A, const float2* exp_tab, int64_t warp,
-                                             int64_t nw, int64_t& done) {
-  const int qi = A.qidx[L];
-  if (qi >= 0) {
-    const unsigned long long c = A.count[qi];
-    const int64_t n = c < (unsigned long long)A.cap ? (int64_t)c : A.cap;
-    const unsigned long long* queue = A.queue + qi * A.cap;
+                                             int64_t nw, int64_t count, int64_t& done) {
+  const int64_t n = __shfl_sync(0xffffffffu, count, L);
+  if (n > 0) {
+    const unsigned long long* queue = A.queue + A.qidx[L] * A.cap;
     int64_t v = (warp - done) % nw;
     if (v < 0) v += nw;
     for (; v < n; v += nw) {
@@ -151,7 +150,7 @@ __device__ __forceinline__ void refine_order(int lane, const GmpRefine& A, const
     }
     done += n;
   }
-  if constexpr (L > 0) refine_order<L - 1>(lane, A, exp_tab, warp, nw, done);
+  if constexpr (L > 0) refine_order<L - 1>(lane, A, exp_tab, warp, nw, count, done);
 }
 
 // A warp per entry, the entries of all orders numbered through, the largest
@@ -169,10 +168,15 @@ __device__ __forceinline__ void refine_order(int lane, const GmpRefine& A, const
 __global__ void __launch_bounds__(256, 2) k_refine(const GmpRefine A) {
   __shared__ float2 exp_tab[64];
   if (threadIdx.x < 64) exp_tab[threadIdx.x] = A.exp_tab[threadIdx.x];
+  const int lane = threadIdx.x & 31;
+  int64_t count = 0;
+#pragma unroll
+  for (int l = 0; l < 7; ++l)
+    if (lane == l && A.qidx[l] >= 0) count = (int64_t)min(A.count[A.qidx[l]], (unsigned long long)A.cap);
   __syncthreads();
   int64_t done = 0;
-  refine_order<6>(threadIdx.x & 31, A, exp_tab, ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5,
-                  ((int64_t)gridDim.x * blockDim.x) >> 5, done);
+  refine_order<6>(lane, A, exp_tab, ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5,
+                  ((int64_t)gridDim.x * blockDim.x) >> 5, count, done);
 }
 
 }  // namespace

@@ -36,6 +36,7 @@ from collections import defaultdict
 from fractions import Fraction
 
 LMAX = 6
+JAC_LMAX = 4  # highest order of the Jacobian kernel that takes gradient coefficients
 
 
 # ---------------------------------------------------------------- polynomials
@@ -501,15 +502,68 @@ def emit_shift_contract(L):
     return "\n".join(lines)
 
 
+def grad_coefs(l):
+    """D[v][k] = {k': c} with dS_k/dv = sum c S_k', k of order l, k' of order
+    l - 1 (independent components): the derivative of a harmonic polynomial is
+    harmonic, so its coefficients of the monomials with at most one x, which
+    fix it, give the combination."""
+    low = indep_components(l - 1)
+    monos = low
+    A = [[Fraction(closed_form(*u).get(mo, 0)) for u in low] for mo in monos]
+    out = []
+    for v in range(3):
+        rows = []
+        for t in indep_components(l):
+            p = deriv(closed_form(*t), v)
+            M = [r[:] + [Fraction(p.get(mo, 0))] for r, mo in zip(A, monos)]
+            n = len(M)
+            for i in range(n):
+                piv = next(r for r in range(i, n) if M[r][i])
+                M[i], M[piv] = M[piv], M[i]
+                M[i] = [x / M[i][i] for x in M[i]]
+                for r in range(n):
+                    if r != i and M[r][i]:
+                        f = M[r][i]
+                        M[r] = [x - f * w for x, w in zip(M[r], M[i])]
+            row = {j: M[j][n] for j in range(n) if M[j][n]}
+            assert padd(*[(c, closed_form(*low[j])) for j, c in row.items()]) == p, (t, v)
+            rows.append(row)
+        out.append(rows)
+    return out
+
+
+def emit_grad_coef_order(l):
+    """Mv[k'] (k' of order l - 1, flat) with d/dv sum_k lam_k S_k = sum_k' Mv[k']
+    S_k', k of order l (flat): once per center, the gradient of a pair then
+    needs no order above l - 1."""
+    D = grad_coefs(l)
+    ind, low = indep_components(l), indep_components(l - 1)
+    L = [f"__device__ __forceinline__ void gmp_mcsh_grad_coef_order_{l}(const float* __restrict__ lam, "
+         f"float* __restrict__ Mx, float* __restrict__ My, float* __restrict__ Mz) {{"]
+    for v in range(3):
+        for j, u in enumerate(low):
+            e = None
+            for k, t in enumerate(ind):
+                c = D[v][k].get(j, 0)
+                if c:
+                    e = f"__fmul_rn({fnum(c)}, lam[{flat(t)}])" if e is None else f"__fmaf_rn({fnum(c)}, lam[{flat(t)}], {e})"
+            L.append(f"  M{'xyz'[v]}[{flat(u)}] = {e or '0.0f'};")
+    L.append("}")
+    return "\n".join(L)
+
+
+def deriv(p, ax):
+    out = {}
+    for m, v in p.items():
+        if m[ax]:
+            mm = list(m)
+            mm[ax] -= 1
+            out[tuple(mm)] = out.get(tuple(mm), 0) + v * m[ax]
+    return {m: v for m, v in out.items() if v}
+
+
 def check_shift_identity():
     """r^2 dS/dv == (2l+1) v S - S_{+v} for all components up to LMAX."""
-    def deriv(p, ax):
-        out = {}
-        for m, v in p.items():
-            if m[ax]:
-                mm = list(m); mm[ax] -= 1
-                out[tuple(mm)] = out.get(tuple(mm), 0) + v * m[ax]
-        return {m: v for m, v in out.items() if v}
     for l in range(LMAX + 1):
         for t in all_components(l):
             S = closed_form(*t)
@@ -547,6 +601,8 @@ def generate() -> str:
         out.append(emit_shift_contract(L))
     for l in range(LMAX + 1):
         out.append(emit_shift_contract_order(l))
+    for l in range(1, JAC_LMAX + 1):
+        out.append(emit_grad_coef_order(l))
     out.append("")
     out.append("template <int L> struct GmpMcsh;")
     for L in range(LMAX + 2):

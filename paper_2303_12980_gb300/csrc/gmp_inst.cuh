@@ -2,6 +2,7 @@
 // seven orders compile in parallel).
 #pragma once
 
+#include "gmp_jacobian.cuh"
 #include "gmp_kernels.cuh"
 #include "gmp_launch.h"
 
@@ -27,9 +28,17 @@ cudaError_t launch(int kind, const KParams& K, GmpShape shape, GmpLaunchPlan* pl
                             ? (K.pass.mixed_sign ? k_backward<L, NS, false, true> : k_backward<L, NS, false, false>)
                         : kind == GMP_KIND_BACKWARD_VIRIAL
                             ? (K.pass.mixed_sign ? k_backward<L, NS, true, true> : k_backward<L, NS, true, false>)
-                            : k_jacobian<L, NS>;
+                            : nullptr;
+  if constexpr (L <= kJacRegOrders) {
+    if (kind == GMP_KIND_JACOBIAN) fn = k_jacobian_r<L, NS>;
+  } else {
+    if (kind == GMP_KIND_JACOBIAN) fn = k_jacobian<L, NS>;
+  }
   const int extra = kind == GMP_KIND_BACKWARD_VIRIAL ? virial_extra_floats<L, NS>() : 0;
-  auto smem_of = [&](int w) {
+  auto smem_of = [&](int w) -> size_t {
+    if constexpr (L <= kJacRegOrders)
+      if (kind == GMP_KIND_JACOBIAN)
+        return sizeof(float) * (table_floats(K.pass.n_el, L, NS, K.pass.kmax) + (size_t)w * JacShape<L, NS>::WARP_FLOATS);
     const bool pad = kind != GMP_KIND_BACKWARD && kind != GMP_KIND_JACOBIAN;  // these two: unpadded table
     return tile == 32 ? smem_bytes<L, NS, 32>(K.pass, w, 0) : smem_bytes<L, NS, 16>(K.pass, w, extra, pad);
   };
@@ -52,17 +61,19 @@ cudaError_t launch(int kind, const KParams& K, GmpShape shape, GmpLaunchPlan* pl
     if (want > 0 && want < warps) warps = want;
     while (warps > 1 && smem_of(warps) > 227 * 1024) --warps;
     if (want <= 0) {
-      // untuned: the CTA size with the most resident warps, the larger of two
-      // equals (registers and the tables' share of the shared memory decide:
-      // the forward kernel at orders 0-4 x 8 sigmas keeps 24 warps in 4-warp
-      // CTAs and 16 in one of 16, 3.40 against 4.03 ms on 10,000 structures)
+      // untuned: the CTA size with the most resident warps, of equals the
+      // smallest with at least 4 (registers and the tables' share of the
+      // shared memory decide: the forward kernel at orders 0-4 x 8 sigmas keeps
+      // 24 warps in 4-warp CTAs and 16 in one of 16, 3.40 against 4.03 ms on
+      // 10,000 structures; 4096 Jacobian centers took 177 us in 12-warp CTAs
+      // and 167 in as many warps of 4-warp ones)
       int best_w = warps, best_res = 0;
       for (int w = warps; w >= 1; --w) {
         if (smem_of(w) > 227 * 1024) continue;
         int ps = 0;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, fn, w * 32, smem_of(w));
         if (e != cudaSuccess) return e;
-        if (ps * w > best_res) { best_res = ps * w; best_w = w; }
+        if (ps * w > best_res || (ps * w == best_res && w >= 4)) { best_res = ps * w; best_w = w; }
       }
       warps = best_w;
     }

@@ -207,6 +207,21 @@ __device__ __forceinline__ float2 gmp_exp_neg2(float2 Bhi, float2 Blo, float2 nr
   return gmp_fma2(E, gmp_mul2(make_float2(-0.69314718055994531f, -0.69314718055994531f), xl), E);
 }
 
+// The same times 2^S (an integer S per lane of the pair, 0..126), with the
+// operations of gmp_exp_neg_shifted_by below in packed form.
+__device__ __forceinline__ float2 gmp_exp_neg2_shifted(float2 Bhi, float2 Blo, float2 nr2h, float2 r2h, float2 r2l,
+                                                       float2 S) {
+  const float2 nxh = gmp_mul2(Bhi, nr2h);
+  float2 xl = gmp_fma2(Bhi, r2h, nxh);
+  xl = gmp_fma2(Bhi, r2l, xl);
+  xl = gmp_fma2(Blo, r2h, xl);
+  const float2 m1 = make_float2(-1.0f, -1.0f);
+  const float2 d = gmp_add2(S, nxh);
+  const float2 e = gmp_add2(gmp_fma2(d, m1, S), nxh);  // (S - xh) - d, exactly
+  const float2 E = make_float2(gmp_ex2(d.x), gmp_ex2(d.y));
+  return gmp_fma2(E, gmp_mul2(make_float2(-0.69314718055994531f, -0.69314718055994531f), gmp_fma2(e, m1, xl)), E);
+}
+
 // exp(-B r^2) with B and r^2 given as double-floats: the product is formed
 // to about 2^-44 relative, the SFU takes its high part and the low part is
 // applied to first order, exp2(-(h+l)) = exp2(-h) (1 - ln2 l).

@@ -1752,6 +1752,62 @@ __device__ __forceinline__ void gmp_mcsh_shift_contract_order_6(const float* __r
   vz = __fmaf_rn(lam[48], S1[63], vz);
   V[0] = vx; V[1] = vy; V[2] = vz;
 }
+__device__ __forceinline__ void gmp_mcsh_grad_coef_order_1(const float* __restrict__ lam, float* __restrict__ Mx, float* __restrict__ My, float* __restrict__ Mz) {
+  Mx[0] = __fmul_rn(1.0f, lam[3]);
+  My[0] = __fmul_rn(1.0f, lam[1]);
+  Mz[0] = __fmul_rn(1.0f, lam[2]);
+}
+__device__ __forceinline__ void gmp_mcsh_grad_coef_order_2(const float* __restrict__ lam, float* __restrict__ Mx, float* __restrict__ My, float* __restrict__ Mz) {
+  Mx[1] = __fmul_rn(3.0f, lam[7]);
+  Mx[2] = __fmul_rn(3.0f, lam[8]);
+  Mx[3] = __fmaf_rn(-2.0f, lam[6], __fmul_rn(-2.0f, lam[4]));
+  My[1] = __fmaf_rn(-2.0f, lam[6], __fmul_rn(4.0f, lam[4]));
+  My[2] = __fmul_rn(3.0f, lam[5]);
+  My[3] = __fmul_rn(3.0f, lam[7]);
+  Mz[1] = __fmul_rn(3.0f, lam[5]);
+  Mz[2] = __fmaf_rn(4.0f, lam[6], __fmul_rn(-2.0f, lam[4]));
+  Mz[3] = __fmul_rn(3.0f, lam[8]);
+}
+__device__ __forceinline__ void gmp_mcsh_grad_coef_order_3(const float* __restrict__ lam, float* __restrict__ Mx, float* __restrict__ My, float* __restrict__ Mz) {
+  Mx[4] = __fmaf_rn(2.0f, lam[15], __fmul_rn(7.0f, lam[13]));
+  Mx[5] = __fmul_rn(5.0f, lam[14]);
+  Mx[6] = __fmaf_rn(7.0f, lam[15], __fmul_rn(2.0f, lam[13]));
+  Mx[7] = __fmaf_rn(-2.0f, lam[11], __fmul_rn(-6.0f, lam[9]));
+  Mx[8] = __fmaf_rn(-6.0f, lam[12], __fmul_rn(-2.0f, lam[10]));
+  My[4] = __fmaf_rn(-2.0f, lam[11], __fmul_rn(9.0f, lam[9]));
+  My[5] = __fmaf_rn(-6.0f, lam[12], __fmul_rn(8.0f, lam[10]));
+  My[6] = __fmul_rn(5.0f, lam[11]);
+  My[7] = __fmaf_rn(-2.0f, lam[15], __fmul_rn(8.0f, lam[13]));
+  My[8] = __fmul_rn(5.0f, lam[14]);
+  Mz[4] = __fmul_rn(5.0f, lam[10]);
+  Mz[5] = __fmaf_rn(8.0f, lam[11], __fmul_rn(-6.0f, lam[9]));
+  Mz[6] = __fmaf_rn(9.0f, lam[12], __fmul_rn(-2.0f, lam[10]));
+  Mz[7] = __fmul_rn(5.0f, lam[14]);
+  Mz[8] = __fmaf_rn(8.0f, lam[15], __fmul_rn(-2.0f, lam[13]));
+}
+__device__ __forceinline__ void gmp_mcsh_grad_coef_order_4(const float* __restrict__ lam, float* __restrict__ Mx, float* __restrict__ My, float* __restrict__ Mz) {
+  Mx[9] = __fmaf_rn(2.0f, lam[23], __fmul_rn(13.0f, lam[21]));
+  Mx[10] = __fmaf_rn(6.0f, lam[24], __fmul_rn(9.0f, lam[22]));
+  Mx[11] = __fmaf_rn(9.0f, lam[23], __fmul_rn(6.0f, lam[21]));
+  Mx[12] = __fmaf_rn(13.0f, lam[24], __fmul_rn(2.0f, lam[22]));
+  Mx[13] = __fmaf_rn(-2.0f, lam[18], __fmul_rn(-12.0f, lam[16]));
+  Mx[14] = __fmaf_rn(-6.0f, lam[19], __fmul_rn(-6.0f, lam[17]));
+  Mx[15] = __fmaf_rn(-12.0f, lam[20], __fmul_rn(-2.0f, lam[18]));
+  My[9] = __fmaf_rn(-2.0f, lam[18], __fmul_rn(16.0f, lam[16]));
+  My[10] = __fmaf_rn(-6.0f, lam[19], __fmul_rn(15.0f, lam[17]));
+  My[11] = __fmaf_rn(-12.0f, lam[20], __fmul_rn(12.0f, lam[18]));
+  My[12] = __fmul_rn(7.0f, lam[19]);
+  My[13] = __fmaf_rn(-2.0f, lam[23], __fmul_rn(15.0f, lam[21]));
+  My[14] = __fmaf_rn(-6.0f, lam[24], __fmul_rn(12.0f, lam[22]));
+  My[15] = __fmul_rn(7.0f, lam[23]);
+  Mz[9] = __fmul_rn(7.0f, lam[17]);
+  Mz[10] = __fmaf_rn(12.0f, lam[18], __fmul_rn(-12.0f, lam[16]));
+  Mz[11] = __fmaf_rn(15.0f, lam[19], __fmul_rn(-6.0f, lam[17]));
+  Mz[12] = __fmaf_rn(16.0f, lam[20], __fmul_rn(-2.0f, lam[18]));
+  Mz[13] = __fmul_rn(7.0f, lam[22]);
+  Mz[14] = __fmaf_rn(12.0f, lam[23], __fmul_rn(-6.0f, lam[21]));
+  Mz[15] = __fmaf_rn(15.0f, lam[24], __fmul_rn(-2.0f, lam[22]));
+}
 
 template <int L> struct GmpMcsh;
 template <> struct GmpMcsh<0> {

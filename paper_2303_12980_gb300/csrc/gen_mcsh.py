@@ -348,7 +348,8 @@ def check_solid():
 
 
 def emit_solid_df(l):
-    """The solid harmonics of order l in double-float arithmetic."""
+    """The solid harmonics of order l in double-float arithmetic.  Products that
+    only enter a sum or a final product stay unnormalised (gmp_df_mul_u)."""
     L = [f"__device__ __forceinline__ void gmp_solid_df_{l}(gmp_f2 x, gmp_f2 y, gmp_f2 z, gmp_f2 r2, gmp_f2* __restrict__ H) {{"]
     if l == 0:
         return "\n".join(L + ["  H[0] = gmp_f2{1.0f, 0.0f};", "}"])
@@ -357,22 +358,22 @@ def emit_solid_df(l):
     for k in range(2, l // 2 + 1):
         L.append(f"  const gmp_f2 r2_{k} = gmp_df_mul(r2, {'r2' if k == 2 else f'r2_{k - 1}'});")
     rk = lambda k: "r2" if k == 1 else f"r2_{k}"
-    times = lambda v, e: e if v == 1 else f"gmp_df_mul_f({e}, {fnum(v)})"
+    times = lambda v, e: e if v == 1 else f"gmp_df_mul_fu({e}, {fnum(v)})"  # (inside sums)
     L.append("  gmp_f2 a = x, b = y;")
     j = 0
     for m, part, _, c, _ in solid_harmonics(l):
         if part:
             continue
         if m > 1:
-            L.append("  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul(x, a), gmp_df_neg(gmp_df_mul(y, b)));")
-            L.append("    b = gmp_df_add_sloppy(gmp_df_mul(x, b), gmp_df_mul(y, a));")
+            L.append("  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul_u(x, a), gmp_df_neg(gmp_df_mul_u(y, b)));")
+            L.append("    b = gmp_df_add_sloppy(gmp_df_mul_u(x, b), gmp_df_mul_u(y, a));")
             L.append("    a = t; }")
         e = None
         for k, v in enumerate(c[1:], 1):
-            lead = times(c[0], "z2") if k == 1 else f"gmp_df_mul({e}, z2)"
+            lead = times(c[0], "z2") if k == 1 else f"gmp_df_mul_u({e}, z2)"
             e = f"gmp_df_add_sloppy({lead}, {times(v, rk(k))})"
         if (l - m) % 2:
-            e = "z" if e is None else f"gmp_df_mul({e}, z)"
+            e = "z" if e is None else f"gmp_df_mul{'_u' if m == 0 else ''}({e}, z)"
         if m == 0:
             L.append(f"  H[0] = {e};")
             j = 1
@@ -380,7 +381,7 @@ def emit_solid_df(l):
         if e is None:
             L.append(f"  H[{j}] = a; H[{j + 1}] = b;")
         else:
-            L.append(f"  {{ const gmp_f2 q = {e}; H[{j}] = gmp_df_mul(q, a); H[{j + 1}] = gmp_df_mul(q, b); }}")
+            L.append(f"  {{ const gmp_f2 q = {e}; H[{j}] = gmp_df_mul_u(q, a); H[{j + 1}] = gmp_df_mul_u(q, b); }}")
         j += 2
     L.append("}")
     return "\n".join(L)

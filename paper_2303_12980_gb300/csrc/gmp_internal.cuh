@@ -147,6 +147,17 @@ __device__ __forceinline__ gmp_f2 gmp_df_mul(gmp_f2 a, gmp_f2 b) {
   float e = __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.lo, b.hi, p.lo));
   return gmp_fast_two_sum(p.hi, e);
 }
+// The same without the renormalisation: the low word may reach a few units in
+// the last place of the high one, which sums and products with further
+// operands take as it is.
+__device__ __forceinline__ gmp_f2 gmp_df_mul_u(gmp_f2 a, gmp_f2 b) {
+  const gmp_f2 p = gmp_two_prod(a.hi, b.hi);
+  return {p.hi, __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.lo, b.hi, p.lo))};
+}
+__device__ __forceinline__ gmp_f2 gmp_df_mul_fu(gmp_f2 a, float b) {
+  const gmp_f2 p = gmp_two_prod(a.hi, b);
+  return {p.hi, __fmaf_rn(a.lo, b, p.lo)};
+}
 // Double-float times a float.
 __device__ __forceinline__ gmp_f2 gmp_df_mul_f(gmp_f2 a, float b) {
   gmp_f2 p = gmp_two_prod(a.hi, b);

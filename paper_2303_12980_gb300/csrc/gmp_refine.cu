@@ -78,10 +78,14 @@ __device__ __forceinline__ void refine_entry(int lane, const GmpRefine& A, const
     for (int k = 0; k < NV; ++k) mu[g][k] = gmp_f2{0.0f, 0.0f};
   for (int64_t p = p0 + lane; p < p1; p += 32) {
     const GmpPair pr = A.pairs[p];
+    // the next pair's atom, whose position is fetched while this one is computed
+    const int jn = p + 32 < p1 ? A.pairs[p + 32].j : pr.j;
     int nn[3];
     gmp_unpack_shift(pr.shift, nn);
     gmp_f2 d[3], r2, H[2 * L + 1];
     gmp_df_disp(xhi, xli, A.atom_xh[pr.j], A.atom_xl[pr.j], st, nn, d, r2);
+    asm volatile("prefetch.global.L1 [%0];" ::"l"(A.atom_xh + jn));
+    asm volatile("prefetch.global.L1 [%0];" ::"l"(A.atom_xl + jn));
     gmp_solid_df<L>(d[0], d[1], d[2], r2, H);
 #pragma unroll
     for (int g = 0; g < 2; ++g) {
@@ -92,7 +96,7 @@ __device__ __forceinline__ void refine_entry(int lane, const GmpRefine& A, const
       gmp_f2 R{0.0f, 0.0f};
       for (int q = 0; q < A.kmax; ++q) {
         const float2 b = __ldg(te + 8 * q), a = __ldg(te + 8 * q + 1 + L);
-        const gmp_f2 E = gmp_df_exp_neg(gmp_df_mul(gmp_f2{b.x, b.y}, r2), exp_tab);
+        const gmp_f2 E = gmp_df_exp_neg(gmp_df_mul_u(gmp_f2{b.x, b.y}, r2), exp_tab);
         const gmp_f2 t = gmp_two_prod(a.x, E.hi);
         const gmp_f2 s = gmp_two_sum(R.hi, t.hi);
         R.hi = s.hi;

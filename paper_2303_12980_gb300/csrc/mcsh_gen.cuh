@@ -537,24 +537,24 @@ __device__ __forceinline__ void gmp_solid_df_1(gmp_f2 x, gmp_f2 y, gmp_f2 z, gmp
 __device__ __forceinline__ void gmp_solid_df_2(gmp_f2 x, gmp_f2 y, gmp_f2 z, gmp_f2 r2, gmp_f2* __restrict__ H) {
   const gmp_f2 z2 = gmp_df_mul(z, z);
   gmp_f2 a = x, b = y;
-  H[0] = gmp_df_add_sloppy(gmp_df_mul_f(z2, 3.0f), gmp_df_mul_f(r2, -1.0f));
-  { const gmp_f2 q = z; H[1] = gmp_df_mul(q, a); H[2] = gmp_df_mul(q, b); }
-  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul(x, a), gmp_df_neg(gmp_df_mul(y, b)));
-    b = gmp_df_add_sloppy(gmp_df_mul(x, b), gmp_df_mul(y, a));
+  H[0] = gmp_df_add_sloppy(gmp_df_mul_fu(z2, 3.0f), gmp_df_mul_fu(r2, -1.0f));
+  { const gmp_f2 q = z; H[1] = gmp_df_mul_u(q, a); H[2] = gmp_df_mul_u(q, b); }
+  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul_u(x, a), gmp_df_neg(gmp_df_mul_u(y, b)));
+    b = gmp_df_add_sloppy(gmp_df_mul_u(x, b), gmp_df_mul_u(y, a));
     a = t; }
   H[3] = a; H[4] = b;
 }
 __device__ __forceinline__ void gmp_solid_df_3(gmp_f2 x, gmp_f2 y, gmp_f2 z, gmp_f2 r2, gmp_f2* __restrict__ H) {
   const gmp_f2 z2 = gmp_df_mul(z, z);
   gmp_f2 a = x, b = y;
-  H[0] = gmp_df_mul(gmp_df_add_sloppy(gmp_df_mul_f(z2, 5.0f), gmp_df_mul_f(r2, -3.0f)), z);
-  { const gmp_f2 q = gmp_df_add_sloppy(gmp_df_mul_f(z2, 5.0f), gmp_df_mul_f(r2, -1.0f)); H[1] = gmp_df_mul(q, a); H[2] = gmp_df_mul(q, b); }
-  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul(x, a), gmp_df_neg(gmp_df_mul(y, b)));
-    b = gmp_df_add_sloppy(gmp_df_mul(x, b), gmp_df_mul(y, a));
+  H[0] = gmp_df_mul_u(gmp_df_add_sloppy(gmp_df_mul_fu(z2, 5.0f), gmp_df_mul_fu(r2, -3.0f)), z);
+  { const gmp_f2 q = gmp_df_add_sloppy(gmp_df_mul_fu(z2, 5.0f), gmp_df_mul_fu(r2, -1.0f)); H[1] = gmp_df_mul_u(q, a); H[2] = gmp_df_mul_u(q, b); }
+  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul_u(x, a), gmp_df_neg(gmp_df_mul_u(y, b)));
+    b = gmp_df_add_sloppy(gmp_df_mul_u(x, b), gmp_df_mul_u(y, a));
     a = t; }
-  { const gmp_f2 q = z; H[3] = gmp_df_mul(q, a); H[4] = gmp_df_mul(q, b); }
-  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul(x, a), gmp_df_neg(gmp_df_mul(y, b)));
-    b = gmp_df_add_sloppy(gmp_df_mul(x, b), gmp_df_mul(y, a));
+  { const gmp_f2 q = z; H[3] = gmp_df_mul_u(q, a); H[4] = gmp_df_mul_u(q, b); }
+  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul_u(x, a), gmp_df_neg(gmp_df_mul_u(y, b)));
+    b = gmp_df_add_sloppy(gmp_df_mul_u(x, b), gmp_df_mul_u(y, a));
     a = t; }
   H[5] = a; H[6] = b;
 }
@@ -562,18 +562,18 @@ __device__ __forceinline__ void gmp_solid_df_4(gmp_f2 x, gmp_f2 y, gmp_f2 z, gmp
   const gmp_f2 z2 = gmp_df_mul(z, z);
   const gmp_f2 r2_2 = gmp_df_mul(r2, r2);
   gmp_f2 a = x, b = y;
-  H[0] = gmp_df_add_sloppy(gmp_df_mul(gmp_df_add_sloppy(gmp_df_mul_f(z2, 35.0f), gmp_df_mul_f(r2, -30.0f)), z2), gmp_df_mul_f(r2_2, 3.0f));
-  { const gmp_f2 q = gmp_df_mul(gmp_df_add_sloppy(gmp_df_mul_f(z2, 7.0f), gmp_df_mul_f(r2, -3.0f)), z); H[1] = gmp_df_mul(q, a); H[2] = gmp_df_mul(q, b); }
-  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul(x, a), gmp_df_neg(gmp_df_mul(y, b)));
-    b = gmp_df_add_sloppy(gmp_df_mul(x, b), gmp_df_mul(y, a));
+  H[0] = gmp_df_add_sloppy(gmp_df_mul_u(gmp_df_add_sloppy(gmp_df_mul_fu(z2, 35.0f), gmp_df_mul_fu(r2, -30.0f)), z2), gmp_df_mul_fu(r2_2, 3.0f));
+  { const gmp_f2 q = gmp_df_mul(gmp_df_add_sloppy(gmp_df_mul_fu(z2, 7.0f), gmp_df_mul_fu(r2, -3.0f)), z); H[1] = gmp_df_mul_u(q, a); H[2] = gmp_df_mul_u(q, b); }
+  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul_u(x, a), gmp_df_neg(gmp_df_mul_u(y, b)));
+    b = gmp_df_add_sloppy(gmp_df_mul_u(x, b), gmp_df_mul_u(y, a));
     a = t; }
-  { const gmp_f2 q = gmp_df_add_sloppy(gmp_df_mul_f(z2, 7.0f), gmp_df_mul_f(r2, -1.0f)); H[3] = gmp_df_mul(q, a); H[4] = gmp_df_mul(q, b); }
-  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul(x, a), gmp_df_neg(gmp_df_mul(y, b)));
-    b = gmp_df_add_sloppy(gmp_df_mul(x, b), gmp_df_mul(y, a));
+  { const gmp_f2 q = gmp_df_add_sloppy(gmp_df_mul_fu(z2, 7.0f), gmp_df_mul_fu(r2, -1.0f)); H[3] = gmp_df_mul_u(q, a); H[4] = gmp_df_mul_u(q, b); }
+  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul_u(x, a), gmp_df_neg(gmp_df_mul_u(y, b)));
+    b = gmp_df_add_sloppy(gmp_df_mul_u(x, b), gmp_df_mul_u(y, a));
     a = t; }
-  { const gmp_f2 q = z; H[5] = gmp_df_mul(q, a); H[6] = gmp_df_mul(q, b); }
-  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul(x, a), gmp_df_neg(gmp_df_mul(y, b)));
-    b = gmp_df_add_sloppy(gmp_df_mul(x, b), gmp_df_mul(y, a));
+  { const gmp_f2 q = z; H[5] = gmp_df_mul_u(q, a); H[6] = gmp_df_mul_u(q, b); }
+  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul_u(x, a), gmp_df_neg(gmp_df_mul_u(y, b)));
+    b = gmp_df_add_sloppy(gmp_df_mul_u(x, b), gmp_df_mul_u(y, a));
     a = t; }
   H[7] = a; H[8] = b;
 }
@@ -581,22 +581,22 @@ __device__ __forceinline__ void gmp_solid_df_5(gmp_f2 x, gmp_f2 y, gmp_f2 z, gmp
   const gmp_f2 z2 = gmp_df_mul(z, z);
   const gmp_f2 r2_2 = gmp_df_mul(r2, r2);
   gmp_f2 a = x, b = y;
-  H[0] = gmp_df_mul(gmp_df_add_sloppy(gmp_df_mul(gmp_df_add_sloppy(gmp_df_mul_f(z2, 63.0f), gmp_df_mul_f(r2, -70.0f)), z2), gmp_df_mul_f(r2_2, 15.0f)), z);
-  { const gmp_f2 q = gmp_df_add_sloppy(gmp_df_mul(gmp_df_add_sloppy(gmp_df_mul_f(z2, 21.0f), gmp_df_mul_f(r2, -14.0f)), z2), r2_2); H[1] = gmp_df_mul(q, a); H[2] = gmp_df_mul(q, b); }
-  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul(x, a), gmp_df_neg(gmp_df_mul(y, b)));
-    b = gmp_df_add_sloppy(gmp_df_mul(x, b), gmp_df_mul(y, a));
+  H[0] = gmp_df_mul_u(gmp_df_add_sloppy(gmp_df_mul_u(gmp_df_add_sloppy(gmp_df_mul_fu(z2, 63.0f), gmp_df_mul_fu(r2, -70.0f)), z2), gmp_df_mul_fu(r2_2, 15.0f)), z);
+  { const gmp_f2 q = gmp_df_add_sloppy(gmp_df_mul_u(gmp_df_add_sloppy(gmp_df_mul_fu(z2, 21.0f), gmp_df_mul_fu(r2, -14.0f)), z2), r2_2); H[1] = gmp_df_mul_u(q, a); H[2] = gmp_df_mul_u(q, b); }
+  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul_u(x, a), gmp_df_neg(gmp_df_mul_u(y, b)));
+    b = gmp_df_add_sloppy(gmp_df_mul_u(x, b), gmp_df_mul_u(y, a));
     a = t; }
-  { const gmp_f2 q = gmp_df_mul(gmp_df_add_sloppy(gmp_df_mul_f(z2, 3.0f), gmp_df_mul_f(r2, -1.0f)), z); H[3] = gmp_df_mul(q, a); H[4] = gmp_df_mul(q, b); }
-  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul(x, a), gmp_df_neg(gmp_df_mul(y, b)));
-    b = gmp_df_add_sloppy(gmp_df_mul(x, b), gmp_df_mul(y, a));
+  { const gmp_f2 q = gmp_df_mul(gmp_df_add_sloppy(gmp_df_mul_fu(z2, 3.0f), gmp_df_mul_fu(r2, -1.0f)), z); H[3] = gmp_df_mul_u(q, a); H[4] = gmp_df_mul_u(q, b); }
+  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul_u(x, a), gmp_df_neg(gmp_df_mul_u(y, b)));
+    b = gmp_df_add_sloppy(gmp_df_mul_u(x, b), gmp_df_mul_u(y, a));
     a = t; }
-  { const gmp_f2 q = gmp_df_add_sloppy(gmp_df_mul_f(z2, 9.0f), gmp_df_mul_f(r2, -1.0f)); H[5] = gmp_df_mul(q, a); H[6] = gmp_df_mul(q, b); }
-  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul(x, a), gmp_df_neg(gmp_df_mul(y, b)));
-    b = gmp_df_add_sloppy(gmp_df_mul(x, b), gmp_df_mul(y, a));
+  { const gmp_f2 q = gmp_df_add_sloppy(gmp_df_mul_fu(z2, 9.0f), gmp_df_mul_fu(r2, -1.0f)); H[5] = gmp_df_mul_u(q, a); H[6] = gmp_df_mul_u(q, b); }
+  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul_u(x, a), gmp_df_neg(gmp_df_mul_u(y, b)));
+    b = gmp_df_add_sloppy(gmp_df_mul_u(x, b), gmp_df_mul_u(y, a));
     a = t; }
-  { const gmp_f2 q = z; H[7] = gmp_df_mul(q, a); H[8] = gmp_df_mul(q, b); }
-  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul(x, a), gmp_df_neg(gmp_df_mul(y, b)));
-    b = gmp_df_add_sloppy(gmp_df_mul(x, b), gmp_df_mul(y, a));
+  { const gmp_f2 q = z; H[7] = gmp_df_mul_u(q, a); H[8] = gmp_df_mul_u(q, b); }
+  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul_u(x, a), gmp_df_neg(gmp_df_mul_u(y, b)));
+    b = gmp_df_add_sloppy(gmp_df_mul_u(x, b), gmp_df_mul_u(y, a));
     a = t; }
   H[9] = a; H[10] = b;
 }
@@ -605,26 +605,26 @@ __device__ __forceinline__ void gmp_solid_df_6(gmp_f2 x, gmp_f2 y, gmp_f2 z, gmp
   const gmp_f2 r2_2 = gmp_df_mul(r2, r2);
   const gmp_f2 r2_3 = gmp_df_mul(r2, r2_2);
   gmp_f2 a = x, b = y;
-  H[0] = gmp_df_add_sloppy(gmp_df_mul(gmp_df_add_sloppy(gmp_df_mul(gmp_df_add_sloppy(gmp_df_mul_f(z2, 231.0f), gmp_df_mul_f(r2, -315.0f)), z2), gmp_df_mul_f(r2_2, 105.0f)), z2), gmp_df_mul_f(r2_3, -5.0f));
-  { const gmp_f2 q = gmp_df_mul(gmp_df_add_sloppy(gmp_df_mul(gmp_df_add_sloppy(gmp_df_mul_f(z2, 33.0f), gmp_df_mul_f(r2, -30.0f)), z2), gmp_df_mul_f(r2_2, 5.0f)), z); H[1] = gmp_df_mul(q, a); H[2] = gmp_df_mul(q, b); }
-  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul(x, a), gmp_df_neg(gmp_df_mul(y, b)));
-    b = gmp_df_add_sloppy(gmp_df_mul(x, b), gmp_df_mul(y, a));
+  H[0] = gmp_df_add_sloppy(gmp_df_mul_u(gmp_df_add_sloppy(gmp_df_mul_u(gmp_df_add_sloppy(gmp_df_mul_fu(z2, 231.0f), gmp_df_mul_fu(r2, -315.0f)), z2), gmp_df_mul_fu(r2_2, 105.0f)), z2), gmp_df_mul_fu(r2_3, -5.0f));
+  { const gmp_f2 q = gmp_df_mul(gmp_df_add_sloppy(gmp_df_mul_u(gmp_df_add_sloppy(gmp_df_mul_fu(z2, 33.0f), gmp_df_mul_fu(r2, -30.0f)), z2), gmp_df_mul_fu(r2_2, 5.0f)), z); H[1] = gmp_df_mul_u(q, a); H[2] = gmp_df_mul_u(q, b); }
+  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul_u(x, a), gmp_df_neg(gmp_df_mul_u(y, b)));
+    b = gmp_df_add_sloppy(gmp_df_mul_u(x, b), gmp_df_mul_u(y, a));
     a = t; }
-  { const gmp_f2 q = gmp_df_add_sloppy(gmp_df_mul(gmp_df_add_sloppy(gmp_df_mul_f(z2, 33.0f), gmp_df_mul_f(r2, -18.0f)), z2), r2_2); H[3] = gmp_df_mul(q, a); H[4] = gmp_df_mul(q, b); }
-  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul(x, a), gmp_df_neg(gmp_df_mul(y, b)));
-    b = gmp_df_add_sloppy(gmp_df_mul(x, b), gmp_df_mul(y, a));
+  { const gmp_f2 q = gmp_df_add_sloppy(gmp_df_mul_u(gmp_df_add_sloppy(gmp_df_mul_fu(z2, 33.0f), gmp_df_mul_fu(r2, -18.0f)), z2), r2_2); H[3] = gmp_df_mul_u(q, a); H[4] = gmp_df_mul_u(q, b); }
+  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul_u(x, a), gmp_df_neg(gmp_df_mul_u(y, b)));
+    b = gmp_df_add_sloppy(gmp_df_mul_u(x, b), gmp_df_mul_u(y, a));
     a = t; }
-  { const gmp_f2 q = gmp_df_mul(gmp_df_add_sloppy(gmp_df_mul_f(z2, 11.0f), gmp_df_mul_f(r2, -3.0f)), z); H[5] = gmp_df_mul(q, a); H[6] = gmp_df_mul(q, b); }
-  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul(x, a), gmp_df_neg(gmp_df_mul(y, b)));
-    b = gmp_df_add_sloppy(gmp_df_mul(x, b), gmp_df_mul(y, a));
+  { const gmp_f2 q = gmp_df_mul(gmp_df_add_sloppy(gmp_df_mul_fu(z2, 11.0f), gmp_df_mul_fu(r2, -3.0f)), z); H[5] = gmp_df_mul_u(q, a); H[6] = gmp_df_mul_u(q, b); }
+  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul_u(x, a), gmp_df_neg(gmp_df_mul_u(y, b)));
+    b = gmp_df_add_sloppy(gmp_df_mul_u(x, b), gmp_df_mul_u(y, a));
     a = t; }
-  { const gmp_f2 q = gmp_df_add_sloppy(gmp_df_mul_f(z2, 11.0f), gmp_df_mul_f(r2, -1.0f)); H[7] = gmp_df_mul(q, a); H[8] = gmp_df_mul(q, b); }
-  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul(x, a), gmp_df_neg(gmp_df_mul(y, b)));
-    b = gmp_df_add_sloppy(gmp_df_mul(x, b), gmp_df_mul(y, a));
+  { const gmp_f2 q = gmp_df_add_sloppy(gmp_df_mul_fu(z2, 11.0f), gmp_df_mul_fu(r2, -1.0f)); H[7] = gmp_df_mul_u(q, a); H[8] = gmp_df_mul_u(q, b); }
+  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul_u(x, a), gmp_df_neg(gmp_df_mul_u(y, b)));
+    b = gmp_df_add_sloppy(gmp_df_mul_u(x, b), gmp_df_mul_u(y, a));
     a = t; }
-  { const gmp_f2 q = z; H[9] = gmp_df_mul(q, a); H[10] = gmp_df_mul(q, b); }
-  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul(x, a), gmp_df_neg(gmp_df_mul(y, b)));
-    b = gmp_df_add_sloppy(gmp_df_mul(x, b), gmp_df_mul(y, a));
+  { const gmp_f2 q = z; H[9] = gmp_df_mul_u(q, a); H[10] = gmp_df_mul_u(q, b); }
+  { const gmp_f2 t = gmp_df_add_sloppy(gmp_df_mul_u(x, a), gmp_df_neg(gmp_df_mul_u(y, b)));
+    b = gmp_df_add_sloppy(gmp_df_mul_u(x, b), gmp_df_mul_u(y, a));
     a = t; }
   H[11] = a; H[12] = b;
 }

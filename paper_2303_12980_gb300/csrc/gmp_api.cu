@@ -1304,7 +1304,11 @@ static gmp_status vjp_impl(gmp_handle h, int32_t n_struct, const int64_t* atom_o
     K.own = h->own.as<double>();
     K.vir_c = vir ? h->vir_c.as<double>() : nullptr;
     take_counter(h, K);
-    GMP_CK(cudaMemsetAsync(K.gbins, 0, sizeof(unsigned long long) * 3 * gmpk::kGradBins * N, st), "memset bins");
+    return GMP_OK;
+  };
+  // ahead of a pass's kernels, so that they follow one another directly
+  auto clear_bins = [&]() -> gmp_status {
+    GMP_CK(cudaMemsetAsync(h->gbins.p, 0, sizeof(unsigned long long) * 3 * gmpk::kGradBins * N, st), "memset bins");
     return GMP_OK;
   };
   auto vjp_end = [&](const gmpk::KParams& K, bool first, bool last) -> gmp_status {
@@ -1319,8 +1323,9 @@ static gmp_status vjp_impl(gmp_handle h, int32_t n_struct, const int64_t* atom_o
     return GMP_OK;
   };
   auto seq = [&](bool capture) -> gmp_status {
-  gmp_status q = build_neighbors(h, n_struct, io.pos, io.species, N, st, false, capture);
+  gmp_status q = clear_bins();
   if (q != GMP_OK) return q;
+  if ((q = build_neighbors(h, n_struct, io.pos, io.species, N, st, false, capture)) != GMP_OK) return q;
   if (io.host && (q = finish_lists(h, st)) != GMP_OK) return q;
   if ((q = begin_compute(h, N)) != GMP_OK) return q;
   bool refined = false, waited = false, pending = false;
@@ -1328,6 +1333,7 @@ static gmp_status vjp_impl(gmp_handle h, int32_t n_struct, const int64_t* atom_o
   for (size_t g = 0; g < h->passes.size(); ++g) {
     PassData& pd = h->passes[g];
     const bool last = g + 1 == h->passes.size();
+    if (g > 0 && (q = clear_bins()) != GMP_OK) return q;
     // forward kernel (features + moments), then the backward kernel reading
     // the moments (or one fused kernel, if the autotuner chose it)
     float* fout = feat ? feat : h->stage_feat.as<float>();

@@ -90,9 +90,8 @@ cudaError_t launch(int kind, const KParams& K, GmpShape shape, GmpLaunchPlan* pl
   const int64_t need = (n + warps - 1) / warps;
   if (blocks > need) blocks = need;
   if (blocks < 1) blocks = 1;
-  fn<<<(unsigned)blocks, warps * 32, smem, st>>>(K);
   ++*launches;
-  return cudaGetLastError();
+  return gmp_launch_next(fn, (unsigned)blocks, warps * 32, smem, st, K);
 }
 
 }  // namespace gmpk

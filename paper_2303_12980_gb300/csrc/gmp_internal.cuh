@@ -111,6 +111,42 @@ struct GmpPass {
   int jac_exp[16];
 };
 
+// ------------------------------------------------- programmatic dependent launch
+// The kernels of a call follow one another in one stream, most of them for a
+// few microseconds.  Each lets the next one start at once (its CTAs then wait
+// where they need the predecessor's results: gmp_after_predecessor returns when
+// that grid is complete and its memory visible) instead of being launched when
+// it has drained.  Everything that a kernel reads from memory another kernel
+// wrote is addressed through the returned thread index or comes after an
+// atomic behind it, so that no load moves ahead of the wait.
+__device__ __forceinline__ unsigned gmp_after_predecessor(unsigned tid) {
+  unsigned t;
+  asm volatile("griddepcontrol.wait;\n\tmov.b32 %0, %1;" : "=r"(t) : "r"(tid) : "memory");
+  return t;
+}
+__device__ __forceinline__ void gmp_let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+#define GMP_TRY(expr)                    \
+  do {                                   \
+    const cudaError_t e_ = (expr);       \
+    if (e_ != cudaSuccess) return e_;    \
+  } while (0)
+
+template <typename... P, typename... A>
+cudaError_t gmp_launch_next(void (*fn)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t stream, A... args) {
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, fn, static_cast<P>(args)...);
+}
+
 // ---------------------------------------------------------------- double-float
 struct gmp_f2 {
   float hi, lo;

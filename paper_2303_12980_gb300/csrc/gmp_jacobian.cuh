@@ -60,8 +60,10 @@ __global__ void __launch_bounds__(384) k_jacobian_r(KParams K) {
   float* s_rad = smem;
   float* s_dens = s_rad + (size_t)P.n_el * rad_elem_stride(L, NS, P.kmax);
   float* s_warp = s_dens + (size_t)P.n_el * dens_elem_stride(P.kmax);
+  gmp_let_next_start();
   load_tables<L>(P, NS, s_rad, s_dens);
   __syncthreads();
+  gmp_after_predecessor(0);  // (the tables belong to the handle)
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int g = lane / NS, s = lane % NS;  // group and, in it, the staged pair or the sigma
   const bool s_ok = s < P.nsig;

@@ -896,8 +896,10 @@ __global__ void __launch_bounds__(512) k_forward(KParams K) {
   float* s_rad = smem;
   float* s_dens = s_rad + (size_t)P.n_el * rad_elem_stride(L, NS, P.kmax);
   float* s_warp = s_dens + (size_t)P.n_el * dens_elem_stride(P.kmax);
+  gmp_let_next_start();
   load_tables<L>(P, NS, s_rad, s_dens);
   __syncthreads();
+  gmp_after_predecessor(0);  // (the tables belong to the handle)
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   float* Rt = s_warp + (size_t)wib * SH::WARP_FLOATS;
   float* St = Rt + SH::TILE * SH::RSTR;
@@ -1106,8 +1108,10 @@ __global__ void __launch_bounds__(256) k_vjp(KParams K) {
   float* s_rad = smem;
   float* s_dens = s_rad + (size_t)P.n_el * rad_elem_stride(L, NS, P.kmax);
   float* s_warp = s_dens + (size_t)P.n_el * dens_elem_stride(P.kmax);
+  gmp_let_next_start();
   load_tables<L>(P, NS, s_rad, s_dens);
   __syncthreads();
+  gmp_after_predecessor(0);  // (the tables belong to the handle)
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   float* Rt = s_warp + (size_t)wib * SH::WARP_FLOATS;
   float* St = Rt + SH::TILE * SH::RSTR;
@@ -1141,8 +1145,10 @@ __global__ void __launch_bounds__(384) k_backward(KParams K) {
   float* s_rad = smem;
   float* s_dens = s_rad + (size_t)P.n_el * rad_elem_stride(L, NS, P.kmax, PADG);
   float* s_warp = s_dens + (size_t)P.n_el * dens_elem_stride(P.kmax);
+  gmp_let_next_start();
   load_tables<L, PADG>(P, NS, s_rad, s_dens);
   __syncthreads();
+  gmp_after_predecessor(0);  // (the tables belong to the handle)
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   constexpr int EXTRA = VIRIAL ? virial_extra_floats<L, NS>() : 0;
   float* Mu = s_warp + (size_t)wib * (SH::WARP_FLOATS + EXTRA);
@@ -1209,8 +1215,10 @@ __global__ void __maxnreg__(L >= 6 ? 168 : 128) k_jacobian(KParams K) {
   float* s_rad = smem;
   float* s_dens = s_rad + (size_t)P.n_el * rad_elem_stride(L, NS, P.kmax, false);
   float* s_warp = s_dens + (size_t)P.n_el * dens_elem_stride(P.kmax);
+  gmp_let_next_start();
   load_tables<L, false>(P, NS, s_rad, s_dens);
   __syncthreads();
+  gmp_after_predecessor(0);  // (the tables belong to the handle)
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int pg = lane / NS, s = lane % NS;
   const bool s_ok = s < P.nsig;

@@ -18,8 +18,10 @@ __global__ void k_struct_of(const int64_t* __restrict__ atom_off, int n_struct,
 __global__ void k_jac_count(int64_t N, const int64_t* __restrict__ nbr_beg, const int64_t* __restrict__ nbr_end,
                             const GmpPair* __restrict__ pairs, int64_t* __restrict__ counts,
                             int32_t* __restrict__ local_row) {
-  const int lane = threadIdx.x & 31;
-  const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  gmp_let_next_start();
+  const unsigned tid = gmp_after_predecessor(threadIdx.x);
+  const int lane = tid & 31;
+  const int64_t i = ((int64_t)blockIdx.x * blockDim.x + tid) >> 5;
   if (i >= N) return;
   const int64_t p0 = nbr_beg[i], p1 = nbr_end[i];
   int c = 0;  // rows so far (warp-uniform)
@@ -46,7 +48,9 @@ __global__ void k_grad_bins_finish(int64_t n, const unsigned long long* __restri
   constexpr int kBins = 12;
   constexpr double kBinUnit[11] = {0x1p-149, 0x1p-125, 0x1p-101, 0x1p-77, 0x1p-53, 0x1p-29,
                                    0x1p-5,   0x1p+19,  0x1p+43,  0x1p+67, 0x1p+91};
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
+  gmp_let_next_start();
+  const unsigned tid = gmp_after_predecessor(threadIdx.x);
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + tid; t < n; t += (int64_t)gridDim.x * blockDim.x) {
     const unsigned long long* bt = bins + t * kBins;
     const unsigned long long fl = bt[11];
     double v;
@@ -69,8 +73,10 @@ __global__ void k_grad_bins_finish(int64_t n, const unsigned long long* __restri
 // vir_c[center] (nine values), one warp per structure, lanes over centers in a fixed order.
 __global__ void k_virial_reduce(int n_struct, const int64_t* __restrict__ atom_off, const double* __restrict__ vir_c,
                                 double* __restrict__ virial, bool first) {
-  const int lane = threadIdx.x & 31;
-  const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  gmp_let_next_start();
+  const unsigned tid = gmp_after_predecessor(threadIdx.x);
+  const int lane = tid & 31;
+  const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + tid) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t s = w0; s < n_struct; s += nw) {
     const int64_t a0 = atom_off[s], a1 = atom_off[s + 1];
@@ -106,7 +112,8 @@ cudaError_t gmp_launch_jacobian_count(int64_t N, const int64_t* nbr_beg, const i
   (void)sm_count;
   if (N <= 0) return cudaSuccess;
   const int64_t threads = N * 32;
-  k_jac_count<<<(unsigned)((threads + 255) / 256), 256, 0, stream>>>(N, nbr_beg, nbr_end, pairs, counts, local_row);
+  GMP_TRY(gmp_launch_next(k_jac_count, (unsigned)((threads + 255) / 256), 256, 0, stream, N, nbr_beg, nbr_end, pairs,
+                          counts, local_row));
   ++*launches;
   return cudaGetLastError();
 }
@@ -121,7 +128,7 @@ cudaError_t gmp_launch_grad_bins_finish(int64_t N, const unsigned long long* bin
   int64_t blocks = (n + nt - 1) / nt;
   const int64_t cap = (int64_t)sm_count * 32;
   if (blocks > cap) blocks = cap;
-  k_grad_bins_finish<<<(unsigned)blocks, nt, 0, stream>>>(n, bins, own, acc_in, acc_out, grad_pos);
+  GMP_TRY(gmp_launch_next(k_grad_bins_finish, (unsigned)blocks, nt, 0, stream, n, bins, own, acc_in, acc_out, grad_pos));
   ++*launches;
   return cudaGetLastError();
 }
@@ -132,7 +139,7 @@ cudaError_t gmp_launch_virial_reduce(int n_struct, const int64_t* atom_off, cons
   int64_t blocks = ((int64_t)n_struct * 32 + 255) / 256;
   const int64_t cap = (int64_t)sm_count * 8;
   if (blocks > cap) blocks = cap;
-  k_virial_reduce<<<(unsigned)blocks, 256, 0, stream>>>(n_struct, atom_off, vir_c, virial, first);
+  GMP_TRY(gmp_launch_next(k_virial_reduce, (unsigned)blocks, 256, 0, stream, n_struct, atom_off, vir_c, virial, first));
   ++*launches;
   return cudaGetLastError();
 }

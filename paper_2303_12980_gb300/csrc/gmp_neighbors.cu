@@ -157,9 +157,11 @@ __global__ void k_prepare(const GmpStruct* __restrict__ S, const int32_t* __rest
                           GmpD4* __restrict__ atom_u, unsigned long long* __restrict__ bbox,
                           int64_t n_bins, int32_t* __restrict__ bin_count, int32_t* __restrict__ bin_cursor,
                           uint32_t* __restrict__ err) {
-  for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < n_bins; b += (int64_t)gridDim.x * blockDim.x)
+  gmp_let_next_start();
+  const unsigned tid = gmp_after_predecessor(threadIdx.x);
+  for (int64_t b = blockIdx.x * (int64_t)blockDim.x + tid; b < n_bins; b += (int64_t)gridDim.x * blockDim.x)
     bin_count[b] = bin_cursor[b] = 0;
-  for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < N;
+  for (int64_t a = blockIdx.x * (int64_t)blockDim.x + tid; a < N;
        a += (int64_t)gridDim.x * blockDim.x)
     prepare_atom(S, struct_of, a, pos, species, n_el, atom_xh, atom_xl, atom_u, bbox, err);
 }
@@ -262,7 +264,9 @@ __host__ __device__ inline bool all_periodic(const GmpStruct& st) {
 __global__ void k_grid(GmpStruct* __restrict__ S, int n_struct,
                        const unsigned long long* __restrict__ bbox, GmpGrid* __restrict__ G,
                        double cutoff, int all) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  gmp_let_next_start();
+  const unsigned tid = gmp_after_predecessor(threadIdx.x);
+  const int s = blockIdx.x * blockDim.x + tid;
   if (s >= n_struct || (!all && all_periodic(S[s]))) return;
   GmpGrid g;
   grid_struct(S[s], bbox + 6 * s, g, cutoff);
@@ -285,12 +289,9 @@ __device__ __forceinline__ int32_t bin_of(const GmpStruct* S, const GmpGrid* G, 
 // Bin slot of atom a: bin_y = (wrapped FP32 position, packed wrap of the
 // atom), bin_je = (atom index, species).
 // (wrap = atom_xl[a].w, spec = atom_xh[a].w: packed wrap and species bits)
-__device__ __forceinline__ void write_slot(const GmpStruct& st, int64_t a, int32_t slot, const GmpD4& u4,
-                                           float spec, float wrap, float4* __restrict__ bin_y,
-                                           int2* __restrict__ bin_je) {
-  float y[3];
-  for (int c = 0; c < 3; ++c) y[c] = (float)(u4.x * st.A[c] + u4.y * st.A[3 + c] + u4.z * st.A[6 + c]);
-  bin_y[slot] = make_float4(y[0], y[1], y[2], wrap);
+__device__ __forceinline__ void write_slot(int64_t a, int32_t slot, const float4& y, float spec, float wrap,
+                                           float4* __restrict__ bin_y, int2* __restrict__ bin_je) {
+  bin_y[slot] = make_float4(y.x, y.y, y.z, wrap);
   bin_je[slot] = make_int2((int32_t)a, __float_as_int(spec));
 }
 
@@ -299,7 +300,9 @@ __device__ __forceinline__ void write_slot(const GmpStruct& st, int64_t a, int32
 __global__ void k_bin_scatter(int64_t N, const int32_t* __restrict__ atom_bin,
                               const int32_t* __restrict__ bin_start, int32_t* __restrict__ bin_cursor,
                               int32_t* __restrict__ slot_atom) {
-  for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < N;
+  gmp_let_next_start();
+  const unsigned tid = gmp_after_predecessor(threadIdx.x);
+  for (int64_t a = blockIdx.x * (int64_t)blockDim.x + tid; a < N;
        a += (int64_t)gridDim.x * blockDim.x) {
     const int32_t bin = atom_bin[a];
     slot_atom[bin_start[bin] + atomicAdd(&bin_cursor[bin], 1)] = (int32_t)a;
@@ -310,19 +313,20 @@ __global__ void k_bin_scatter(int64_t N, const int32_t* __restrict__ atom_bin,
 // (bins in atom-index order, which makes neighbor enumeration
 // deterministic); the bin's slot list is read in parallel, not sorted in
 // place.
-__global__ void k_bin_place(const GmpStruct* __restrict__ S, const int32_t* __restrict__ struct_of, int64_t N,
-                            const int32_t* __restrict__ atom_bin, const int32_t* __restrict__ bin_start,
-                            const int32_t* __restrict__ slot_atom, const GmpD4* __restrict__ atom_u,
+__global__ void k_bin_place(int64_t N, const int32_t* __restrict__ atom_bin, const int32_t* __restrict__ bin_start,
+                            const int32_t* __restrict__ slot_atom, const float4* __restrict__ atom_y,
                             const float4* __restrict__ atom_xh, const float4* __restrict__ atom_xl,
                             float4* __restrict__ bin_y, int2* __restrict__ bin_je) {
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < N;
+  gmp_let_next_start();
+  const unsigned tid = gmp_after_predecessor(threadIdx.x);
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + tid; t < N;
        t += (int64_t)gridDim.x * blockDim.x) {
     const int32_t a = slot_atom[t];
     const int32_t bin = atom_bin[a];
     const int32_t b0 = bin_start[bin], b1 = bin_start[bin + 1];
     int32_t rank = 0;
     for (int32_t u = b0; u < b1; ++u) rank += slot_atom[u] < a ? 1 : 0;
-    write_slot(S[struct_of[a]], a, b0 + rank, atom_u[a], atom_xh[a].w, atom_xl[a].w, bin_y, bin_je);
+    write_slot(a, b0 + rank, atom_y[a], atom_xh[a].w, atom_xl[a].w, bin_y, bin_je);
   }
 }
 
@@ -346,7 +350,9 @@ __global__ void k_bin_assign(const GmpStruct* __restrict__ S, const GmpGrid* __r
                              const GmpD4* __restrict__ atom_u, int32_t* __restrict__ atom_bin,
                              int32_t* __restrict__ bin_count, float4* __restrict__ atom_t,
                              float4* __restrict__ atom_y) {
-  for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < N;
+  gmp_let_next_start();
+  const unsigned tid = gmp_after_predecessor(threadIdx.x);
+  for (int64_t a = blockIdx.x * (int64_t)blockDim.x + tid; a < N;
        a += (int64_t)gridDim.x * blockDim.x) {
     const int s = struct_of[a];
     const GmpD4 u4 = atom_u[a];
@@ -365,7 +371,9 @@ __global__ void k_point_prepare(const GmpStruct* __restrict__ S, const GmpGrid* 
                                 const double* __restrict__ atom_pos, float4* __restrict__ pt_xh,
                                 float4* __restrict__ pt_xl, float4* __restrict__ pt_t, float4* __restrict__ pt_y,
                                 uint32_t* __restrict__ err) {
-  for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < n;
+  gmp_let_next_start();
+  const unsigned tid = gmp_after_predecessor(threadIdx.x);
+  for (int64_t a = blockIdx.x * (int64_t)blockDim.x + tid; a < n;
        a += (int64_t)gridDim.x * blockDim.x) {
     const int s = point_struct[a];
     const GmpStruct& st = S[s];
@@ -418,7 +426,8 @@ __global__ void __launch_bounds__(1024) k_bin_small(GmpStruct* S, int n_struct, 
   int32_t* cnt = reinterpret_cast<int32_t*>(bbox + 6 * n_struct);  // [n_bins] counts, then cursors
   int32_t* start = cnt + n_bins;                                    // [n_bins + 1] exclusive offsets
   int32_t* slot_atom = start + n_bins + 1;                          // [N] atom of each slot
-  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wid = tid >> 5;
+  gmp_let_next_start();
+  const int tid = (int)gmp_after_predecessor(threadIdx.x), nt = blockDim.x, lane = tid & 31, wid = tid >> 5;
   for (int t = tid; t < 6 * n_struct; t += nt) bbox[t] = ~0ull;
   for (int64_t b = tid; b < n_bins; b += nt) cnt[b] = 0;
   __syncthreads();
@@ -481,16 +490,17 @@ __global__ void __launch_bounds__(1024) k_bin_small(GmpStruct* S, int n_struct, 
     }
   }
   __syncthreads();
+  for (int64_t b = tid; b <= n_bins; b += nt) bin_start[b] = start[b];
   for (int64_t t = tid; t < N; t += nt) {
     const int64_t a = slot_atom[t];
-    write_slot(S[struct_of[a]], a, (int32_t)t, atom_u[a], atom_xh[a].w, atom_xl[a].w, bin_y, bin_je);
-  }
-  for (int64_t b = tid; b <= n_bins; b += nt) bin_start[b] = start[b];
-  for (int64_t a = tid; a < N; a += nt) {
     const int s = struct_of[a];
     const GmpD4 u4 = atom_u[a];
     const double u[3] = {u4.x, u4.y, u4.z};
-    center_place(S[s], G[s], u, atom_t[a], atom_y[a]);
+    float4 place, y;
+    center_place(S[s], G[s], u, place, y);
+    atom_t[a] = place;
+    atom_y[a] = y;
+    write_slot(a, (int32_t)t, y, atom_xh[a].w, atom_xl[a].w, bin_y, bin_je);
   }
 }
 
@@ -500,7 +510,8 @@ __global__ void k_scan_block(const T* __restrict__ in, T* __restrict__ out, T* _
                              int64_t n) {
   __shared__ T sh[1024];
   const int64_t base = (int64_t)blockIdx.x * 1024;
-  const int t = threadIdx.x;
+  gmp_let_next_start();
+  const int t = gmp_after_predecessor(threadIdx.x);
   T v = (base + t < n) ? in[base + t] : T(0);
   sh[t] = v;
   __syncthreads();
@@ -516,7 +527,9 @@ __global__ void k_scan_block(const T* __restrict__ in, T* __restrict__ out, T* _
 
 template <typename T>
 __global__ void k_scan_add(T* __restrict__ out, const T* __restrict__ offs, int64_t n) {
-  const int64_t i = (int64_t)blockIdx.x * 1024 + threadIdx.x;
+  gmp_let_next_start();
+  const unsigned tid = gmp_after_predecessor(threadIdx.x);
+  const int64_t i = (int64_t)blockIdx.x * 1024 + tid;
   if (i < n) out[i] += offs[blockIdx.x];
   if (i == 0) out[n] = offs[gridDim.x];  // the total
 }
@@ -528,7 +541,8 @@ constexpr int64_t kScanOneCta = 16384;
 template <typename T>
 __global__ void __launch_bounds__(1024) k_scan_one(const T* __restrict__ in, T* __restrict__ out, int64_t n) {
   __shared__ T tot[32];
-  const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+  gmp_let_next_start();
+  const int t = gmp_after_predecessor(threadIdx.x), lane = t & 31, wid = t >> 5;
   T carry = 0;
   for (int64_t base = 0; base < n; base += 4096) {
     const int64_t i0 = base + 4 * t;
@@ -572,7 +586,7 @@ cudaError_t exclusive_scan(const T* in, T* out, int64_t n, void* tmp, cudaStream
     return cudaMemsetAsync(out, 0, sizeof(T), st);
   }
   if (n <= kScanOneCta) {
-    k_scan_one<T><<<1, 1024, 0, st>>>(in, out, n);
+    GMP_TRY(gmp_launch_next(k_scan_one<T>, 1, 1024, 0, st, in, out, n));
     ++*launches;
     return cudaGetLastError();
   }
@@ -580,11 +594,11 @@ cudaError_t exclusive_scan(const T* in, T* out, int64_t n, void* tmp, cudaStream
   T* sums = (T*)tmp;
   T* sums_scan = sums + nb + 1;
   void* rest = (void*)(sums_scan + nb + 1);
-  k_scan_block<T><<<(unsigned)nb, 1024, 0, st>>>(in, out, sums, n);
+  GMP_TRY(gmp_launch_next(k_scan_block<T>, (unsigned)nb, 1024, 0, st, in, out, sums, n));
   ++*launches;
   const cudaError_t e = exclusive_scan<T>(sums, sums_scan, nb, rest, st, launches);
   if (e != cudaSuccess) return e;
-  k_scan_add<T><<<(unsigned)nb, 1024, 0, st>>>(out, sums_scan, n);
+  GMP_TRY(gmp_launch_next(k_scan_add<T>, (unsigned)nb, 1024, 0, st, out, sums_scan, n));
   ++*launches;
   return cudaGetLastError();
 }
@@ -671,8 +685,10 @@ __global__ void __launch_bounds__(128, 8) k_neighbors(const GmpStruct* __restric
                             int32_t* __restrict__ maxm, uint32_t* __restrict__ err) {
   extern __shared__ __align__(16) unsigned char sh_fill[];
   constexpr int fill = FILL;
-  const int lane = threadIdx.x & 31;
-  const int wib = threadIdx.x >> 5;
+  gmp_let_next_start();
+  const unsigned tid = gmp_after_predecessor(threadIdx.x);
+  const int lane = tid & 31;
+  const int wib = tid >> 5;
   const int64_t i = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib;
   if (i >= N) return;
   unsigned char* wbase = sh_fill + (size_t)wib * (fill ? fill_warp_bytes(max_keys, n_el) : kSegBytes);
@@ -970,7 +986,9 @@ __global__ void __launch_bounds__(128, 8) k_neighbors(const GmpStruct* __restric
 
 __global__ void k_unpack(int64_t P, const GmpPair* __restrict__ pairs, int32_t* __restrict__ nbr_j,
                          int32_t* __restrict__ nbr_shift) {
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < P;
+  gmp_let_next_start();
+  const unsigned tid = gmp_after_predecessor(threadIdx.x);
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + tid; t < P;
        t += (int64_t)gridDim.x * blockDim.x) {
     GmpPair p = pairs[t];
     int n[3];
@@ -1032,13 +1050,12 @@ cudaError_t gmp_launch_neighbors_prepare(GmpStruct* d_structs, int n_struct,
     if (e != cudaSuccess) return e;
   }
   const int nt = atom_threads(N, sm_count);
-  k_prepare<<<grid_for(N, nt, sm_count), nt, 0, stream>>>(d_structs, d_struct_of, N, pos, species,
-                                                            n_el, atom_xh, atom_xl, atom_u, d_bbox, n_bins,
-                                                            bin_count, bin_cursor, d_err);
+  GMP_TRY(gmp_launch_next(k_prepare, grid_for(N, nt, sm_count), nt, 0, stream, d_structs, d_struct_of, N, pos,
+                          species, n_el, atom_xh, atom_xl, atom_u, d_bbox, n_bins, bin_count, bin_cursor, d_err));
   ++*launches;
   if (mode != GmpGridMode::kGiven) {
-    k_grid<<<(n_struct + 31) / 32, 32, 0, stream>>>(d_structs, n_struct, d_bbox, d_grid, cutoff,
-                                                    mode == GmpGridMode::kAll ? 1 : 0);
+    GMP_TRY(gmp_launch_next(k_grid, (n_struct + 31) / 32, 32, 0, stream, d_structs, n_struct, d_bbox, d_grid,
+                            cutoff, mode == GmpGridMode::kAll ? 1 : 0));
     ++*launches;
   }
   return cudaGetLastError();
@@ -1051,17 +1068,18 @@ cudaError_t gmp_launch_bins(const GmpStruct* d_structs, const GmpGrid* d_grid,
                             const GmpD4* atom_u, const float4* atom_xh, const float4* atom_xl, void* scan_tmp,
                             cudaStream_t stream, int sm_count, int64_t* launches) {
   const int nt = atom_threads(N, sm_count);
-  k_bin_assign<<<grid_for(N, nt, sm_count), nt, 0, stream>>>(d_structs, d_grid, d_struct_of, N,
-                                                               atom_u, atom_bin, bin_count, atom_t, atom_y);
+  GMP_TRY(gmp_launch_next(k_bin_assign, grid_for(N, nt, sm_count), nt, 0, stream, d_structs, d_grid, d_struct_of, N,
+                          atom_u, atom_bin, bin_count, atom_t, atom_y));
   ++*launches;
   cudaError_t e = exclusive_scan<int32_t>(bin_count, bin_start, n_bins, scan_tmp, stream, launches);
   if (e != cudaSuccess) return e;
   // bin_count is free once scanned: it holds the slot lists (room for
   // max(n_bins, N) values)
-  k_bin_scatter<<<grid_for(N, 256, sm_count), 256, 0, stream>>>(N, atom_bin, bin_start, bin_cursor, bin_count);
+  GMP_TRY(gmp_launch_next(k_bin_scatter, grid_for(N, 256, sm_count), 256, 0, stream, N, atom_bin, bin_start,
+                          bin_cursor, bin_count));
   ++*launches;
-  k_bin_place<<<grid_for(N, nt, sm_count), nt, 0, stream>>>(d_structs, d_struct_of, N, atom_bin, bin_start,
-                                                              bin_count, atom_u, atom_xh, atom_xl, bin_y, bin_je);
+  GMP_TRY(gmp_launch_next(k_bin_place, grid_for(N, nt, sm_count), nt, 0, stream, N, atom_bin, bin_start, bin_count,
+                          atom_y, atom_xh, atom_xl, bin_y, bin_je));
   ++*launches;
   return cudaGetLastError();
 }
@@ -1082,9 +1100,9 @@ cudaError_t gmp_launch_bin_small(GmpStruct* d_structs, int n_struct, const int32
     const cudaError_t e = cudaFuncSetAttribute(k_bin_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  k_bin_small<<<1, 1024, smem, stream>>>(d_structs, n_struct, d_struct_of, N, cutoff, pos, species, n_el, d_grid,
-                                         n_bins, atom_xh, atom_xl, atom_u, atom_bin, bin_start, bin_y, bin_je,
-                                         atom_t, atom_y, d_err);
+  GMP_TRY(gmp_launch_next(k_bin_small, 1, 1024, smem, stream, d_structs, n_struct, d_struct_of, N, cutoff, pos,
+                          species, n_el, d_grid, n_bins, atom_xh, atom_xl, atom_u, atom_bin, bin_start, bin_y,
+                          bin_je, atom_t, atom_y, d_err));
   ++*launches;
   return cudaGetLastError();
 }
@@ -1096,8 +1114,8 @@ cudaError_t gmp_launch_point_prepare(const GmpStruct* d_structs, const GmpGrid* 
                                      int64_t* launches) {
   if (n_points <= 0) return cudaSuccess;
   const int nt = atom_threads(n_points, sm_count);
-  k_point_prepare<<<grid_for(n_points, nt, sm_count), nt, 0, stream>>>(
-      d_structs, d_grid, point_struct, n_points, points, atom_pos, pt_xh, pt_xl, pt_t, pt_y, d_err);
+  GMP_TRY(gmp_launch_next(k_point_prepare, grid_for(n_points, nt, sm_count), nt, 0, stream, d_structs, d_grid,
+                          point_struct, n_points, points, atom_pos, pt_xh, pt_xl, pt_t, pt_y, d_err));
   ++*launches;
   return cudaGetLastError();
 }
@@ -1127,9 +1145,9 @@ cudaError_t gmp_launch_neighbor_pass(int fill, const GmpStruct* d_structs, const
     }
   }
   const unsigned blocks = (unsigned)((N + warps - 1) / warps);
-  fn<<<blocks, warps * 32, smem, stream>>>(d_structs, d_grid, C, N, (float)cutoff, rc2hi, rc2lo, rc2, pos,
-                                           atom_xh, atom_xl, bin_start, bin_y, bin_je, n_el, counts, offsets,
-                                           cursor, rng, pairs, pair_cap, max_keys, d_maxm, d_err);
+  GMP_TRY(gmp_launch_next(fn, blocks, warps * 32, smem, stream, d_structs, d_grid, C, N, (float)cutoff, rc2hi,
+                          rc2lo, rc2, pos, atom_xh, atom_xl, bin_start, bin_y, bin_je, n_el, counts, offsets,
+                          cursor, rng, pairs, pair_cap, max_keys, d_maxm, d_err));
   ++*launches;
   return cudaGetLastError();
 }
@@ -1138,7 +1156,7 @@ cudaError_t gmp_launch_unpack_neighbors(int64_t P, const GmpPair* pairs, int32_t
                                         int32_t* nbr_shift, cudaStream_t stream,
                                         int64_t* launches) {
   if (P <= 0) return cudaSuccess;
-  k_unpack<<<grid_for(P, 256, 152), 256, 0, stream>>>(P, pairs, nbr_j, nbr_shift);
+  GMP_TRY(gmp_launch_next(k_unpack, grid_for(P, 256, 152), 256, 0, stream, P, pairs, nbr_j, nbr_shift));
   ++*launches;
   return cudaGetLastError();
 }

@@ -171,8 +171,9 @@ __device__ __forceinline__ void refine_order(int lane, const GmpRefine& A, const
 // dependent double-float chains at 16 warps per SM (128 registers).
 __global__ void __launch_bounds__(256, 2) k_refine(const GmpRefine A) {
   __shared__ float2 exp_tab[64];
+  gmp_let_next_start();
   if (threadIdx.x < 64) exp_tab[threadIdx.x] = A.exp_tab[threadIdx.x];
-  const int lane = threadIdx.x & 31;
+  const int lane = gmp_after_predecessor(threadIdx.x) & 31;
   int64_t count = 0;
 #pragma unroll
   for (int l = 0; l < 7; ++l)
@@ -197,7 +198,6 @@ cudaError_t gmp_launch_refine(const GmpRefine& A, int sm_count, int* per_sm, cud
     if (e != cudaSuccess) return e;
     if (*per_sm < 1) *per_sm = 1;
   }
-  k_refine<<<(unsigned)(sm_count * *per_sm), 256, 0, stream>>>(A);
   ++*launches;
-  return cudaGetLastError();
+  return gmp_launch_next(k_refine, (unsigned)(sm_count * *per_sm), 256, 0, stream, A);
 }

@@ -246,7 +246,8 @@ gmp_status gmp_set_graph(gmp_handle h, int enable);
 /* Autotuner (not part of the method): builds the neighbor lists of the given
  * batch, then times on it (CUDA events, `reps` launches after a warm-up)
  * the candidate launch shapes of each compute kernel -- forward tile of 16
- * or 32 pairs x 4/8/16 warps per CTA, backward 4/6/12 warps, the fused
+ * or 32 pairs with up to 16 warps per CTA, backward 4, 12 or the untuned
+ * number of warps, the fused
  * forward+backward VJP kernel 4/8 warps versus the forward + backward pair
  * -- and keeps the fastest in the handle for later calls.  Synchronises
  * `stream`; writes the number of neighbor pairs to *pairs_out (host, may be
@@ -257,7 +258,8 @@ gmp_status gmp_tune(gmp_handle h, int32_t n_struct, const int64_t *atom_off, con
 
 /* The handle's launch shapes as 6 int32 per sigma pass (forward tile,
  * forward warps, backward warps, fused-VJP flag, fused warps, Jacobian
- * warps; 0 warps = largest that fits), for persisting tuning results.
+ * warps; 0 warps = the CTA size with the most resident warps), for
+ * persisting tuning results.
  * gmp_tuning_get needs n >= 6 * passes (GMP_ERR_CAPACITY otherwise);
  * gmp_tuning_set needs exactly that many values in range. */
 gmp_status gmp_tuning_get(gmp_handle h, int32_t *values, int32_t n);

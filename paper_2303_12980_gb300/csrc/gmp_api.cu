@@ -68,7 +68,8 @@ struct PassData {
   int L;
   int NS;
   DevBuf rad;
-  // launch shapes (defaults until gmp_tune / gmp_tuning_set)
+  // launch shapes (0 warps: the CTA size with the most resident warps, until
+  // gmp_tune / gmp_tuning_set)
   GmpShape fwd{16, 0};
   GmpShape bwd{16, 0};
   GmpShape fused{16, 0};
@@ -1624,12 +1625,13 @@ gmp_status gmp_tune(gmp_handle h, int32_t n_struct, const int64_t* atom_off, con
     K.mu_out = h->mu.as<float>();
     float best_f = 1e30f, t = 0.0f;
     GmpShape fwd_best = pd.fwd;
-    for (int tile : {16, 32})
-      for (int warps : {4, 8, 16}) {
-        cudaError_t e = timed(GMP_KIND_FORWARD, pd, K, GmpShape{tile, warps}, &t);
-        if (e != cudaSuccess) { out = cuda_fail(h, e, "tune forward"); break; }
-        if (t < best_f) { best_f = t; fwd_best = GmpShape{tile, warps}; }
-      }
+    // (0 warps: the untuned choice, the CTA size with the most resident warps)
+    for (const GmpShape c : {GmpShape{16, 0}, GmpShape{16, 4}, GmpShape{16, 8}, GmpShape{16, 16}, GmpShape{32, 0},
+                             GmpShape{32, 8}}) {
+      cudaError_t e = timed(GMP_KIND_FORWARD, pd, K, c, &t);
+      if (e != cudaSuccess) { out = cuda_fail(h, e, "tune forward"); break; }
+      if (t < best_f) { best_f = t; fwd_best = c; }
+    }
     if (out != GMP_OK) break;
     // moments for the backward candidates
     if (cudaError_t e = launch_cleared(GMP_KIND_FORWARD, pd, K, fwd_best)) {
@@ -1641,7 +1643,7 @@ gmp_status gmp_tune(gmp_handle h, int32_t n_struct, const int64_t* atom_off, con
     Kb.grad_feat = h->stage_gradf.as<float>();
     float best_b = 1e30f;
     GmpShape bwd_best = pd.bwd;
-    for (int warps : {4, 6, 12}) {
+    for (int warps : {0, 4, 12}) {
       cudaError_t e = timed(GMP_KIND_BACKWARD, pd, Kb, GmpShape{16, warps}, &t);
       if (e != cudaSuccess) { out = cuda_fail(h, e, "tune backward"); break; }
       if (t < best_b) { best_b = t; bwd_best = GmpShape{16, warps}; }

@@ -11,13 +11,13 @@
 namespace gmpk {
 
 template <int L, int NS, int TILE>
-size_t smem_bytes(const GmpPass& P, int warps, int extra_per_warp, bool pad = true) {
+size_t smem_bytes(const GmpPass& P, int warps, bool pad = true) {
   return sizeof(float) * (table_floats(P.n_el, L, NS, P.kmax, pad) +
-                          (size_t)warps * (Shape<L, NS, TILE>::WARP_FLOATS + extra_per_warp));
+                          (size_t)warps * Shape<L, NS, TILE>::WARP_FLOATS);
 }
 
 // shape.tile: 16 or 32 pairs per forward tile; shape.warps: warps per CTA
-// (0 = as many as the launch bounds and 227 KB of shared memory allow).
+// (0 = the size with the most resident warps).
 template <int L, int NS>
 cudaError_t launch(int kind, const KParams& K, GmpShape shape, GmpLaunchPlan* plan, cudaStream_t st, int sm_count,
                    int64_t* launches) {
@@ -34,13 +34,17 @@ cudaError_t launch(int kind, const KParams& K, GmpShape shape, GmpLaunchPlan* pl
   } else {
     if (kind == GMP_KIND_JACOBIAN) fn = k_jacobian<L, NS>;
   }
-  const int extra = kind == GMP_KIND_BACKWARD_VIRIAL ? virial_extra_floats<L, NS>() : 0;
   auto smem_of = [&](int w) -> size_t {
     if constexpr (L <= kJacRegOrders)
       if (kind == GMP_KIND_JACOBIAN)
         return sizeof(float) * (table_floats(K.pass.n_el, L, NS, K.pass.kmax) + (size_t)w * JacShape<L, NS>::WARP_FLOATS);
-    const bool pad = kind != GMP_KIND_BACKWARD && kind != GMP_KIND_JACOBIAN;  // these two: unpadded table
-    return tile == 32 ? smem_bytes<L, NS, 32>(K.pass, w, 0) : smem_bytes<L, NS, 16>(K.pass, w, extra, pad);
+    if (kind == GMP_KIND_BACKWARD || kind == GMP_KIND_BACKWARD_VIRIAL) {
+      const bool vir = kind == GMP_KIND_BACKWARD_VIRIAL;
+      return sizeof(float) * (table_floats(K.pass.n_el, L, NS, K.pass.kmax, vir ? back_pad<L, true>() : back_pad<L, false>()) +
+                              (size_t)w * back_warp_floats<L, NS>(vir));
+    }
+    const bool pad = kind != GMP_KIND_JACOBIAN;  // the general Jacobian kernel: unpadded table
+    return tile == 32 ? smem_bytes<L, NS, 32>(K.pass, w) : smem_bytes<L, NS, 16>(K.pass, w, pad);
   };
   const int64_t n = K.N - K.center0;
   // fewer centers than a CTA of the usual size on every SM would take: as
@@ -57,7 +61,7 @@ cudaError_t launch(int kind, const KParams& K, GmpShape shape, GmpLaunchPlan* pl
     e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     if (e != cudaSuccess) return e;
     int warps = fa.maxThreadsPerBlock / 32;
-    if (warps > 16) warps = 16;
+    if (warps > 20) warps = 20;
     if (want > 0 && want < warps) warps = want;
     while (warps > 1 && smem_of(warps) > 227 * 1024) --warps;
     if (want <= 0) {

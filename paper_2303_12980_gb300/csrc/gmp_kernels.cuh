@@ -143,14 +143,15 @@ struct Shape {
   static_assert(NS * NINDP <= TILE * SSTR, "adjoints must fit the S tile");
 };
 
-// Per-warp shared floats of the backward kernel's strain-derivative sums
-// ([9][32]: one column per lane).  They reuse the moment block of the
-// warp's region (dead once the adjoints are formed) when it is large
-// enough, else they take extra space after the region.
+// Shared floats of the backward kernel's strain-derivative sums ([9][32]: one
+// column per lane).  They reuse the warp's moment block (dead once the
+// adjoints are formed), which is at least that large.
 constexpr int kVirialFloats = 9 * 32;
+// Per-warp shared floats of the backward kernel: adjoints, then moments.
 template <int L, int NS>
-constexpr int virial_extra_floats() {
-  return Shape<L, NS>::TILE * Shape<L, NS>::RSTR >= kVirialFloats ? 0 : kVirialFloats;
+__host__ __device__ constexpr int back_warp_floats(bool vir) {
+  const int mu = (NS * Shape<L, NS>::NIND + 3) / 4 * 4;
+  return NS * Shape<L, NS>::NINDP + (vir && mu < kVirialFloats ? kVirialFloats : mu);
 }
 
 // Strides of the shared-memory radial table: within an element, the
@@ -329,6 +330,7 @@ __device__ __forceinline__ void radial4d(const float* __restrict__ tab_e, int km
   }
 }
 
+// (Below, NL orders from LA on: the backward takes its orders in ranges.)
 // Radial factors scaled by 2^32 for the backward, with scalar FP32
 // operations (the backward kernel keeps its 168-register budget with these;
 // packed pairs need aligned register pairs and spill there).  The exponent
@@ -339,7 +341,7 @@ __device__ __forceinline__ void radial4d(const float* __restrict__ tab_e, int km
 // down to exp(-B r^2) = 2^-158, with room for the amplitudes (alpha/gamma)^l
 // of the higher orders: a gradient term of a far pair, multiplied by large
 // adjoints, keeps its digits; the kernel scales its sums back by 2^-32.
-template <int L, int NL = L + 2, bool PADG = true>
+template <int L, int NL = L + 2, bool PADG = true, int LA = 0>
 __device__ __forceinline__ void radial4s(const float* __restrict__ tab_e, int kmax, int sg, float r2h,
                                          float (&R)[4][NL]) {
   constexpr int RB = gmp_rad_block(L);
@@ -358,7 +360,7 @@ __device__ __forceinline__ void radial4s(const float* __restrict__ tab_e, int km
     E[3] = gmp_ex2(__fmaf_rn(bh.w, -r2h, GMP_EXP_SHIFT));
 #pragma unroll
     for (int l = 0; l < NL; ++l) {
-      const float4 a = blk[2 + l];
+      const float4 a = blk[2 + LA + l];
       const float av[4] = {a.x, a.y, a.z, a.w};
 #pragma unroll
       for (int u = 0; u < 4; ++u) R[u][l] = __fmaf_rn(av[u], E[u], R[u][l]);
@@ -372,7 +374,7 @@ __device__ __forceinline__ void radial4s(const float* __restrict__ tab_e, int km
 // pair, and the exponentials' errors count against sum_q |A_q| E_q rather
 // than against the factor.  (A separate instantiation of the backward
 // kernel: a runtime branch would raise the register count of every one.)
-template <int L, int NL = L + 2, bool PADG = true>
+template <int L, int NL = L + 2, bool PADG = true, int LA = 0>
 __device__ __forceinline__ void radial4x(const float* __restrict__ tab_e, int kmax, int sg, float r2h,
                                          float r2l, float (&R)[4][NL]) {
   constexpr int RB = gmp_rad_block(L);
@@ -391,7 +393,7 @@ __device__ __forceinline__ void radial4x(const float* __restrict__ tab_e, int km
     E[3] = gmp_exp_neg_shifted(bh.w, bl.w, r2h, r2l);
 #pragma unroll
     for (int l = 0; l < NL; ++l) {
-      const float4 a = blk[2 + l];
+      const float4 a = blk[2 + LA + l];
       const float av[4] = {a.x, a.y, a.z, a.w};
 #pragma unroll
       for (int u = 0; u < 4; ++u) R[u][l] = __fmaf_rn(av[u], E[u], R[u][l]);
@@ -402,7 +404,7 @@ __device__ __forceinline__ void radial4x(const float* __restrict__ tab_e, int km
 // The scaled radial factors of radial4s on packed FP32 pairs, sigmas (0,1)
 // and (2,3) of the group: bit-identical to the scalar form, half the issue
 // slots.
-template <int L, int NL = L + 2, bool PADG = true>
+template <int L, int NL = L + 2, bool PADG = true, int LA = 0>
 __device__ __forceinline__ void radial4p(const float* __restrict__ tab_e, int kmax, int sg, float r2h,
                                          float (&R)[4][NL]) {
   constexpr int RB = gmp_rad_block(L);
@@ -420,7 +422,7 @@ __device__ __forceinline__ void radial4p(const float* __restrict__ tab_e, int km
     const float2 E0 = make_float2(gmp_ex2(x0.x), gmp_ex2(x0.y)), E1 = make_float2(gmp_ex2(x1.x), gmp_ex2(x1.y));
 #pragma unroll
     for (int l = 0; l < NL; ++l) {
-      const float4 a = blk[2 + l];
+      const float4 a = blk[2 + LA + l];
       Rp[0][l] = gmp_fma2(make_float2(a.x, a.y), E0, Rp[0][l]);
       Rp[1][l] = gmp_fma2(make_float2(a.z, a.w), E1, Rp[1][l]);
     }
@@ -942,37 +944,115 @@ __device__ __forceinline__ void adjoints(const GmpPass& P, const float* __restri
   __syncwarp();
 }
 
-// d/dd of sum_k lam_k R(r^2) S_k(d) for one pair, from
-//   A = sum_k lamd_k S_k (lamd carries dR/dr^2), B = sum_k (2l_k+1) lam_k S_k,
-//   V = sum_k lam_k S_{k+e}:   grad = d (2 A + B / r^2) - V / r^2   (r^2 > 0)
-// where lam already carries R.  At d = 0 only order 1 has a gradient:
-// (lam_x, lam_y, lam_z).  S1 holds the MCSH values of orders 0..L+1.
-template <int L>
-__device__ __forceinline__ void pair_gradient(const float* lam, float A, float dx, float dy, float dz, float r2,
-                                              const float* S1, float* g) {
-  float B = 0.0f;
+// gmp_mcsh_shift_contract_order_<l> by a compile-time order.
+template <int l>
+__device__ __forceinline__ void shift_contract_order(const float* lam, const float* S1, float* V) {
+  if constexpr (l == 0) gmp_mcsh_shift_contract_order_0(lam, S1, V);
+  else if constexpr (l == 1) gmp_mcsh_shift_contract_order_1(lam, S1, V);
+  else if constexpr (l == 2) gmp_mcsh_shift_contract_order_2(lam, S1, V);
+  else if constexpr (l == 3) gmp_mcsh_shift_contract_order_3(lam, S1, V);
+  else if constexpr (l == 4) gmp_mcsh_shift_contract_order_4(lam, S1, V);
+  else if constexpr (l == 5) gmp_mcsh_shift_contract_order_5(lam, S1, V);
+  else gmp_mcsh_shift_contract_order_6(lam, S1, V);
+}
+
+// One pair's part of the gradient of sum_k lam_k R_l(r^2) S_k(d) from the
+// orders LA .. LB, lam_k = sum_s Lam_{s,k} R_{s,l} and lamd_k with dR_l/dr^2 =
+// -beta R_{l+1}: adds to
+//   A = sum_k lamd_k S_k, B = sum_k (2l_k+1) lam_k S_k, V = sum_k lam_k S_{k+e},
+// from which grad = d (2 A + B / r^2) - V / r^2 (r^2 > 0).  At d = 0 only order
+// 1 has a gradient: g1 = (lam_x, lam_y, lam_z).
+// PACKED: radial factors on packed FP32 pairs (same results, fewer issue
+// slots); MIXED: exact exponentials (coefficients of both signs).
+template <int L, int NS, int LA, int LB, bool PACKED, bool PADG, bool MIXED>
+__device__ __forceinline__ void adjoint_range(const GmpPass& P, const float* __restrict__ tab_e,
+                                              const float* __restrict__ Lam, float dx, float dy, float dz, float r2h,
+                                              float r2l, float r2c, float& A, float& B, float (&V)[3], float (&g1)[3]) {
+  using SH = Shape<L, NS>;
+  constexpr int K0 = LA * LA, K1 = (LB + 1) * (LB + 1), NL = LB - LA + 2;
+  // MCSH values of orders up to LB first (order LB + 1 after the sigma loop):
+  // the sigma loop then contracts them directly, so that only the
+  // radial-weighted adjoints lam (not their derivative counterparts) are live
+  // beside them
+  float S[(LB + 2) * (LB + 2)];
+  GmpMcsh<LB>::eval(dx, dy, dz, r2c, S);
+  float lam[K1];
 #pragma unroll
-  for (int l = 0; l <= L; ++l) {
+  for (int k = K0; k < K1; ++k) lam[k] = 0.0f;
+  for (int sg = 0; sg < SH::NSB; ++sg) {
+    float R[4][NL];  // orders LA .. LB + 1
+    if constexpr (MIXED)
+      radial4x<L, NL, PADG, LA>(tab_e, P.kmax, sg, r2h, r2l, R);
+    else if constexpr (PACKED)
+      radial4p<L, NL, PADG, LA>(tab_e, P.kmax, sg, r2h, R);
+    else
+      radial4s<L, NL, PADG, LA>(tab_e, P.kmax, sg, r2h, R);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const float nb = P.nbeta[4 * sg + u];
+      const float* lrow = Lam + (4 * sg + u) * SH::NINDP;
+      float pl[NL - 1];
+#pragma unroll
+      for (int l = 0; l < NL - 1; ++l) pl[l] = 0.0f;
+      static_for<(K1 + 3) / 4 - K0 / 4>([&](auto cq) {
+        constexpr int c4 = K0 / 4 + decltype(cq)::value;
+        const float4 lv4 = *reinterpret_cast<const float4*>(lrow + 4 * c4);
+        const float lv[4] = {lv4.x, lv4.y, lv4.z, lv4.w};
+        static_for<4>([&](auto tt) {
+          constexpr int k = 4 * c4 + decltype(tt)::value;
+          if constexpr (k >= K0 && k < K1) {
+            constexpr int l = order_of(k) - LA;
+            lam[k] = __fmaf_rn(lv[decltype(tt)::value], R[u][l], lam[k]);
+            pl[l] = __fmaf_rn(lv[decltype(tt)::value], S[k], pl[l]);
+          }
+        });
+      });
+      // dR_l/dr^2 = -beta R_{l+1}: A += -beta sum_l R_{l+1} pl_l
+      float a = 0.0f;
+#pragma unroll
+      for (int l = 0; l < NL - 1; ++l) a = __fmaf_rn(R[u][l + 1], pl[l], a);
+      A = __fmaf_rn(nb, a, A);
+    }
+  }
+  GmpMcsh<LB + 1>::eval_top(dx, dy, dz, r2c, S);
+  if constexpr (LA == 0) GmpMcsh<LB>::shift_contract(lam, S, V);
+  static_for<LB - LA + 1>([&](auto ll) {
+    constexpr int l = LA + decltype(ll)::value;
     float b = 0.0f;
 #pragma unroll
-    for (int k = l * l; k < (l + 1) * (l + 1); ++k) b = __fmaf_rn(lam[k], S1[k], b);
+    for (int k = l * l; k < (l + 1) * (l + 1); ++k) b = __fmaf_rn(lam[k], S[k], b);
     B = __fmaf_rn((float)(2 * l + 1), b, B);
-  }
-  float V[3];
-  GmpMcsh<L>::shift_contract(lam, S1, V);
-  if (r2 > 0.0f) {
-    const float inv = 1.0f / r2;
-    const float c = 2.0f * A + B * inv;
-    g[0] = dx * c - V[0] * inv;
-    g[1] = dy * c - V[1] * inv;
-    g[2] = dz * c - V[2] * inv;
-  } else if (L >= 1) {
-    // independent order-1 components: (0,1,0), (0,0,1), (1,0,0) at flat 1, 2, 3
-    g[0] = lam[3]; g[1] = lam[1]; g[2] = lam[2];
-  } else {
-    g[0] = g[1] = g[2] = 0.0f;
-  }
+    if constexpr (LA > 0) {
+      float W[3];
+      shift_contract_order<l>(lam, S, W);
+#pragma unroll
+      for (int v = 0; v < 3; ++v) V[v] = __fadd_rn(V[v], W[v]);
+    }
+    if constexpr (l == 1) {  // independent order-1 components: (0,1,0), (0,0,1), (1,0,0) at flat 1, 2, 3
+      g1[0] = lam[3];
+      g1[1] = lam[1];
+      g1[2] = lam[2];
+    }
+  });
 }
+
+// The backward kernels' time follows their resident warps as long as the
+// sums and MCSH values of a pair stay in registers.  Orders 0-4 do in 96
+// registers, 20 warps per SM (10,000 structures, orders 0-4 x 8 sigmas, GB300:
+// 5.76 ms at 12 warps, 4.80 at 16, 4.67 at 20), orders 0-5 in 128, orders 0-6
+// in 168 (12 warps).  The strain derivative's kernel takes orders 0-6 in two
+// ranges, 0-4 and the rest, which repeat the exponentials (10% more
+// instructions) but fit 128 registers: 1.70 -> 1.66 ms on a 32,768-atom slab.
+// Without the strain sums the two ranges lose: 6.95 against 6.80 ms on the
+// 262,144-atom slab.
+template <int L, bool VIRIAL>
+constexpr int back_split() { return L >= 6 && VIRIAL ? 5 : L + 1; }
+template <int L, bool VIRIAL>
+constexpr int back_threads() { return L <= 4 ? 640 : L == 5 || VIRIAL ? 512 : 384; }
+// the radial table's sigma groups padded, but for the kernel whose 168
+// registers the padded stride would exceed
+template <int L, bool VIRIAL>
+constexpr bool back_pad() { return VIRIAL || L < 6; }
 
 // ------------------------------------------------------------------------
 // Backward only: moments come from the forward kernel (K.mu_out, read), the
@@ -981,16 +1061,13 @@ __device__ __forceinline__ void pair_gradient(const float* lam, float A, float d
 // (positions and lattice vectors strained alike move every d to (I+eps) d),
 // each lane's partial sums kept in its column of Wv ([9][32] floats of
 // warp-private shared memory) rather than in registers.
-// PACKED: radial factors on packed FP32 pairs (same results, fewer issue
-// slots; the plain backward kernel uses them, the strain-derivative variant
-// would spill at the 168 registers of the 12-warp launch).
 template <int L, int NS, bool VIRIAL = false, bool PACKED = false, bool PADG = true, bool MIXED = false>
 __device__ __forceinline__ void backward_sweep(const KParams& K, const float* __restrict__ s_rad,
                                                const float* __restrict__ s_dens, int64_t i, int64_t p0, int M,
                                                const float* __restrict__ Lam, float gd, float* Wv = nullptr) {
-  using SH = Shape<L, NS>;
   const GmpPass& P = K.pass;
   const int lane = threadIdx.x & 31;
+  constexpr int SPLIT = back_split<L, VIRIAL>();
   float own[3] = {0.0f, 0.0f, 0.0f};
   if constexpr (VIRIAL) {
 #pragma unroll
@@ -1001,56 +1078,24 @@ __device__ __forceinline__ void backward_sweep(const KParams& K, const float* __
     int e, j;
     load_pair(K.pairs, p0 + pp, dx, dy, dz, r2h, r2l, e, j);
     if (pp + 32 < M) prefetch_pair(K.pairs + p0 + pp + 32);
-    // MCSH values of orders 0..L first (order L+1 after the sigma loop):
-    // the sigma loop then contracts them directly, so that only the
-    // radial-weighted adjoints lam (not their derivative counterparts) are
-    // live beside them
     const float r2c = mcsh_r2(dx, dy, dz);
-    float S[SH::NIND1];
-    GmpMcsh<L>::eval(dx, dy, dz, r2c, S);
-    float lam[SH::NIND];
-#pragma unroll
-    for (int k = 0; k < SH::NIND; ++k) lam[k] = 0.0f;
-    float A = 0.0f;  // sum over sigma and order of dR_l/dr^2 * sum_{k in l} Lam_k S_k
     const float* tab_e = s_rad + (size_t)e * rad_elem_stride(L, NS, P.kmax, PADG);
-    for (int sg = 0; sg < SH::NSB; ++sg) {
-      float R[4][L + 2];
-      if constexpr (MIXED)
-        radial4x<L, L + 2, PADG>(tab_e, P.kmax, sg, r2h, r2l, R);
-      else if constexpr (PACKED)
-        radial4p<L, L + 2, PADG>(tab_e, P.kmax, sg, r2h, R);
-      else
-        radial4s<L, L + 2, PADG>(tab_e, P.kmax, sg, r2h, R);
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const float nb = P.nbeta[4 * sg + u];
-        const float* lrow = Lam + (4 * sg + u) * SH::NINDP;
-        float pl[L + 1];
-#pragma unroll
-        for (int l = 0; l <= L; ++l) pl[l] = 0.0f;
-        static_for<SH::NINDP / 4>([&](auto cq) {
-          constexpr int c4 = decltype(cq)::value;
-          const float4 lv4 = *reinterpret_cast<const float4*>(lrow + 4 * c4);
-          const float lv[4] = {lv4.x, lv4.y, lv4.z, lv4.w};
-          static_for<4>([&](auto tt) {
-            constexpr int k = 4 * c4 + decltype(tt)::value;
-            if constexpr (k < SH::NIND) {
-              constexpr int l = order_of(k);
-              lam[k] = __fmaf_rn(lv[decltype(tt)::value], R[u][l], lam[k]);
-              pl[l] = __fmaf_rn(lv[decltype(tt)::value], S[k], pl[l]);
-            }
-          });
-        });
-        // dR_l/dr^2 = -beta R_{l+1}: A += -beta sum_l R_{l+1} pl_l
-        float a = 0.0f;
-#pragma unroll
-        for (int l = 0; l <= L; ++l) a = __fmaf_rn(R[u][l + 1], pl[l], a);
-        A = __fmaf_rn(nb, a, A);
-      }
-    }
-    GmpMcsh<L + 1>::eval_top(dx, dy, dz, r2c, S);
+    float A = 0.0f, B = 0.0f, V[3] = {0.0f, 0.0f, 0.0f}, g1[3] = {0.0f, 0.0f, 0.0f};
+    adjoint_range<L, NS, 0, SPLIT - 1, PACKED, PADG, MIXED>(P, tab_e, Lam, dx, dy, dz, r2h, r2l, r2c, A, B, V, g1);
+    if constexpr (SPLIT <= L)
+      adjoint_range<L, NS, SPLIT, L, PACKED, PADG, MIXED>(P, tab_e, Lam, dx, dy, dz, r2h, r2l, r2c, A, B, V, g1);
     float g[3];
-    pair_gradient<L>(lam, A, dx, dy, dz, r2c, S, g);
+    if (r2c > 0.0f) {
+      const float inv = 1.0f / r2c;
+      const float c = 2.0f * A + B * inv;
+      g[0] = dx * c - V[0] * inv;
+      g[1] = dy * c - V[1] * inv;
+      g[2] = dz * c - V[2] * inv;
+    } else {
+      g[0] = g1[0];
+      g[1] = g1[1];
+      g[2] = g1[2];
+    }
     // the radial factors carried 2^32
     g[0] = __fmul_rn(g[0], GMP_EXP_UNSHIFT);
     g[1] = __fmul_rn(g[1], GMP_EXP_UNSHIFT);
@@ -1135,13 +1180,11 @@ __global__ void __launch_bounds__(256) k_vjp(KParams K) {
 }
 
 template <int L, int NS, bool VIRIAL = false, bool MIXED = false>
-__global__ void __launch_bounds__(384) k_backward(KParams K) {
+__global__ void __launch_bounds__(back_threads<L, VIRIAL>()) k_backward(KParams K) {
   using SH = Shape<L, NS>;
   extern __shared__ __align__(16) float smem[];
   const GmpPass& P = K.pass;
-  // table layout by register budget: each variant with the one it keeps
-  // 168 registers without spilling
-  constexpr bool PADG = VIRIAL;
+  constexpr bool PADG = back_pad<L, VIRIAL>();
   float* s_rad = smem;
   float* s_dens = s_rad + (size_t)P.n_el * rad_elem_stride(L, NS, P.kmax, PADG);
   float* s_warp = s_dens + (size_t)P.n_el * dens_elem_stride(P.kmax);
@@ -1150,10 +1193,9 @@ __global__ void __launch_bounds__(384) k_backward(KParams K) {
   __syncthreads();
   gmp_after_predecessor(0);  // (the tables belong to the handle)
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  constexpr int EXTRA = VIRIAL ? virial_extra_floats<L, NS>() : 0;
-  float* Mu = s_warp + (size_t)wib * (SH::WARP_FLOATS + EXTRA);
-  float* Lam = Mu + SH::TILE * SH::RSTR;
-  float* Wv = EXTRA ? Mu + SH::WARP_FLOATS : Mu;  // Mu is dead once Lam is formed
+  float* Lam = s_warp + (size_t)wib * back_warp_floats<L, NS>(VIRIAL);
+  float* Mu = Lam + NS * SH::NINDP;
+  float* Wv = Mu;  // Mu is dead once Lam is formed
   for (int64_t i = next_center(K); i < K.N; i = next_center(K)) {
     const int64_t p0 = K.nbr_beg[i], p1 = K.nbr_end[i];
     if (p1 > K.pair_cap) continue;  // over capacity: flagged by the fill pass
@@ -1164,21 +1206,9 @@ __global__ void __launch_bounds__(384) k_backward(KParams K) {
     const float* grow = K.grad_feat + i * P.F;
     adjoints<L, NS>(P, Mu, grow, Lam);
     const float gd = P.want_density ? grow[P.dens_col] : 0.0f;
-    backward_sweep<L, NS, VIRIAL, !VIRIAL && !MIXED, PADG, MIXED>(K, s_rad, s_dens, i, p0, M, Lam, gd, Wv);
+    backward_sweep<L, NS, VIRIAL, !MIXED, PADG, MIXED>(K, s_rad, s_dens, i, p0, M, Lam, gd, Wv);
     __syncwarp();
   }
-}
-
-// gmp_mcsh_shift_contract_order_<l> by a compile-time order.
-template <int l>
-__device__ __forceinline__ void shift_contract_order(const float* lam, const float* S1, float* V) {
-  if constexpr (l == 0) gmp_mcsh_shift_contract_order_0(lam, S1, V);
-  else if constexpr (l == 1) gmp_mcsh_shift_contract_order_1(lam, S1, V);
-  else if constexpr (l == 2) gmp_mcsh_shift_contract_order_2(lam, S1, V);
-  else if constexpr (l == 3) gmp_mcsh_shift_contract_order_3(lam, S1, V);
-  else if constexpr (l == 4) gmp_mcsh_shift_contract_order_4(lam, S1, V);
-  else if constexpr (l == 5) gmp_mcsh_shift_contract_order_5(lam, S1, V);
-  else gmp_mcsh_shift_contract_order_6(lam, S1, V);
 }
 
 // ------------------------------------------------------------------------

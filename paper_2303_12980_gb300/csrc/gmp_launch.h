@@ -17,7 +17,7 @@ struct KParams;
 // Launch shape of a compute kernel (chosen by the autotuner or defaults).
 struct GmpShape {
   int tile;   // forward tile: 16 pairs (two lanes per pair) or 32 (one lane per pair)
-  int warps;  // warps per CTA, 0 = largest that fits
+  int warps;  // warps per CTA, 0 = the CTA size with the most resident warps
 };
 
 // The launch worked out for a request (shape and number of centers' class):

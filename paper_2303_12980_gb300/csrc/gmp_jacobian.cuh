@@ -60,7 +60,6 @@ __global__ void __launch_bounds__(384) k_jacobian_r(KParams K) {
   float* s_rad = smem;
   float* s_dens = s_rad + (size_t)P.n_el * rad_elem_stride(L, NS, P.kmax);
   float* s_warp = s_dens + (size_t)P.n_el * dens_elem_stride(P.kmax);
-  gmp_let_next_start();
   load_tables<L>(P, NS, s_rad, s_dens);
   __syncthreads();
   gmp_after_predecessor(0);  // (the tables belong to the handle)

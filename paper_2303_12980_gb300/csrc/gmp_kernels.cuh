@@ -898,7 +898,6 @@ __global__ void __launch_bounds__(512) k_forward(KParams K) {
   float* s_rad = smem;
   float* s_dens = s_rad + (size_t)P.n_el * rad_elem_stride(L, NS, P.kmax);
   float* s_warp = s_dens + (size_t)P.n_el * dens_elem_stride(P.kmax);
-  gmp_let_next_start();
   load_tables<L>(P, NS, s_rad, s_dens);
   __syncthreads();
   gmp_after_predecessor(0);  // (the tables belong to the handle)
@@ -1153,7 +1152,6 @@ __global__ void __launch_bounds__(256) k_vjp(KParams K) {
   float* s_rad = smem;
   float* s_dens = s_rad + (size_t)P.n_el * rad_elem_stride(L, NS, P.kmax);
   float* s_warp = s_dens + (size_t)P.n_el * dens_elem_stride(P.kmax);
-  gmp_let_next_start();
   load_tables<L>(P, NS, s_rad, s_dens);
   __syncthreads();
   gmp_after_predecessor(0);  // (the tables belong to the handle)
@@ -1188,7 +1186,6 @@ __global__ void __launch_bounds__(back_threads<L, VIRIAL>()) k_backward(KParams 
   float* s_rad = smem;
   float* s_dens = s_rad + (size_t)P.n_el * rad_elem_stride(L, NS, P.kmax, PADG);
   float* s_warp = s_dens + (size_t)P.n_el * dens_elem_stride(P.kmax);
-  gmp_let_next_start();
   load_tables<L, PADG>(P, NS, s_rad, s_dens);
   __syncthreads();
   gmp_after_predecessor(0);  // (the tables belong to the handle)
@@ -1245,7 +1242,6 @@ __global__ void __maxnreg__(L >= 6 ? 168 : 128) k_jacobian(KParams K) {
   float* s_rad = smem;
   float* s_dens = s_rad + (size_t)P.n_el * rad_elem_stride(L, NS, P.kmax, false);
   float* s_warp = s_dens + (size_t)P.n_el * dens_elem_stride(P.kmax);
-  gmp_let_next_start();
   load_tables<L, false>(P, NS, s_rad, s_dens);
   __syncthreads();
   gmp_after_predecessor(0);  // (the tables belong to the handle)

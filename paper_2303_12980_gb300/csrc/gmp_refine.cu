@@ -171,7 +171,6 @@ __device__ __forceinline__ void refine_order(int lane, const GmpRefine& A, const
 // dependent double-float chains at 16 warps per SM (128 registers).
 __global__ void __launch_bounds__(256, 2) k_refine(const GmpRefine A) {
   __shared__ float2 exp_tab[64];
-  gmp_let_next_start();
   if (threadIdx.x < 64) exp_tab[threadIdx.x] = A.exp_tab[threadIdx.x];
   const int lane = gmp_after_predecessor(threadIdx.x) & 31;
   int64_t count = 0;

@@ -5,6 +5,7 @@
 #include "gmp_kernels.cuh"
 #include "gmp_launch.h"
 
+#include <atomic>
 #include <chrono>
 #include <cmath>
 #include <cstdio>
@@ -118,6 +119,7 @@ struct gmp_ctx {
   // VJP sums without float atomics: fixed-point bins per (atom,
   // component), per-center own terms and strain-derivative sums
   DevBuf gbins, own, vir_c;
+  bool gbins_empty = false;
   DevBuf mu;     // per-center moments between the forward and backward kernels
   DevBuf ktab;   // double-float radial constants [n_el][n_sigmas][kmax][16] for the refinement kernel
   DevBuf exptab; // [64] 2^(-j/64) as double-floats (the refinement's exponential)
@@ -143,7 +145,10 @@ struct gmp_ctx {
   int size_kind = 0;           // of the current lists
   int64_t cap_cur = 0;         // pair capacity of the current lists
   int64_t nc_cur = 0;          // ... and their centers
-  bool lists_pending = false;  // single-pass lists whose outcome is not read yet (ev_lists)
+  bool lists_pending = false;  // single-pass lists whose outcome is not read yet
+  bool lists_report = false;   // ... it comes from the next compute kernel (else a copy, ev_lists)
+  unsigned long long build = 0;      // number of that build
+  GmpListReport* report = nullptr;   // pinned
   bool lists_outgrown = false; // ... and found to exceed its capacities
   bool exact_lists = false;    // count before filling (set for a rerun)
   cudaEvent_t ev_lists = nullptr;
@@ -431,9 +436,10 @@ gmp_status bin_atoms(gmp_ctx* h, int32_t S, const double* pos, const int32_t* sp
   GMP_CK(h->nbr_off.ensure(sizeof(int64_t) * (n_centers + 1)), "nbr_off");
   const int64_t scan_n = std::max<int64_t>(std::max<int64_t>(N, n_centers), h->n_bins);
   GMP_CK(h->scan_tmp.ensure(gmp_scan_tmp_bytes(scan_n)), "scan_tmp");
-  // the error word is cleared after it is read, so a condition raised after
-  // the read of the previous call is reported here
-  GMP_CK(cudaMemsetAsync(h->scalars.as<char>() + kScalarMaxM, 0, kScalarBytes - kScalarMaxM, st), "clear scalars");
+  // the first kernel clears everything in scalars but the error word, which is
+  // cleared after it is read, so a condition raised after the read of the
+  // previous call is reported here
+  constexpr int n_clear = (int)(kScalarBytes / 4) - 1;
   h->next_counter = 0;
 
   if (gmp_bin_small_fits(N, h->n_bins, S)) {
@@ -441,7 +447,7 @@ gmp_status bin_atoms(gmp_ctx* h, int32_t S, const double* pos, const int32_t* sp
                                 h->n_el, h->grid.as<GmpGrid>(), h->n_bins, h->atom_xh.as<float4>(),
                                 h->atom_xl.as<float4>(), h->atom_u.as<GmpD4>(), h->atom_bin.as<int32_t>(),
                                 h->bin_start.as<int32_t>(), h->bin_y.as<float4>(), h->bin_je.as<int2>(),
-                                h->atom_t.as<float4>(), h->atom_y.as<float4>(), d_err, st, L),
+                                h->atom_t.as<float4>(), h->atom_y.as<float4>(), d_err, n_clear, st, L),
            "bins (one block)");
     return GMP_OK;
   }
@@ -449,7 +455,7 @@ gmp_status bin_atoms(gmp_ctx* h, int32_t S, const double* pos, const int32_t* sp
                                       pos, species, h->n_el, h->grid_mode, h->grid.as<GmpGrid>(),
                                       h->atom_xh.as<float4>(), h->atom_xl.as<float4>(), h->atom_u.as<GmpD4>(),
                                       h->bbox.as<unsigned long long>(), h->n_bins, h->bin_count.as<int32_t>(),
-                                      h->bin_cursor.as<int32_t>(), d_err, st, h->sm_count, L),
+                                      h->bin_cursor.as<int32_t>(), d_err, n_clear, st, h->sm_count, L),
          "prepare");
   GMP_CK(gmp_launch_bins(h->structs.as<GmpStruct>(), h->grid.as<GmpGrid>(), h->struct_of.as<int32_t>(), N,
                          h->n_bins, h->atom_bin.as<int32_t>(), h->bin_count.as<int32_t>(),
@@ -471,11 +477,30 @@ void note_sizes(gmp_ctx* h) {
 gmp_status finish_lists(gmp_ctx* h, cudaStream_t st) {
   if (!h->lists_pending) return GMP_OK;
   h->lists_pending = false;
-  GMP_CK(cudaEventSynchronize(h->ev_lists), "neighbor sync");
-  const uint32_t w = (uint32_t)(h->h_small[0] & 0xffffffffu);
+  unsigned long long err_maxm, pairs;
+  if (h->lists_report) {
+    // the first compute kernel writes it when it starts; the stream's state is
+    // looked at now and then, so that a kernel that never comes is noticed
+    volatile GmpListReport* r = h->report;
+    for (uint32_t n = 1; r->build != h->build; ++n) {
+      if (n % 4096 != 0) continue;
+      const cudaError_t e = cudaStreamQuery(st);
+      if (e == cudaErrorNotReady) continue;
+      if (e != cudaSuccess) return cuda_fail(h, e, "neighbor wait");
+      if (r->build != h->build) return fail(h, GMP_ERR_CUDA, "the neighbor lists' outcome was not reported");
+    }
+    std::atomic_thread_fence(std::memory_order_acquire);
+    err_maxm = r->err_maxm;
+    pairs = r->pairs;
+  } else {
+    GMP_CK(cudaEventSynchronize(h->ev_lists), "neighbor sync");
+    err_maxm = (unsigned long long)h->h_small[0];
+    pairs = (unsigned long long)h->h_small[1];
+  }
+  const uint32_t w = (uint32_t)(err_maxm & 0xffffffffu);
   if (!w) {
-    h->P = h->h_small[1];
-    h->max_m = (int)(h->h_small[0] >> 32);
+    h->P = (int64_t)pairs;
+    h->max_m = (int)(err_maxm >> 32);
     note_sizes(h);
     return GMP_OK;
   }
@@ -502,10 +527,11 @@ gmp_status run_sequence(gmp_ctx* h, cudaStream_t st, Seq& seq) {
 // Exact neighbor lists of the NC centers C over the binned atoms into
 // h->pairs / h->nbr_off.  With single_ok and an earlier build to guess the
 // capacities from, one enumeration pass whose outcome finish_lists reads
-// later; otherwise (unless capturing) synchronises `st` once to size the pair
+// later (with report, from the compute kernel that the caller launches next;
+// else from a copy); otherwise (unless capturing) synchronises `st` once to size the pair
 // buffer.
 gmp_status neighbor_lists(gmp_ctx* h, const GmpCenters& C, int64_t NC, const double* pos, cudaStream_t st,
-                          bool sorted, bool capture, bool single_ok, int size_kind) {
+                          bool sorted, bool capture, bool single_ok, int size_kind, bool report) {
   int64_t* L = &h->launches;
   uint32_t* d_err = h->scalars.as<uint32_t>();
   int32_t* d_maxm = reinterpret_cast<int32_t*>(h->scalars.as<char>() + kScalarMaxM);
@@ -532,8 +558,12 @@ gmp_status neighbor_lists(gmp_ctx* h, const GmpCenters& C, int64_t NC, const dou
                                       h->pairs.as<GmpPair>(), cap, keys, d_maxm, d_err, st, h->sm_count, L, d_cursor,
                                       h->nbr_rng.as<int64_t>()),
              "neighbor single pass");
-      GMP_CK(cudaMemcpyAsync(h->h_small, d_err, 16, cudaMemcpyDeviceToHost, st), "read err, longest, P");
-      GMP_CK(cudaEventRecord(h->ev_lists, st), "event");
+      h->lists_report = report;
+      ++h->build;
+      if (!report) {
+        GMP_CK(cudaMemcpyAsync(h->h_small, d_err, 16, cudaMemcpyDeviceToHost, st), "read err, longest, P");
+        GMP_CK(cudaEventRecord(h->ev_lists, st), "event");
+      }
       h->cap_cur = cap;
       h->rng_mode = true;
       h->lists_pending = true;
@@ -602,14 +632,15 @@ gmp_status neighbor_lists(gmp_ctx* h, const GmpCenters& C, int64_t NC, const dou
 // Binning + exact neighbor lists of every atom into h->pairs / h->nbr_off
 // (see neighbor_lists).
 gmp_status build_neighbors(gmp_ctx* h, int32_t S, const double* pos, const int32_t* species,
-                           int64_t N, cudaStream_t st, bool sorted, bool capture = false, bool need_csr = false) {
+                           int64_t N, cudaStream_t st, bool sorted, bool capture = false, bool need_csr = false,
+                           bool report = false) {
   if (!capture) h->graph_valid = false;  // buffers may move: a captured graph is stale
   GMP_CK(prof_mark(h, 0, true, st), "profile");
   gmp_status r = bin_atoms(h, S, pos, species, N, N, st);
   if (r != GMP_OK) return r;
   const GmpCenters C{h->struct_of.as<int32_t>(), pos, h->atom_xh.as<float4>(), h->atom_xl.as<float4>(),
                      h->atom_t.as<float4>(), h->atom_y.as<float4>()};
-  if ((r = neighbor_lists(h, C, N, pos, st, sorted, capture, !need_csr, 0)) != GMP_OK) return r;
+  if ((r = neighbor_lists(h, C, N, pos, st, sorted, capture, !need_csr, 0, report)) != GMP_OK) return r;
   GMP_CK(prof_mark(h, 0, false, st), "profile");
   return GMP_OK;
 }
@@ -655,8 +686,12 @@ gmpk::KParams base_params(gmp_ctx* h, const PassData& pd, int pass_index, int64_
   return K;
 }
 
-// The next of the call's work counters (cleared when the call began).
+// The next of the call's work counters (cleared when the call began); the
+// first compute kernel also reports the neighbor lists.
 void take_counter(gmp_ctx* h, gmpk::KParams& K) {
+  K.report = h->next_counter == 0 && h->lists_pending && h->lists_report ? h->report : nullptr;
+  K.list_state = h->scalars.as<unsigned long long>();
+  K.build = h->build;
   K.counter = reinterpret_cast<int32_t*>(h->scalars.as<char>() + kScalarCounters) + h->next_counter++;
 }
 
@@ -1158,7 +1193,10 @@ gmp_status gmp_create(const gmp_params* p, int device, gmp_handle* out) {
     }
     for (auto& pd : h->passes) pd.pass.exp_tab = h->exptab.as<float2>();
   }
-  if (cudaMallocHost((void**)&h->h_small, 64) != cudaSuccess) { cudaGetLastError(); return bad("pinned alloc failed"); }
+  // small readbacks, then the neighbor lists' report
+  if (cudaMallocHost((void**)&h->h_small, 128) != cudaSuccess) { cudaGetLastError(); return bad("pinned alloc failed"); }
+  std::memset(h->h_small, 0, 128);
+  h->report = reinterpret_cast<GmpListReport*>(h->h_small + 8);
   if (cudaEventCreateWithFlags(&h->ev, cudaEventDisableTiming) != cudaSuccess) { cudaGetLastError(); return bad("event"); }
   if (cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking) != cudaSuccess ||
       cudaEventCreateWithFlags(&h->ev_desc, cudaEventDisableTiming) != cudaSuccess ||
@@ -1208,7 +1246,7 @@ gmp_status gmp_featurize(gmp_handle h, int32_t n_struct, const int64_t* atom_off
                                       (uintptr_t)N, (uintptr_t)n_struct, (uintptr_t)h->struct_gen};
   if (use_graph && (r = replay_graph(h, key, st)) != GMP_ERR_CAPACITY) return r;
   auto seq = [&](bool capture) -> gmp_status {
-    gmp_status q = build_neighbors(h, n_struct, io.pos, io.species, N, st, false, capture);
+    gmp_status q = build_neighbors(h, n_struct, io.pos, io.species, N, st, false, capture, false, !io.host);
     if (q != GMP_OK) return q;
     if (io.host && (q = finish_lists(h, st)) != GMP_OK) return q;
     if ((q = begin_compute(h, N)) != GMP_OK) return q;
@@ -1290,7 +1328,15 @@ static gmp_status vjp_impl(gmp_handle h, int32_t n_struct, const int64_t* atom_o
   if (use_graph && (r = replay_graph(h, key, st)) != GMP_ERR_CAPACITY) return r;
   // buffers first (no allocation may happen while a graph is captured)
   if (h->passes.size() > 1) GMP_CK(h->grad_acc.ensure(sizeof(double) * 3 * N), "grad_acc");
-  GMP_CK(h->gbins.ensure(sizeof(unsigned long long) * 3 * gmpk::kGradBins * N), "gradient bins");
+  {
+    // the finishing kernel leaves the bins empty; new ones, and those of a call
+    // that did not get that far, are cleared here
+    void* const old = h->gbins.p;
+    GMP_CK(h->gbins.ensure(sizeof(unsigned long long) * 3 * gmpk::kGradBins * N), "gradient bins");
+    if (h->gbins.p != old || !h->gbins_empty)
+      GMP_CK(cudaMemsetAsync(h->gbins.p, 0, h->gbins.bytes, st), "clear bins");
+    h->gbins_empty = true;
+  }
   GMP_CK(h->own.ensure(sizeof(double) * 3 * N), "own");
   if (vir) GMP_CK(h->vir_c.ensure(sizeof(double) * 9 * N), "vir_c");
   for (const PassData& pd : h->passes)
@@ -1305,11 +1351,7 @@ static gmp_status vjp_impl(gmp_handle h, int32_t n_struct, const int64_t* atom_o
     K.own = h->own.as<double>();
     K.vir_c = vir ? h->vir_c.as<double>() : nullptr;
     take_counter(h, K);
-    return GMP_OK;
-  };
-  // ahead of a pass's kernels, so that they follow one another directly
-  auto clear_bins = [&]() -> gmp_status {
-    GMP_CK(cudaMemsetAsync(h->gbins.p, 0, sizeof(unsigned long long) * 3 * gmpk::kGradBins * N, st), "memset bins");
+    h->gbins_empty = false;
     return GMP_OK;
   };
   auto vjp_end = [&](const gmpk::KParams& K, bool first, bool last) -> gmp_status {
@@ -1317,6 +1359,7 @@ static gmp_status vjp_impl(gmp_handle h, int32_t n_struct, const int64_t* atom_o
                                        last ? nullptr : h->grad_acc.as<double>(), last ? gp : nullptr, st, h->sm_count,
                                        &h->launches),
            "gradient sums");
+    h->gbins_empty = true;
     if (vir)
       GMP_CK(gmp_launch_virial_reduce(n_struct, h->atom_off.as<int64_t>(), K.vir_c, vir, first, st, h->sm_count,
                                       &h->launches),
@@ -1324,9 +1367,8 @@ static gmp_status vjp_impl(gmp_handle h, int32_t n_struct, const int64_t* atom_o
     return GMP_OK;
   };
   auto seq = [&](bool capture) -> gmp_status {
-  gmp_status q = clear_bins();
+  gmp_status q = build_neighbors(h, n_struct, io.pos, io.species, N, st, false, capture, false, !io.host);
   if (q != GMP_OK) return q;
-  if ((q = build_neighbors(h, n_struct, io.pos, io.species, N, st, false, capture)) != GMP_OK) return q;
   if (io.host && (q = finish_lists(h, st)) != GMP_OK) return q;
   if ((q = begin_compute(h, N)) != GMP_OK) return q;
   bool refined = false, waited = false, pending = false;
@@ -1334,7 +1376,6 @@ static gmp_status vjp_impl(gmp_handle h, int32_t n_struct, const int64_t* atom_o
   for (size_t g = 0; g < h->passes.size(); ++g) {
     PassData& pd = h->passes[g];
     const bool last = g + 1 == h->passes.size();
-    if (g > 0 && (q = clear_bins()) != GMP_OK) return q;
     // forward kernel (features + moments), then the backward kernel reading
     // the moments (or one fused kernel, if the autotuner chose it)
     float* fout = feat ? feat : h->stage_feat.as<float>();
@@ -1409,6 +1450,7 @@ static gmp_status vjp_impl(gmp_handle h, int32_t n_struct, const int64_t* atom_o
   return GMP_OK;
   };
   if ((r = run_sequence(h, st, seq)) != GMP_OK) {
+    h->gbins_empty = false;
     if (io.host) cudaStreamSynchronize(h->side);  // no copy may outlive the call
     return r;
   }
@@ -1506,7 +1548,7 @@ gmp_status gmp_featurize_points(gmp_handle h, int32_t n_struct, const int64_t* a
            "point prepare");
     const GmpCenters C{h->pt_struct.as<int32_t>(), pts, h->pt_xh.as<float4>(), h->pt_xl.as<float4>(),
                        h->pt_t.as<float4>(), h->pt_y.as<float4>()};
-    if ((q = neighbor_lists(h, C, NP, io.pos, st, false, false, true, 1)) != GMP_OK) return q;
+    if ((q = neighbor_lists(h, C, NP, io.pos, st, false, false, true, 1, !host)) != GMP_OK) return q;
     GMP_CK(prof_mark(h, 0, false, st), "profile");
     if (host && (q = finish_lists(h, st)) != GMP_OK) return q;
     if ((q = begin_compute(h, NP)) != GMP_OK) return q;

@@ -410,8 +410,9 @@ cudaError_t gmp_launch_bin_small(GmpStruct* d_structs, int n_struct, const int32
                                  double cutoff, const double* pos, const int32_t* species, int n_el,
                                  GmpGrid* d_grid, int64_t n_bins, float4* atom_xh, float4* atom_xl, GmpD4* atom_u,
                                  int32_t* atom_bin, int32_t* bin_start, float4* bin_y, int2* bin_je,
-                                 float4* atom_t, float4* atom_y, uint32_t* d_err, cudaStream_t stream,
+                                 float4* atom_t, float4* atom_y, uint32_t* d_err, int n_clear, cudaStream_t stream,
                                  int64_t* launches);
+// n_clear words behind *d_err are cleared (gmp_launch_bin_small too).
 // Where the structures' bin grids come from: given (uploaded with the batch
 // description: every structure is periodic along all axes, gmp_periodic_grid),
 // from the atoms' range for the structures with a non-periodic axis (the
@@ -425,7 +426,7 @@ cudaError_t gmp_launch_neighbors_prepare(GmpStruct* d_structs, int n_struct,
                                          const double* pos, const int32_t* species, int n_el, GmpGridMode mode,
                                          GmpGrid* d_grid, float4* atom_xh, float4* atom_xl,
                                          GmpD4* atom_u, unsigned long long* d_bbox, int64_t n_bins,
-                                         int32_t* bin_count, int32_t* bin_cursor, uint32_t* d_err,
+                                         int32_t* bin_count, int32_t* bin_cursor, uint32_t* d_err, int n_clear,
                                          cudaStream_t stream, int sm_count, int64_t* launches);
 cudaError_t gmp_launch_bins(const GmpStruct* d_structs, const GmpGrid* d_grid,
                             const int32_t* d_struct_of, int64_t N, int64_t n_bins,
@@ -471,6 +472,12 @@ cudaError_t gmp_launch_neighbor_pass(int fill, const GmpStruct* d_structs, const
                                      GmpPair* pairs, int64_t pair_cap, int max_keys, int32_t* d_maxm,
                                      uint32_t* d_err, cudaStream_t stream, int sm_count, int64_t* launches,
                                      unsigned long long* cursor = nullptr, int64_t* rng = nullptr);
+// What the host reads of a single-pass build: error word and longest list,
+// pairs, then the number of the build, written last.  The first compute
+// kernel behind the build writes it (KParams::report), to pinned host memory.
+struct GmpListReport {
+  unsigned long long err_maxm, pairs, build;
+};
 // Distinct neighbor atoms per center (counts [N]) and each pair's row
 // among them (local_row [P]); center i's pairs are [nbr_beg[i], nbr_end[i]),
 // sorted by atom.
@@ -478,10 +485,11 @@ cudaError_t gmp_launch_jacobian_count(int64_t N, const int64_t* nbr_beg, const i
                                       int64_t* counts, int32_t* local_row, cudaStream_t stream, int sm_count,
                                       int64_t* launches);
 // Gradient of atom j: own[j] + the value of j's exact fixed-point bins (filled
-// by the backward kernels without float atomics; 12 per atom and component),
+// by the backward kernels without float atomics; 12 per atom and component, left
+// empty again),
 // plus acc_in[j] (earlier passes, may be null), to acc_out[j], or rounded to
 // grad_pos[j] when that is given (the last pass).
-cudaError_t gmp_launch_grad_bins_finish(int64_t N, const unsigned long long* bins, const double* own,
+cudaError_t gmp_launch_grad_bins_finish(int64_t N, unsigned long long* bins, const double* own,
                                         const double* acc_in, double* acc_out, float* grad_pos, cudaStream_t stream,
                                         int sm_count, int64_t* launches);
 // virial[s] = (first) or += sum of vir_c over the centers atom_off[s] .. atom_off[s+1]-1 (fixed order).

@@ -189,6 +189,11 @@ struct KParams {
   int32_t* jac_j;
   float* jac;             // [nnz, F, 3]
   int32_t* counter;       // the launch's work counter, zero at its start
+  // outcome of the neighbor lists for the waiting host (null: not asked):
+  // list_state holds the error word and longest list, then the pairs
+  GmpListReport* report;
+  const unsigned long long* list_state;
+  unsigned long long build;
   int64_t center0;        // centers center0 .. N-1;
                           // jac_off row 0 belongs to center center0 (jacobian)
   // features too ill-conditioned for FP32 (recomputed in double-float
@@ -828,6 +833,23 @@ __device__ __forceinline__ void setup_items(int (&it_l)[Shape<L, NS>::Q], int (&
   }
 }
 
+// The outcome of the neighbor build before this kernel, for the host that
+// waits for it while the call's kernels run.  A copy in the stream between the
+// two would hold this kernel back until the copy engine is done, and the
+// memsets of the counters and of the gradient bins did the same to theirs
+// (the first kernel of a call and the last user of the bins clear them now).
+// Without the three, a call of a 64-atom box takes 58 us instead of 71
+// (with gradients 63 instead of 82), of a 4,096-atom crystal 112 instead of
+// 126 (176 instead of 194), of 400 mixed structures 1072 instead of 1152.
+__device__ __forceinline__ void report_lists(const KParams& K) {
+  if (!K.report || blockIdx.x != 0 || threadIdx.x != 0) return;
+  volatile GmpListReport* r = K.report;
+  r->err_maxm = K.list_state[0];
+  r->pairs = K.list_state[1];
+  __threadfence_system();
+  r->build = K.build;
+}
+
 __device__ __forceinline__ int64_t next_center(const KParams& K) {
   int c = 0;
   if ((threadIdx.x & 31) == 0) c = atomicAdd(K.counter, 1);
@@ -901,6 +923,7 @@ __global__ void __launch_bounds__(512) k_forward(KParams K) {
   load_tables<L>(P, NS, s_rad, s_dens);
   __syncthreads();
   gmp_after_predecessor(0);  // (the tables belong to the handle)
+  report_lists(K);
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   float* Rt = s_warp + (size_t)wib * SH::WARP_FLOATS;
   float* St = Rt + SH::TILE * SH::RSTR;
@@ -1155,6 +1178,7 @@ __global__ void __launch_bounds__(256) k_vjp(KParams K) {
   load_tables<L>(P, NS, s_rad, s_dens);
   __syncthreads();
   gmp_after_predecessor(0);  // (the tables belong to the handle)
+  report_lists(K);
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   float* Rt = s_warp + (size_t)wib * SH::WARP_FLOATS;
   float* St = Rt + SH::TILE * SH::RSTR;

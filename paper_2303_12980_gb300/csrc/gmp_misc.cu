@@ -41,8 +41,9 @@ __global__ void k_jac_count(int64_t N, const int64_t* __restrict__ nbr_beg, cons
 // units of 2^(24 b - 149); added in a fixed order, so the result does not
 // depend on the order in which the bins were filled).  Bin 11 holds flags
 // of non-finite contributions: NaN if any was NaN or infinities of both
-// signs came in, else that infinity.  One thread per (atom, component).
-__global__ void k_grad_bins_finish(int64_t n, const unsigned long long* __restrict__ bins,
+// signs came in, else that infinity.  The bins are left empty for the next
+// pass.  One thread per (atom, component).
+__global__ void k_grad_bins_finish(int64_t n, unsigned long long* __restrict__ bins,
                                    const double* __restrict__ own, const double* acc_in, double* acc_out,
                                    float* __restrict__ grad_pos) {
   constexpr int kBins = 12;
@@ -51,16 +52,21 @@ __global__ void k_grad_bins_finish(int64_t n, const unsigned long long* __restri
   gmp_let_next_start();
   const unsigned tid = gmp_after_predecessor(threadIdx.x);
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + tid; t < n; t += (int64_t)gridDim.x * blockDim.x) {
-    const unsigned long long* bt = bins + t * kBins;
+    unsigned long long* bt = bins + t * kBins;
     const unsigned long long fl = bt[11];
     double v;
     if (fl) {
+#pragma unroll
+      for (int b = 0; b < kBins; ++b) bt[b] = 0;
       v = ((fl & 1ull) || ((fl & 6ull) == 6ull)) ? (double)NAN : ((fl & 2ull) ? (double)INFINITY : -(double)INFINITY);
     } else {
       v = 0.0;
 #pragma unroll
       for (int b = 0; b < 11; ++b)  // most are empty; the product is exact
-        if (const long long x = (long long)bt[b]) v = __fma_rn((double)x, kBinUnit[b], v);
+        if (const long long x = (long long)bt[b]) {
+          v = __fma_rn((double)x, kBinUnit[b], v);
+          bt[b] = 0;
+        }
     }
     v = own[t] + v;
     if (acc_in) v = acc_in[t] + v;
@@ -118,7 +124,7 @@ cudaError_t gmp_launch_jacobian_count(int64_t N, const int64_t* nbr_beg, const i
   return cudaGetLastError();
 }
 
-cudaError_t gmp_launch_grad_bins_finish(int64_t N, const unsigned long long* bins, const double* own,
+cudaError_t gmp_launch_grad_bins_finish(int64_t N, unsigned long long* bins, const double* own,
                                         const double* acc_in, double* acc_out, float* grad_pos, cudaStream_t stream,
                                         int sm_count, int64_t* launches) {
   if (N <= 0) return cudaSuccess;

@@ -24,6 +24,8 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
+
 namespace {
 
 __device__ __forceinline__ unsigned long long order_key(double v) {
@@ -107,6 +109,8 @@ __device__ inline int wrap_axis(double& u, double f0, uint32_t* err) {
   return w;
 }
 
+// (The first kernel of a call also clears the n_clear words behind the error
+// word: counters and sizes of the call, which later kernels use.)
 // Per atom: checks, fractional coordinates, wrap, double-float split, bbox.
 // bbox (6 keys per structure: min and complemented max of each
 // non-periodic fractional axis) may be global or shared memory.
@@ -156,9 +160,11 @@ __global__ void k_prepare(const GmpStruct* __restrict__ S, const int32_t* __rest
                           float4* __restrict__ atom_xh, float4* __restrict__ atom_xl,
                           GmpD4* __restrict__ atom_u, unsigned long long* __restrict__ bbox,
                           int64_t n_bins, int32_t* __restrict__ bin_count, int32_t* __restrict__ bin_cursor,
-                          uint32_t* __restrict__ err) {
+                          uint32_t* __restrict__ err, int n_clear) {
   gmp_let_next_start();
   const unsigned tid = gmp_after_predecessor(threadIdx.x);
+  if (blockIdx.x == 0)
+    for (int t = tid; t < n_clear; t += blockDim.x) err[1 + t] = 0;
   for (int64_t b = blockIdx.x * (int64_t)blockDim.x + tid; b < n_bins; b += (int64_t)gridDim.x * blockDim.x)
     bin_count[b] = bin_cursor[b] = 0;
   for (int64_t a = blockIdx.x * (int64_t)blockDim.x + tid; a < N;
@@ -419,7 +425,7 @@ __global__ void __launch_bounds__(1024) k_bin_small(GmpStruct* S, int n_struct, 
                                                    int32_t* atom_bin, int32_t* __restrict__ bin_start,
                                                    float4* __restrict__ bin_y, int2* __restrict__ bin_je,
                                                    float4* __restrict__ atom_t, float4* __restrict__ atom_y,
-                                                   uint32_t* __restrict__ err) {
+                                                   uint32_t* __restrict__ err, int n_clear) {
   extern __shared__ __align__(16) unsigned char sm_small[];
   __shared__ int32_t warp_tot[32];
   unsigned long long* bbox = reinterpret_cast<unsigned long long*>(sm_small);
@@ -428,6 +434,7 @@ __global__ void __launch_bounds__(1024) k_bin_small(GmpStruct* S, int n_struct, 
   int32_t* slot_atom = start + n_bins + 1;                          // [N] atom of each slot
   gmp_let_next_start();
   const int tid = (int)gmp_after_predecessor(threadIdx.x), nt = blockDim.x, lane = tid & 31, wid = tid >> 5;
+  for (int t = tid; t < n_clear; t += nt) err[1 + t] = 0;
   for (int t = tid; t < 6 * n_struct; t += nt) bbox[t] = ~0ull;
   for (int64_t b = tid; b < n_bins; b += nt) cnt[b] = 0;
   __syncthreads();
@@ -1043,7 +1050,7 @@ cudaError_t gmp_launch_neighbors_prepare(GmpStruct* d_structs, int n_struct,
                                          const double* pos, const int32_t* species, int n_el, GmpGridMode mode,
                                          GmpGrid* d_grid, float4* atom_xh, float4* atom_xl,
                                          GmpD4* atom_u, unsigned long long* d_bbox, int64_t n_bins,
-                                         int32_t* bin_count, int32_t* bin_cursor, uint32_t* d_err,
+                                         int32_t* bin_count, int32_t* bin_cursor, uint32_t* d_err, int n_clear,
                                          cudaStream_t stream, int sm_count, int64_t* launches) {
   if (mode != GmpGridMode::kGiven) {
     const cudaError_t e = cudaMemsetAsync(d_bbox, 0xFF, sizeof(unsigned long long) * 6 * n_struct, stream);
@@ -1051,7 +1058,7 @@ cudaError_t gmp_launch_neighbors_prepare(GmpStruct* d_structs, int n_struct,
   }
   const int nt = atom_threads(N, sm_count);
   GMP_TRY(gmp_launch_next(k_prepare, grid_for(N, nt, sm_count), nt, 0, stream, d_structs, d_struct_of, N, pos,
-                          species, n_el, atom_xh, atom_xl, atom_u, d_bbox, n_bins, bin_count, bin_cursor, d_err));
+                          species, n_el, atom_xh, atom_xl, atom_u, d_bbox, n_bins, bin_count, bin_cursor, d_err, n_clear));
   ++*launches;
   if (mode != GmpGridMode::kGiven) {
     GMP_TRY(gmp_launch_next(k_grid, (n_struct + 31) / 32, 32, 0, stream, d_structs, n_struct, d_bbox, d_grid,
@@ -1092,7 +1099,7 @@ cudaError_t gmp_launch_bin_small(GmpStruct* d_structs, int n_struct, const int32
                                  double cutoff, const double* pos, const int32_t* species, int n_el,
                                  GmpGrid* d_grid, int64_t n_bins, float4* atom_xh, float4* atom_xl, GmpD4* atom_u,
                                  int32_t* atom_bin, int32_t* bin_start, float4* bin_y, int2* bin_je,
-                                 float4* atom_t, float4* atom_y, uint32_t* d_err, cudaStream_t stream,
+                                 float4* atom_t, float4* atom_y, uint32_t* d_err, int n_clear, cudaStream_t stream,
                                  int64_t* launches) {
   if (!gmp_bin_small_fits(N, n_bins, n_struct)) return cudaErrorInvalidValue;
   const size_t smem = small_bin_smem(N, n_bins, n_struct);
@@ -1100,9 +1107,11 @@ cudaError_t gmp_launch_bin_small(GmpStruct* d_structs, int n_struct, const int32
     const cudaError_t e = cudaFuncSetAttribute(k_bin_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  GMP_TRY(gmp_launch_next(k_bin_small, 1, 1024, smem, stream, d_structs, n_struct, d_struct_of, N, cutoff, pos,
+  // (as many threads as atoms: fewer warps to wait for at each step)
+  const int nt = (int)std::min<int64_t>(1024, std::max<int64_t>(128, (N + 31) / 32 * 32));
+  GMP_TRY(gmp_launch_next(k_bin_small, 1, nt, smem, stream, d_structs, n_struct, d_struct_of, N, cutoff, pos,
                           species, n_el, d_grid, n_bins, atom_xh, atom_xl, atom_u, atom_bin, bin_start, bin_y,
-                          bin_je, atom_t, atom_y, d_err));
+                          bin_je, atom_t, atom_y, d_err, n_clear));
   ++*launches;
   return cudaGetLastError();
 }

@@ -185,7 +185,7 @@ extern "C" gmp_status gmp_neighbor_counts_noalloc(int32_t n_atoms, const double*
   if (e == cudaSuccess) e = cudaMemsetAsync(d_species, 0, sizeof(int32_t) * n_atoms, st);
   if (e == cudaSuccess)
     e = gmp_launch_neighbors_prepare(d_st, 1, d_struct_of, n_atoms, cutoff, pos, d_species, 1, GmpGridMode::kAll,
-                                     d_grid, d_xh, d_xl, d_u, d_bbox, n_bins, d_bcount, d_bcursor, d_err, st, sm_count,
+                                     d_grid, d_xh, d_xl, d_u, d_bbox, n_bins, d_bcount, d_bcursor, d_err, 1, st, sm_count,
                                      &launches);
   if (e == cudaSuccess)
     e = gmp_launch_bins(d_st, d_grid, d_struct_of, n_atoms, n_bins, d_bin, d_bcount, d_bstart, d_bcursor, d_t,

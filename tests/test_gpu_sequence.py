@@ -94,3 +94,36 @@ def test_bins_around_the_scan_limit(torch, oracle_mod, n, periodic):
     F = GMPFeaturizer.from_workload(w)
     f = F.featurize(torch.from_numpy(w.positions).cuda(), torch.from_numpy(w.species).cuda(), w.atom_off, w.cells, w.pbc)
     assert feature_errors(f.cpu().numpy()[centers], ref, fabs).max() <= FEAT_TOL
+
+
+@pytest.mark.parametrize("on_dev", [True, False])
+@pytest.mark.parametrize("n_sig", [3, 18])  # 18: two passes over the same bins
+@pytest.mark.parametrize("virial", [False, True])
+def test_gradient_bins_are_left_empty(torch, on_dev, n_sig, virial):
+    """Gradients of a handle whose bins held another batch, a refused call's
+    sums, infinities, or grew in between, to the bit of a fresh handle's."""
+    from paper_2303_12980_gb300.binding import GMPError, GMPFeaturizer
+    small, large = _wl(2, n_sig=n_sig), _wl(4, n_sig=n_sig)
+    put = (lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()) if on_dev else (lambda a: a)
+
+    def call(F, w, bad=False, scale=1.0):
+        sp = w.species.copy()
+        if bad:
+            sp[-1] = 9
+        g = (synth.upstream_gradient(w.n_atoms, w.n_features, seed=1) * np.float32(scale)).astype(np.float32)
+        f = F.featurize_vjp_virial if virial else F.featurize_vjp
+        return [torch.as_tensor(x).cpu() for x in f(put(w.positions), put(sp), w.atom_off, w.cells, w.pbc, put(g))]
+
+    want = {id(w): call(GMPFeaturizer.from_workload(w), w) for w in (small, large)}
+    F = GMPFeaturizer.from_workload(small)
+    steps = [(small, {}), (small, {"scale": np.inf}), (small, {}), (small, {"bad": True}), (small, {}), (large, {}),
+             (large, {"bad": True}), (small, {}), (large, {})]
+    for w, how in steps:
+        if how.get("bad"):
+            with pytest.raises(GMPError, match="species"):
+                call(F, w, **how)
+            continue
+        got = call(F, w, **how)
+        if not how:
+            for a, b in zip(got, want[id(w)]):
+                assert torch.equal(a, b)

@@ -177,13 +177,15 @@ __global__ void k_prepare(const GmpStruct* __restrict__ S, const int32_t* __rest
 // from its cell and is made on the host, with the batch description).
 __host__ __device__ inline void grid_struct(GmpStruct& st, const unsigned long long* bbox, GmpGrid& g,
                                             double cutoff) {
+  // half a cutoff wide, along axis 0, which the neighbor search takes a row at
+  // a time, a quarter (a row's ends overshoot the sphere's chord by a bin)
   double umax[3], ext[3];
   for (int k = 0; k < 3; ++k) {
     if (st.periodic[k]) {
       g.umin[k] = 0.0;
       umax[k] = 1.0;
       ext[k] = 1.0;
-      double target = 0.5 * st.reach[k];
+      double target = (k == 0 ? 0.25 : 0.5) * st.reach[k];
       double nbf = target > 0.0 ? floor(1.0 / target) : 1.0;
       g.nb[k] = (int)fmin(fmax(nbf, 1.0), 1024.0);
       g.binw[k] = 1.0 / g.nb[k];
@@ -193,7 +195,7 @@ __host__ __device__ inline void grid_struct(GmpStruct& st, const unsigned long l
       g.umin[k] = lo;
       umax[k] = hi;
       ext[k] = hi - lo;
-      g.binw[k] = fmax(0.5 * st.reach[k], 1e-12);
+      g.binw[k] = fmax((k == 0 ? 0.25 : 0.5) * st.reach[k], 1e-12);
       double nbf = floor(ext[k] / g.binw[k]) + 1.0;
       g.nb[k] = (int)fmin(fmax(nbf, 1.0), 1024.0);
       if (g.nb[k] == 1024) g.binw[k] = fmax(ext[k] / 1023.0, g.binw[k]);
@@ -649,12 +651,12 @@ __device__ __forceinline__ bool out_of_range(const int* n) {
   return abs(n[0]) >= 512 || abs(n[1]) >= 512 || abs(n[2]) >= 512;
 }
 
-// Per-warp shared memory: 32 bin segments (float4 + int2); in the fill
-// passes also keys [max_keys] u64, species of each key [max_keys] u16
-// (FILL 1), per-species counters [n_el] int.
-constexpr size_t kSegBytes = 32 * (sizeof(float4) + sizeof(int2));
+// Per-warp shared memory: 32 bin segments (float4 + int); in the fill
+// passes also keys [max_keys] u64, species and rank of each key
+// [max_keys] u32 (FILL 1), per-species counters [n_el] int.
+constexpr size_t kSegBytes = 32 * (sizeof(float4) + sizeof(int));
 __host__ __device__ inline size_t fill_warp_bytes(int max_keys, int n_el) {
-  return kSegBytes + ((size_t)max_keys * 10 + (size_t)n_el * 4 + 15) / 16 * 16;
+  return kSegBytes + ((size_t)max_keys * 12 + (size_t)n_el * 4 + 15) / 16 * 16;
 }
 
 // Warp per center.  The center's cutoff sphere is covered by segments: the
@@ -664,16 +666,18 @@ __host__ __device__ inline size_t fill_warp_bytes(int max_keys, int n_el) {
 // orthogonal axes the row is cut to the sphere's chord (bounds on the
 // distance between planes, with a slack of kSlack bins that covers the FP32
 // rounding of t; the test of each candidate is exact, so the bounds only have
-// to keep every neighbor).  Then groups of 8 lanes walk the segments that
-// are not empty, 4 at a time: consecutive lanes read consecutive slots.
+// to keep every neighbor).  The slots of the segments that are not empty are
+// then numbered through and taken 32 at a time, a lane's segment found from a
+// bit mask of the segments that start among the 32: every lane has a
+// candidate, and consecutive lanes read consecutive slots.
 // An accepted candidate is kept as (slot, image) and completed afterwards,
 // with all lanes busy; a row costs two bin offsets instead of two per bin.
 // Bound by instruction issue (64%) and the loads' latency; 64 registers, 32
 // resident warps per SM (a few words spilled; 80 registers and 24 warps:
-// 147 us on the slab of 32,768 atoms, 130 at 64).  Against one bin per lane,
-// its slots in turn, and general double-float sums in the records (GB300):
-// neighbor stage of 2,500 small structures 946 -> 634 us, alloy slab of
-// 262,144 atoms 1774 -> 1087 us.
+// 147 us on the slab of 32,768 atoms, 130 at 64).  Neighbor stage of 2,500 small
+// structures / of the alloy slab of 262,144 atoms (GB300): 946 / 1774 us with
+// one bin per lane, its slots in turn; 562 / 1004 with groups of 8 lanes walking
+// the segments, 4 at a time; 508 / 900 now.
 // FILL = 0: count exact neighbors; FILL = 1: write the
 // pair records grouped by neighbor species, in enumeration order within a
 // species (segments in a fixed order, atoms in index order within a bin:
@@ -699,10 +703,11 @@ __global__ void __launch_bounds__(128, 8) k_neighbors(const GmpStruct* __restric
   const int64_t i = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib;
   if (i >= N) return;
   unsigned char* wbase = sh_fill + (size_t)wib * (fill ? fill_warp_bytes(max_keys, n_el) : kSegBytes);
-  float4* seg_sh = reinterpret_cast<float4*>(wbase);          // image shift of the segment, first slot
-  int2* seg_cm = reinterpret_cast<int2*>(seg_sh + 32);        // slots, packed image (m0, m1, m2)
+  float4* seg_sh = reinterpret_cast<float4*>(wbase);          // image shift of the segment, slot of candidate 0
+  int* seg_m = reinterpret_cast<int*>(seg_sh + 32);           // packed image (m0, m1, m2)
+  const unsigned below = (1u << lane) - 1u;
   int2* keys = reinterpret_cast<int2*>(wbase + kSegBytes);    // accepted: slot, packed image (m0, m1, m2)
-  uint16_t* kel = reinterpret_cast<uint16_t*>(keys + max_keys);
+  uint32_t* kel = reinterpret_cast<uint32_t*>(keys + max_keys);
   int* ecnt = reinterpret_cast<int*>(kel + max_keys);  // max_keys: a power of 2 >= 32
 
   const int s = C.sid[i];
@@ -780,61 +785,69 @@ __global__ void __launch_bounds__(128, 8) k_neighbors(const GmpStruct* __restric
           }
         }
       }
+      // the candidates of the segments that are not empty, numbered through:
+      // lane's segment starts at candidate `start`
+      int incl = cm.x;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+      }
+      const int start = incl - cm.x, n_cand = __shfl_sync(0xffffffffu, incl, 31);
       const unsigned some = __ballot_sync(0xffffffffu, cm.x > 0);
-      const int nseg = __popc(some);
       if (cm.x > 0) {
-        const int at = __popc(some & ((1u << lane) - 1u));
+        const int at = __popc(some & below);
+        sg.w = __int_as_float(__float_as_int(sg.w) - start);
         seg_sh[at] = sg;
-        seg_cm[at] = cm;
+        seg_m[at] = cm.y;
       }
       __syncwarp();
-      for (int q0 = 0; q0 < nseg; q0 += 4) {
-        const int q = q0 + (lane >> 3);
-        float4 sh = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        int2 c = make_int2(0, 0);
-        if (q < nseg) {
-          sh = seg_sh[q];
-          c = seg_cm[q];
-        }
-        const int len = __reduce_max_sync(0xffffffffu, c.x);
-        for (int u = lane & 7; u - (lane & 7) < len; u += 8) {
-          const int slot = __float_as_int(sh.w) + u;
-          bool acc = false;
-          if (u < c.x) {
-            const float4 yj = bin_y[slot];
-            const float dx = (yj.x - yi.x) + sh.x;
-            const float dy = (yj.y - yi.y) + sh.y;
-            const float dz = (yj.z - yi.z) + sh.z;
-            // three roundings of non-negative terms: within 3 x 2^-24 relative
-            const float r2 = __fmaf_rn(dx, dx, __fmaf_rn(dy, dy, __fmul_rn(dz, dz)));
-            acc = r2 <= p2;
-            // the image index is needed for the boundary shell's exact
-            // decision, and in the count pass (whose caller reports it) for
-            // its range
-            if (acc && (!fill || r2 >= q2)) {
-              int wj[3], m[3];
-              gmp_unpack_shift(__float_as_int(yj.w), wj);
-              gmp_unpack_shift(c.y, m);
-              const int n[3] = {m[0] + wi[0] - wj[0], m[1] + wi[1] - wj[1], m[2] + wi[2] - wj[2]};
-              if (r2 >= q2) {
-                const int64_t j = bin_je[slot].x;
-                const float4 xhj = atom_xh[j], xlj = atom_xl[j];
-                acc = exact_accept(pos, xi, j, xhi, xli, xhj, xlj, st, n, rc2hi, rc2lo, rc2, cutoff);
-              }
-              if (!fill && acc && out_of_range(n)) {
-                atomicOr(err, GMP_DEV_SHIFT_RANGE);  // reported after the count pass
-                acc = false;
-              }
+      int q0 = -1;  // segments that start before candidate c0, less one
+      for (int c0 = 0; c0 < n_cand; c0 += 32) {
+        // bit b: a segment starts at candidate c0 + b
+        const unsigned heads = __reduce_or_sync(0xffffffffu, cm.x > 0 && (unsigned)(start - c0) < 32u ? 1u << (start - c0) : 0u);
+        const int q = q0 + __popc(heads & (below << 1 | 1u));
+        q0 += __popc(heads);
+        const int cand = c0 + lane;
+        int slot = 0, cy = 0;
+        bool acc = false;
+        if (cand < n_cand) {
+          const float4 sh = seg_sh[q];
+          cy = seg_m[q];
+          slot = __float_as_int(sh.w) + cand;
+          const float4 yj = bin_y[slot];
+          const float dx = (yj.x - yi.x) + sh.x;
+          const float dy = (yj.y - yi.y) + sh.y;
+          const float dz = (yj.z - yi.z) + sh.z;
+          // three roundings of non-negative terms: within 3 x 2^-24 relative
+          const float r2 = __fmaf_rn(dx, dx, __fmaf_rn(dy, dy, __fmul_rn(dz, dz)));
+          acc = r2 <= p2;
+          // the image index is needed for the boundary shell's exact
+          // decision, and in the count pass (whose caller reports it) for
+          // its range
+          if (acc && (!fill || r2 >= q2)) {
+            int wj[3], m[3];
+            gmp_unpack_shift(__float_as_int(yj.w), wj);
+            gmp_unpack_shift(cy, m);
+            const int n[3] = {m[0] + wi[0] - wj[0], m[1] + wi[1] - wj[1], m[2] + wi[2] - wj[2]};
+            if (r2 >= q2) {
+              const int64_t j = bin_je[slot].x;
+              const float4 xhj = atom_xh[j], xlj = atom_xl[j];
+              acc = exact_accept(pos, xi, j, xhi, xli, xhj, xlj, st, n, rc2hi, rc2lo, rc2, cutoff);
+            }
+            if (!fill && acc && out_of_range(n)) {
+              atomicOr(err, GMP_DEV_SHIFT_RANGE);  // reported after the count pass
+              acc = false;
             }
           }
-          if (!fill) {
-            count += acc ? 1 : 0;
-          } else {
-            const unsigned mask = __ballot_sync(0xffffffffu, acc);
-            const int slot_k = count + __popc(mask & ((1u << lane) - 1u));
-            if (acc && slot_k < max_keys) keys[slot_k] = make_int2(slot, c.y);
-            count += __popc(mask);
-          }
+        }
+        if (!fill) {
+          count += acc ? 1 : 0;
+        } else {
+          const unsigned mask = __ballot_sync(0xffffffffu, acc);
+          const int slot_k = count + __popc(mask & below);
+          if (acc && slot_k < max_keys) keys[slot_k] = make_int2(slot, cy);
+          count += __popc(mask);
         }
       }
       __syncwarp();
@@ -923,18 +936,29 @@ __global__ void __launch_bounds__(128, 8) k_neighbors(const GmpStruct* __restric
   const bool by_species = fill == 1 && n_el > 1;
   if (by_species) {
     // destination of key t: species-major, enumeration order within a
-    // species (counting sort; lanes of one match group have one species)
+    // species (counting sort; lanes of one match group have one species).
+    // The key's rank within its species is kept with the species, and its
+    // slot makes way for its atom (neither exceeds 16 bits: max_keys records
+    // fit the shared memory).
     for (int e = lane; e < n_el; e += 32) ecnt[e] = 0;
     __syncwarp();
     for (int t0 = 0; t0 < M; t0 += 32) {
       const int t = t0 + lane;
       int e = -1;
       if (t < M) {
-        e = bin_je[keys[t].x].y;
-        kel[t] = (uint16_t)e;
+        const int2 je = bin_je[keys[t].x];
+        e = je.y;
+        keys[t].x = je.x;
       }
       const unsigned grp = __match_any_sync(0xffffffffu, e);
-      if (t < M && lane == __ffs(grp) - 1) ecnt[e] += __popc(grp);
+      const int rank = __popc(grp & ((1u << lane) - 1u));
+      int before = 0;
+      if (t < M) {
+        before = ecnt[e];
+        kel[t] = (uint32_t)e << 16 | (uint32_t)(before + rank);
+      }
+      __syncwarp();
+      if (t < M && rank == 0) ecnt[e] = before + __popc(grp);
       __syncwarp();
     }
     // exclusive prefix over the species
@@ -954,18 +978,9 @@ __global__ void __launch_bounds__(128, 8) k_neighbors(const GmpStruct* __restric
     __syncwarp();
   }
   // records: the double-float displacement, rounded to FP32
-  for (int t0 = 0; t0 < M; t0 += 32) {
-    const int t = t0 + lane;
+  for (int t = lane; t < M; t += 32) {
     int dst = t;
-    if (by_species) {
-      const int e = t < M ? (int)kel[t] : -1;
-      const unsigned grp = __match_any_sync(0xffffffffu, e);
-      if (t < M) dst = ecnt[e] + __popc(grp & ((1u << lane) - 1u));
-      __syncwarp();
-      if (t < M && lane == __ffs(grp) - 1) ecnt[e] += __popc(grp);
-      __syncwarp();
-    }
-    if (t >= M) continue;
+    if (by_species) dst = ecnt[kel[t] >> 16] + (int)(kel[t] & 0xffffu);
     int64_t j;
     int n[3];
     float4 xhj, xlj;
@@ -977,7 +992,7 @@ __global__ void __launch_bounds__(128, 8) k_neighbors(const GmpStruct* __restric
       xlj = atom_xl[j];
     } else {
       const int2 k = keys[t];
-      j = bin_je[k.x].x;
+      j = by_species ? k.x : bin_je[k.x].x;
       xhj = atom_xh[j];
       xlj = atom_xl[j];
       image(k.y, __float_as_int(xlj.w), n);

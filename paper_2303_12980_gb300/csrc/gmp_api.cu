@@ -108,6 +108,7 @@ struct gmp_ctx {
   size_t h_desc_bytes = 0;
   cudaEvent_t ev_desc = nullptr;    // the copy is done with the staging
   GmpGridMode grid_mode = GmpGridMode::kGiven;
+  int max_atoms = 0, max_bins = 0;  // of one structure of the batch
   DevBuf struct_of, bbox, atom_xh, atom_xl, atom_u, atom_bin, atom_t, atom_y;
   DevBuf bin_count, bin_cursor, bin_start, bin_y, bin_je, counts, nbr_off, scan_tmp, pairs;
   // error word, longest list, pair cursor, refinement queue counts and the
@@ -327,6 +328,7 @@ gmp_status upload_structures(gmp_ctx* h, int32_t S, const int64_t* atom_off, con
   GmpGrid* const grids = reinterpret_cast<GmpGrid*>(static_cast<char*>(h->h_desc) + o_grid);
   GmpGridMode mode = GmpGridMode::kGiven;
   int64_t bin_base = 0;
+  int max_atoms = 0, max_bins = 0;
   for (int s = 0; s < S; ++s) {
     GmpStruct& g = info[s];
     std::memset(&g, 0, sizeof(g));
@@ -366,11 +368,15 @@ gmp_status upload_structures(gmp_ctx* h, int32_t S, const int64_t* atom_off, con
     g.bin_cap = 2 * g.n_atoms + 8;
     gmp_periodic_grid(g, grids[s], h->cutoff);
     bin_base += g.bin_cap;
+    max_atoms = std::max(max_atoms, g.n_atoms);
+    max_bins = std::max(max_bins, g.bin_cap);
     if (!(g.periodic[0] && g.periodic[1] && g.periodic[2])) mode = GmpGridMode::kOpen;
   }
   std::memcpy(static_cast<char*>(h->h_desc) + o_off, atom_off, sizeof(int64_t) * (S + 1));
   h->n_bins = bin_base;
   h->grid_mode = mode;
+  h->max_atoms = max_atoms;
+  h->max_bins = max_bins;
   GMP_CK(h->desc.ensure(bytes), "structs");
   h->structs.p = h->desc.p;
   h->grid.p = h->desc.as<char>() + o_grid;
@@ -379,7 +385,8 @@ gmp_status upload_structures(gmp_ctx* h, int32_t S, const int64_t* atom_off, con
   GMP_CK(h->struct_of.ensure(sizeof(int32_t) * (N > 0 ? N : 1)), "struct_of");
   GMP_CK(cudaMemcpyAsync(h->desc.p, h->h_desc, bytes, cudaMemcpyHostToDevice, st), "upload structs");
   GMP_CK(cudaEventRecord(h->ev_desc, st), "event");
-  if (N > 0) GMP_CK(gmp_launch_struct_of(h->atom_off.as<int64_t>(), S, h->struct_of.as<int32_t>(), st, &h->launches), "struct_of");
+  if (N > 0 && !gmp_bin_structs_fits(N, max_atoms, max_bins))  // (that kernel writes it, on each call)
+    GMP_CK(gmp_launch_struct_of(h->atom_off.as<int64_t>(), S, h->struct_of.as<int32_t>(), st, &h->launches), "struct_of");
   ++h->struct_gen;
   h->last_off.assign(atom_off, atom_off + S + 1);
   h->last_cell.assign(cell, cell + 9 * S);
@@ -442,13 +449,13 @@ gmp_status bin_atoms(gmp_ctx* h, int32_t S, const double* pos, const int32_t* sp
   constexpr int n_clear = (int)(kScalarBytes / 4) - 1;
   h->next_counter = 0;
 
-  if (gmp_bin_small_fits(N, h->n_bins, S)) {
-    GMP_CK(gmp_launch_bin_small(h->structs.as<GmpStruct>(), S, h->struct_of.as<int32_t>(), N, h->cutoff, pos, species,
-                                h->n_el, h->grid.as<GmpGrid>(), h->n_bins, h->atom_xh.as<float4>(),
-                                h->atom_xl.as<float4>(), h->atom_u.as<GmpD4>(), h->atom_bin.as<int32_t>(),
-                                h->bin_start.as<int32_t>(), h->bin_y.as<float4>(), h->bin_je.as<int2>(),
-                                h->atom_t.as<float4>(), h->atom_y.as<float4>(), d_err, n_clear, st, L),
-           "bins (one block)");
+  if (gmp_bin_structs_fits(N, h->max_atoms, h->max_bins)) {
+    GMP_CK(gmp_launch_bin_structs(h->structs.as<GmpStruct>(), S, N, h->max_atoms, h->max_bins, h->cutoff, pos, species,
+                                  h->n_el, h->grid.as<GmpGrid>(), h->struct_of.as<int32_t>(),
+                                  h->atom_xh.as<float4>(), h->atom_xl.as<float4>(), h->bin_start.as<int32_t>(),
+                                  h->bin_y.as<float4>(), h->bin_je.as<int2>(), h->atom_t.as<float4>(),
+                                  h->atom_y.as<float4>(), d_err, n_clear, st, h->sm_count, L),
+           "bins (a block per structure)");
     return GMP_OK;
   }
   GMP_CK(gmp_launch_neighbors_prepare(h->structs.as<GmpStruct>(), S, h->struct_of.as<int32_t>(), N, h->cutoff,

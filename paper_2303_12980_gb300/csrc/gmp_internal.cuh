@@ -40,8 +40,7 @@ struct GmpStruct {
 // Per-structure bin grid (device-built from bounding boxes).
 struct GmpGrid {
   double umin[3];     // fractional coordinate of bin 0 edge
-  double binw[3];     // bin width (fractional)
-  double inv_binw[3]; // 1 / binw
+  double inv_binw[3]; // 1 / the bin width (fractional)
   int nb[3];          // bins per axis
   int ortho;          // the cell's axes are orthogonal (up to rounding)
   // for the neighbor search, in FP32: the cutoff in bins, the distance
@@ -395,24 +394,18 @@ __device__ __forceinline__ void gmp_df_disp(const float4& xhi, const float4& xli
 struct GmpWorkspace;
 
 // Launchers implemented in the .cu files (all asynchronous on `stream`).
-// Binning of a small batch (at most kSmallBinAtoms atoms, 256 structures)
-// in one launch of one CTA: the outputs of gmp_launch_neighbors_prepare +
-// gmp_launch_bins (atom_xh/xl/u/bin/t/y, grid, pre-screen bounds,
-// bin_start/bin_y/bin_je), bit for bit.  gmp_bin_small_fits says whether
-// a batch qualifies (shared memory for its bins and slots).
-// One SM runs the batch's FP64 set-up (GB300: 1/64 of the FP32 rate), so
-// the single CTA wins only for small batches: on a GB300, 64 atoms took
-// 0.054 ms against 0.088 for the multi-kernel path, 4096 atoms 0.34 against
-// 0.17.
-constexpr int64_t kSmallBinAtoms = 1024;
-bool gmp_bin_small_fits(int64_t N, int64_t n_bins, int n_struct);
-cudaError_t gmp_launch_bin_small(GmpStruct* d_structs, int n_struct, const int32_t* d_struct_of, int64_t N,
-                                 double cutoff, const double* pos, const int32_t* species, int n_el,
-                                 GmpGrid* d_grid, int64_t n_bins, float4* atom_xh, float4* atom_xl, GmpD4* atom_u,
-                                 int32_t* atom_bin, int32_t* bin_start, float4* bin_y, int2* bin_je,
-                                 float4* atom_t, float4* atom_y, uint32_t* d_err, int n_clear, cudaStream_t stream,
-                                 int64_t* launches);
-// n_clear words behind *d_err are cleared (gmp_launch_bin_small too).
+// Binning of a batch of small structures (N atoms; none of more than max_atoms
+// atoms or max_bins bins) in one launch: the outputs of
+// gmp_launch_neighbors_prepare + gmp_launch_bins that later kernels read
+// (atom_xh/xl/t/y, grid, pre-screen bounds, bin_start/bin_y/bin_je), bit for
+// bit, and struct_of.  gmp_bin_structs_fits says whether a batch qualifies.
+bool gmp_bin_structs_fits(int64_t N, int max_atoms, int max_bins);
+cudaError_t gmp_launch_bin_structs(GmpStruct* d_structs, int n_struct, int64_t N, int max_atoms, int max_bins,
+                                   double cutoff, const double* pos, const int32_t* species, int n_el, GmpGrid* d_grid,
+                                   int32_t* d_struct_of, float4* atom_xh, float4* atom_xl, int32_t* bin_start,
+                                   float4* bin_y, int2* bin_je, float4* atom_t, float4* atom_y, uint32_t* d_err,
+                                   int n_clear, cudaStream_t stream, int sm_count, int64_t* launches);
+// n_clear words behind *d_err are cleared (gmp_launch_bin_structs too).
 // Where the structures' bin grids come from: given (uploaded with the batch
 // description: every structure is periodic along all axes, gmp_periodic_grid),
 // from the atoms' range for the structures with a non-periodic axis (the

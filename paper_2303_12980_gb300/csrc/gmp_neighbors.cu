@@ -109,19 +109,22 @@ __device__ inline int wrap_axis(double& u, double f0, uint32_t* err) {
   return w;
 }
 
-// (The first kernel of a call also clears the n_clear words behind the error
-// word: counters and sizes of the call, which later kernels use.)
-// Per atom: checks, fractional coordinates, wrap, double-float split, bbox.
-// bbox (6 keys per structure: min and complemented max of each
-// non-periodic fractional axis) may be global or shared memory.
-__device__ __forceinline__ void prepare_atom(const GmpStruct* S, const int32_t* __restrict__ struct_of, int64_t a,
-                                             const double* __restrict__ pos, const int32_t* __restrict__ species,
-                                             int n_el, float4* __restrict__ atom_xh, float4* __restrict__ atom_xl,
-                                             GmpD4* __restrict__ atom_u, unsigned long long* bbox,
-                                             uint32_t* __restrict__ err) {
-  const int s = struct_of[a];
-  const GmpStruct& st = S[s];
-  double x[3] = {pos[3 * a], pos[3 * a + 1], pos[3 * a + 2]};
+// The double-float split of a position, with the species and the packed wrap.
+__device__ __forceinline__ void write_split(int64_t a, const double (&x)[3], int e, const int (&w)[3], float4* xh,
+                                            float4* xl) {
+  float h[3], l[3];
+  for (int k = 0; k < 3; ++k) {
+    h[k] = (float)x[k];
+    l[k] = (float)(x[k] - (double)h[k]);
+  }
+  xh[a] = make_float4(h[0], h[1], h[2], __int_as_float(e));
+  xl[a] = make_float4(l[0], l[1], l[2], __int_as_float(pack_wrap(w[0], w[1], w[2])));
+}
+
+// Position and species of atom a, checked (flagged ones are replaced).
+__device__ __forceinline__ int load_atom(int64_t a, const double* __restrict__ pos, const int32_t* __restrict__ species,
+                                         int n_el, double (&x)[3], uint32_t* __restrict__ err) {
+  for (int k = 0; k < 3; ++k) x[k] = pos[3 * a + k];
   int e = species[a];
   if (e < 0 || e >= n_el) {
     atomicOr(err, GMP_DEV_BAD_SPECIES);
@@ -131,6 +134,21 @@ __device__ __forceinline__ void prepare_atom(const GmpStruct* S, const int32_t* 
     atomicOr(err, GMP_DEV_NONFINITE);
     x[0] = x[1] = x[2] = 0.0;
   }
+  return e;
+}
+
+// Per atom: checks, fractional coordinates, wrap, double-float split, bbox.
+// bbox: 6 keys per structure (min and complemented max of each non-periodic
+// fractional axis).
+__device__ __forceinline__ void prepare_atom(const GmpStruct* S, const int32_t* __restrict__ struct_of, int64_t a,
+                                             const double* __restrict__ pos, const int32_t* __restrict__ species,
+                                             int n_el, float4* __restrict__ atom_xh, float4* __restrict__ atom_xl,
+                                             GmpD4* __restrict__ atom_u, unsigned long long* bbox,
+                                             uint32_t* __restrict__ err) {
+  const int s = struct_of[a];
+  const GmpStruct& st = S[s];
+  double x[3];
+  const int e = load_atom(a, pos, species, n_el, x, err);
   double u[3], f0[3];
   int w[3] = {0, 0, 0};
   struct_ref_cell(st, pos, f0);
@@ -144,16 +162,12 @@ __device__ __forceinline__ void prepare_atom(const GmpStruct* S, const int32_t* 
       atomicMin(&bbox[6 * s + 2 * k + 1], ~order_key(u[k]));
     }
   }
-  float h[3], l[3];
-  for (int k = 0; k < 3; ++k) {
-    h[k] = (float)x[k];
-    l[k] = (float)(x[k] - (double)h[k]);
-  }
-  atom_xh[a] = make_float4(h[0], h[1], h[2], __int_as_float(e));
-  atom_xl[a] = make_float4(l[0], l[1], l[2], __int_as_float(pack_wrap(w[0], w[1], w[2])));
+  write_split(a, x, e, w, atom_xh, atom_xl);
   atom_u[a] = GmpD4{u[0], u[1], u[2], 0.0};
 }
 
+// (The first kernel of a call also clears the n_clear words behind the error
+// word: counters and sizes of the call, which later kernels use.)
 __global__ void k_prepare(const GmpStruct* __restrict__ S, const int32_t* __restrict__ struct_of,
                           int64_t N, const double* __restrict__ pos,
                           const int32_t* __restrict__ species, int n_el,
@@ -175,30 +189,38 @@ __global__ void k_prepare(const GmpStruct* __restrict__ S, const int32_t* __rest
 // Bin grid and FP32 pre-screen bound of one structure.  bbox: its 6 keys,
 // read for non-periodic axes only (a fully periodic structure's grid follows
 // from its cell and is made on the host, with the batch description).
+// The bins are half a cutoff wide, along axis 0, which the neighbor search
+// takes a row at a time, a quarter (a row's ends overshoot the sphere's chord
+// by a bin: 508 against 512 us for the neighbor stage of 2,500 small
+// structures, 45 against 47 of a 4,096-atom crystal).  One thread runs this
+// for a structure, at 1/64 of the FP32 rate in FP64: one division an axis, and
+// the bounds, which carry a margin, in FP32.
 __host__ __device__ inline void grid_struct(GmpStruct& st, const unsigned long long* bbox, GmpGrid& g,
                                             double cutoff) {
-  // half a cutoff wide, along axis 0, which the neighbor search takes a row at
-  // a time, a quarter (a row's ends overshoot the sphere's chord by a bin)
-  double umax[3], ext[3];
+  double w[3], ext[3];
+  float uk[3];  // bound on the fractional coordinates
   for (int k = 0; k < 3; ++k) {
+    const double target = (k == 0 ? 0.25 : 0.5) * st.reach[k];
     if (st.periodic[k]) {
       g.umin[k] = 0.0;
-      umax[k] = 1.0;
-      ext[k] = 1.0;
-      double target = (k == 0 ? 0.25 : 0.5) * st.reach[k];
-      double nbf = target > 0.0 ? floor(1.0 / target) : 1.0;
+      ext[k] = w[k] = 1.0;
+      const double nbf = target > 0.0 ? floor(1.0 / target) : 1.0;
       g.nb[k] = (int)fmin(fmax(nbf, 1.0), 1024.0);
-      g.binw[k] = 1.0 / g.nb[k];
+      g.inv_binw[k] = g.nb[k];
+      uk[k] = 2.0f;
     } else {
-      double lo = st.n_atoms ? key_to_double(bbox[2 * k]) : 0.0;
-      double hi = st.n_atoms ? key_to_double(~bbox[2 * k + 1]) : 0.0;
+      const double lo = st.n_atoms ? key_to_double(bbox[2 * k]) : 0.0;
+      const double hi = st.n_atoms ? key_to_double(~bbox[2 * k + 1]) : 0.0;
       g.umin[k] = lo;
-      umax[k] = hi;
       ext[k] = hi - lo;
-      g.binw[k] = fmax((k == 0 ? 0.25 : 0.5) * st.reach[k], 1e-12);
-      double nbf = floor(ext[k] / g.binw[k]) + 1.0;
-      g.nb[k] = (int)fmin(fmax(nbf, 1.0), 1024.0);
-      if (g.nb[k] == 1024) g.binw[k] = fmax(ext[k] / 1023.0, g.binw[k]);
+      w[k] = fmax(target, 1e-12);
+      g.inv_binw[k] = 1.0 / w[k];
+      g.nb[k] = (int)fmin(floor(ext[k] * g.inv_binw[k]) + 1.0, 1024.0);
+      if (g.nb[k] == 1024) {
+        w[k] = fmax(ext[k] / 1023.0, w[k]);
+        g.inv_binw[k] = 1.0 / w[k];
+      }
+      uk[k] = fmaxf(fabsf((float)lo), fabsf((float)hi)) + 1.0f;
     }
   }
   // keep the grid within the reserved bin slots
@@ -208,10 +230,11 @@ __host__ __device__ inline void grid_struct(GmpStruct& st, const unsigned long l
     if (g.nb[2] > g.nb[k]) k = 2;
     if (st.periodic[k]) {
       g.nb[k] = (g.nb[k] + 1) / 2;
-      g.binw[k] = 1.0 / g.nb[k];
+      g.inv_binw[k] = g.nb[k];
     } else {
-      g.binw[k] *= 2.0;
-      g.nb[k] = (int)fmin(floor(ext[k] / g.binw[k]) + 1.0, 1024.0);
+      w[k] *= 2.0;
+      g.inv_binw[k] *= 0.5;
+      g.nb[k] = (int)fmin(floor(ext[k] * g.inv_binw[k]) + 1.0, 1024.0);
     }
   }
   // Rigorous two-sided FP32 bounds.  Wrapped Cartesian coordinates are
@@ -227,40 +250,46 @@ __host__ __device__ inline void grid_struct(GmpStruct& st, const unsigned long l
   // Centers need not be atoms (reference points): along a non-periodic axis
   // a center scans some bin only if its coordinate lies within reach + one
   // bin width of the atoms' range, which the bound on |y| covers.
-  double Y = 0.0, Sh = 0.0;
-  for (int c = 0; c < 3; ++c) {
-    double yc = 0.0, sc = 0.0;
-    for (int k = 0; k < 3; ++k) {
-      double a = fabs(st.A[3 * k + c]);
-      double uk = fmax(fabs(g.umin[k]), fabs(umax[k])) + 1.0 +
-                  (st.periodic[k] ? 0.0 : st.reach[k] + 2.0 * g.binw[k]);
-      yc += uk * a;
-      sc += (ceil(st.reach[k]) + 2.0) * a;
-    }
-    Y = fmax(Y, yc);
-    Sh = fmax(Sh, sc);
+  // (FP32 sums of at most 10 roundings, a relative 2^-20 at most; coordinates
+  // beyond FP32's range leave everything to the exact test.)
+  float sk[3], Y = 0.0f, Sh = 0.0f;
+  for (int k = 0; k < 3; ++k) {
+    const float r = (float)st.reach[k] * 1.000001f;
+    uk[k] = fminf(uk[k] + (st.periodic[k] ? 0.0f : r + 2.0f * (float)w[k]), 1e30f);
+    sk[k] = ceilf(r) + 2.0f;
   }
-  double delta = ldexp(Y + Sh + cutoff, -21);
+  for (int c = 0; c < 3; ++c) {
+    float yc = 0.0f, sc = 0.0f;
+    for (int k = 0; k < 3; ++k) {
+      const float a = fabsf(st.Ahi[3 * k + c]);
+      yc += uk[k] * a;
+      sc += sk[k] * a;
+    }
+    Y = fmaxf(Y, yc);
+    Sh = fmaxf(Sh, sc);
+  }
+  const double delta = (double)((Y + Sh + (float)cutoff) * 1.00001f) * 0x1p-21;
   double b = (cutoff + 2.0 * delta);
   g.ortho = 1;
-  double bk[3];  // |b_k|^2, b_k = column k of Ainv
-  for (int k = 0; k < 3; ++k) bk[k] = st.Ainv[k] * st.Ainv[k] + st.Ainv[3 + k] * st.Ainv[3 + k] + st.Ainv[6 + k] * st.Ainv[6 + k];
-  for (int k = 0; k < 3; ++k) {
-    const int m = k == 2 ? 0 : k + 1;
-    const double d = st.Ainv[k] * st.Ainv[m] + st.Ainv[3 + k] * st.Ainv[3 + m] + st.Ainv[6 + k] * st.Ainv[6 + m];
-    if (!(d * d <= 1e-18 * bk[k] * bk[m])) g.ortho = 0;
+  if (!st.diag) {
+    double bk[3];  // |b_k|^2, b_k = column k of Ainv
+    for (int k = 0; k < 3; ++k) bk[k] = st.Ainv[k] * st.Ainv[k] + st.Ainv[3 + k] * st.Ainv[3 + k] + st.Ainv[6 + k] * st.Ainv[6 + k];
+    for (int k = 0; k < 3; ++k) {
+      const int m = k == 2 ? 0 : k + 1;
+      const double d = st.Ainv[k] * st.Ainv[m] + st.Ainv[3 + k] * st.Ainv[3 + m] + st.Ainv[6 + k] * st.Ainv[6 + m];
+      if (!(d * d <= 1e-18 * bk[k] * bk[m])) g.ortho = 0;
+    }
   }
   for (int k = 0; k < 3; ++k) {
-    g.inv_binw[k] = 1.0 / g.binw[k];
     g.rb[k] = (float)(st.reach[k] * g.inv_binw[k]);
-    g.h[k] = (float)(cutoff / (st.reach[k] * g.inv_binw[k]));
+    g.h[k] = (float)cutoff / g.rb[k];
   }
   g.inv_h0 = g.rb[0] / (float)cutoff;
   g.pad = 0.0f;
-  float p2 = (float)(b * b * (1.0 + ldexp(1.0, -20)));
+  float p2 = (float)(b * b * (1.0 + 0x1p-20));
   st.prescreen2 = nextafterf(p2, INFINITY);
   const double bi = fmax(cutoff - 2.0 * delta, 0.0);
-  float q2 = (float)(bi * bi * (1.0 - ldexp(1.0, -20)));
+  float q2 = (float)(bi * bi * (1.0 - 0x1p-20));
   st.inside2 = fmaxf(nextafterf(q2, 0.0f), 0.0f);
 }
 
@@ -281,17 +310,15 @@ __global__ void k_grid(GmpStruct* __restrict__ S, int n_struct,
   G[s] = g;
 }
 
-// Bin of an atom at wrapped fractional coordinates u4 in structure s.
-__device__ __forceinline__ int32_t bin_of(const GmpStruct* S, const GmpGrid* G, int s, const GmpD4& u4) {
-  const GmpGrid& g = G[s];
-  const double u[3] = {u4.x, u4.y, u4.z};
+// Bin, in its structure's grid, of an atom at wrapped fractional coordinates u.
+__device__ __forceinline__ int64_t bin_of(const GmpGrid& g, const double* u) {
   int b[3];
   for (int k = 0; k < 3; ++k) {
     double t = floor((u[k] - g.umin[k]) * g.inv_binw[k]);  // as center_place scales
     t = fmin(fmax(t, 0.0), (double)(g.nb[k] - 1));
     b[k] = (int)t;
   }
-  return (int32_t)(S[s].bin_base + b[0] + (int64_t)g.nb[0] * (b[1] + (int64_t)g.nb[1] * b[2]));
+  return b[0] + (int64_t)g.nb[0] * (b[1] + (int64_t)g.nb[1] * b[2]);
 }
 
 // Bin slot of atom a: bin_y = (wrapped FP32 position, packed wrap of the
@@ -364,10 +391,10 @@ __global__ void k_bin_assign(const GmpStruct* __restrict__ S, const GmpGrid* __r
        a += (int64_t)gridDim.x * blockDim.x) {
     const int s = struct_of[a];
     const GmpD4 u4 = atom_u[a];
-    const int32_t bin = bin_of(S, G, s, u4);
+    const double u[3] = {u4.x, u4.y, u4.z};
+    const int32_t bin = (int32_t)(S[s].bin_base + bin_of(G[s], u));
     atom_bin[a] = bin;
     atomicAdd(&bin_count[bin], 1);
-    const double u[3] = {u4.x, u4.y, u4.z};
     center_place(S[s], G[s], u, atom_t[a], atom_y[a]);
   }
 }
@@ -397,96 +424,158 @@ __global__ void k_point_prepare(const GmpStruct* __restrict__ S, const GmpGrid* 
       u[k] = x[0] * st.Ainv[k] + x[1] * st.Ainv[3 + k] + x[2] * st.Ainv[6 + k];
       if (st.periodic[k]) w[k] = wrap_axis(u[k], f0[k], err);
     }
-    float h[3], l[3];
-    for (int k = 0; k < 3; ++k) {
-      h[k] = (float)x[k];
-      l[k] = (float)(x[k] - (double)h[k]);
-    }
-    pt_xh[a] = make_float4(h[0], h[1], h[2], 0.0f);
-    pt_xl[a] = make_float4(l[0], l[1], l[2], __int_as_float(pack_wrap(w[0], w[1], w[2])));
+    write_split(a, x, 0, w, pt_xh, pt_xl);
     center_place(st, G[s], u, pt_t[a], pt_y[a]);
   }
 }
 
-// Small batches: the whole binning (k_prepare, k_grid, k_bin_assign, the
-// scan, k_bin_scatter, k_bin_place) in one CTA, the bin counts,
-// offsets and slot lists in shared memory; same outputs as those kernels
-// (bins hold their atoms in index order).  A batch of up to about a
-// thousand atoms spends most of its multi-kernel binning time in launch and
-// tail latency, not work; past that the one SM's FP64 set-up dominates.
-// The pointers written here and read back by other threads are plain
-// (no __restrict__), so those reads see the writes after __syncthreads().
-__host__ __device__ inline size_t small_bin_smem(int64_t N, int64_t n_bins, int n_struct) {
-  return sizeof(unsigned long long) * 6 * (size_t)n_struct + sizeof(int32_t) * (size_t)(2 * n_bins + 1 + N);
+// Batches of small structures: the whole binning (k_prepare, k_grid,
+// k_bin_assign, the scan, k_bin_scatter, k_bin_place) in one launch, a CTA per
+// structure, with its coordinates, bin counts, offsets and slot lists in shared
+// memory; same outputs as those kernels (bins hold their atoms in index order).
+// A structure's atoms and bins are contiguous in the batch, so its bin offsets
+// need no scan over the others.  Small structures spend most of the
+// multi-kernel binning in launch and tail latency, not work.  Also writes
+// struct_of.  Measured on a GB300 (neighbor stage; this kernel / the several):
+// one structure of 16 atoms 22 / 27 us, of 256 28 / 28, of 512 38 / 29; 16 of
+// 512 53 / 65; 150 of 64 47 / 61; eight batches of 100 structures of 8-256
+// atoms 384 / 451.  So it takes batches whose largest structure has up to 256
+// atoms, or 512 when the batch holds at least 16 times as many (with larger
+// ones the shared memory keeps small structures from filling the chip).
+struct StructBins {
+  GmpStruct st;
+  GmpGrid g;
+  double f0[3];                // reference cell (struct_ref_cell)
+  unsigned long long bbox[6];  // as prepare_atom's
+  int32_t warp_tot[32];
+};
+__host__ __device__ inline size_t struct_bins_smem(int n_atoms, int n_bins) {
+  return sizeof(StructBins) + (3 * sizeof(double) + 2 * sizeof(int32_t)) * (size_t)n_atoms +
+         sizeof(int32_t) * (2 * (size_t)n_bins + 1);
 }
 
-__global__ void __launch_bounds__(1024) k_bin_small(GmpStruct* S, int n_struct, const int32_t* __restrict__ struct_of,
-                                                   int64_t N, double cutoff, const double* __restrict__ pos,
-                                                   const int32_t* __restrict__ species, int n_el, GmpGrid* G,
-                                                   int64_t n_bins, float4* atom_xh, float4* atom_xl, GmpD4* atom_u,
-                                                   int32_t* atom_bin, int32_t* __restrict__ bin_start,
-                                                   float4* __restrict__ bin_y, int2* __restrict__ bin_je,
-                                                   float4* __restrict__ atom_t, float4* __restrict__ atom_y,
-                                                   uint32_t* __restrict__ err, int n_clear) {
-  extern __shared__ __align__(16) unsigned char sm_small[];
-  __shared__ int32_t warp_tot[32];
-  unsigned long long* bbox = reinterpret_cast<unsigned long long*>(sm_small);
-  int32_t* cnt = reinterpret_cast<int32_t*>(bbox + 6 * n_struct);  // [n_bins] counts, then cursors
-  int32_t* start = cnt + n_bins;                                    // [n_bins + 1] exclusive offsets
-  int32_t* slot_atom = start + n_bins + 1;                          // [N] atom of each slot
+__global__ void __launch_bounds__(1024) k_bin_structs(GmpStruct* __restrict__ S, double cutoff, const double* __restrict__ pos,
+                                                     const int32_t* __restrict__ species, int n_el,
+                                                     GmpGrid* __restrict__ G, int32_t* __restrict__ struct_of,
+                                                     float4* atom_xh, float4* atom_xl, int32_t* __restrict__ bin_start,
+                                                     float4* __restrict__ bin_y, int2* __restrict__ bin_je,
+                                                     float4* __restrict__ atom_t, float4* __restrict__ atom_y,
+                                                     uint32_t* __restrict__ err, int n_clear) {
+  extern __shared__ __align__(16) unsigned char sm_bins[];
+  StructBins& B = *reinterpret_cast<StructBins*>(sm_bins);
   gmp_let_next_start();
   const int tid = (int)gmp_after_predecessor(threadIdx.x), nt = blockDim.x, lane = tid & 31, wid = tid >> 5;
-  for (int t = tid; t < n_clear; t += nt) err[1 + t] = 0;
-  for (int t = tid; t < 6 * n_struct; t += nt) bbox[t] = ~0ull;
-  for (int64_t b = tid; b < n_bins; b += nt) cnt[b] = 0;
+  const int s = blockIdx.x;
+  if (s == 0)
+    for (int t = tid; t < n_clear; t += nt) err[1 + t] = 0;
+  {
+    const int32_t* src = reinterpret_cast<const int32_t*>(S + s);
+    int32_t* dst = reinterpret_cast<int32_t*>(&B.st);
+    for (int t = tid; t < (int)(sizeof(GmpStruct) / 4); t += nt) dst[t] = src[t];
+    src = reinterpret_cast<const int32_t*>(G + s);
+    dst = reinterpret_cast<int32_t*>(&B.g);
+    for (int t = tid; t < (int)(sizeof(GmpGrid) / 4); t += nt) dst[t] = src[t];
+    if (tid < 6) B.bbox[tid] = ~0ull;
+  }
   __syncthreads();
-  for (int64_t a = tid; a < N; a += nt)
-    prepare_atom(S, struct_of, a, pos, species, n_el, atom_xh, atom_xl, atom_u, bbox, err);
+  const GmpStruct& st = B.st;
+  const int n = st.n_atoms;
+  const int64_t a0 = st.atom_base;
+  const bool open = !all_periodic(st);
+  double* const us = reinterpret_cast<double*>(sm_bins + sizeof(StructBins));  // [n][3]
+  int32_t* const slot_atom = reinterpret_cast<int32_t*>(us + 3 * (size_t)n);   // [n] atom of each slot
+  int32_t* const bin = slot_atom + n;                                          // [n]
+  if (tid == 0) {
+    double f0[3];
+    struct_ref_cell(st, pos, f0);
+    for (int k = 0; k < 3; ++k) B.f0[k] = f0[k];
+  }
   __syncthreads();
-  for (int s = tid; s < n_struct; s += nt)
-    if (!all_periodic(S[s])) grid_struct(S[s], bbox + 6 * s, G[s], cutoff);
+  for (int t0 = 0; t0 < n; t0 += nt) {
+    const int t = t0 + tid;
+    unsigned long long lo[3], hi[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) lo[k] = hi[k] = ~0ull;
+    if (t < n) {
+      double x[3];
+      const int e = load_atom(a0 + t, pos, species, n_el, x, err);
+      int w[3] = {0, 0, 0};
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        double u = x[0] * st.Ainv[k] + x[1] * st.Ainv[3 + k] + x[2] * st.Ainv[6 + k];
+        if (st.periodic[k]) {
+          w[k] = wrap_axis(u, B.f0[k], err);
+        } else {
+          lo[k] = order_key(u);
+          hi[k] = ~lo[k];
+        }
+        us[3 * t + k] = u;
+      }
+      write_split(a0 + t, x, e, w, atom_xh, atom_xl);
+      struct_of[a0 + t] = s;
+    }
+    if (open) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        if (st.periodic[k]) continue;
+        for (int o = 16; o; o >>= 1) {
+          lo[k] = min(lo[k], __shfl_xor_sync(0xffffffffu, lo[k], o));
+          hi[k] = min(hi[k], __shfl_xor_sync(0xffffffffu, hi[k], o));
+        }
+        if (lane == 0) {
+          atomicMin(&B.bbox[2 * k], lo[k]);
+          atomicMin(&B.bbox[2 * k + 1], hi[k]);
+        }
+      }
+    }
+  }
   __syncthreads();
-  for (int64_t a = tid; a < N; a += nt) {
-    const int32_t b = bin_of(S, G, struct_of[a], atom_u[a]);
-    atom_bin[a] = b;
+  if (open && tid == 0) {
+    grid_struct(B.st, B.bbox, B.g, cutoff);
+    G[s] = B.g;
+    S[s].prescreen2 = st.prescreen2;
+    S[s].inside2 = st.inside2;
+  }
+  __syncthreads();
+  const GmpGrid& g = B.g;
+  const int n_bins = g.nb[0] * g.nb[1] * g.nb[2];  // at most bin_cap
+  int32_t* const cnt = bin + n;                    // [n_bins] counts, then cursors
+  int32_t* const start = cnt + n_bins;             // [n_bins + 1] exclusive offsets
+  for (int b = tid; b < n_bins; b += nt) cnt[b] = 0;
+  __syncthreads();
+  for (int t = tid; t < n; t += nt) {
+    const int b = (int)bin_of(g, us + 3 * t);
+    bin[t] = b;
     atomicAdd(&cnt[b], 1);
   }
   __syncthreads();
   // exclusive scan of the counts: a contiguous chunk per thread, then the
   // chunk totals across the block
-  const int64_t chunk = (n_bins + nt - 1) / nt;
-  const int64_t c0 = min((int64_t)tid * chunk, n_bins), c1 = min(c0 + chunk, n_bins);
+  const int chunk = (n_bins + nt - 1) / nt;
+  const int c0 = min(tid * chunk, n_bins), c1 = min(c0 + chunk, n_bins);
   int32_t run = 0;
-  for (int64_t b = c0; b < c1; ++b) run += cnt[b];
+  for (int b = c0; b < c1; ++b) run += cnt[b];
   int32_t incl = run;
   for (int o = 1; o < 32; o <<= 1) {
     const int32_t v = __shfl_up_sync(0xffffffffu, incl, o);
     if (lane >= o) incl += v;
   }
-  if (lane == 31) warp_tot[wid] = incl;
+  if (lane == 31) B.warp_tot[wid] = incl;
   __syncthreads();
-  if (wid == 0) {
-    int32_t w = lane < (nt >> 5) ? warp_tot[lane] : 0;
-    for (int o = 1; o < 32; o <<= 1) {
-      const int32_t v = __shfl_up_sync(0xffffffffu, w, o);
-      if (lane >= o) w += v;
-    }
-    warp_tot[lane] = w;  // inclusive over warps
-  }
-  __syncthreads();
-  int32_t off = incl - run + (wid > 0 ? warp_tot[wid - 1] : 0);
-  for (int64_t b = c0; b < c1; ++b) {
+  int32_t off = incl - run;
+  for (int w = 0; w < wid; ++w) off += B.warp_tot[w];
+  for (int b = c0; b < c1; ++b) {
     const int32_t c = cnt[b];
     start[b] = off;
     cnt[b] = off;  // cursor
     off += c;
   }
-  if (tid == 0) start[n_bins] = (int32_t)N;
+  if (tid == 0) start[n_bins] = n;
   __syncthreads();
-  for (int64_t a = tid; a < N; a += nt) slot_atom[atomicAdd(&cnt[atom_bin[a]], 1)] = (int32_t)a;
+  for (int t = tid; t < n; t += nt) slot_atom[atomicAdd(&cnt[bin[t]], 1)] = t;
   __syncthreads();
   // each bin's atoms in index order (insertion sort; a bin holds few atoms)
-  for (int64_t b = tid; b < n_bins; b += nt) {
+  for (int b = tid; b < n_bins; b += nt) {
     const int b0 = start[b], b1 = start[b + 1];
     for (int t = b0 + 1; t < b1; ++t) {
       const int32_t v = slot_atom[t];
@@ -499,17 +588,16 @@ __global__ void __launch_bounds__(1024) k_bin_small(GmpStruct* S, int n_struct, 
     }
   }
   __syncthreads();
-  for (int64_t b = tid; b <= n_bins; b += nt) bin_start[b] = start[b];
-  for (int64_t t = tid; t < N; t += nt) {
-    const int64_t a = slot_atom[t];
-    const int s = struct_of[a];
-    const GmpD4 u4 = atom_u[a];
-    const double u[3] = {u4.x, u4.y, u4.z};
+  // (the last offset, n, is also the next structure's first: same value)
+  for (int b = tid; b <= n_bins; b += nt) bin_start[st.bin_base + b] = (int32_t)a0 + start[b];
+  for (int t = tid; t < n; t += nt) {
+    const int v = slot_atom[t];
+    const int64_t a = a0 + v;
     float4 place, y;
-    center_place(S[s], G[s], u, place, y);
+    center_place(st, g, us + 3 * v, place, y);
     atom_t[a] = place;
     atom_y[a] = y;
-    write_slot(a, (int32_t)t, y, atom_xh[a].w, atom_xl[a].w, bin_y, bin_je);
+    write_slot(a, (int32_t)(a0 + t), y, atom_xh[a].w, atom_xl[a].w, bin_y, bin_je);
   }
 }
 
@@ -1106,27 +1194,29 @@ cudaError_t gmp_launch_bins(const GmpStruct* d_structs, const GmpGrid* d_grid,
   return cudaGetLastError();
 }
 
-bool gmp_bin_small_fits(int64_t N, int64_t n_bins, int n_struct) {
-  return N > 0 && N <= kSmallBinAtoms && n_struct <= 256 && small_bin_smem(N, n_bins, n_struct) <= 200 * 1024;
+bool gmp_bin_structs_fits(int64_t N, int max_atoms, int max_bins) {
+  if (max_atoms > 256 && (max_atoms > 512 || N < 16 * (int64_t)max_atoms)) return false;
+  return struct_bins_smem(max_atoms, max_bins) <= 200 * 1024;
 }
 
-cudaError_t gmp_launch_bin_small(GmpStruct* d_structs, int n_struct, const int32_t* d_struct_of, int64_t N,
-                                 double cutoff, const double* pos, const int32_t* species, int n_el,
-                                 GmpGrid* d_grid, int64_t n_bins, float4* atom_xh, float4* atom_xl, GmpD4* atom_u,
-                                 int32_t* atom_bin, int32_t* bin_start, float4* bin_y, int2* bin_je,
-                                 float4* atom_t, float4* atom_y, uint32_t* d_err, int n_clear, cudaStream_t stream,
-                                 int64_t* launches) {
-  if (!gmp_bin_small_fits(N, n_bins, n_struct)) return cudaErrorInvalidValue;
-  const size_t smem = small_bin_smem(N, n_bins, n_struct);
+cudaError_t gmp_launch_bin_structs(GmpStruct* d_structs, int n_struct, int64_t N, int max_atoms, int max_bins,
+                                   double cutoff, const double* pos, const int32_t* species, int n_el, GmpGrid* d_grid,
+                                   int32_t* d_struct_of, float4* atom_xh, float4* atom_xl, int32_t* bin_start,
+                                   float4* bin_y, int2* bin_je, float4* atom_t, float4* atom_y, uint32_t* d_err,
+                                   int n_clear, cudaStream_t stream, int sm_count, int64_t* launches) {
+  if (!gmp_bin_structs_fits(N, max_atoms, max_bins)) return cudaErrorInvalidValue;
+  const size_t smem = struct_bins_smem(max_atoms, max_bins);
   if (smem > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(k_bin_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = cudaFuncSetAttribute(k_bin_structs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  // (as many threads as atoms: fewer warps to wait for at each step)
-  const int nt = (int)std::min<int64_t>(1024, std::max<int64_t>(128, (N + 31) / 32 * 32));
-  GMP_TRY(gmp_launch_next(k_bin_small, 1, nt, smem, stream, d_structs, n_struct, d_struct_of, N, cutoff, pos,
-                          species, n_el, d_grid, n_bins, atom_xh, atom_xl, atom_u, atom_bin, bin_start, bin_y,
-                          bin_je, atom_t, atom_y, d_err, n_clear));
+  // as many threads as atoms: fewer warps to wait for at each step; with more
+  // structures than SMs small CTAs, which leave room for one another
+  const int most = n_struct > sm_count ? 128 : 1024;
+  const int nt = std::min(most, std::max(64, (max_atoms + 31) / 32 * 32));
+  GMP_TRY(gmp_launch_next(k_bin_structs, (unsigned)n_struct, nt, smem, stream, d_structs, cutoff, pos, species, n_el,
+                          d_grid, d_struct_of, atom_xh, atom_xl, bin_start, bin_y, bin_je, atom_t, atom_y, d_err,
+                          n_clear));
   ++*launches;
   return cudaGetLastError();
 }

@@ -153,6 +153,7 @@ struct gmp_ctx {
   bool lists_outgrown = false; // ... and found to exceed its capacities
   bool exact_lists = false;    // count before filling (set for a rerun)
   cudaEvent_t ev_lists = nullptr;
+  cudaEvent_t ev_rows = nullptr;  // the number of Jacobian rows is read
   // pinned host scratch for small readbacks
   int64_t* h_small = nullptr;
   std::string err;
@@ -887,52 +888,20 @@ gmp_status grad_impl(gmp_ctx* h, int32_t n_struct, const int64_t* atom_off, cons
   if (N == 0) return GMP_OK;
   if (!jac_off) return fail(h, GMP_ERR_INVALID_ARG, "jac_off is required");
   const int64_t n = c1 - c0;
-  const bool whole = c0 == 0 && c1 == N;
   Io io;
   if ((r = stage_inputs(h, N, pos, species, io, st)) != GMP_OK) return r;
   GMP_CK(h->jac_counts.ensure(sizeof(int64_t) * (2 * n + 1)), "jac counts");
   int64_t* cnt = h->jac_counts.as<int64_t>();
   int64_t* joff = cnt + n;
-  auto lists = [&](bool) -> gmp_status {
-    gmp_status q = build_neighbors(h, n_struct, io.pos, io.species, N, st, true);
-    if (q != GMP_OK) return q;
-    GMP_CK(h->jac_rows.ensure(sizeof(int32_t) * std::max<int64_t>(h->cap_cur, 1)), "jac rows");
-    const int64_t* nbeg = h->rng_mode ? h->nbr_rng.as<int64_t>() : h->nbr_off.as<int64_t>();
-    const int64_t* nend = h->rng_mode ? h->nbr_rng.as<int64_t>() + N : h->nbr_off.as<int64_t>() + 1;
-    GMP_CK(gmp_launch_jacobian_count(n, nbeg + c0, nend + c0, h->pairs.as<GmpPair>(), cnt,
-                                     h->jac_rows.as<int32_t>(), st, h->sm_count, &h->launches), "jac count");
-    GMP_CK(gmp_exclusive_scan_i64(cnt, joff, n, h->scan_tmp.p, st, &h->launches), "jac scan");
-    GMP_CK(cudaMemcpyAsync(h->h_small + 2, joff + n, sizeof(int64_t), cudaMemcpyDeviceToHost, st), "read nnz");
-    GMP_CK(cudaStreamSynchronize(st), "jac sync");
-    return GMP_OK;
-  };
-  if ((r = run_sequence(h, st, lists)) != GMP_OK) return r;
-  const int64_t nnz = h->h_small[2];
-  *nnz_out = nnz;
-  if (nnz > cap) return fail(h, GMP_ERR_CAPACITY, "jacobian needs " + std::to_string(nnz) + " rows, cap is " + std::to_string(cap));
-  if (nnz > 0 && (!jac_j || !jac)) return fail(h, GMP_ERR_INVALID_ARG, "jac_j and jac are required");
-  // features: straight into a device output of the whole batch, else into
-  // the [N, F] scratch and the range's rows copied out at the end
-  float* jd = jac;
-  int32_t* jj = jac_j;
-  DevBuf tmp_jac, tmp_jj;
-  if (io.host && nnz > 0) {
-    GMP_CK(tmp_jac.ensure(sizeof(float) * nnz * h->F * 3), "stage jac");
-    GMP_CK(tmp_jj.ensure(sizeof(int32_t) * nnz), "stage jac_j");
-    jd = tmp_jac.as<float>();
-    jj = tmp_jj.as<int32_t>();
-  }
   for (const PassData& pd : h->passes)
     GMP_CK(h->mu.ensure(sizeof(float) * (size_t)N * std::max(pd.pass.nsig, 1) * (pd.L + 1) * (pd.L + 1)), "moments");
-  float* fout = (whole && features && !io.host) ? features : nullptr;
-  if (!fout) {
-    GMP_CK(h->stage_feat.ensure(sizeof(float) * N * h->F), "feature scratch");
-    fout = h->stage_feat.as<float>();
-  }
-  if ((r = begin_compute(h, N)) != GMP_OK) return r;
-  for (size_t g = 0; g < h->passes.size(); ++g) {
-    // forward kernel (features, moments), refinement of the flagged
-    // features and their moments, then the Jacobian rows from the moments
+  // features: into scratch, from which they are copied at the end (nothing is
+  // written when the rows exceed `cap`)
+  GMP_CK(h->stage_feat.ensure(sizeof(float) * N * h->F), "feature scratch");
+  float* const fout = h->stage_feat.as<float>();
+  // one pass's forward kernel (features, moments) and the refinement of the
+  // flagged features and their moments, ahead of the pass's Jacobian rows
+  auto forward = [&](size_t g) -> gmp_status {
     PassData& pd = h->passes[g];
     gmpk::KParams K = base_params(h, pd, (int)g, N);
     K.N = c1;
@@ -944,9 +913,50 @@ gmp_status grad_impl(gmp_ctx* h, int32_t n_struct, const int64_t* atom_off, cons
     GMP_CK(launch_compute(pd, GMP_KIND_FORWARD, K, pd.fwd, st, h->sm_count, &h->launches), "forward");
     GMP_CK(prof_mark(h, 1, false, st), "profile");
     GMP_CK(prof_mark(h, 3, true, st), "profile");
-    if ((r = refine(h, N, fout, st, nullptr, nullptr, nullptr, pass_moments(h, pd, (int)g))) != GMP_OK) return r;
-    if (g + 1 < h->passes.size() && (r = reset_flags(h, st)) != GMP_OK) return r;
+    gmp_status q = refine(h, N, fout, st, nullptr, nullptr, nullptr, pass_moments(h, pd, (int)g));
+    if (q != GMP_OK) return q;
+    if (g + 1 < h->passes.size() && (q = reset_flags(h, st)) != GMP_OK) return q;
     GMP_CK(prof_mark(h, 3, false, st), "profile");
+    return GMP_OK;
+  };
+  // lists, row counts, and the first pass's features, which run while the host
+  // reads the number of rows
+  auto lists = [&](bool) -> gmp_status {
+    gmp_status q = build_neighbors(h, n_struct, io.pos, io.species, N, st, true);
+    if (q != GMP_OK) return q;
+    GMP_CK(h->jac_rows.ensure(sizeof(int32_t) * std::max<int64_t>(h->cap_cur, 1)), "jac rows");
+    if ((q = begin_compute(h, N)) != GMP_OK) return q;
+    const int64_t* nbeg = h->rng_mode ? h->nbr_rng.as<int64_t>() : h->nbr_off.as<int64_t>();
+    const int64_t* nend = h->rng_mode ? h->nbr_rng.as<int64_t>() + N : h->nbr_off.as<int64_t>() + 1;
+    GMP_CK(gmp_launch_jacobian_count(n, nbeg + c0, nend + c0, h->pairs.as<GmpPair>(), cnt,
+                                     h->jac_rows.as<int32_t>(), st, h->sm_count, &h->launches), "jac count");
+    GMP_CK(gmp_exclusive_scan_i64(cnt, joff, n, h->scan_tmp.p, st, &h->launches), "jac scan");
+    GMP_CK(cudaMemcpyAsync(h->h_small + 2, joff + n, sizeof(int64_t), cudaMemcpyDeviceToHost, st), "read nnz");
+    GMP_CK(cudaEventRecord(h->ev_rows, st), "event");
+    return forward(0);
+  };
+  if ((r = run_sequence(h, st, lists)) != GMP_OK) return r;
+  GMP_CK(cudaEventSynchronize(h->ev_rows), "jac sync");
+  const int64_t nnz = h->h_small[2];
+  *nnz_out = nnz;
+  if (nnz > cap) return fail(h, GMP_ERR_CAPACITY, "jacobian needs " + std::to_string(nnz) + " rows, cap is " + std::to_string(cap));
+  if (nnz > 0 && (!jac_j || !jac)) return fail(h, GMP_ERR_INVALID_ARG, "jac_j and jac are required");
+  float* jd = jac;
+  int32_t* jj = jac_j;
+  DevBuf tmp_jac, tmp_jj;
+  if (io.host && nnz > 0) {
+    GMP_CK(tmp_jac.ensure(sizeof(float) * nnz * h->F * 3), "stage jac");
+    GMP_CK(tmp_jj.ensure(sizeof(int32_t) * nnz), "stage jac_j");
+    jd = tmp_jac.as<float>();
+    jj = tmp_jj.as<int32_t>();
+  }
+  for (size_t g = 0; g < h->passes.size(); ++g) {
+    if (g > 0 && (r = forward(g)) != GMP_OK) return r;
+    PassData& pd = h->passes[g];
+    gmpk::KParams K = base_params(h, pd, (int)g, N);
+    K.N = c1;
+    K.center0 = c0;
+    K.mu_out = h->mu.as<float>();
     K.features = nullptr;
     K.flags = nullptr;
     K.jac_off = joff;
@@ -960,7 +970,7 @@ gmp_status grad_impl(gmp_ctx* h, int32_t n_struct, const int64_t* atom_off, cons
   }
   const cudaMemcpyKind k_out = io.host ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
   GMP_CK(cudaMemcpyAsync(jac_off, joff, sizeof(int64_t) * (n + 1), k_out, st), "copy jac_off");
-  if (features && fout != features)
+  if (features)
     GMP_CK(cudaMemcpyAsync(features, fout + c0 * h->F, sizeof(float) * n * h->F, k_out, st), "copy features");
   if (io.host) {
     if (nnz > 0) {
@@ -1208,6 +1218,7 @@ gmp_status gmp_create(const gmp_params* p, int device, gmp_handle* out) {
   if (cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking) != cudaSuccess ||
       cudaEventCreateWithFlags(&h->ev_desc, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&h->ev_lists, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&h->ev_rows, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&h->ev_in, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&h->ev_feat, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&h->ev_out, cudaEventDisableTiming) != cudaSuccess) {
@@ -1826,7 +1837,7 @@ void gmp_destroy(gmp_handle h) {
     for (cudaEvent_t e : v) cudaEventDestroy(e);
   if (h->ev) cudaEventDestroy(h->ev);
   if (h->h_desc) cudaFreeHost(h->h_desc);
-  for (cudaEvent_t e : {h->ev_in, h->ev_feat, h->ev_out, h->ev_desc, h->ev_lists})
+  for (cudaEvent_t e : {h->ev_in, h->ev_feat, h->ev_out, h->ev_desc, h->ev_lists, h->ev_rows})
     if (e) cudaEventDestroy(e);
   if (h->side) cudaStreamDestroy(h->side);
   delete h;  // the device buffers free themselves, with this device current

@@ -1006,15 +1006,12 @@ __global__ void __launch_bounds__(128, 8) k_neighbors(const GmpStruct* __restric
     __syncwarp();
     for (int k = 2; k <= P2; k <<= 1) {
       for (int jj = k >> 1; jj > 0; jj >>= 1) {
-        for (int t = lane; t < P2; t += 32) {
-          int partner = t ^ jj;
-          if (partner > t) {
-            unsigned long long a = skey[t], b = skey[partner];
-            bool up = (t & k) == 0;
-            if ((a > b) == up) {
-              skey[t] = b;
-              skey[partner] = a;
-            }
+        for (int c = lane; c < P2 / 2; c += 32) {  // comparison c: keys t and t + jj
+          const int t = 2 * c - (c & (jj - 1));
+          const unsigned long long a = skey[t], b = skey[t + jj];
+          if ((a > b) == ((t & k) == 0)) {
+            skey[t] = b;
+            skey[t + jj] = a;
           }
         }
         __syncwarp();

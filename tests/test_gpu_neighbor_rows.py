@@ -61,3 +61,24 @@ def test_neighbor_rows(torch, oracle_mod, kind, edge, n, pbc):
     pref, pabs = oracle_mod.point_features(w, pts, np.zeros(40, np.int64), want_abs=True)
     fp = F.featurize_points(*dev, w.atom_off, w.cells, w.pbc, torch.from_numpy(pts).cuda(), [0, 40]).cpu().numpy()
     assert (np.abs(fp - pref) <= 1e-5 * np.maximum(np.maximum(np.abs(pref), 1e-6 * pabs), 2.0 ** -126)).all()
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 17, 32, 33, 34, 64, 65, 66, 129, 130, 257, 258, 600])
+def test_sorted_lists(torch, oracle_mod, n):
+    """n atoms all within the cutoff of one another (lists of n, the center's
+    own entry included), and the same periodic along one axis (3 n): ascending
+    (atom, image)."""
+    from paper_2303_12980_gb300.binding import GMPFeaturizer
+    rng = np.random.default_rng(n)
+    pos = rng.permutation(n)[:, None] * np.array([[0.002, 0.0, 0.0]]) + rng.uniform(0, 1e-3, (n, 3))
+    for pbc in ([0, 0, 0], [0, 0, 1]):
+        w = synth._single("line", pos, np.eye(3) * 3.7, pbc, np.zeros(n, np.int32), synth.gaussian_table(rng, [4], 2), [0],
+                          [0.6], 4.0)
+        F = GMPFeaturizer.from_workload(w)
+        off, j, s = (x.cpu().numpy().astype(np.int64) for x in F.neighbors(
+            torch.from_numpy(w.positions).cuda(), torch.from_numpy(w.species).cuda(), w.atom_off, w.cells, w.pbc))
+        s = s.reshape(-1, 3)
+        key = ((j * 1024 + s[:, 0] + 512) * 1024 + s[:, 1] + 512) * 1024 + s[:, 2] + 512
+        assert np.array_equal(off, oracle_mod.neighbors(w)[0]) and off[-1] == n * n * (3 if pbc[2] else 1)
+        for i in range(0, n, max(1, n // 9)):
+            assert (np.diff(key[off[i]:off[i + 1]]) > 0).all()

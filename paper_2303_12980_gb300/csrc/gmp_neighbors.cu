@@ -78,17 +78,16 @@ __device__ __forceinline__ void sort_key_image(unsigned long long key, int* n) {
 // it, so a structure placed any number of cells away from its cell keeps
 // small stored indices; pair image indices, which are differences of the
 // stored indices, do not change.
-__device__ inline void struct_ref_cell(const GmpStruct& st, const double* __restrict__ atom_pos, double (&f0)[3]) {
-  f0[0] = f0[1] = f0[2] = 0.0;
-  if (st.n_atoms <= 0) return;
+__device__ inline double ref_cell_axis(const GmpStruct& st, const double* __restrict__ atom_pos, int k) {
+  if (st.n_atoms <= 0 || !st.periodic[k]) return 0.0;
   const double* x = atom_pos + 3 * st.atom_base;
   const double x0 = x[0], x1 = x[1], x2 = x[2];
-  if (!isfinite(x0) || !isfinite(x1) || !isfinite(x2)) return;
-  for (int k = 0; k < 3; ++k) {
-    if (!st.periodic[k]) continue;
-    const double f = floor(x0 * st.Ainv[k] + x1 * st.Ainv[3 + k] + x2 * st.Ainv[6 + k]);
-    if (fabs(f) < 1e9) f0[k] = f;
-  }
+  if (!isfinite(x0) || !isfinite(x1) || !isfinite(x2)) return 0.0;
+  const double f = floor(x0 * st.Ainv[k] + x1 * st.Ainv[3 + k] + x2 * st.Ainv[6 + k]);
+  return fabs(f) < 1e9 ? f : 0.0;
+}
+__device__ inline void struct_ref_cell(const GmpStruct& st, const double* __restrict__ atom_pos, double (&f0)[3]) {
+  for (int k = 0; k < 3; ++k) f0[k] = ref_cell_axis(st, atom_pos, k);
 }
 
 // Wraps the fractional coordinate u of a periodic axis into [0, 1) and
@@ -195,33 +194,43 @@ __global__ void k_prepare(const GmpStruct* __restrict__ S, const int32_t* __rest
 // structures, 45 against 47 of a 4,096-atom crystal).  One thread runs this
 // for a structure, at 1/64 of the FP32 rate in FP64: one division an axis, and
 // the bounds, which carry a margin, in FP32.
-__host__ __device__ inline void grid_struct(GmpStruct& st, const unsigned long long* bbox, GmpGrid& g,
-                                            double cutoff) {
-  double w[3], ext[3];
-  float uk[3];  // bound on the fractional coordinates
-  for (int k = 0; k < 3; ++k) {
-    const double target = (k == 0 ? 0.25 : 0.5) * st.reach[k];
-    if (st.periodic[k]) {
-      g.umin[k] = 0.0;
-      ext[k] = w[k] = 1.0;
-      const double nbf = target > 0.0 ? floor(1.0 / target) : 1.0;
-      g.nb[k] = (int)fmin(fmax(nbf, 1.0), 1024.0);
-      g.inv_binw[k] = g.nb[k];
-      uk[k] = 2.0f;
-    } else {
-      const double lo = st.n_atoms ? key_to_double(bbox[2 * k]) : 0.0;
-      const double hi = st.n_atoms ? key_to_double(~bbox[2 * k + 1]) : 0.0;
-      g.umin[k] = lo;
-      ext[k] = hi - lo;
-      w[k] = fmax(target, 1e-12);
-      g.inv_binw[k] = 1.0 / w[k];
-      g.nb[k] = (int)fmin(floor(ext[k] * g.inv_binw[k]) + 1.0, 1024.0);
-      if (g.nb[k] == 1024) {
-        w[k] = fmax(ext[k] / 1023.0, w[k]);
-        g.inv_binw[k] = 1.0 / w[k];
-      }
-      uk[k] = fmaxf(fabsf((float)lo), fabsf((float)hi)) + 1.0f;
+// In two parts: an axis (they may be taken by different threads), then the rest.
+struct GridAxes {
+  double w[3], ext[3];  // bin width, extent of the bins
+  float uk[3];          // bound on the fractional coordinates
+};
+__host__ __device__ inline void grid_axis(const GmpStruct& st, const unsigned long long* bbox, GmpGrid& g, GridAxes& x,
+                                          int k) {
+  const double target = (k == 0 ? 0.25 : 0.5) * st.reach[k];
+  if (st.periodic[k]) {
+    g.umin[k] = 0.0;
+    x.ext[k] = x.w[k] = 1.0;
+    const double nbf = target > 0.0 ? floor(1.0 / target) : 1.0;
+    g.nb[k] = (int)fmin(fmax(nbf, 1.0), 1024.0);
+    g.inv_binw[k] = g.nb[k];
+    x.uk[k] = 2.0f;
+  } else {
+    const double lo = st.n_atoms ? key_to_double(bbox[2 * k]) : 0.0;
+    const double hi = st.n_atoms ? key_to_double(~bbox[2 * k + 1]) : 0.0;
+    g.umin[k] = lo;
+    x.ext[k] = hi - lo;
+    x.w[k] = fmax(target, 1e-12);
+    g.inv_binw[k] = 1.0 / x.w[k];
+    // (fmax: 1 for a NaN, which an extent beyond FP64's range would make here)
+    g.nb[k] = (int)fmin(fmax(floor(x.ext[k] * g.inv_binw[k]) + 1.0, 1.0), 1024.0);
+    if (g.nb[k] == 1024) {
+      x.w[k] = fmax(x.ext[k] / 1023.0, x.w[k]);
+      g.inv_binw[k] = 1.0 / x.w[k];
     }
+    x.uk[k] = fmaxf(fabsf((float)lo), fabsf((float)hi)) + 1.0f;
+  }
+}
+__host__ __device__ inline void grid_rest(GmpStruct& st, GmpGrid& g, const GridAxes& x, double cutoff) {
+  double w[3];
+  float uk[3];
+  for (int k = 0; k < 3; ++k) {
+    w[k] = x.w[k];
+    uk[k] = x.uk[k];
   }
   // keep the grid within the reserved bin slots
   while ((int64_t)g.nb[0] * g.nb[1] * g.nb[2] > st.bin_cap) {
@@ -234,7 +243,7 @@ __host__ __device__ inline void grid_struct(GmpStruct& st, const unsigned long l
     } else {
       w[k] *= 2.0;
       g.inv_binw[k] *= 0.5;
-      g.nb[k] = (int)fmin(floor(ext[k] * g.inv_binw[k]) + 1.0, 1024.0);
+      g.nb[k] = (int)fmin(fmax(floor(x.ext[k] * g.inv_binw[k]) + 1.0, 1.0), 1024.0);
     }
   }
   // Rigorous two-sided FP32 bounds.  Wrapped Cartesian coordinates are
@@ -291,6 +300,12 @@ __host__ __device__ inline void grid_struct(GmpStruct& st, const unsigned long l
   const double bi = fmax(cutoff - 2.0 * delta, 0.0);
   float q2 = (float)(bi * bi * (1.0 - 0x1p-20));
   st.inside2 = fmaxf(nextafterf(q2, 0.0f), 0.0f);
+}
+
+__host__ __device__ inline void grid_struct(GmpStruct& st, const unsigned long long* bbox, GmpGrid& g, double cutoff) {
+  GridAxes x;
+  for (int k = 0; k < 3; ++k) grid_axis(st, bbox, g, x, k);
+  grid_rest(st, g, x, cutoff);
 }
 
 __host__ __device__ inline bool all_periodic(const GmpStruct& st) {
@@ -447,6 +462,7 @@ struct StructBins {
   GmpGrid g;
   double f0[3];                // reference cell (struct_ref_cell)
   unsigned long long bbox[6];  // as prepare_atom's
+  GridAxes axes;
   int32_t warp_tot[32];
 };
 __host__ __device__ inline size_t struct_bins_smem(int n_atoms, int n_bins) {
@@ -485,11 +501,7 @@ __global__ void __launch_bounds__(1024) k_bin_structs(GmpStruct* __restrict__ S,
   double* const us = reinterpret_cast<double*>(sm_bins + sizeof(StructBins));  // [n][3]
   int32_t* const slot_atom = reinterpret_cast<int32_t*>(us + 3 * (size_t)n);   // [n] atom of each slot
   int32_t* const bin = slot_atom + n;                                          // [n]
-  if (tid == 0) {
-    double f0[3];
-    struct_ref_cell(st, pos, f0);
-    for (int k = 0; k < 3; ++k) B.f0[k] = f0[k];
-  }
+  if (tid < 3) B.f0[tid] = ref_cell_axis(st, pos, tid);
   __syncthreads();
   for (int t0 = 0; t0 < n; t0 += nt) {
     const int t = t0 + tid;
@@ -530,11 +542,15 @@ __global__ void __launch_bounds__(1024) k_bin_structs(GmpStruct* __restrict__ S,
     }
   }
   __syncthreads();
-  if (open && tid == 0) {
-    grid_struct(B.st, B.bbox, B.g, cutoff);
-    G[s] = B.g;
-    S[s].prescreen2 = st.prescreen2;
-    S[s].inside2 = st.inside2;
+  if (open && tid < 32) {
+    if (tid < 3) grid_axis(st, B.bbox, B.g, B.axes, tid);
+    __syncwarp();
+    if (tid == 0) {
+      grid_rest(B.st, B.g, B.axes, cutoff);
+      G[s] = B.g;
+      S[s].prescreen2 = st.prescreen2;
+      S[s].inside2 = st.inside2;
+    }
   }
   __syncthreads();
   const GmpGrid& g = B.g;

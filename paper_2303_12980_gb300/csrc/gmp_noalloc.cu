@@ -2,7 +2,7 @@
 //
 // gmp_neighbor_counts_noalloc runs the same binning and exact neighbor-count
 // kernels as gmp_neighbors (always the multi-kernel binning, whose bins equal
-// those of the single-CTA binning gmp_neighbors uses for small batches), but
+// those of the binning gmp_neighbors uses for batches of small structures), but
 // every scratch buffer they need (per-atom
 // fractional coordinates, the bin grid, bin counts and offsets, the scan
 // workspace, the error word) lives in one file-scope device array of fixed

@@ -18,7 +18,7 @@
 //
 // Layout: one warp per center (persistent warps take centers from an atomic
 // counter).  The forward kernel walks its center's neighbor list in tiles of
-// 16 pairs (two lanes per pair) or 32 (one lane per pair):
+// 16 pairs (two lanes per pair) or 32 (gmp_forward_tile):
 //   phase 1, lane = pair (and half of its sigma groups): exps and radial
 //            factors R[l][s] (double-float exponent argument, four sigmas per
 //            16-byte table load, packed FP32 pairs), MCSH values S[k] ->
@@ -335,6 +335,51 @@ __device__ __forceinline__ void radial4d(const float* __restrict__ tab_e, int km
   }
 }
 
+// The same for two pairs of one element (r^2 a and b): every table load serves
+// both.
+template <int L, int NL = L + 2>
+__device__ __forceinline__ void radial4d2(const float* __restrict__ tab_e, int kmax, int sg, const float (&r2h)[2],
+                                          const float (&r2l)[2], float4 (&R)[2][NL]) {
+  constexpr int RB = gmp_rad_block(L);
+  float2 Rp[2][2][NL];
+  float2 nr2h[2], r2h2[2], r2l2[2];
+#pragma unroll
+  for (int p = 0; p < 2; ++p) {
+    nr2h[p] = make_float2(-r2h[p], -r2h[p]);
+    r2h2[p] = make_float2(r2h[p], r2h[p]);
+    r2l2[p] = make_float2(r2l[p], r2l[p]);
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int l = 0; l < NL; ++l) Rp[p][h][l] = make_float2(0.0f, 0.0f);
+  }
+#pragma unroll 1
+  for (int q = 0; q < kmax; ++q) {
+    const float4* blk = reinterpret_cast<const float4*>(tab_e) + sg * rad_sg_stride(L, kmax) + q * RB;
+    const float4 bh = blk[0];
+    const float4 bl = blk[1];
+    float2 E[2][2];
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      E[p][0] = gmp_exp_neg2(make_float2(bh.x, bh.y), make_float2(bl.x, bl.y), nr2h[p], r2h2[p], r2l2[p]);
+      E[p][1] = gmp_exp_neg2(make_float2(bh.z, bh.w), make_float2(bl.z, bl.w), nr2h[p], r2h2[p], r2l2[p]);
+    }
+#pragma unroll
+    for (int l = 0; l < NL; ++l) {
+      const float4 a = blk[2 + l];
+#pragma unroll
+      for (int p = 0; p < 2; ++p) {
+        Rp[p][0][l] = gmp_fma2(make_float2(a.x, a.y), E[p][0], Rp[p][0][l]);
+        Rp[p][1][l] = gmp_fma2(make_float2(a.z, a.w), E[p][1], Rp[p][1][l]);
+      }
+    }
+  }
+#pragma unroll
+  for (int p = 0; p < 2; ++p)
+#pragma unroll
+    for (int l = 0; l < NL; ++l) R[p][l] = make_float4(Rp[p][0][l].x, Rp[p][0][l].y, Rp[p][1][l].x, Rp[p][1][l].y);
+}
+
 // (Below, NL orders from LA on: the backward takes its orders in ranges.)
 // Radial factors scaled by 2^32 for the backward, with scalar FP32
 // operations (the backward kernel keeps its 168-register budget with these;
@@ -600,19 +645,30 @@ __device__ __forceinline__ float forward_sweep(const GmpPass& P, const float* __
   const bool mixed = P.mixed_sign != 0;
 
   constexpr int LPP = 32 / TILE;      // phase 1: lanes per pair (2 or 1)
+  // Tile of 32: every lane evaluates the MCSH values of one pair, then the radial
+  // factors of two neighboring pairs for half of the sigma groups (its own and
+  // that of lane ^ 16): with one element a table load serves both.  At orders 5
+  // and 6 two pairs' factors do not fit the registers beside the moments.
+  constexpr bool TWO = LPP == 1 && SH::NSB % 2 == 0 && L <= 4;
   const int half = LPP == 2 ? (lane >> 4) : 0;
   const int pl = LPP == 2 ? (lane & 15) : lane;
   constexpr int SG_LO = LPP == 2 ? (SH::NSB + 1) / 2 : SH::NSB;  // sigma groups of half 0: [0, SG_LO)
   const int sg0 = half ? SG_LO : 0, sg1 = half ? SH::NSB : SG_LO;
   for (int base = 0; base < M; base += SH::TILE) {
     const int np = min(SH::TILE, M - base);
+    float own_r2h = 0.0f, own_r2l = 0.0f;
+    int own_e = 0;
+    // the lane's tile row `pl` takes pair `own`: pair p is in row p or, woven, in
+    // row p / 2 + 16 (p mod 2)
+    const bool woven = TWO && np > 16;
+    const int own = woven ? 2 * (lane & 15) + (lane >> 4) : pl;
     // ---- phase 1: lanes (pair, half); both halves evaluate S and store
     // alternate chunks, each half computes the radial factors of half the
     // sigma groups
-    if (pl < np) {
+    if (own < np) {
       float dx, dy, dz, r2h, r2l;
       int e, j;
-      load_pair(pairs, p0 + base + pl, dx, dy, dz, r2h, r2l, e, j);
+      load_pair(pairs, p0 + base + own, dx, dy, dz, r2h, r2l, e, j);
       if (half == 0 && base + SH::TILE + pl < M) prefetch_pair(pairs + p0 + base + SH::TILE + pl);
       float* srow = St + pl * SH::SSTR;
       if constexpr (CW == 2) {
@@ -675,14 +731,20 @@ __device__ __forceinline__ float forward_sweep(const GmpPass& P, const float* __
                 make_float4(rl[4 * c], rl[4 * c + 1], rl[4 * c + 2], rl[4 * c + 3]);
         }
       }
-      const float* tab_e = s_rad + (size_t)e * rad_elem_stride(L, NS, P.kmax);
-      float* rrow = Rt + pl * SH::RSTR;
-      for (int sg = sg0; sg < sg1; ++sg) {
-        float R[4][L + 1];
-        radial4d<L, L + 1>(tab_e, P.kmax, sg, r2h, r2l, R);
-#pragma unroll
-        for (int l = 0; l <= L; ++l)
-          *reinterpret_cast<float4*>(rrow + l * NS + 4 * sg) = make_float4(R[0][l], R[1][l], R[2][l], R[3][l]);
+      if constexpr (TWO) {
+        own_r2h = r2h;
+        own_r2l = r2l;
+        own_e = e;
+      } else {
+        const float* tab_e = s_rad + (size_t)e * rad_elem_stride(L, NS, P.kmax);
+        float* rrow = Rt + pl * SH::RSTR;
+        for (int sg = sg0; sg < sg1; ++sg) {
+          float R[4][L + 1];
+          radial4d<L, L + 1>(tab_e, P.kmax, sg, r2h, r2l, R);
+  #pragma unroll
+          for (int l = 0; l <= L; ++l)
+            *reinterpret_cast<float4*>(rrow + l * NS + 4 * sg) = make_float4(R[0][l], R[1][l], R[2][l], R[3][l]);
+        }
       }
       if (P.want_density && half == 0) {
         const float* dens_e = s_dens + (size_t)e * dens_elem_stride(P.kmax);
@@ -696,6 +758,59 @@ __device__ __forceinline__ float forward_sweep(const GmpPass& P, const float* __
           const gmp_f2 s2 = gmp_two_sum(rho_hi, t);
           rho_hi = s2.hi;
           rho_lo += s2.lo;
+        }
+      }
+    }
+    if constexpr (TWO) {
+      // radial factors for half of the sigma groups a lane: of the pairs of rows
+      // lane and lane ^ 16 (neighbors in the list, mostly of one element), or of
+      // one pair when the tile has no more than 16
+      const int sgb = (lane >> 4) * (SH::NSB / 2), sge = sgb + SH::NSB / 2;
+      if (np <= 16) {
+        const int row = lane & 15;
+        const float h = __shfl_sync(0xffffffffu, own_r2h, row), l2 = __shfl_sync(0xffffffffu, own_r2l, row);
+        const int e = __shfl_sync(0xffffffffu, own_e, row);
+        if (row < np) {
+          const float* tab_e = s_rad + (size_t)e * rad_elem_stride(L, NS, P.kmax);
+          for (int sg = sgb; sg < sge; ++sg) {
+            float R[4][L + 1];
+            radial4d<L, L + 1>(tab_e, P.kmax, sg, h, l2, R);
+#pragma unroll
+            for (int l = 0; l <= L; ++l)
+              *reinterpret_cast<float4*>(Rt + row * SH::RSTR + l * NS + 4 * sg) = make_float4(R[0][l], R[1][l], R[2][l], R[3][l]);
+          }
+        }
+      } else {
+        const float r2h2[2] = {own_r2h, __shfl_xor_sync(0xffffffffu, own_r2h, 16)};
+        const float r2l2[2] = {own_r2l, __shfl_xor_sync(0xffffffffu, own_r2l, 16)};
+        const int e2 = __shfl_xor_sync(0xffffffffu, own_e, 16);
+        const bool ok0 = own < np, ok1 = (own ^ 1) < np;
+        const int eo[2] = {ok0 ? own_e : e2, ok1 ? e2 : own_e};
+        const bool one = __all_sync(0xffffffffu, eo[0] == eo[1]);
+        float* const row0 = Rt + lane * SH::RSTR;
+        float* const row1 = Rt + (lane ^ 16) * SH::RSTR;
+        for (int sg = sgb; sg < sge; ++sg) {
+          if (one) {
+            float4 R[2][L + 1];
+            radial4d2<L, L + 1>(s_rad + (size_t)eo[0] * rad_elem_stride(L, NS, P.kmax), P.kmax, sg, r2h2, r2l2, R);
+#pragma unroll
+            for (int l = 0; l <= L; ++l) {
+              if (ok0) *reinterpret_cast<float4*>(row0 + l * NS + 4 * sg) = R[0][l];
+              if (ok1) *reinterpret_cast<float4*>(row1 + l * NS + 4 * sg) = R[1][l];
+            }
+          } else {
+#pragma unroll 1
+            for (int p = 0; p < 2; ++p) {
+              float R[4][L + 1];
+              radial4d<L, L + 1>(s_rad + (size_t)eo[p] * rad_elem_stride(L, NS, P.kmax), P.kmax, sg, p ? r2h2[1] : r2h2[0],
+                                 p ? r2l2[1] : r2l2[0], R);
+              float* const row = p ? row1 : row0;
+              if (p ? ok1 : ok0)
+#pragma unroll
+                for (int l = 0; l <= L; ++l)
+                  *reinterpret_cast<float4*>(row + l * NS + 4 * sg) = make_float4(R[0][l], R[1][l], R[2][l], R[3][l]);
+            }
+          }
         }
       }
     }
@@ -713,7 +828,8 @@ __device__ __forceinline__ float forward_sweep(const GmpPass& P, const float* __
         if (mixed_last) {
           // the free slot holds 0: B from |R| r^l, r^l read after the chunks
           const float* rlp = St + 4 * SH::NCH + it_l[q];
-          for (int pp = 0; pp < np; ++pp) {
+          for (int t = 0; t < np; ++t) {
+            const int pp = woven ? (t >> 1) + 16 * (t & 1) : t;
             const float4 r = *reinterpret_cast<const float4*>(rp + pp * SH::RSTR);
             const float rl = rlp[pp * SH::SSTR];
             hi[q][3] = __fmaf_rn(fabsf(r.x), rl, hi[q][3]);
@@ -725,13 +841,27 @@ __device__ __forceinline__ float forward_sweep(const GmpPass& P, const float* __
       }
       for (int b0 = 0; b0 < np; b0 += SH::FOLD) {
         const int b1 = min(np, b0 + SH::FOLD);
+        // step(row) for the pairs b0 .. b1-1 in list order
+        auto each_row = [&](auto&& step) {
+          if (TWO && woven) {
+            const int i0 = b0 >> 1, i1 = b1 >> 1;
+#pragma unroll 4
+            for (int i = i0; i < i1; ++i) {
+              step(i);
+              step(16 + i);
+            }
+            if (b1 & 1) step(i1);
+          } else {
+#pragma unroll 8
+            for (int pp = b0; pp < b1; ++pp) step(pp);
+          }
+        };
         // acc2[v]: components (2h, 2h+1) of sigma u as a packed pair, v = (CW / 2) u + h
         float2 acc2[2 * CW];
 #pragma unroll
         for (int v = 0; v < 2 * CW; ++v) acc2[v] = make_float2(0.0f, 0.0f);
         if constexpr (CW == 4) {
-#pragma unroll 8
-          for (int pp = b0; pp < b1; ++pp) {
+          each_row([&](int pp) {
             const float4 r = *reinterpret_cast<const float4*>(rp + pp * SH::RSTR);
             const float4 s = *reinterpret_cast<const float4*>(sp + pp * SH::SSTR);
             const float rv[4] = {r.x, r.y, r.z, r.w};
@@ -742,18 +872,18 @@ __device__ __forceinline__ float forward_sweep(const GmpPass& P, const float* __
               acc2[2 * u] = gmp_fma2(ru, s01, acc2[2 * u]);
               acc2[2 * u + 1] = gmp_fma2(ru, s23, acc2[2 * u + 1]);
             }
-          }
+          });
         } else if (!mixed_last) {
-#pragma unroll 8
-          for (int pp = b0; pp < b1; ++pp) {
+          each_row([&](int pp) {
             const float4 r = *reinterpret_cast<const float4*>(rp + pp * SH::RSTR);
             const float2 s = *reinterpret_cast<const float2*>(sp + pp * SH::SSTR);
             const float rv[4] = {r.x, r.y, r.z, r.w};
 #pragma unroll
             for (int u = 0; u < 4; ++u) acc2[u] = gmp_fma2(make_float2(rv[u], rv[u]), s, acc2[u]);
-          }
+          });
         } else {  // the r^l slot takes |R|, so that it sums B
-          for (int pp = b0; pp < b1; ++pp) {
+          for (int t = b0; t < b1; ++t) {
+            const int pp = woven ? (t >> 1) + 16 * (t & 1) : t;
             const float4 r = *reinterpret_cast<const float4*>(rp + pp * SH::RSTR);
             const float2 s = *reinterpret_cast<const float2*>(sp + pp * SH::SSTR);
             const float rv[4] = {r.x, r.y, r.z, r.w};
@@ -913,7 +1043,7 @@ __device__ __forceinline__ void write_features(const KParams& K, int64_t i, cons
 
 // ------------------------------------------------------------------------
 template <int L, int NS, int TILE>
-__global__ void __launch_bounds__(512) k_forward(KParams K) {
+__global__ void __launch_bounds__(TILE == 32 && L <= 4 ? 640 : 512) k_forward(KParams K) {
   using SH = Shape<L, NS, TILE>;
   extern __shared__ __align__(16) float smem[];
   const GmpPass& P = K.pass;

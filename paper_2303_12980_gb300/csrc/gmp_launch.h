@@ -16,9 +16,29 @@ struct KParams;
 
 // Launch shape of a compute kernel (chosen by the autotuner or defaults).
 struct GmpShape {
-  int tile;   // forward tile: 16 pairs (two lanes per pair) or 32 (one lane per pair)
+  int tile;   // forward tile: 16 pairs (two lanes per pair) or 32
   int warps;  // warps per CTA, 0 = the CTA size with the most resident warps
 };
+
+// The untuned forward tile of highest order L, ns padded sigmas and n_el
+// elements.  In a tile of 32 (orders up to 4, 8 or 16 sigmas) a lane takes the
+// radial factors of two neighboring pairs, so that a table load serves both when
+// they are of one element, as the lists are sorted by; the kernel is bound by
+// shared-memory wavefronts.  It keeps 20 instead of 28 warps per SM, and with many
+// elements the tables take more of that away and fewer pairs agree.  Forward
+// kernel, GB300, us, tile 16 -> 32, crystals of 4,096 / 32,768 atoms (183 pairs
+// a center) and 2,500 small structures (10 elements, 74 pairs):
+//   8 sigmas, orders 0-2   47 -> 43 / 275 -> 253   775 -> 679
+//             orders 0-3   55 -> 45 / 333 -> 274   938 -> 737
+//             orders 0-4   53 -> 52 / 319 -> 299 with 3 elements, 53 -> 56 /
+//                          324 -> 320 with 6, 54 -> 58 / 330 -> 349 with 10;  856 -> 868
+//             orders 0-1   38 -> 40                546 -> 607
+//  16 sigmas, orders 0-2   59 -> 58 / 384 -> 360  1060 -> 953
+//             orders 0-3   72 -> 77               1313 -> 1350
+//             orders 0-4   86 -> 92               1608 -> 2129
+constexpr int gmp_forward_tile(int L, int ns, int n_el) {
+  return (ns == 8 && (L == 2 || L == 3 || (L == 4 && n_el <= 4))) || (ns == 16 && L == 2) ? 32 : 16;
+}
 
 // The launch worked out for a request (shape and number of centers' class):
 // kept by the handle, so that a call repeats neither the attribute nor the

@@ -380,7 +380,6 @@ __device__ __forceinline__ void radial4d2(const float* __restrict__ tab_e, int k
     for (int l = 0; l < NL; ++l) R[p][l] = make_float4(Rp[p][0][l].x, Rp[p][0][l].y, Rp[p][1][l].x, Rp[p][1][l].y);
 }
 
-// (Below, NL orders from LA on: the backward takes its orders in ranges.)
 // Radial factors scaled by 2^32 for the backward, with scalar FP32
 // operations (the backward kernel keeps its 168-register budget with these;
 // packed pairs need aligned register pairs and spill there).  The exponent
@@ -391,7 +390,7 @@ __device__ __forceinline__ void radial4d2(const float* __restrict__ tab_e, int k
 // down to exp(-B r^2) = 2^-158, with room for the amplitudes (alpha/gamma)^l
 // of the higher orders: a gradient term of a far pair, multiplied by large
 // adjoints, keeps its digits; the kernel scales its sums back by 2^-32.
-template <int L, int NL = L + 2, bool PADG = true, int LA = 0>
+template <int L, int NL = L + 2, bool PADG = true>
 __device__ __forceinline__ void radial4s(const float* __restrict__ tab_e, int kmax, int sg, float r2h,
                                          float (&R)[4][NL]) {
   constexpr int RB = gmp_rad_block(L);
@@ -410,7 +409,7 @@ __device__ __forceinline__ void radial4s(const float* __restrict__ tab_e, int km
     E[3] = gmp_ex2(__fmaf_rn(bh.w, -r2h, GMP_EXP_SHIFT));
 #pragma unroll
     for (int l = 0; l < NL; ++l) {
-      const float4 a = blk[2 + LA + l];
+      const float4 a = blk[2 + l];
       const float av[4] = {a.x, a.y, a.z, a.w};
 #pragma unroll
       for (int u = 0; u < 4; ++u) R[u][l] = __fmaf_rn(av[u], E[u], R[u][l]);
@@ -424,7 +423,7 @@ __device__ __forceinline__ void radial4s(const float* __restrict__ tab_e, int km
 // pair, and the exponentials' errors count against sum_q |A_q| E_q rather
 // than against the factor.  (A separate instantiation of the backward
 // kernel: a runtime branch would raise the register count of every one.)
-template <int L, int NL = L + 2, bool PADG = true, int LA = 0>
+template <int L, int NL = L + 2, bool PADG = true>
 __device__ __forceinline__ void radial4x(const float* __restrict__ tab_e, int kmax, int sg, float r2h,
                                          float r2l, float (&R)[4][NL]) {
   constexpr int RB = gmp_rad_block(L);
@@ -443,7 +442,7 @@ __device__ __forceinline__ void radial4x(const float* __restrict__ tab_e, int km
     E[3] = gmp_exp_neg_shifted(bh.w, bl.w, r2h, r2l);
 #pragma unroll
     for (int l = 0; l < NL; ++l) {
-      const float4 a = blk[2 + LA + l];
+      const float4 a = blk[2 + l];
       const float av[4] = {a.x, a.y, a.z, a.w};
 #pragma unroll
       for (int u = 0; u < 4; ++u) R[u][l] = __fmaf_rn(av[u], E[u], R[u][l]);
@@ -454,7 +453,7 @@ __device__ __forceinline__ void radial4x(const float* __restrict__ tab_e, int km
 // The scaled radial factors of radial4s on packed FP32 pairs, sigmas (0,1)
 // and (2,3) of the group: bit-identical to the scalar form, half the issue
 // slots.
-template <int L, int NL = L + 2, bool PADG = true, int LA = 0>
+template <int L, int NL = L + 2, bool PADG = true>
 __device__ __forceinline__ void radial4p(const float* __restrict__ tab_e, int kmax, int sg, float r2h,
                                          float (&R)[4][NL]) {
   constexpr int RB = gmp_rad_block(L);
@@ -472,7 +471,7 @@ __device__ __forceinline__ void radial4p(const float* __restrict__ tab_e, int km
     const float2 E0 = make_float2(gmp_ex2(x0.x), gmp_ex2(x0.y)), E1 = make_float2(gmp_ex2(x1.x), gmp_ex2(x1.y));
 #pragma unroll
     for (int l = 0; l < NL; ++l) {
-      const float4 a = blk[2 + LA + l];
+      const float4 a = blk[2 + l];
       Rp[0][l] = gmp_fma2(make_float2(a.x, a.y), E0, Rp[0][l]);
       Rp[1][l] = gmp_fma2(make_float2(a.z, a.w), E1, Rp[1][l]);
     }
@@ -1109,36 +1108,36 @@ __device__ __forceinline__ void shift_contract_order(const float* lam, const flo
 }
 
 // One pair's part of the gradient of sum_k lam_k R_l(r^2) S_k(d) from the
-// orders LA .. LB, lam_k = sum_s Lam_{s,k} R_{s,l} and lamd_k with dR_l/dr^2 =
+// orders 0 .. L, lam_k = sum_s Lam_{s,k} R_{s,l} and lamd_k with dR_l/dr^2 =
 // -beta R_{l+1}: adds to
 //   A = sum_k lamd_k S_k, B = sum_k (2l_k+1) lam_k S_k, V = sum_k lam_k S_{k+e},
 // from which grad = d (2 A + B / r^2) - V / r^2 (r^2 > 0).  At d = 0 only order
 // 1 has a gradient: g1 = (lam_x, lam_y, lam_z).
 // PACKED: radial factors on packed FP32 pairs (same results, fewer issue
 // slots); MIXED: exact exponentials (coefficients of both signs).
-template <int L, int NS, int LA, int LB, bool PACKED, bool PADG, bool MIXED>
-__device__ __forceinline__ void adjoint_range(const GmpPass& P, const float* __restrict__ tab_e,
+template <int L, int NS, bool PACKED, bool PADG, bool MIXED>
+__device__ __forceinline__ void pair_adjoint(const GmpPass& P, const float* __restrict__ tab_e,
                                               const float* __restrict__ Lam, float dx, float dy, float dz, float r2h,
                                               float r2l, float r2c, float& A, float& B, float (&V)[3], float (&g1)[3]) {
   using SH = Shape<L, NS>;
-  constexpr int K0 = LA * LA, K1 = (LB + 1) * (LB + 1), NL = LB - LA + 2;
-  // MCSH values of orders up to LB first (order LB + 1 after the sigma loop):
+  constexpr int K1 = (L + 1) * (L + 1), NL = L + 2;
+  // MCSH values of orders up to L first (order L + 1 after the sigma loop):
   // the sigma loop then contracts them directly, so that only the
   // radial-weighted adjoints lam (not their derivative counterparts) are live
   // beside them
-  float S[(LB + 2) * (LB + 2)];
-  GmpMcsh<LB>::eval(dx, dy, dz, r2c, S);
+  float S[(L + 2) * (L + 2)];
+  GmpMcsh<L>::eval(dx, dy, dz, r2c, S);
   float lam[K1];
 #pragma unroll
-  for (int k = K0; k < K1; ++k) lam[k] = 0.0f;
+  for (int k = 0; k < K1; ++k) lam[k] = 0.0f;
   for (int sg = 0; sg < SH::NSB; ++sg) {
-    float R[4][NL];  // orders LA .. LB + 1
+    float R[4][NL];  // orders 0 .. L + 1
     if constexpr (MIXED)
-      radial4x<L, NL, PADG, LA>(tab_e, P.kmax, sg, r2h, r2l, R);
+      radial4x<L, NL, PADG>(tab_e, P.kmax, sg, r2h, r2l, R);
     else if constexpr (PACKED)
-      radial4p<L, NL, PADG, LA>(tab_e, P.kmax, sg, r2h, R);
+      radial4p<L, NL, PADG>(tab_e, P.kmax, sg, r2h, R);
     else
-      radial4s<L, NL, PADG, LA>(tab_e, P.kmax, sg, r2h, R);
+      radial4s<L, NL, PADG>(tab_e, P.kmax, sg, r2h, R);
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const float nb = P.nbeta[4 * sg + u];
@@ -1146,14 +1145,14 @@ __device__ __forceinline__ void adjoint_range(const GmpPass& P, const float* __r
       float pl[NL - 1];
 #pragma unroll
       for (int l = 0; l < NL - 1; ++l) pl[l] = 0.0f;
-      static_for<(K1 + 3) / 4 - K0 / 4>([&](auto cq) {
-        constexpr int c4 = K0 / 4 + decltype(cq)::value;
+      static_for<(K1 + 3) / 4>([&](auto cq) {
+        constexpr int c4 = decltype(cq)::value;
         const float4 lv4 = *reinterpret_cast<const float4*>(lrow + 4 * c4);
         const float lv[4] = {lv4.x, lv4.y, lv4.z, lv4.w};
         static_for<4>([&](auto tt) {
           constexpr int k = 4 * c4 + decltype(tt)::value;
-          if constexpr (k >= K0 && k < K1) {
-            constexpr int l = order_of(k) - LA;
+          if constexpr (k < K1) {
+            constexpr int l = order_of(k);
             lam[k] = __fmaf_rn(lv[decltype(tt)::value], R[u][l], lam[k]);
             pl[l] = __fmaf_rn(lv[decltype(tt)::value], S[k], pl[l]);
           }
@@ -1166,20 +1165,14 @@ __device__ __forceinline__ void adjoint_range(const GmpPass& P, const float* __r
       A = __fmaf_rn(nb, a, A);
     }
   }
-  GmpMcsh<LB + 1>::eval_top(dx, dy, dz, r2c, S);
-  if constexpr (LA == 0) GmpMcsh<LB>::shift_contract(lam, S, V);
-  static_for<LB - LA + 1>([&](auto ll) {
-    constexpr int l = LA + decltype(ll)::value;
+  GmpMcsh<L + 1>::eval_top(dx, dy, dz, r2c, S);
+  GmpMcsh<L>::shift_contract(lam, S, V);
+  static_for<L + 1>([&](auto ll) {
+    constexpr int l = decltype(ll)::value;
     float b = 0.0f;
 #pragma unroll
     for (int k = l * l; k < (l + 1) * (l + 1); ++k) b = __fmaf_rn(lam[k], S[k], b);
     B = __fmaf_rn((float)(2 * l + 1), b, B);
-    if constexpr (LA > 0) {
-      float W[3];
-      shift_contract_order<l>(lam, S, W);
-#pragma unroll
-      for (int v = 0; v < 3; ++v) V[v] = __fadd_rn(V[v], W[v]);
-    }
     if constexpr (l == 1) {  // independent order-1 components: (0,1,0), (0,0,1), (1,0,0) at flat 1, 2, 3
       g1[0] = lam[3];
       g1[1] = lam[1];
@@ -1192,15 +1185,12 @@ __device__ __forceinline__ void adjoint_range(const GmpPass& P, const float* __r
 // sums and MCSH values of a pair stay in registers.  Orders 0-4 do in 96
 // registers, 20 warps per SM (10,000 structures, orders 0-4 x 8 sigmas, GB300:
 // 5.76 ms at 12 warps, 4.80 at 16, 4.67 at 20), orders 0-5 in 128, orders 0-6
-// in 168 (12 warps).  The strain derivative's kernel takes orders 0-6 in two
-// ranges, 0-4 and the rest, which repeat the exponentials (10% more
-// instructions) but fit 128 registers: 1.70 -> 1.66 ms on a 32,768-atom slab.
-// Without the strain sums the two ranges lose: 6.95 against 6.80 ms on the
-// 262,144-atom slab.
+// in 168 (12 warps).  Orders 0-6 in two ranges at 128 registers repeat the
+// exponentials: 6.95 against 6.80 ms on the 262,144-atom slab; with the strain
+// sums 1661 against 1673 us on 32,768 atoms, but the strain derivative came out
+// 3% further off.
 template <int L, bool VIRIAL>
-constexpr int back_split() { return L >= 6 && VIRIAL ? 5 : L + 1; }
-template <int L, bool VIRIAL>
-constexpr int back_threads() { return L <= 4 ? 640 : L == 5 || VIRIAL ? 512 : 384; }
+constexpr int back_threads() { return L <= 4 ? 640 : L == 5 ? 512 : 384; }
 // the radial table's sigma groups padded, but for the kernel whose 168
 // registers the padded stride would exceed
 template <int L, bool VIRIAL>
@@ -1219,7 +1209,6 @@ __device__ __forceinline__ void backward_sweep(const KParams& K, const float* __
                                                const float* __restrict__ Lam, float gd, float* Wv = nullptr) {
   const GmpPass& P = K.pass;
   const int lane = threadIdx.x & 31;
-  constexpr int SPLIT = back_split<L, VIRIAL>();
   float own[3] = {0.0f, 0.0f, 0.0f};
   if constexpr (VIRIAL) {
 #pragma unroll
@@ -1233,9 +1222,7 @@ __device__ __forceinline__ void backward_sweep(const KParams& K, const float* __
     const float r2c = mcsh_r2(dx, dy, dz);
     const float* tab_e = s_rad + (size_t)e * rad_elem_stride(L, NS, P.kmax, PADG);
     float A = 0.0f, B = 0.0f, V[3] = {0.0f, 0.0f, 0.0f}, g1[3] = {0.0f, 0.0f, 0.0f};
-    adjoint_range<L, NS, 0, SPLIT - 1, PACKED, PADG, MIXED>(P, tab_e, Lam, dx, dy, dz, r2h, r2l, r2c, A, B, V, g1);
-    if constexpr (SPLIT <= L)
-      adjoint_range<L, NS, SPLIT, L, PACKED, PADG, MIXED>(P, tab_e, Lam, dx, dy, dz, r2h, r2l, r2c, A, B, V, g1);
+    pair_adjoint<L, NS, PACKED, PADG, MIXED>(P, tab_e, Lam, dx, dy, dz, r2h, r2l, r2c, A, B, V, g1);
     float g[3];
     if (r2c > 0.0f) {
       const float inv = 1.0f / r2c;

@@ -997,14 +997,19 @@ __global__ void __launch_bounds__(128, 8) k_neighbors(const GmpStruct* __restric
       return;
     }
   }
-  // image index of an accepted slot's atom from its packed (m0, m1, m2) and wrap
+  // image index of an accepted slot's atom from its packed (m0, m1, m2) and
+  // wrap; one that does not fit is flagged and replaced, so that the sort keys
+  // and records made from it keep naming their atom (10 bits an axis)
   auto image = [&](int m, int wrap, int* n) {
     int wj[3], mm[3];
     gmp_unpack_shift(wrap, wj);
     gmp_unpack_shift(m, mm);
 #pragma unroll
     for (int k = 0; k < 3; ++k) n[k] = mm[k] + wi[k] - wj[k];
-    if (out_of_range(n)) atomicOr(err, GMP_DEV_SHIFT_RANGE);
+    if (out_of_range(n)) {
+      atomicOr(err, GMP_DEV_SHIFT_RANGE);
+      n[0] = n[1] = n[2] = 0;
+    }
   };
   unsigned long long* skey = reinterpret_cast<unsigned long long*>(keys);
   if (fill == 2) {

@@ -1349,12 +1349,15 @@ static gmp_status vjp_impl(gmp_handle h, int32_t n_struct, const int64_t* atom_o
   if (h->passes.size() > 1) GMP_CK(h->grad_acc.ensure(sizeof(double) * 3 * N), "grad_acc");
   {
     // the finishing kernel leaves the bins empty; new ones, and those of a call
-    // that did not get that far, are cleared here
-    void* const old = h->gbins.p;
+    // that did not get that far, are cleared here (a buffer that grew may well
+    // lie where it lay before: its size tells)
+    const size_t old = h->gbins.bytes;
     GMP_CK(h->gbins.ensure(sizeof(unsigned long long) * 3 * gmpk::kGradBins * N), "gradient bins");
-    if (h->gbins.p != old || !h->gbins_empty)
+    if (h->gbins.bytes != old || !h->gbins_empty) {
+      h->gbins_empty = false;
       GMP_CK(cudaMemsetAsync(h->gbins.p, 0, h->gbins.bytes, st), "clear bins");
-    h->gbins_empty = true;
+      h->gbins_empty = true;
+    }
   }
   GMP_CK(h->own.ensure(sizeof(double) * 3 * N), "own");
   if (vir) GMP_CK(h->vir_c.ensure(sizeof(double) * 9 * N), "vir_c");

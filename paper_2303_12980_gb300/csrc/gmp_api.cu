@@ -532,6 +532,18 @@ gmp_status run_sequence(gmp_ctx* h, cudaStream_t st, Seq& seq) {
   return r;
 }
 
+// Room for a guessed number of pairs.  A buffer that has to grow for a guess
+// takes at most a sixteenth of the free memory (a batch unlike the last one can
+// ask for any multiple of what it needs); false: count instead.
+bool room_for_guess(gmp_ctx* h, size_t bytes) {
+  if (bytes <= h->pairs.bytes) return true;
+  size_t free_b = 0, total = 0;
+  if (cudaMemGetInfo(&free_b, &total) == cudaSuccess && bytes <= free_b / 16 && h->pairs.ensure(bytes) == cudaSuccess)
+    return true;
+  cudaGetLastError();
+  return false;
+}
+
 // Exact neighbor lists of the NC centers C over the binned atoms into
 // h->pairs / h->nbr_off.  With single_ok and an earlier build to guess the
 // capacities from, one enumeration pass whose outcome finish_lists reads
@@ -557,8 +569,7 @@ gmp_status neighbor_lists(gmp_ctx* h, const GmpCenters& C, int64_t NC, const dou
     const int64_t cap = (int64_t)(last.per_center * 1.125 * (double)NC) + 4096;
     int keys = 32;
     while (keys < last.max_m + last.max_m / 8 + 8) keys <<= 1;
-    if ((size_t)keys * 8 <= 200 * 1024) {
-      GMP_CK(h->pairs.ensure(sizeof(GmpPair) * cap), "pairs");
+    if ((size_t)keys * 8 <= 200 * 1024 && room_for_guess(h, sizeof(GmpPair) * cap)) {
       GMP_CK(h->nbr_rng.ensure(sizeof(int64_t) * 2 * NC), "nbr_rng");
       GMP_CK(gmp_launch_neighbor_pass(sorted ? 2 : 1, h->structs.as<GmpStruct>(), h->grid.as<GmpGrid>(), C, NC, h->cutoff, pos,
                                       h->atom_xh.as<float4>(), h->atom_xl.as<float4>(), h->bin_start.as<int32_t>(),
@@ -627,7 +638,8 @@ gmp_status neighbor_lists(gmp_ctx* h, const GmpCenters& C, int64_t NC, const dou
   while (keys < maxm) keys <<= 1;
   if ((size_t)keys * 8 > 200 * 1024)
     return fail(h, GMP_ERR_CAPACITY, "a center has " + std::to_string(maxm) + " neighbor images (limit 25600)");
-  GMP_CK(h->pairs.ensure(sizeof(GmpPair) * (h->P > 0 ? h->P : 1)), "pairs");
+  // (ensure's slack and these 4,096 hold what the next batch of this kind guesses)
+  GMP_CK(h->pairs.ensure(sizeof(GmpPair) * (h->P + 4096)), "pairs");
   GMP_CK(gmp_launch_neighbor_pass(sorted ? 2 : 1, h->structs.as<GmpStruct>(), h->grid.as<GmpGrid>(), C, NC,
                                   h->cutoff, pos, h->atom_xh.as<float4>(), h->atom_xl.as<float4>(),
                                   h->bin_start.as<int32_t>(), h->bin_y.as<float4>(), h->bin_je.as<int2>(), h->n_el,

@@ -21,23 +21,27 @@ size_t smem_bytes(const GmpPass& P, int warps, bool pad = true) {
 template <int L, int NS>
 cudaError_t launch(int kind, const KParams& K, GmpShape shape, GmpLaunchPlan* plan, cudaStream_t st, int sm_count,
                    int64_t* launches) {
-  const int tile = (kind == GMP_KIND_FORWARD && shape.tile == 32) ? 32 : 16;
+  constexpr size_t kMaxSmem = 227 * 1024;
+  // the kernels that stage more a warp give way to the ones that stage less
+  // where not even one of their warps fits beside the tables
+  const int tile = kind == GMP_KIND_FORWARD && shape.tile == 32 && smem_bytes<L, NS, 32>(K.pass, 1) <= kMaxSmem ? 32 : 16;
+  size_t jac_r_floats = 0;  // per warp of k_jacobian_r (0: not used)
   void (*fn)(KParams) = kind == GMP_KIND_FORWARD    ? (tile == 32 ? k_forward<L, NS, 32> : k_forward<L, NS, 16>)
                         : kind == GMP_KIND_VJP      ? k_vjp<L, NS>
                         : kind == GMP_KIND_BACKWARD
                             ? (K.pass.mixed_sign ? k_backward<L, NS, false, true> : k_backward<L, NS, false, false>)
                         : kind == GMP_KIND_BACKWARD_VIRIAL
                             ? (K.pass.mixed_sign ? k_backward<L, NS, true, true> : k_backward<L, NS, true, false>)
-                            : nullptr;
+                            : k_jacobian<L, NS>;
   if constexpr (L <= kJacRegOrders) {
-    if (kind == GMP_KIND_JACOBIAN) fn = k_jacobian_r<L, NS>;
-  } else {
-    if (kind == GMP_KIND_JACOBIAN) fn = k_jacobian<L, NS>;
+    if (kind == GMP_KIND_JACOBIAN &&
+        sizeof(float) * (table_floats(K.pass.n_el, L, NS, K.pass.kmax) + JacShape<L, NS>::WARP_FLOATS) <= kMaxSmem) {
+      fn = k_jacobian_r<L, NS>;
+      jac_r_floats = JacShape<L, NS>::WARP_FLOATS;
+    }
   }
   auto smem_of = [&](int w) -> size_t {
-    if constexpr (L <= kJacRegOrders)
-      if (kind == GMP_KIND_JACOBIAN)
-        return sizeof(float) * (table_floats(K.pass.n_el, L, NS, K.pass.kmax) + (size_t)w * JacShape<L, NS>::WARP_FLOATS);
+    if (jac_r_floats) return sizeof(float) * (table_floats(K.pass.n_el, L, NS, K.pass.kmax) + (size_t)w * jac_r_floats);
     if (kind == GMP_KIND_BACKWARD || kind == GMP_KIND_BACKWARD_VIRIAL) {
       const bool vir = kind == GMP_KIND_BACKWARD_VIRIAL;
       return sizeof(float) * (table_floats(K.pass.n_el, L, NS, K.pass.kmax, vir ? back_pad<L, true>() : back_pad<L, false>()) +
@@ -58,12 +62,12 @@ cudaError_t launch(int kind, const KParams& K, GmpShape shape, GmpLaunchPlan* pl
     if (e != cudaSuccess) return e;
     // always the same limit, so that no handle's launch depends on which one
     // set it last
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
     if (e != cudaSuccess) return e;
     int warps = fa.maxThreadsPerBlock / 32;
     if (warps > 20) warps = 20;
     if (want > 0 && want < warps) warps = want;
-    while (warps > 1 && smem_of(warps) > 227 * 1024) --warps;
+    while (warps > 1 && smem_of(warps) > kMaxSmem) --warps;
     if (want <= 0) {
       // untuned: the CTA size with the most resident warps, of equals the
       // smallest with at least 4 (registers and the tables' share of the
@@ -73,7 +77,7 @@ cudaError_t launch(int kind, const KParams& K, GmpShape shape, GmpLaunchPlan* pl
       // and 167 in as many warps of 4-warp ones)
       int best_w = warps, best_res = 0;
       for (int w = warps; w >= 1; --w) {
-        if (smem_of(w) > 227 * 1024) continue;
+        if (smem_of(w) > kMaxSmem) continue;
         int ps = 0;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, fn, w * 32, smem_of(w));
         if (e != cudaSuccess) return e;
@@ -81,7 +85,7 @@ cudaError_t launch(int kind, const KParams& K, GmpShape shape, GmpLaunchPlan* pl
       }
       warps = best_w;
     }
-    if (smem_of(warps) > 227 * 1024) return cudaErrorInvalidConfiguration;
+    if (smem_of(warps) > kMaxSmem) return cudaErrorInvalidConfiguration;
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, warps * 32, smem_of(warps));
     if (e != cudaSuccess) return e;

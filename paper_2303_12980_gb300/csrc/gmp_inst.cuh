@@ -16,14 +16,31 @@ size_t smem_bytes(const GmpPass& P, int warps, bool pad = true) {
                           (size_t)warps * Shape<L, NS, TILE>::WARP_FLOATS);
 }
 
+// Whether k_jacobian_r (orders up to kJacRegOrders) is faster than k_jacobian
+// beside these tables: it stages 2.6 times as much a warp, and with fewer than 6
+// of its warps per SM that costs more than its fewer instructions spare.
+// Jacobian kernel, 3,072 centers of 79 pairs, us, k_jacobian -> k_jacobian_r (GB300;
+// elements x Gaussians, warps that fit beside the tables):
+//   orders 0-4, 16 sigmas   12 x 16 (6) 387 -> 224, 24 x 8 (6) 242 -> 184,
+//                           24 x 16 (1) 596 -> 962, 48 x 8 (1) 494 -> 802
+//   orders 0-3              8 sigmas 48 x 16 (3) 151 -> 189, 16 sigmas 12 x 16 (9)
+//                           381 -> 165, 48 x 8 (2) 234 -> 348
+//   orders 0-2, 16 sigmas   24 x 8 (12) 155 -> 131, 48 x 8 (5) 178 -> 230
+//   orders 0-2, 4 sigmas    6 x 8 44 -> 42, 12 x 8 45 -> 46, 24 x 16 56 -> 64
+template <int L, int NS>
+bool jacobian_r_pays(const GmpPass& P, size_t max_smem) {
+  if (L == 2 && NS == 4 && P.n_el > 6) return false;
+  return sizeof(float) * (table_floats(P.n_el, L, NS, P.kmax) + 6 * (size_t)JacShape<L, NS>::WARP_FLOATS) <= max_smem;
+}
+
 // shape.tile: 16 or 32 pairs per forward tile; shape.warps: warps per CTA
 // (0 = the size with the most resident warps).
 template <int L, int NS>
 cudaError_t launch(int kind, const KParams& K, GmpShape shape, GmpLaunchPlan* plan, cudaStream_t st, int sm_count,
                    int64_t* launches) {
   constexpr size_t kMaxSmem = 227 * 1024;
-  // the kernels that stage more a warp give way to the ones that stage less
-  // where not even one of their warps fits beside the tables
+  // a tile of 32 pairs gives way to one of 16 where not even one warp of it fits
+  // beside the tables
   const int tile = kind == GMP_KIND_FORWARD && shape.tile == 32 && smem_bytes<L, NS, 32>(K.pass, 1) <= kMaxSmem ? 32 : 16;
   size_t jac_r_floats = 0;  // per warp of k_jacobian_r (0: not used)
   void (*fn)(KParams) = kind == GMP_KIND_FORWARD    ? (tile == 32 ? k_forward<L, NS, 32> : k_forward<L, NS, 16>)
@@ -34,8 +51,7 @@ cudaError_t launch(int kind, const KParams& K, GmpShape shape, GmpLaunchPlan* pl
                             ? (K.pass.mixed_sign ? k_backward<L, NS, true, true> : k_backward<L, NS, true, false>)
                             : k_jacobian<L, NS>;
   if constexpr (L <= kJacRegOrders) {
-    if (kind == GMP_KIND_JACOBIAN &&
-        sizeof(float) * (table_floats(K.pass.n_el, L, NS, K.pass.kmax) + JacShape<L, NS>::WARP_FLOATS) <= kMaxSmem) {
+    if (kind == GMP_KIND_JACOBIAN && jacobian_r_pays<L, NS>(K.pass, kMaxSmem)) {
       fn = k_jacobian_r<L, NS>;
       jac_r_floats = JacShape<L, NS>::WARP_FLOATS;
     }

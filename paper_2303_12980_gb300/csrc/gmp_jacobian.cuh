@@ -1,7 +1,6 @@
 // Jacobian rows for orders up to 4 (k_jacobian in gmp_kernels.cuh takes the
 // higher ones, whose coefficients below do not fit the registers, and tables
-// that leave no room for a warp's rows below: 18.9 KB at orders 0-4 x 16 sigmas
-// against 7.3).
+// that leave room for few warps' rows below: jacobian_r_pays).
 //
 // For center i, order l and sigma s, with P = sum_k lam_k S_k(d) and lam = d f /
 // d mu, a pair contributes d f / d d = 2 d (-beta R_{l+1}) P + R_l grad P.  The

@@ -49,3 +49,10 @@ def test_large_tables(torch, oracle_mod, lmax, n_sig, n_el, n_gauss):
     _, goff, gj, gjac = (x.cpu().numpy() for x in F.featurize_grad(*a))
     assert np.array_equal(goff, off) and np.array_equal(gj, j)
     assert grad_errors(gjac, jac, jabs, tau=JAC_TAU).max() <= GRAD_TOL
+
+
+# either side of the lines where the Jacobian kernel for orders up to 4 gives way
+@pytest.mark.parametrize("lmax,n_sig,n_el,n_gauss", [(4, 16, 21, 10), (4, 16, 22, 10), (2, 4, 6, 4), (2, 4, 7, 4), (2, 16, 38, 10),
+                                                     (2, 16, 39, 10)])
+def test_rows_either_side(torch, oracle_mod, lmax, n_sig, n_el, n_gauss):
+    test_large_tables(torch, oracle_mod, lmax, n_sig, n_el, n_gauss)

@@ -1081,7 +1081,7 @@ gmp_status gmp_create(const gmp_params* p, int device, gmp_handle* out) {
     GmpPass& P = pd.pass;
     P.lmax = L;
     P.nsig = ns;
-    pd.fwd.tile = gmp_forward_tile(pd.L, pd.NS, h->n_el);
+    pd.fwd.tile = gmp_forward_tile(pd.L, pd.NS, h->n_el, h->kmax);
     P.nsig_pad = pd.NS;
     P.kmax = h->kmax;
     P.n_el = h->n_el;

@@ -56,3 +56,13 @@ def test_large_tables(torch, oracle_mod, lmax, n_sig, n_el, n_gauss):
                                                      (2, 16, 39, 10)])
 def test_rows_either_side(torch, oracle_mod, lmax, n_sig, n_el, n_gauss):
     test_large_tables(torch, oracle_mod, lmax, n_sig, n_el, n_gauss)
+
+
+# the untuned forward tile of 32 pairs pays beside small tables only
+@pytest.mark.parametrize("lmax,n_sig,n_el,n_gauss,tile", [(2, 8, 10, 8, 32), (2, 8, 40, 8, 16), (3, 7, 20, 4, 32), (3, 7, 6, 32, 16),
+                                                          (4, 8, 3, 5, 32), (4, 8, 3, 16, 16), (4, 8, 10, 1, 16), (2, 16, 10, 4, 32),
+                                                          (2, 16, 20, 4, 16), (1, 8, 1, 4, 16), (6, 16, 1, 4, 16)])
+def test_untuned_tile(torch, lmax, n_sig, n_el, n_gauss, tile):
+    from paper_2303_12980_gb300.binding import GMPFeaturizer
+    F = GMPFeaturizer.from_workload(_workload(lmax, n_sig, n_el, n_gauss))
+    assert F.tuning()[0] == tile

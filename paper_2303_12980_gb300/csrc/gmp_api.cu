@@ -518,6 +518,16 @@ gmp_status finish_lists(gmp_ctx* h, cudaStream_t st) {
   return GMP_ERR_CAPACITY;
 }
 
+// The end of a call's device sequence: one that failed takes along what its
+// lists flagged and nobody read.
+gmp_status settle(gmp_ctx* h, cudaStream_t st, gmp_status r) {
+  if (r != GMP_OK) {
+    h->lists_pending = false;
+    cudaMemsetAsync(h->scalars.p, 0, 4, st);  // (r is the error to report)
+  }
+  return r;
+}
+
 // Runs a call's device sequence and then reads the outcome of its neighbor
 // lists; a sequence whose lists outgrew the guess runs again, counting first.
 template <typename Seq>
@@ -525,11 +535,11 @@ gmp_status run_sequence(gmp_ctx* h, cudaStream_t st, Seq& seq) {
   h->lists_pending = h->lists_outgrown = h->exact_lists = false;
   gmp_status r = seq(false);
   if (r == GMP_OK) r = finish_lists(h, st);
-  if (!h->lists_outgrown) return r;
+  if (!h->lists_outgrown) return settle(h, st, r);
   h->exact_lists = true;
   r = seq(false);
   h->exact_lists = false;
-  return r;
+  return settle(h, st, r);
 }
 
 // Room for a guessed number of pairs.  A buffer that has to grow for a guess
@@ -1622,7 +1632,8 @@ gmp_status gmp_neighbors(gmp_handle h, int32_t n_struct, const int64_t* atom_off
   if (!nbr_off) return fail(h, GMP_ERR_INVALID_ARG, "nbr_off is required");
   Io io;
   if ((r = stage_inputs(h, N, pos, species, io, st)) != GMP_OK) return r;
-  if ((r = build_neighbors(h, n_struct, io.pos, io.species, N, st, true, false, true)) != GMP_OK) return r;
+  r = settle(h, st, build_neighbors(h, n_struct, io.pos, io.species, N, st, true, false, true));
+  if (r != GMP_OK) return r;
   *nnz_out = h->P;
   if (h->P > cap) return fail(h, GMP_ERR_CAPACITY, "neighbor list needs " + std::to_string(h->P) + " entries");
   if (h->P > 0 && (!nbr_j || !nbr_shift)) return fail(h, GMP_ERR_INVALID_ARG, "nbr_j and nbr_shift are required");

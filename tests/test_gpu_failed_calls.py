@@ -1,0 +1,44 @@
+"""A call that fails after its neighbor lists were queued (here: tables that no
+compute kernel fits beside) leaves nothing of them to the next one."""
+import numpy as np
+import pytest
+
+from paper_2303_12980_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def torch():
+    t = pytest.importorskip("torch")
+    if not t.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    return t
+
+
+@pytest.mark.parametrize("call", ["features", "vjp", "jacobian", "points"])
+@pytest.mark.parametrize("what", ["outgrown", "species"])
+def test_no_condition_is_left(torch, call, what):
+    from paper_2303_12980_gb300.binding import GMPError, GMPFeaturizer
+    rng = np.random.default_rng(4)
+    n_el = 2000
+    table = synth.gaussian_table(rng, [3] * n_el, 1)
+    pos, cell = synth.fcc_supercell(rng, 3.6, (4, 4, 4), 0.1)
+    n = len(pos)
+    put = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    sp = np.arange(n, dtype=np.int32)
+    lone = (put(np.arange(2)[:, None] * np.array([[3.0, 0, 0]])), put(sp[:2]), [0, 2], np.zeros((1, 3, 3)), [[0, 0, 0]])
+    dense = (put(pos), put(sp), [0, n], cell[None], [[1, 1, 1]])
+    bad = (dense[0], put(sp + n_el - 5), *dense[2:])
+    new = lambda: GMPFeaturizer([0], [0.5], 6.0, *table)
+    want = new().neighbors(*dense)
+    F = new()
+    F.neighbors(*(lone if what == "outgrown" else dense))  # the capacities of the next lists
+    a = dense if what == "outgrown" else bad
+    calls = {"features": lambda: F.featurize(*a), "vjp": lambda: F.featurize_vjp(*a, torch.ones((n, 1), device="cuda")),
+             "jacobian": lambda: F.featurize_grad(*a), "points": lambda: F.featurize_points(*a, a[0], [0, n])}
+    with pytest.raises(GMPError):
+        calls[call]()
+    F.sync()
+    for x, y in zip(F.neighbors(*dense), want):
+        assert torch.equal(x, y)

@@ -106,7 +106,8 @@ struct gmp_ctx {
   DevView structs, grid, atom_off;
   void* h_desc = nullptr;           // pinned staging of that copy
   size_t h_desc_bytes = 0;
-  cudaEvent_t ev_desc = nullptr;    // the copy is done with the staging
+  cudaEvent_t ev_desc = nullptr;    // the copy is done with the staging, struct_of written
+  bool desc_pending = false;        // ... and that is not known to have happened yet
   GmpGridMode grid_mode = GmpGridMode::kGiven;
   int max_atoms = 0, max_bins = 0;  // of one structure of the batch
   DevBuf struct_of, bbox, atom_xh, atom_xl, atom_u, atom_bin, atom_t, atom_y;
@@ -310,7 +311,14 @@ gmp_status upload_structures(gmp_ctx* h, int32_t S, const int64_t* atom_off, con
                     std::memcmp(h->last_off.data(), atom_off, sizeof(int64_t) * (S + 1)) == 0 &&
                     std::memcmp(h->last_cell.data(), cell, sizeof(double) * 9 * S) == 0 &&
                     std::memcmp(h->last_pbc.data(), pbc, S * 3) == 0;
-  if (same) return GMP_OK;
+  if (same) {
+    // (the call that uploaded it may have ended without waiting, on another stream)
+    if (h->desc_pending) {
+      h->desc_pending = cudaEventQuery(h->ev_desc) == cudaErrorNotReady;
+      if (h->desc_pending) GMP_CK(cudaStreamWaitEvent(st, h->ev_desc, 0), "batch description");
+    }
+    return GMP_OK;
+  }
   // one pinned staging block [structs | grid | atom_off], one copy
   const size_t o_grid = sizeof(GmpStruct) * (size_t)S, o_off = o_grid + sizeof(GmpGrid) * (size_t)S;
   const size_t bytes = o_off + sizeof(int64_t) * (size_t)(S + 1);
@@ -385,9 +393,10 @@ gmp_status upload_structures(gmp_ctx* h, int32_t S, const int64_t* atom_off, con
   GMP_CK(h->bbox.ensure(sizeof(unsigned long long) * 6 * S), "bbox");
   GMP_CK(h->struct_of.ensure(sizeof(int32_t) * (N > 0 ? N : 1)), "struct_of");
   GMP_CK(cudaMemcpyAsync(h->desc.p, h->h_desc, bytes, cudaMemcpyHostToDevice, st), "upload structs");
-  GMP_CK(cudaEventRecord(h->ev_desc, st), "event");
   if (N > 0 && !gmp_bin_structs_fits(N, max_atoms, max_bins))  // (that kernel writes it, on each call)
     GMP_CK(gmp_launch_struct_of(h->atom_off.as<int64_t>(), S, h->struct_of.as<int32_t>(), st, &h->launches), "struct_of");
+  GMP_CK(cudaEventRecord(h->ev_desc, st), "event");
+  h->desc_pending = true;
   ++h->struct_gen;
   h->last_off.assign(atom_off, atom_off + S + 1);
   h->last_cell.assign(cell, cell + 9 * S);

@@ -42,3 +42,26 @@ def test_no_condition_is_left(torch, call, what):
     F.sync()
     for x, y in zip(F.neighbors(*dense), want):
         assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("n", [2, 8])  # 32 and 2,048 atoms: one CTA a structure, or several kernels
+def test_description_uploaded_on_another_stream(torch, n):
+    """A call without points uploads the batch description behind what its stream
+    holds, and returns; the next call, on another stream, waits for it."""
+    from paper_2303_12980_gb300.binding import GMPFeaturizer
+    rng = np.random.default_rng(6)
+    pos, cell = synth.fcc_supercell(rng, 3.6, (n, n, n), 0.1)
+    w = synth._single("fcc", pos, cell, [1, 1, 0], rng.integers(0, 2, len(pos)).astype(np.int32),
+                      synth.gaussian_table(rng, [3, 4], 2), [0, 1, 2], [0.4, 0.8], 5.0)
+    a = (torch.from_numpy(w.positions).cuda(), torch.from_numpy(w.species).cuda(), w.atom_off, w.cells, w.pbc)
+    want = GMPFeaturizer.from_workload(w).featurize(*a)
+    F, s1, s2 = GMPFeaturizer.from_workload(w), torch.cuda.Stream(), torch.cuda.Stream()
+    none = torch.empty((0, 3), dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    with torch.cuda.stream(s1):
+        torch.cuda._sleep(200_000_000)  # about 0.1 s
+    F.featurize_points(*a, none, [0, 0], stream=s1)
+    got = F.featurize(*a, stream=s2)
+    assert s1.query()
+    s2.synchronize()
+    assert torch.equal(got, want)

@@ -113,8 +113,8 @@ struct gmp_ctx {
   DevBuf struct_of, bbox, atom_xh, atom_xl, atom_u, atom_bin, atom_t, atom_y;
   DevBuf bin_count, bin_cursor, bin_start, bin_y, bin_je, counts, nbr_off, scan_tmp, pairs;
   // error word, longest list, pair cursor, refinement queue counts and the
-  // work counters of a call's compute launches (kScalar* below); everything
-  // but the error word is cleared at the start of a call
+  // work counters of a call's compute launches (kScalar*); everything but the
+  // error word is cleared at the start of a call
   DevBuf scalars;
   int next_counter = 0;
   DevBuf grad_acc, jac_counts, jac_rows;
@@ -180,11 +180,6 @@ struct gmp_ctx {
 };
 
 namespace {
-
-// Byte offsets in gmp_ctx::scalars.
-constexpr size_t kScalarMaxM = 4, kScalarCursor = 8, kScalarFlags = 16, kScalarCounters = 80;  // the error word at 0
-constexpr int kCounters = 160;  // two per sigma pass (at most 64) and spares
-constexpr size_t kScalarBytes = kScalarCounters + 4 * kCounters;
 
 gmp_status fail(gmp_ctx* h, gmp_status st, const std::string& msg) {
   if (h) h->err = msg;

@@ -15,6 +15,15 @@
 #define GMP_DEV_SHIFT_RANGE 8u
 #define GMP_DEV_CAPACITY 16u
 
+// A handle's device words: the error word, the longest list, the pair cursor
+// (u64), the refinement queues' counts (u64 each), then the work counters of a
+// call's compute launches (byte offsets).
+constexpr size_t kScalarMaxM = 4, kScalarCursor = 8, kScalarFlags = 16, kScalarCounters = 80;
+constexpr int kCounters = 160;  // two per sigma pass (at most 64) and spares
+constexpr size_t kScalarBytes = kScalarCounters + 4 * kCounters;
+// A counter at or above this hands out no center (batches hold fewer).
+constexpr int kCounterClosed = 1 << 30;
+
 struct __align__(32) GmpD4 {
   double x, y, z, w;
 };
@@ -456,7 +465,9 @@ cudaError_t gmp_launch_point_prepare(const GmpStruct* d_structs, const GmpGrid* 
 // are the binned atoms (pos, atom_xh, atom_xl).  Records go to the CSR
 // offsets (from a count pass), or, with cursor (fill 1 or 2), to blocks
 // allocated from *cursor whose ranges are written to rng[i], rng[N + i].
-// Over-capacity blocks set GMP_DEV_CAPACITY.
+// Over-capacity blocks set GMP_DEV_CAPACITY, with cursor also the work counters
+// behind d_err (kScalarCounters) to kCounterClosed: the compute kernels that were
+// queued behind lists that are built again then have nothing to do.
 cudaError_t gmp_launch_neighbor_pass(int fill, const GmpStruct* d_structs, const GmpGrid* d_grid,
                                      const GmpCenters& C, int64_t N, double cutoff,
                                      const double* pos, const float4* atom_xh, const float4* atom_xl,

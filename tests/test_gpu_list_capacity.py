@@ -45,3 +45,36 @@ def test_guess_beyond_the_memory(torch, call):
         got = run(F, grid)
         torch.cuda.synchronize()
         assert torch.equal(got, want)
+
+
+def test_outgrown_lists_are_not_computed_on(torch):
+    """A batch with a fifth more pairs than the last one outgrows the guess: its
+    forward kernels together take about as long as the one of a batch that fits."""
+    from paper_2303_12980_gb300.binding import GMPFeaturizer
+    rng = np.random.default_rng(3)
+    table = synth.gaussian_table(rng, [3, 5], 6)
+
+    def batch(a):
+        pos, cell = synth.fcc_supercell(rng, a, (20, 20, 20), 0.1)
+        sp = torch.from_numpy(rng.integers(0, 2, len(pos)).astype(np.int32)).cuda()
+        return torch.from_numpy(pos).cuda(), sp, [0, len(pos)], cell[None], [[1, 1, 1]]
+
+    dense, sparse = batch(3.7), batch(3.95)
+    F = GMPFeaturizer(list(range(7)), np.geomspace(0.05, 1.5, 16), 8.0, *table)
+    want = F.featurize(*dense)
+
+    def forward_ms(n):
+        F.profile(True)
+        got = F.featurize(*dense)
+        torch.cuda.synchronize()
+        ms, count = F.profile_read()["features"]
+        F.profile(False)
+        assert count == n and torch.equal(got, want)
+        return ms
+
+    fits = min(forward_ms(1) for _ in range(3))
+    outgrown = []
+    for _ in range(3):
+        F.featurize(*sparse)
+        outgrown.append(forward_ms(2))
+    assert min(outgrown) < 1.4 * fits  # 1.9 when the partial lists are computed on

@@ -919,12 +919,16 @@ gmp_status grad_impl(gmp_ctx* h, int32_t n_struct, const int64_t* atom_off, cons
   GMP_CK(h->jac_counts.ensure(sizeof(int64_t) * (2 * n + 1)), "jac counts");
   int64_t* cnt = h->jac_counts.as<int64_t>();
   int64_t* joff = cnt + n;
-  for (const PassData& pd : h->passes)
-    GMP_CK(h->mu.ensure(sizeof(float) * (size_t)N * std::max(pd.pass.nsig, 1) * (pd.L + 1) * (pd.L + 1)), "moments");
   // features: into scratch, from which they are copied at the end (nothing is
   // written when the rows exceed `cap`)
-  GMP_CK(h->stage_feat.ensure(sizeof(float) * N * h->F), "feature scratch");
-  float* const fout = h->stage_feat.as<float>();
+  float* fout = nullptr;
+  auto buffers = [&]() -> gmp_status {
+    for (const PassData& pd : h->passes)
+      GMP_CK(h->mu.ensure(sizeof(float) * (size_t)N * std::max(pd.pass.nsig, 1) * (pd.L + 1) * (pd.L + 1)), "moments");
+    GMP_CK(h->stage_feat.ensure(sizeof(float) * N * h->F), "feature scratch");
+    fout = h->stage_feat.as<float>();
+    return begin_compute(h, N);
+  };
   // one pass's forward kernel (features, moments) and the refinement of the
   // flagged features and their moments, ahead of the pass's Jacobian rows
   auto forward = [&](size_t g) -> gmp_status {
@@ -946,12 +950,14 @@ gmp_status grad_impl(gmp_ctx* h, int32_t n_struct, const int64_t* atom_off, cons
     return GMP_OK;
   };
   // lists, row counts, and the first pass's features, which run while the host
-  // reads the number of rows
+  // reads the number of rows (unless they cannot fit: every center has a row; so a
+  // call that asks for their number computes and allocates no more than that)
+  const bool ahead = cap >= n;
   auto lists = [&](bool) -> gmp_status {
     gmp_status q = build_neighbors(h, n_struct, io.pos, io.species, N, st, true);
     if (q != GMP_OK) return q;
     GMP_CK(h->jac_rows.ensure(sizeof(int32_t) * std::max<int64_t>(h->cap_cur, 1)), "jac rows");
-    if ((q = begin_compute(h, N)) != GMP_OK) return q;
+    if (ahead && (q = buffers()) != GMP_OK) return q;
     const int64_t* nbeg = h->rng_mode ? h->nbr_rng.as<int64_t>() : h->nbr_off.as<int64_t>();
     const int64_t* nend = h->rng_mode ? h->nbr_rng.as<int64_t>() + N : h->nbr_off.as<int64_t>() + 1;
     GMP_CK(gmp_launch_jacobian_count(n, nbeg + c0, nend + c0, h->pairs.as<GmpPair>(), cnt,
@@ -959,7 +965,7 @@ gmp_status grad_impl(gmp_ctx* h, int32_t n_struct, const int64_t* atom_off, cons
     GMP_CK(gmp_exclusive_scan_i64(cnt, joff, n, h->scan_tmp.p, st, &h->launches), "jac scan");
     GMP_CK(cudaMemcpyAsync(h->h_small + 2, joff + n, sizeof(int64_t), cudaMemcpyDeviceToHost, st), "read nnz");
     GMP_CK(cudaEventRecord(h->ev_rows, st), "event");
-    return forward(0);
+    return ahead ? forward(0) : GMP_OK;
   };
   if ((r = run_sequence(h, st, lists)) != GMP_OK) return r;
   GMP_CK(cudaEventSynchronize(h->ev_rows), "jac sync");
@@ -976,8 +982,9 @@ gmp_status grad_impl(gmp_ctx* h, int32_t n_struct, const int64_t* atom_off, cons
     jd = tmp_jac.as<float>();
     jj = tmp_jj.as<int32_t>();
   }
+  if (!ahead && (r = buffers()) != GMP_OK) return r;
   for (size_t g = 0; g < h->passes.size(); ++g) {
-    if (g > 0 && (r = forward(g)) != GMP_OK) return r;
+    if ((g > 0 || !ahead) && (r = forward(g)) != GMP_OK) return r;
     PassData& pd = h->passes[g];
     gmpk::KParams K = base_params(h, pd, (int)g, N);
     K.N = c1;

@@ -78,3 +78,24 @@ def test_outgrown_lists_are_not_computed_on(torch):
         F.featurize(*sparse)
         outgrown.append(forward_ms(2))
     assert min(outgrown) < 1.4 * fits  # 1.9 when the partial lists are computed on
+
+
+def test_query_of_the_rows(torch):
+    """A Jacobian call whose buffers hold fewer rows than there are centers reads
+    their number and computes no features."""
+    from paper_2303_12980_gb300.binding import GMPFeaturizer
+    rng = np.random.default_rng(5)
+    pos, cell = synth.fcc_supercell(rng, 3.6, (3, 3, 3), 0.1)
+    n = len(pos)
+    a = (torch.from_numpy(pos).cuda(), torch.zeros(n, dtype=torch.int32, device="cuda"), [0, n], cell[None], [[1, 1, 1]])
+    F = GMPFeaturizer([0, 1, 2], [0.4, 0.8], 5.0, *synth.gaussian_table(rng, [3], 2))
+    F.profile(True)
+    first = F.featurize_grad(*a)  # asks for the rows, then takes them
+    torch.cuda.synchronize()
+    assert F.profile_read()["features"][1] == 1
+    for b, e in ((0, n), (5, 9), (3, 3)):
+        F._rows["grad"] = 0
+        got = F.featurize_grad(*a, centers=(b, e))
+        lo, hi = int(first[1][b]), int(first[1][e])
+        assert torch.equal(got[0], first[0][b:e]) and torch.equal(got[1], first[1][b:e + 1] - lo)
+        assert torch.equal(got[2], first[2][lo:hi]) and torch.equal(got[3], first[3][lo:hi])

@@ -154,6 +154,8 @@ struct gmp_ctx {
   bool lists_outgrown = false; // ... and found to exceed its capacities
   bool exact_lists = false;    // count before filling (set for a rerun)
   cudaEvent_t ev_lists = nullptr;
+  bool wait_blocks = false;    // the process waits for the device blocked (cudaDeviceScheduleBlockingSync)
+  bool wait_yields = false;    // ... or yielding
   cudaEvent_t ev_rows = nullptr;  // the number of Jacobian rows is read
   // pinned host scratch for small readbacks
   int64_t* h_small = nullptr;
@@ -492,10 +494,12 @@ gmp_status finish_lists(gmp_ctx* h, cudaStream_t st) {
   unsigned long long err_maxm, pairs;
   if (h->lists_report) {
     // the first compute kernel writes it when it starts; the stream's state is
-    // looked at now and then, so that a kernel that never comes is noticed
+    // looked at now and then, so that a kernel that never comes is noticed, and
+    // other threads get the core meanwhile
     volatile GmpListReport* r = h->report;
     for (uint32_t n = 1; r->build != h->build; ++n) {
-      if (n % 4096 != 0) continue;
+      if (n % (h->wait_yields ? 64 : 4096) != 0) continue;
+      std::this_thread::yield();
       const cudaError_t e = cudaStreamQuery(st);
       if (e == cudaErrorNotReady) continue;
       if (e != cudaSuccess) return cuda_fail(h, e, "neighbor wait");
@@ -591,9 +595,9 @@ gmp_status neighbor_lists(gmp_ctx* h, const GmpCenters& C, int64_t NC, const dou
                                       h->pairs.as<GmpPair>(), cap, keys, d_maxm, d_err, st, h->sm_count, L, d_cursor,
                                       h->nbr_rng.as<int64_t>()),
              "neighbor single pass");
-      h->lists_report = report;
+      h->lists_report = report && !h->wait_blocks;
       ++h->build;
-      if (!report) {
+      if (!h->lists_report) {
         GMP_CK(cudaMemcpyAsync(h->h_small, d_err, 16, cudaMemcpyDeviceToHost, st), "read err, longest, P");
         GMP_CK(cudaEventRecord(h->ev_lists, st), "event");
       }
@@ -1249,10 +1253,16 @@ gmp_status gmp_create(const gmp_params* p, int device, gmp_handle* out) {
   std::memset(h->h_small, 0, 128);
   h->report = reinterpret_cast<GmpListReport*>(h->h_small + 8);
   if (cudaEventCreateWithFlags(&h->ev, cudaEventDisableTiming) != cudaSuccess) { cudaGetLastError(); return bad("event"); }
+  // the host waits for events as the process asked the device to be waited for
+  unsigned dev_flags = 0;
+  if (cudaGetDeviceFlags(&dev_flags) != cudaSuccess) { cudaGetLastError(); dev_flags = 0; }
+  h->wait_blocks = (dev_flags & cudaDeviceScheduleMask) == cudaDeviceScheduleBlockingSync;
+  h->wait_yields = (dev_flags & cudaDeviceScheduleMask) == cudaDeviceScheduleYield;
+  const unsigned ev_waited = cudaEventDisableTiming | (h->wait_blocks ? cudaEventBlockingSync : 0);
   if (cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking) != cudaSuccess ||
-      cudaEventCreateWithFlags(&h->ev_desc, cudaEventDisableTiming) != cudaSuccess ||
-      cudaEventCreateWithFlags(&h->ev_lists, cudaEventDisableTiming) != cudaSuccess ||
-      cudaEventCreateWithFlags(&h->ev_rows, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&h->ev_desc, ev_waited) != cudaSuccess ||
+      cudaEventCreateWithFlags(&h->ev_lists, ev_waited) != cudaSuccess ||
+      cudaEventCreateWithFlags(&h->ev_rows, ev_waited) != cudaSuccess ||
       cudaEventCreateWithFlags(&h->ev_in, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&h->ev_feat, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&h->ev_out, cudaEventDisableTiming) != cudaSuccess) {

@@ -128,9 +128,14 @@ struct GmpPass {
 // kernels let the next one start at once; the compute kernels do not, since
 // CTAs that wait for a kernel of a millisecond only take room from it (262,144
 // atom slab 13.39 ms a pass with, 13.19 without; 4,096-atom crystal features 136
-// us with no dependents at all, 128 so).  Everything that a kernel reads from
-// memory another kernel wrote is addressed through the returned thread index
-// or comes after an atomic behind it, so that no load moves ahead of the wait.
+// us with no dependents at all, 128 so).  What a kernel reads from memory that
+// another kernel wrote is addressed through the returned thread index, comes after
+// an atomic behind it, or is read through a pointer that is not const __restrict__,
+// so that no load moves ahead of the wait.  Several kernels of a chain may be
+// resident at once, so a non-coherent load (const __restrict__) could find a line
+// that an earlier one of them brought into the SM's L1: what one kernel reads and
+// another rewrites before a third reads it (the structures' bounds and grids, the
+// bin counts that become slot lists, a scan's sums) is read through plain pointers.
 __device__ __forceinline__ unsigned gmp_after_predecessor(unsigned tid) {
   unsigned t;
   asm volatile("griddepcontrol.wait;\n\tmov.b32 %0, %1;" : "=r"(t) : "r"(tid) : "memory");

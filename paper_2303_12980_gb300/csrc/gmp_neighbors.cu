@@ -364,7 +364,7 @@ __global__ void k_bin_scatter(int64_t N, const int32_t* __restrict__ atom_bin,
 // deterministic); the bin's slot list is read in parallel, not sorted in
 // place.
 __global__ void k_bin_place(int64_t N, const int32_t* __restrict__ atom_bin, const int32_t* __restrict__ bin_start,
-                            const int32_t* __restrict__ slot_atom, const float4* __restrict__ atom_y,
+                            const int32_t* slot_atom, const float4* __restrict__ atom_y,
                             const float4* __restrict__ atom_xh, const float4* __restrict__ atom_xl,
                             float4* __restrict__ bin_y, int2* __restrict__ bin_je) {
   gmp_let_next_start();
@@ -395,7 +395,7 @@ __device__ __forceinline__ void center_place(const GmpStruct& st, const GmpGrid&
 
 // Per atom: its bin, its place in the bin grid and its wrapped FP32 position
 // (so that the neighbor kernels need no FP64 set-up).
-__global__ void k_bin_assign(const GmpStruct* __restrict__ S, const GmpGrid* __restrict__ G,
+__global__ void k_bin_assign(const GmpStruct* S, const GmpGrid* G,
                              const int32_t* __restrict__ struct_of, int64_t N,
                              const GmpD4* __restrict__ atom_u, int32_t* __restrict__ atom_bin,
                              int32_t* __restrict__ bin_count, float4* __restrict__ atom_t,
@@ -416,7 +416,7 @@ __global__ void k_bin_assign(const GmpStruct* __restrict__ S, const GmpGrid* __r
 
 // Per reference point: the checks, wrap and double-float split of
 // k_prepare and the place of k_bin_assign, in the structure's atom grid.
-__global__ void k_point_prepare(const GmpStruct* __restrict__ S, const GmpGrid* __restrict__ G,
+__global__ void k_point_prepare(const GmpStruct* S, const GmpGrid* G,
                                 const int32_t* __restrict__ point_struct, int64_t n, const double* __restrict__ pts,
                                 const double* __restrict__ atom_pos, float4* __restrict__ pt_xh,
                                 float4* __restrict__ pt_xl, float4* __restrict__ pt_t, float4* __restrict__ pt_y,
@@ -639,7 +639,7 @@ __global__ void k_scan_block(const T* __restrict__ in, T* __restrict__ out, T* _
 }
 
 template <typename T>
-__global__ void k_scan_add(T* __restrict__ out, const T* __restrict__ offs, int64_t n) {
+__global__ void k_scan_add(T* out, const T* offs, int64_t n) {
   gmp_let_next_start();
   const unsigned tid = gmp_after_predecessor(threadIdx.x);
   const int64_t i = (int64_t)blockIdx.x * 1024 + tid;
@@ -788,7 +788,7 @@ __host__ __device__ inline size_t fill_warp_bytes(int max_keys, int n_el) {
 // deterministic); FILL = 2: sorted by (neighbor atom, image).
 constexpr float kSlack = 1e-3f;
 template <int FILL>
-__global__ void __launch_bounds__(128, 8) k_neighbors(const GmpStruct* __restrict__ S, const GmpGrid* __restrict__ G,
+__global__ void __launch_bounds__(128, 8) k_neighbors(const GmpStruct* S, const GmpGrid* G,
                             const GmpCenters C, int64_t N, float cutoff,
                             float rc2hi, float rc2lo, double rc2, const double* __restrict__ pos,
                             const float4* __restrict__ atom_xh, const float4* __restrict__ atom_xl,

@@ -587,7 +587,7 @@ gmp_status neighbor_lists(gmp_ctx* h, const GmpCenters& C, int64_t NC, const dou
     const int64_t cap = (int64_t)(last.per_center * 1.125 * (double)NC) + 4096;
     int keys = 32;
     while (keys < last.max_m + last.max_m / 8 + 8) keys <<= 1;
-    if ((size_t)keys * 8 <= 200 * 1024 && room_for_guess(h, sizeof(GmpPair) * cap)) {
+    if (gmp_neighbor_keys_fit(sorted ? 2 : 1, keys, h->n_el) && room_for_guess(h, sizeof(GmpPair) * cap)) {
       GMP_CK(h->nbr_rng.ensure(sizeof(int64_t) * 2 * NC), "nbr_rng");
       GMP_CK(gmp_launch_neighbor_pass(sorted ? 2 : 1, h->structs.as<GmpStruct>(), h->grid.as<GmpGrid>(), C, NC, h->cutoff, pos,
                                       h->atom_xh.as<float4>(), h->atom_xl.as<float4>(), h->bin_start.as<int32_t>(),
@@ -654,8 +654,8 @@ gmp_status neighbor_lists(gmp_ctx* h, const GmpCenters& C, int64_t NC, const dou
   h->cap_cur = h->P;
   int keys = 32;
   while (keys < maxm) keys <<= 1;
-  if ((size_t)keys * 8 > 200 * 1024)
-    return fail(h, GMP_ERR_CAPACITY, "a center has " + std::to_string(maxm) + " neighbor images (limit 25600)");
+  if (!gmp_neighbor_keys_fit(sorted ? 2 : 1, keys, h->n_el))
+    return fail(h, GMP_ERR_CAPACITY, "a center has " + std::to_string(maxm) + " neighbor images (limit 16384)");
   // (ensure's slack and these 4,096 hold what the next batch of this kind guesses)
   GMP_CK(h->pairs.ensure(sizeof(GmpPair) * (h->P + 4096)), "pairs");
   GMP_CK(gmp_launch_neighbor_pass(sorted ? 2 : 1, h->structs.as<GmpStruct>(), h->grid.as<GmpGrid>(), C, NC,
@@ -870,7 +870,7 @@ gmp_status capture_graph(gmp_ctx* h, const std::vector<uintptr_t>& key, cudaStre
   h->cap_pairs = h->P + h->P / 8 + 4096;
   int keys = 32;
   while (keys < h->max_m + h->max_m / 8 + 8) keys <<= 1;
-  if ((size_t)keys * 8 > 200 * 1024) return GMP_OK;  // too large for a fixed capacity: stay eager
+  if (!gmp_neighbor_keys_fit(1, keys, h->n_el)) return GMP_OK;  // too large for a fixed capacity: stay eager
   h->cap_keys = keys;
   // every buffer the captured sequence uses exists before the capture
   GMP_CK(h->pairs.ensure(sizeof(GmpPair) * h->cap_pairs), "pairs");

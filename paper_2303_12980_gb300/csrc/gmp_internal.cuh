@@ -481,6 +481,9 @@ cudaError_t gmp_launch_neighbor_pass(int fill, const GmpStruct* d_structs, const
                                      GmpPair* pairs, int64_t pair_cap, int max_keys, int32_t* d_maxm,
                                      uint32_t* d_err, cudaStream_t stream, int sm_count, int64_t* launches,
                                      unsigned long long* cursor = nullptr, int64_t* rng = nullptr);
+// Whether the fill pass has the shared memory for lists of max_keys (a power of
+// two; 16,384 is the most).
+bool gmp_neighbor_keys_fit(int fill, int max_keys, int n_el);
 // What the host reads of a single-pass build: error word and longest list,
 // pairs, then the number of the build, written last.  The first compute
 // kernel behind the build writes it (KParams::report), to pinned host memory.

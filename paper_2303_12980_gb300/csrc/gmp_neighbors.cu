@@ -755,12 +755,13 @@ __device__ __forceinline__ bool out_of_range(const int* n) {
   return abs(n[0]) >= 512 || abs(n[1]) >= 512 || abs(n[2]) >= 512;
 }
 
-// Per-warp shared memory: 32 bin segments (float4 + int); in the fill
-// passes also keys [max_keys] u64, species and rank of each key
-// [max_keys] u32 (FILL 1), per-species counters [n_el] int.
+// Per-warp shared memory: 32 bin segments (float4 + int); in the fill passes also
+// keys [max_keys] u64, and to group them by species (FILL 1) species and rank of
+// each key [max_keys] u32, per-species counters [n_el] int.
 constexpr size_t kSegBytes = 32 * (sizeof(float4) + sizeof(int));
-__host__ __device__ inline size_t fill_warp_bytes(int max_keys, int n_el) {
-  return kSegBytes + ((size_t)max_keys * 12 + (size_t)n_el * 4 + 15) / 16 * 16;
+__host__ __device__ inline size_t warp_bytes(int fill, int max_keys, int n_el) {
+  if (fill == 0) return kSegBytes;
+  return kSegBytes + ((size_t)max_keys * (fill == 1 ? 12 : 8) + (fill == 1 ? (size_t)n_el * 4 : 0) + 15) / 16 * 16;
 }
 
 // Warp per center.  The center's cutoff sphere is covered by segments: the
@@ -806,7 +807,7 @@ __global__ void __launch_bounds__(128, 8) k_neighbors(const GmpStruct* S, const 
   const int wib = tid >> 5;
   const int64_t i = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib;
   if (i >= N) return;
-  unsigned char* wbase = sh_fill + (size_t)wib * (fill ? fill_warp_bytes(max_keys, n_el) : kSegBytes);
+  unsigned char* wbase = sh_fill + (size_t)wib * warp_bytes(fill, max_keys, n_el);
   float4* seg_sh = reinterpret_cast<float4*>(wbase);          // image shift of the segment, slot of candidate 0
   int* seg_m = reinterpret_cast<int*>(seg_sh + 32);           // packed image (m0, m1, m2)
   const unsigned below = (1u << lane) - 1u;
@@ -1261,6 +1262,8 @@ cudaError_t gmp_launch_point_prepare(const GmpStruct* d_structs, const GmpGrid* 
   return cudaGetLastError();
 }
 
+bool gmp_neighbor_keys_fit(int fill, int max_keys, int n_el) { return warp_bytes(fill, max_keys, n_el) <= 227 * 1024; }
+
 cudaError_t gmp_launch_neighbor_pass(int fill, const GmpStruct* d_structs, const GmpGrid* d_grid,
                                      const GmpCenters& C, int64_t N, double cutoff,
                                      const double* pos, const float4* atom_xh, const float4* atom_xl,
@@ -1276,10 +1279,9 @@ cudaError_t gmp_launch_neighbor_pass(int fill, const GmpStruct* d_structs, const
   auto fn = fill == 0 ? k_neighbors<0> : fill == 1 ? k_neighbors<1> : k_neighbors<2>;
   // few centers: one warp per CTA, so that they spread over the SMs
   int warps = N >= 16 * (int64_t)sm_count ? 4 : 1;
-  size_t smem = warps * kSegBytes;
+  while (warps > 1 && (size_t)warps * warp_bytes(fill, max_keys, n_el) > 96 * 1024) warps >>= 1;
+  const size_t smem = (size_t)warps * warp_bytes(fill, max_keys, n_el);
   if (fill) {
-    while (warps > 1 && (size_t)warps * fill_warp_bytes(max_keys, n_el) > 96 * 1024) warps >>= 1;
-    smem = (size_t)warps * fill_warp_bytes(max_keys, n_el);
     if (smem > 48 * 1024) {
       cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       if (e != cudaSuccess) return e;

@@ -99,3 +99,26 @@ def test_query_of_the_rows(torch):
         lo, hi = int(first[1][b]), int(first[1][e])
         assert torch.equal(got[0], first[0][b:e]) and torch.equal(got[1], first[1][b:e + 1] - lo)
         assert torch.equal(got[2], first[2][lo:hi]) and torch.equal(got[3], first[3][lo:hi])
+
+
+@pytest.mark.parametrize("n_el", [1, 9000])
+@pytest.mark.parametrize("rc", [12.8, 15.5, 15.9])  # 8,733, 15,515 and 16,831 images
+def test_longest_list(torch, n_el, rc):
+    """One atom in a cell of 1 A: lists of its images up to 16,384, the limit that the
+    error names, whatever the number of elements."""
+    from paper_2303_12980_gb300.binding import GMPError, GMPFeaturizer
+    F = GMPFeaturizer([0], [0.5], rc, *synth.gaussian_table(np.random.default_rng(1), [3] * n_el, 1))
+    a = (torch.zeros((1, 3), dtype=torch.float64, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda"), [0, 1],
+         np.eye(3)[None], [[1, 1, 1]])
+    k = np.arange(-16, 17)
+    x = np.stack(np.meshgrid(k, k, k, indexing="ij"), -1).reshape(-1, 3)
+    x = x[(x * x).sum(1) < rc * rc]
+    for _ in range(2):
+        if len(x) > 16384:
+            with pytest.raises(GMPError, match=f"{len(x)} neighbor images .limit 16384."):
+                F.neighbors(*a)
+            continue
+        off, j, s = F.neighbors(*a)
+        assert off.tolist() == [0, len(x)] and np.array_equal(s.cpu().numpy(), x) and not j.any()
+        if n_el == 1:
+            assert np.isfinite(F.featurize(*a).cpu().numpy()).all()

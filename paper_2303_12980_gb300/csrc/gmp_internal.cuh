@@ -211,12 +211,6 @@ __device__ __forceinline__ gmp_f2 gmp_df_mul_fu(gmp_f2 a, float b) {
   const gmp_f2 p = gmp_two_prod(a.hi, b);
   return {p.hi, __fmaf_rn(a.lo, b, p.lo)};
 }
-// Double-float times a float.
-__device__ __forceinline__ gmp_f2 gmp_df_mul_f(gmp_f2 a, float b) {
-  gmp_f2 p = gmp_two_prod(a.hi, b);
-  float e = __fmaf_rn(a.lo, b, p.lo);
-  return gmp_fast_two_sum(p.hi, e);
-}
 // Addition with one renormalisation: the low words are added in FP32, an
 // error of 2^-48 of the larger operand (not of a cancelling result).  For
 // sums whose accuracy counts against the size of their terms.

@@ -380,9 +380,8 @@ __device__ __forceinline__ void radial4d2(const float* __restrict__ tab_e, int k
     for (int l = 0; l < NL; ++l) R[p][l] = make_float4(Rp[p][0][l].x, Rp[p][0][l].y, Rp[p][1][l].x, Rp[p][1][l].y);
 }
 
-// Radial factors scaled by 2^32 for the backward, with scalar FP32
-// operations (the backward kernel keeps its 168-register budget with these;
-// packed pairs need aligned register pairs and spill there).  The exponent
+// Radial factors scaled by 2^32 for the backward, on packed FP32 pairs, sigmas
+// (0,1) and (2,3) of the group.  The exponent
 // argument 32 - B r^2 is one FMA, rounded once: an absolute error of at most
 // 2^-18 while the scaled factor is normal (|32 - B r^2| < 128), so each
 // exponential is within ~2e-6 relative: ample for derivatives, checked to
@@ -391,29 +390,34 @@ __device__ __forceinline__ void radial4d2(const float* __restrict__ tab_e, int k
 // of the higher orders: a gradient term of a far pair, multiplied by large
 // adjoints, keeps its digits; the kernel scales its sums back by 2^-32.
 template <int L, int NL = L + 2, bool PADG = true>
-__device__ __forceinline__ void radial4s(const float* __restrict__ tab_e, int kmax, int sg, float r2h,
+__device__ __forceinline__ void radial4p(const float* __restrict__ tab_e, int kmax, int sg, float r2h,
                                          float (&R)[4][NL]) {
   constexpr int RB = gmp_rad_block(L);
+  float2 Rp[2][NL];
 #pragma unroll
-  for (int u = 0; u < 4; ++u)
+  for (int h = 0; h < 2; ++h)
 #pragma unroll
-    for (int l = 0; l < NL; ++l) R[u][l] = 0.0f;
+    for (int l = 0; l < NL; ++l) Rp[h][l] = make_float2(0.0f, 0.0f);
+  const float2 nr2 = make_float2(-r2h, -r2h), sh = make_float2(GMP_EXP_SHIFT, GMP_EXP_SHIFT);
 #pragma unroll 1
   for (int q = 0; q < kmax; ++q) {
     const float4* blk = reinterpret_cast<const float4*>(tab_e) + sg * rad_sg_stride(L, kmax, PADG) + q * RB;
     const float4 bh = blk[0];
-    float E[4];
-    E[0] = gmp_ex2(__fmaf_rn(bh.x, -r2h, GMP_EXP_SHIFT));
-    E[1] = gmp_ex2(__fmaf_rn(bh.y, -r2h, GMP_EXP_SHIFT));
-    E[2] = gmp_ex2(__fmaf_rn(bh.z, -r2h, GMP_EXP_SHIFT));
-    E[3] = gmp_ex2(__fmaf_rn(bh.w, -r2h, GMP_EXP_SHIFT));
+    const float2 x0 = gmp_fma2(make_float2(bh.x, bh.y), nr2, sh), x1 = gmp_fma2(make_float2(bh.z, bh.w), nr2, sh);
+    const float2 E0 = make_float2(gmp_ex2(x0.x), gmp_ex2(x0.y)), E1 = make_float2(gmp_ex2(x1.x), gmp_ex2(x1.y));
 #pragma unroll
     for (int l = 0; l < NL; ++l) {
       const float4 a = blk[2 + l];
-      const float av[4] = {a.x, a.y, a.z, a.w};
-#pragma unroll
-      for (int u = 0; u < 4; ++u) R[u][l] = __fmaf_rn(av[u], E[u], R[u][l]);
+      Rp[0][l] = gmp_fma2(make_float2(a.x, a.y), E0, Rp[0][l]);
+      Rp[1][l] = gmp_fma2(make_float2(a.z, a.w), E1, Rp[1][l]);
     }
+  }
+#pragma unroll
+  for (int l = 0; l < NL; ++l) {
+    R[0][l] = Rp[0][l].x;
+    R[1][l] = Rp[0][l].y;
+    R[2][l] = Rp[1][l].x;
+    R[3][l] = Rp[1][l].y;
   }
 }
 
@@ -447,41 +451,6 @@ __device__ __forceinline__ void radial4x(const float* __restrict__ tab_e, int km
 #pragma unroll
       for (int u = 0; u < 4; ++u) R[u][l] = __fmaf_rn(av[u], E[u], R[u][l]);
     }
-  }
-}
-
-// The scaled radial factors of radial4s on packed FP32 pairs, sigmas (0,1)
-// and (2,3) of the group: bit-identical to the scalar form, half the issue
-// slots.
-template <int L, int NL = L + 2, bool PADG = true>
-__device__ __forceinline__ void radial4p(const float* __restrict__ tab_e, int kmax, int sg, float r2h,
-                                         float (&R)[4][NL]) {
-  constexpr int RB = gmp_rad_block(L);
-  float2 Rp[2][NL];
-#pragma unroll
-  for (int h = 0; h < 2; ++h)
-#pragma unroll
-    for (int l = 0; l < NL; ++l) Rp[h][l] = make_float2(0.0f, 0.0f);
-  const float2 nr2 = make_float2(-r2h, -r2h), sh = make_float2(GMP_EXP_SHIFT, GMP_EXP_SHIFT);
-#pragma unroll 1
-  for (int q = 0; q < kmax; ++q) {
-    const float4* blk = reinterpret_cast<const float4*>(tab_e) + sg * rad_sg_stride(L, kmax, PADG) + q * RB;
-    const float4 bh = blk[0];
-    const float2 x0 = gmp_fma2(make_float2(bh.x, bh.y), nr2, sh), x1 = gmp_fma2(make_float2(bh.z, bh.w), nr2, sh);
-    const float2 E0 = make_float2(gmp_ex2(x0.x), gmp_ex2(x0.y)), E1 = make_float2(gmp_ex2(x1.x), gmp_ex2(x1.y));
-#pragma unroll
-    for (int l = 0; l < NL; ++l) {
-      const float4 a = blk[2 + l];
-      Rp[0][l] = gmp_fma2(make_float2(a.x, a.y), E0, Rp[0][l]);
-      Rp[1][l] = gmp_fma2(make_float2(a.z, a.w), E1, Rp[1][l]);
-    }
-  }
-#pragma unroll
-  for (int l = 0; l < NL; ++l) {
-    R[0][l] = Rp[0][l].x;
-    R[1][l] = Rp[0][l].y;
-    R[2][l] = Rp[1][l].x;
-    R[3][l] = Rp[1][l].y;
   }
 }
 
@@ -1113,9 +1082,8 @@ __device__ __forceinline__ void shift_contract_order(const float* lam, const flo
 //   A = sum_k lamd_k S_k, B = sum_k (2l_k+1) lam_k S_k, V = sum_k lam_k S_{k+e},
 // from which grad = d (2 A + B / r^2) - V / r^2 (r^2 > 0).  At d = 0 only order
 // 1 has a gradient: g1 = (lam_x, lam_y, lam_z).
-// PACKED: radial factors on packed FP32 pairs (same results, fewer issue
-// slots); MIXED: exact exponentials (coefficients of both signs).
-template <int L, int NS, bool PACKED, bool PADG, bool MIXED>
+// MIXED: exact exponentials (coefficients of both signs).
+template <int L, int NS, bool PADG, bool MIXED>
 __device__ __forceinline__ void pair_adjoint(const GmpPass& P, const float* __restrict__ tab_e,
                                               const float* __restrict__ Lam, float dx, float dy, float dz, float r2h,
                                               float r2l, float r2c, float& A, float& B, float (&V)[3], float (&g1)[3]) {
@@ -1134,10 +1102,8 @@ __device__ __forceinline__ void pair_adjoint(const GmpPass& P, const float* __re
     float R[4][NL];  // orders 0 .. L + 1
     if constexpr (MIXED)
       radial4x<L, NL, PADG>(tab_e, P.kmax, sg, r2h, r2l, R);
-    else if constexpr (PACKED)
-      radial4p<L, NL, PADG>(tab_e, P.kmax, sg, r2h, R);
     else
-      radial4s<L, NL, PADG>(tab_e, P.kmax, sg, r2h, R);
+      radial4p<L, NL, PADG>(tab_e, P.kmax, sg, r2h, R);
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const float nb = P.nbeta[4 * sg + u];
@@ -1189,7 +1155,7 @@ __device__ __forceinline__ void pair_adjoint(const GmpPass& P, const float* __re
 // exponentials: 6.95 against 6.80 ms on the 262,144-atom slab; with the strain
 // sums 1661 against 1673 us on 32,768 atoms, but the strain derivative came out
 // 3% further off.
-template <int L, bool VIRIAL>
+template <int L>
 constexpr int back_threads() { return L <= 4 ? 640 : L == 5 ? 512 : 384; }
 // the radial table's sigma groups padded, but for the kernel whose 168
 // registers the padded stride would exceed
@@ -1203,7 +1169,7 @@ constexpr bool back_pad() { return VIRIAL || L < 6; }
 // (positions and lattice vectors strained alike move every d to (I+eps) d),
 // each lane's partial sums kept in its column of Wv ([9][32] floats of
 // warp-private shared memory) rather than in registers.
-template <int L, int NS, bool VIRIAL = false, bool PACKED = false, bool PADG = true, bool MIXED = false>
+template <int L, int NS, bool VIRIAL = false, bool PADG = true, bool MIXED = false>
 __device__ __forceinline__ void backward_sweep(const KParams& K, const float* __restrict__ s_rad,
                                                const float* __restrict__ s_dens, int64_t i, int64_t p0, int M,
                                                const float* __restrict__ Lam, float gd, float* Wv = nullptr) {
@@ -1222,7 +1188,7 @@ __device__ __forceinline__ void backward_sweep(const KParams& K, const float* __
     const float r2c = mcsh_r2(dx, dy, dz);
     const float* tab_e = s_rad + (size_t)e * rad_elem_stride(L, NS, P.kmax, PADG);
     float A = 0.0f, B = 0.0f, V[3] = {0.0f, 0.0f, 0.0f}, g1[3] = {0.0f, 0.0f, 0.0f};
-    pair_adjoint<L, NS, PACKED, PADG, MIXED>(P, tab_e, Lam, dx, dy, dz, r2h, r2l, r2c, A, B, V, g1);
+    pair_adjoint<L, NS, PADG, MIXED>(P, tab_e, Lam, dx, dy, dz, r2h, r2l, r2c, A, B, V, g1);
     float g[3];
     if (r2c > 0.0f) {
       const float inv = 1.0f / r2c;
@@ -1313,13 +1279,13 @@ __global__ void __launch_bounds__(256) k_vjp(KParams K) {
     if (K.features) write_features<L, NS>(K, i, Mu, rho);
     adjoints<L, NS>(P, Mu, grow, Lam);
     const float gd = P.want_density ? grow[P.dens_col] : 0.0f;
-    backward_sweep<L, NS, false, true>(K, s_rad, s_dens, i, p0, M, Lam, gd);
+    backward_sweep<L, NS>(K, s_rad, s_dens, i, p0, M, Lam, gd);
     __syncwarp();
   }
 }
 
 template <int L, int NS, bool VIRIAL = false, bool MIXED = false>
-__global__ void __launch_bounds__(back_threads<L, VIRIAL>()) k_backward(KParams K) {
+__global__ void __launch_bounds__(back_threads<L>()) k_backward(KParams K) {
   using SH = Shape<L, NS>;
   extern __shared__ __align__(16) float smem[];
   const GmpPass& P = K.pass;
@@ -1344,7 +1310,7 @@ __global__ void __launch_bounds__(back_threads<L, VIRIAL>()) k_backward(KParams 
     const float* grow = K.grad_feat + i * P.F;
     adjoints<L, NS>(P, Mu, grow, Lam);
     const float gd = P.want_density ? grow[P.dens_col] : 0.0f;
-    backward_sweep<L, NS, VIRIAL, !MIXED, PADG, MIXED>(K, s_rad, s_dens, i, p0, M, Lam, gd, Wv);
+    backward_sweep<L, NS, VIRIAL, PADG, MIXED>(K, s_rad, s_dens, i, p0, M, Lam, gd, Wv);
     __syncwarp();
   }
 }

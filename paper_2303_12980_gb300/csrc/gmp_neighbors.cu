@@ -717,11 +717,6 @@ cudaError_t exclusive_scan(const T* in, T* out, int64_t n, void* tmp, cudaStream
 }
 
 // ----------------------------------------------------------- neighbor pass
-struct Cand {
-  bool ok;
-  int n[3];
-};
-
 // The FP64 expression of the neighbor definition, evaluated exactly as written.
 __device__ __noinline__ bool fp64_within(const double* __restrict__ pos, const double* __restrict__ xi,
                                          int64_t j, const GmpStruct& st, const int* n, double rc2) {
@@ -1223,8 +1218,8 @@ cudaError_t gmp_launch_bins(const GmpStruct* d_structs, const GmpGrid* d_grid,
 }
 
 bool gmp_bin_structs_fits(int64_t N, int max_atoms, int max_bins) {
-  if (max_atoms > 256 && (max_atoms > 512 || N < 16 * (int64_t)max_atoms)) return false;
-  return struct_bins_smem(max_atoms, max_bins) <= 200 * 1024;
+  // (at most 2 bins an atom and 8: 26 KB of shared memory at 512 atoms)
+  return max_bins <= 2 * max_atoms + 8 && (max_atoms <= 256 || (max_atoms <= 512 && N >= 16 * (int64_t)max_atoms));
 }
 
 cudaError_t gmp_launch_bin_structs(GmpStruct* d_structs, int n_struct, int64_t N, int max_atoms, int max_bins,
@@ -1234,10 +1229,6 @@ cudaError_t gmp_launch_bin_structs(GmpStruct* d_structs, int n_struct, int64_t N
                                    int n_clear, cudaStream_t stream, int sm_count, int64_t* launches) {
   if (!gmp_bin_structs_fits(N, max_atoms, max_bins)) return cudaErrorInvalidValue;
   const size_t smem = struct_bins_smem(max_atoms, max_bins);
-  if (smem > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(k_bin_structs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
   // as many threads as atoms: fewer warps to wait for at each step; with more
   // structures than SMs small CTAs, which leave room for one another
   const int most = n_struct > sm_count ? 128 : 1024;

@@ -495,11 +495,12 @@ gmp_status finish_lists(gmp_ctx* h, cudaStream_t st) {
   if (h->lists_report) {
     // the first compute kernel writes it when it starts; the stream's state is
     // looked at now and then, so that a kernel that never comes is noticed, and
-    // other threads get the core meanwhile
+    // other threads get the core where the process asked for that, or after
+    // a long wait (a millisecond or so)
     volatile GmpListReport* r = h->report;
     for (uint32_t n = 1; r->build != h->build; ++n) {
       if (n % (h->wait_yields ? 64 : 4096) != 0) continue;
-      std::this_thread::yield();
+      if (h->wait_yields || n >= 1u << 20) std::this_thread::yield();
       const cudaError_t e = cudaStreamQuery(st);
       if (e == cudaErrorNotReady) continue;
       if (e != cudaSuccess) return cuda_fail(h, e, "neighbor wait");

@@ -150,6 +150,8 @@ gmp_status gmp_featurize_vjp_virial(gmp_handle h, int32_t n_struct, const int64_
  *   jac [cap, F, 3] float32 = d features[i, :] / d pos[j, :].
  * If the total nnz exceeds `cap`, nothing but *nnz_out is written and
  * GMP_ERR_CAPACITY is returned; call again with cap >= *nnz_out.
+ * (A cap below the number of centers, each of which has a row, asks for
+ * *nnz_out only: no features are computed for it.)
  * nnz_out is a host pointer; this call synchronises `stream`. */
 gmp_status gmp_featurize_grad(gmp_handle h, int32_t n_struct, const int64_t *atom_off,
                                   const double *pos, const double *cell, const uint8_t *pbc,

@@ -88,7 +88,7 @@ cudaError_t launch(int kind, const KParams& K, GmpShape shape, GmpLaunchPlan* pl
       // untuned: the CTA size with the most resident warps, of equals the
       // smallest with at least 4 (registers and the tables' share of the
       // shared memory decide: the forward kernel at orders 0-4 x 8 sigmas keeps
-      // 24 warps in 4-warp CTAs and 16 in one of 16, 3.40 against 4.03 ms on
+      // 28 warps in CTAs of 7 and 16 in one of 16, 3.40 against 4.03 ms on
       // 10,000 structures; 4096 Jacobian centers took 177 us in 12-warp CTAs
       // and 167 in as many warps of 4-warp ones)
       int best_w = warps, best_res = 0;

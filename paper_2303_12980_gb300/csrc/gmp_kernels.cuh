@@ -1147,11 +1147,13 @@ __device__ __forceinline__ void pair_adjoint(const GmpPass& P, const float* __re
   });
 }
 
-// The backward kernels' time follows their resident warps as long as the
-// sums and MCSH values of a pair stay in registers.  Orders 0-4 do in 96
-// registers, 20 warps per SM (10,000 structures, orders 0-4 x 8 sigmas, GB300:
-// 5.76 ms at 12 warps, 4.80 at 16, 4.67 at 20), orders 0-5 in 128, orders 0-6
-// in 168 (12 warps).  Orders 0-6 in two ranges at 128 registers repeat the
+// The backward kernels' time follows their resident warps as long as most of
+// the sums and MCSH values of a pair stay in registers.  Orders 0-4 do in 96
+// registers, 20 warps per SM (20-80 bytes spilled; 10,000 structures, orders 0-4 x 8
+// sigmas, GB300: 5.76 ms at 12 warps, 4.80 at 16, 4.67 at 20), orders 0-5 in 128,
+// orders 0-6 in 168 (12 warps; up to 76 bytes spilled since the packed radial
+// factors and the 64-bit center index, which a 32-bit one would spare).
+// Orders 0-6 in two ranges at 128 registers repeat the
 // exponentials: 6.95 against 6.80 ms on the 262,144-atom slab; with the strain
 // sums 1661 against 1673 us on 32,768 atoms, but the strain derivative came out
 // 3% further off.

@@ -772,8 +772,8 @@ __host__ __device__ inline size_t warp_bytes(int fill, int max_keys, int n_el) {
 // candidate, and consecutive lanes read consecutive slots.
 // An accepted candidate is kept as (slot, image) and completed afterwards,
 // with all lanes busy; a row costs two bin offsets instead of two per bin.
-// Bound by instruction issue (64%) and the loads' latency; 64 registers, 32
-// resident warps per SM (a few words spilled; 80 registers and 24 warps:
+// Bound by instruction issue (60-65%) and the loads' latency; 64 registers, 32
+// resident warps per SM (14 words spilled; 80 registers and 24 warps:
 // 147 us on the slab of 32,768 atoms, 130 at 64).  Neighbor stage of 2,500 small
 // structures / of the alloy slab of 262,144 atoms (GB300): 946 / 1774 us with
 // one bin per lane, its slots in turn; 562 / 1004 with groups of 8 lanes walking

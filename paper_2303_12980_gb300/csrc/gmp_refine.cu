@@ -163,12 +163,12 @@ __device__ __forceinline__ void refine_order(int lane, const GmpRefine& A, const
 // what a warp mostly waits for at orders 4-6).  One launch for all orders:
 // a typical batch flags a few thousand features per order, one round of
 // warps each, and a launch per order paid that round's latency five times.
-// Measured on a GB300 with the solid harmonics and the cheaper exponential
-// (before: one launch per order, raising recurrences): perfect FCC crystal of
-// 32,768 atoms, orders 0-6 x 16 sigmas, 2565 -> 717 us; 4,096-atom alloy
-// crystal, orders 0-4 x 8 sigmas, 82 -> 27 us; alloy slab of 262,144 atoms
-// 482 -> 135 us.  Outputs bit for bit the same.  Bound by the FP32 pipe's
-// dependent double-float chains at 16 warps per SM (128 registers).
+// Measured on a GB300 with the solid harmonics, the cheaper exponential and sums
+// left unnormalised (before: one launch per order, raising recurrences): perfect
+// FCC crystal of 32,768 atoms, orders 0-6 x 16 sigmas, 2565 -> 589 us; 4,096-atom
+// alloy crystal, orders 0-4 x 8 sigmas, 82 -> 24 us; alloy slab of 262,144 atoms
+// 482 -> 104 us.  Bound by the double-float instructions themselves (issue 77%) at
+// 16 warps per SM (128 registers).
 __global__ void __launch_bounds__(256, 2) k_refine(const GmpRefine A) {
   __shared__ float2 exp_tab[64];
   if (threadIdx.x < 64) exp_tab[threadIdx.x] = A.exp_tab[threadIdx.x];

@@ -528,11 +528,13 @@ gmp_status finish_lists(gmp_ctx* h, cudaStream_t st) {
 }
 
 // The end of a call's device sequence: one that failed takes along what its
-// lists flagged and nobody read.
+// lists flagged and nobody read, and leaves nothing in flight (its kernels and
+// copies write the handle's pinned memory).
 gmp_status settle(gmp_ctx* h, cudaStream_t st, gmp_status r) {
   if (r != GMP_OK) {
     h->lists_pending = false;
     cudaMemsetAsync(h->scalars.p, 0, 4, st);  // (r is the error to report)
+    cudaStreamSynchronize(st);
   }
   return r;
 }
@@ -1879,6 +1881,7 @@ gmp_status gmp_profile_read(gmp_handle h, double* ms, int64_t* count, int n_stag
 void gmp_destroy(gmp_handle h) {
   if (!h) return;
   cudaSetDevice(h->device);
+  if (h->ev_desc) cudaEventSynchronize(h->ev_desc);  // (an upload whose call waited for nothing)
   for (auto& pd : h->passes) pd.rad.release();
   if (h->graph_exec) cudaGraphExecDestroy(h->graph_exec);
   if (h->h_small) cudaFreeHost(h->h_small);

@@ -65,3 +65,30 @@ def test_description_uploaded_on_another_stream(torch, n):
     assert s1.query()
     s2.synchronize()
     assert torch.equal(got, want)
+
+
+def test_nothing_is_in_flight_after_a_failure(torch):
+    """A failed call returns when what it queued is done; a handle is destroyed only
+    when its last upload is."""
+    from paper_2303_12980_gb300.binding import GMPError, GMPFeaturizer
+    rng = np.random.default_rng(4)
+    pos, cell = synth.fcc_supercell(rng, 3.6, (3, 3, 3), 0.1)
+    n = len(pos)
+    a = (torch.from_numpy(pos).cuda(), torch.zeros(n, dtype=torch.int32, device="cuda"), [0, n], cell[None], [[1, 1, 1]])
+    F = GMPFeaturizer([0, 1], [0.4], 5.0, *synth.gaussian_table(rng, [3], 2))
+    F.featurize(*a)
+    torch.cuda.synchronize()
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        torch.cuda._sleep(100_000_000)
+    with pytest.raises(GMPError, match="species"):
+        F.featurize(a[0], a[1] + 7, *a[2:], stream=s)
+    assert s.query()
+    none = torch.empty((0, 3), dtype=torch.float64, device="cuda")
+    G = GMPFeaturizer([0, 1], [0.4], 5.0, *synth.gaussian_table(rng, [3], 2))
+    torch.cuda.synchronize()
+    with torch.cuda.stream(s):
+        torch.cuda._sleep(100_000_000)
+    G.featurize_points(*a, none, [0, 0], stream=s)
+    G.close()
+    assert s.query()
